@@ -76,7 +76,7 @@ __device__ __forceinline__ void normalise(const float *__restrict__ w, const flo
 }
 
 // B fragments of layer 2 (B[k][n] = W2[n][k]: a lane's registers are
-// consecutive pairs along a row of W2), from the float32 master weights...
+// consecutive pairs along a row of W2), from the float32 master weights
 struct W2FromGlobal {
     const float *w;
     __device__ __forceinline__ void operator()(int ks, int nt, int g, int t, uint32_t &b0,
@@ -88,28 +88,13 @@ struct W2FromGlobal {
         b1 = pack2(hi.x, hi.y);
     }
 };
-// ... or from a bf16 copy in shared memory, rows of `ld` bf16 (ld even):
-// s[n * ld + k] = bf16(W2[n][k]) (or any other matrix stored that way).
-struct BFromShared {
-    const uint32_t *s;
-    int ld;
-    __device__ __forceinline__ void operator()(int ks, int nt, int g, int t, uint32_t &b0,
-                                               uint32_t &b1) const {
-        const int base = (8 * nt + g) * ld + 16 * ks + 2 * t;
-        b0 = s[base >> 1];
-        b1 = s[(base + 8) >> 1];
-    }
-};
-
 // Layers 1 and 2 of one 16-row tile of a warp. fa, fb: normalised features of
 // rows g and g+8. Out: A = bf16(h1) as the A fragments of the four k-steps of
-// layer 2, acc = p2 = W2 h1 + b2 in C layout (n-tile nt: cols 8 nt + 2t, +1),
-// and with KEEP_D1 d1 = gelu'(p1) in C layout.
-template <bool KEEP_D1, class BLoad>
+// layer 2, acc = p2 = W2 h1 + b2 in C layout (n-tile nt: cols 8 nt + 2t, +1).
+template <class BLoad>
 __device__ __forceinline__ void layers12(const float *__restrict__ w, const BLoad &bload,
                                          const float (&fa)[4], const float (&fb)[4], int g, int t,
-                                         uint32_t (&A)[4][4], float (&acc)[8][4],
-                                         float (&d1)[8][4]) {
+                                         uint32_t (&A)[4][4], float (&acc)[8][4]) {
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
         float h[4];
@@ -121,13 +106,8 @@ __device__ __forceinline__ void layers12(const float *__restrict__ w, const BLoa
             const float bb = w[B1 + c];
             const float pa = fmaf(w3, fa[3], fmaf(w2, fa[2], fmaf(w1, fa[1], fmaf(w0, fa[0], bb))));
             const float pb = fmaf(w3, fb[3], fmaf(w2, fb[2], fmaf(w1, fb[1], fmaf(w0, fb[0], bb))));
-            float da, db;
-            h[e] = gelu(pa, da);
-            h[2 + e] = gelu(pb, db);
-            if (KEEP_D1) {
-                d1[nt][e] = da;
-                d1[nt][2 + e] = db;
-            }
+            h[e] = gelu(pa);
+            h[2 + e] = gelu(pb);
         }
         const int ks = nt >> 1, half = nt & 1;
         A[ks][2 * half] = pack2(h[0], h[1]);       // row g
@@ -189,8 +169,8 @@ __device__ __forceinline__ float warp_forward(const float *__restrict__ w, const
             fb[i] = __shfl_sync(0xffffffffu, fn[i], 16 * mt + g + 8);
         }
         uint32_t A[4][4];
-        float acc[8][4], d1[8][4];
-        layers12<false>(w, W2FromGlobal{w}, fa, fb, g, t, A, acc, d1);
+        float acc[8][4];
+        layers12(w, W2FromGlobal{w}, fa, fb, g, t, A, acc);
         float ya, yb;
         output(w, acc, t, ya, yb);
         // lane l owns row l & 15 of tile l >> 4, held by lane 4 (row & 7)
