@@ -393,24 +393,17 @@ __global__ void k_aos_from_soa(int64_t R, const double *soa, double *aos) {
     for (int c = 0; c < 3; ++c) aos[3 * r + c] = soa[c * R + r];
 }
 
-// Launch shape of the kick for this batch: enough CTAs to fill the GPU
-// several times, each CTA at least a tile of j rows per split.
+// Launch shape of the kick for this batch
 static KickTune default_tune(const std::vector<int64_t> &off, int prec) {
-    KickTune t;
-    t.threads = 128;
-    t.ipt = prec == QYM_KICK_MIXED ? 2 : 1;
-    int32_t nsys = (int32_t)off.size() - 1;
+    const int32_t nsys = (int32_t)off.size() - 1;
+    const int64_t ti = prec == QYM_KICK_MIXED ? 256 : 128;
     int64_t ib = 0, nbmax = 0;
     for (int32_t s = 0; s < nsys; ++s) {
-        int64_t nb = off[s + 1] - off[s] - 1;
-        ib += (nb + t.threads * t.ipt - 1) / (t.threads * t.ipt);
+        const int64_t nb = off[s + 1] - off[s] - 1;
+        ib += (nb + ti - 1) / ti;
         nbmax = std::max(nbmax, nb);
     }
-    int64_t want = 4 * 152;
-    int64_t sp = (want + ib - 1) / std::max<int64_t>(ib, 1);
-    int64_t maxsp = std::max<int64_t>(1, nbmax / 256);
-    t.splits = (int32_t)std::max<int64_t>(1, std::min(sp, maxsp));
-    return t;
+    return default_kick_tune(ib * ti, nbmax, prec);
 }
 
 static qym_status upload_state(qym_ctx *c, const double *q, const double *v) {

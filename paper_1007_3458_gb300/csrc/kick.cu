@@ -16,6 +16,9 @@
 // are folded every FOLD pairs into a float two-sum (hi, lo) accumulator that
 // is returned as a double. The FP32 arithmetic runs on Blackwell's packed
 // FP32x2 instructions, two j rows per instruction.
+#include <algorithm>
+
+#include "pair64.cuh"
 #include "qym_internal.cuh"
 
 namespace qym {
@@ -28,8 +31,9 @@ constexpr int FOLD = 64;
 constexpr int kPairUnroll = QYM_KICK_UNROLL;  // j pairs per unrolled step
 
 struct KickArgs {
-    const int4 *items;
+    const int4 *items;      // NULL: one system of `rows` rows, items by kick_item
     const int32_t *slots;
+    int32_t chunk = 0;      // j rows per split (items == NULL)
     const float4 *pos;      // (x_hi, y_hi, z_hi, G m)
     const float4 *lo;       // (x_lo, y_lo, z_lo, c = 2 rho^2 of the crude reach rho)
     const double *q;        // [3][rows] (FP64 path)
@@ -51,6 +55,20 @@ struct KickArgs {
     int32_t *blk_cnt = nullptr;  // arrivals per i-block (NULL: each slot stays for the finisher)
     int32_t splits = 1;          // items (slots) per i-block
 };
+
+// The item of CTA b: its rows [x, y), its j-range [z, w) and its slot; for one
+// system (items == NULL) i-blocks of `ti` rows times `splits` ranges of `chunk`
+__device__ __forceinline__ int4 kick_item(const KickArgs &a, int ti, int &slot) {
+    if (a.items) {
+        slot = a.slots[blockIdx.x];
+        return a.items[blockIdx.x];
+    }
+    const int64_t ib = blockIdx.x / a.splits;
+    slot = (int)(blockIdx.x - ib * a.splits);
+    const int64_t i0 = 1 + ib * ti, j0 = 1 + (int64_t)slot * a.chunk;
+    return make_int4((int)i0, (int)min(i0 + ti, a.rows), (int)min(j0, a.rows),
+                     (int)min(j0 + a.chunk, a.rows));
+}
 
 // The last CTA of an i-block to finish (arrivals counted per i-block, the
 // counter reset by that CTA for the next launch) adds the block's `splits`
@@ -287,8 +305,8 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
     __shared__ float4 s_fa[TILE / 2], s_fb[TILE / 2];
     const JPairs sp{s_a, s_b, s_c, s_d};
     const JFar sf{s_fa, s_fb, s_d};
-    const int4 it = a.items[blockIdx.x];
-    const int slot = a.slots[blockIdx.x];
+    int slot;
+    const int4 it = kick_item(a, IPT * (int)blockDim.x, slot);
     float rho[IPT];
     float2 nxh[IPT], nyh[IPT], nzh[IPT], nxl[IPT], nyl[IPT], nzl[IPT];  // -Q_i, duplicated
     int gi[IPT];
@@ -496,56 +514,112 @@ __global__ void __launch_bounds__(256) k_flag_chunks(KickArgs a, unsigned long l
 }
 
 // ---------------------------------------------------------------- FP64 form
+// G m_j / r^3 of a pair in FP64, where the float form does not hold
+__device__ __noinline__ double weight_fp64(double dx, double dy, double dz, double gm) {
+    const long long ux = __double_as_longlong(dx), uy = __double_as_longlong(dy);
+    const long long uz = __double_as_longlong(dz);
+    // a body and itself, or a massless partner: no FP64 instruction
+    if (((ux | uy | uz) << 1) == 0 || (__double_as_longlong(gm) << 1) == 0) return 0.0;
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double ri = rsqrt(r2);
+    const double s = gm * (ri * ri) * ri;
+    return (r2 > 0.0) ? s : 0.0;
+}
+
+// The FP64 kick. The separations, r^2 and G m / r^3 of a pair are formed to FP64
+// accuracy on the FP32 pipes (pair64.cuh); the FP64 pipe, one warp instruction
+// per ~19 cycles and SM, keeps the separation and the sum of a pair's
+// acceleration, six instructions where the plain form has 22. Rows and partners
+// are split into three floats once per CTA and tile, scaled by powers of two;
+// pairs outside the float range take weight_fp64.
 template <int IPT, bool FLAG, bool FORCE>
 __global__ void __launch_bounds__(256) k_kick_fp64(KickArgs a) {
     __shared__ D4 s_q[TILE];
+    __shared__ float4 s_h[TILE], s_m[TILE], s_l[TILE];  // (x, y, z, G m) in three parts
     __shared__ float s_rho[TILE];
-    const int4 it = a.items[blockIdx.x];
-    const int slot = a.slots[blockIdx.x];
+    __shared__ int s_hi[2][8];
+    int slot;
+    const int4 it = kick_item(a, IPT * (int)blockDim.x, slot);
     const int64_t rows = a.rows;
+    const double G = a.G;
     double xi[IPT], yi[IPT], zi[IPT], ax[IPT], ay[IPT], az[IPT];
     float rho[IPT];
     int gi[IPT];
+    int hl = 0, hw = 0;
 #pragma unroll
     for (int k = 0; k < IPT; ++k) {
-        int i = it.x + threadIdx.x + k * blockDim.x;
+        const int i = it.x + threadIdx.x + k * blockDim.x;
         gi[k] = i;
-        if (i < it.y) {
-            xi[k] = a.q[i]; yi[k] = a.q[rows + i]; zi[k] = a.q[2 * rows + i];
-            rho[k] = FLAG ? a.lo[i].w : 0.0f;
-        } else {
-            xi[k] = yi[k] = zi[k] = 1e18;
-            rho[k] = -1e30f;
-        }
+        const int r = min(i, it.y - 1);  // an idle lane repeats the last row
+        xi[k] = a.q[r]; yi[k] = a.q[rows + r]; zi[k] = a.q[2 * rows + r];
+        rho[k] = FLAG && i < it.y ? a.lo[i].w : -1e30f;
+        hl = max(hl, max(p64::hi_abs(xi[k]), max(p64::hi_abs(yi[k]), p64::hi_abs(zi[k]))));
         ax[k] = ay[k] = az[k] = 0.0;
     }
-    const double G = a.G;
+    if (it.z + (int)threadIdx.x < it.w) hw = p64::hi_abs(G * a.m[it.z + threadIdx.x]);
+    hl = __reduce_max_sync(0xffffffffu, hl);
+    hw = __reduce_max_sync(0xffffffffu, hw);
+    if ((threadIdx.x & 31) == 0) {
+        s_hi[0][threadIdx.x >> 5] = hl;
+        s_hi[1][threadIdx.x >> 5] = hw;
+    }
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        hl = max(hl, s_hi[0][w]);
+        hw = max(hw, s_hi[1][w]);
+    }
+    const p64::Scale sc(hl, hw);
+    const uint64_t bias = sc.bias(3);
+    // r^2 back to the caller's units for the encounter search
+    const bool r2_ok = sc.kb >= -60 && sc.kb <= 60;
+    const float r2u = r2_ok ? __int_as_float((127 + 2 * sc.kb) << 23) : 1.0f;
+    p64::F3 px[IPT], py[IPT], pz[IPT];
+#pragma unroll
+    for (int k = 0; k < IPT; ++k) {
+        px[k] = p64::split3(xi[k] * sc.len);
+        py[k] = p64::split3(yi[k] * sc.len);
+        pz[k] = p64::split3(zi[k] * sc.len);
+    }
     for (int jt = it.z; jt < it.w; jt += TILE) {
         const int n = min(TILE, it.w - jt);
         __syncthreads();
         for (int t = threadIdx.x; t < n; t += blockDim.x) {
-            int j = jt + t;
-            s_q[t] = D4{a.q[j], a.q[rows + j], a.q[2 * rows + j], G * a.m[j]};
+            const int j = jt + t;
+            const D4 p{a.q[j], a.q[rows + j], a.q[2 * rows + j], G * a.m[j]};
+            const p64::F3 x = p64::split3(p.x * sc.len), y = p64::split3(p.y * sc.len);
+            const p64::F3 z = p64::split3(p.z * sc.len), g = p64::split3(p.w * sc.wt);
+            s_q[t] = p;
+            s_h[t] = make_float4(x.h, y.h, z.h, g.h);
+            s_m[t] = make_float4(x.m, y.m, z.m, g.m);
+            s_l[t] = make_float4(x.l, y.l, z.l, g.l);
             if (FLAG) s_rho[t] = a.lo[j].w;
         }
         __syncthreads();
-#pragma unroll 2
+#pragma unroll 1
         for (int j = 0; j < n; ++j) {
             const D4 p = s_q[j];
+            const float4 H = s_h[j], M = s_m[j], L = s_l[j];
+            const bool g_ok = sc.ok && p64::g_fits(H.w);
 #pragma unroll
             for (int k = 0; k < IPT; ++k) {
-                double dx = xi[k] - p.x, dy = yi[k] - p.y, dz = zi[k] - p.z;
-                double r2 = dx * dx + dy * dy + dz * dz;
+                const p64::F3 r2 = p64::norm2(p64::diff(px[k], p64::F3{H.x, M.x, L.x}),
+                                              p64::diff(py[k], p64::F3{H.y, M.y, L.y}),
+                                              p64::diff(pz[k], p64::F3{H.z, M.z, L.z}));
+                const bool fits = p64::r2_fits(r2.h);
+                const double dx = xi[k] - p.x, dy = yi[k] - p.y, dz = zi[k] - p.z;
                 if (FORCE) {
-                    double ri = rsqrt(r2);
-                    double s = p.w * (ri * ri) * ri;
-                    s = (r2 > 0.0) ? s : 0.0;
+                    double s;
+                    if (!(p64::g_over_r3(p64::F3{H.w, M.w, L.w}, r2, rsqrt_ftz(r2.h), bias, s) &&
+                          fits && g_ok))
+                        s = weight_fp64(dx, dy, dz, p.w);
                     ax[k] -= s * dx;
                     ay[k] -= s * dy;
                     az[k] -= s * dz;
                 }
                 if (FLAG) {
-                    if ((float)r2 < rho[k] + s_rho[j]) {
+                    float r2f = __fadd_rn(r2.h, r2.m) * r2u;
+                    if (!(fits && r2_ok && sc.ok)) r2f = (float)(dx * dx + dy * dy + dz * dz);
+                    if (r2f < rho[k] + s_rho[j]) {
                         int gj = jt + j;
                         if (gi[k] < gj) push_candidate(a, gi[k], gj);
                     }
@@ -615,6 +689,26 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t, in
     }
     *nitems = n;
     *splits_used = t.splits;
+}
+
+// Default launch shape for i-blocks of nb bodies in all (nbmax in the largest
+// system). Mixed: about four CTAs per SM, at least a tile of j rows per split.
+// FP64: as many CTAs as fit the GPU at once (eight of 128 threads per SM),
+// since a pair takes some 300 issue slots: 10240 bodies on 80 i-blocks fill
+// the chip with 15 splits; small systems take splits of at least 16 rows (a
+// 260-body kick is one warp's walk over its j-range: 185 us in one range, a
+// plain FP64 form, 7 us in 16).
+KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec) {
+    KickTune t;
+    const bool mixed = prec == QYM_KICK_MIXED;
+    t.threads = 128;
+    t.ipt = mixed ? 2 : 1;
+    const int64_t ib = std::max<int64_t>(1, (iblocks_nb + t.threads * t.ipt - 1) / (t.threads * t.ipt));
+    const int64_t want = (mixed ? 4 : 8) * 152;
+    const int64_t sp = mixed ? (want + ib - 1) / ib : want / ib;
+    const int64_t maxsp = mixed ? (nbmax + 255) / 256 : nbmax / 16;
+    t.splits = (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min(sp, maxsp), 128));
+    return t;
 }
 
 template <bool FLAG, bool FORCE>
@@ -719,6 +813,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     a.tile = d.tile;
     a.blk_cnt = d.kick_cnt;
     a.splits = d.splits;
+    a.chunk = d.item_chunk;
     if (a.far_tiles) {
         const int64_t ntiles = (d.rows - 1 + TILE - 1) / TILE;
         k_tile_prep<<<(unsigned)ntiles, TILE, 0, st>>>(d.rows, d.pk_pos, d.pk_lo, d.far, d.tile);
@@ -748,8 +843,8 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
 // ---------------------------------------------------------------- single system
 // Workspace for qym_accel_dev: packs + items + partials for one system.
 struct SingleLayout {
-    size_t off_pos, off_lo, off_items, off_slots, off_apart, off_heavy, total;
-    int32_t nitems, splits;
+    size_t off_pos, off_lo, off_apart, off_heavy, total;
+    int32_t nitems, chunk;
     KickTune tune;
     bool sorted;   // bodies held in Morton order (mixed kick, >= kSortMinBodies bodies)
     size_t off_perm, off_inv, off_box, off_k0, off_k1, off_v0, off_v1, off_hist, off_far, off_tile;
@@ -760,30 +855,24 @@ constexpr int64_t kSingleSortMin = 2048;
 
 static SingleLayout single_layout(int64_t rows, int prec) {
     SingleLayout L;
-    KickTune t;
-    t.threads = 128;
-    t.ipt = prec == QYM_KICK_MIXED ? 2 : 1;
     int64_t nb = rows - 1;
-    int64_t ib = (nb + t.threads * t.ipt - 1) / (t.threads * t.ipt);
-    // enough CTAs to cover the GPU a few times over
-    int64_t want = 4 * 152;
-    int64_t sp = (want + ib - 1) / ib;
-    int64_t maxsp = (nb + 255) / 256;  // at least a tile of j per split
-    if (sp > maxsp) sp = maxsp;
-    if (sp < 1) sp = 1;
-    t.splits = (int32_t)sp;
-    L.tune = t;
-    L.splits = t.splits;
-    L.nitems = (int32_t)(ib * sp);
+    L.tune = default_kick_tune(nb, nb, prec);
+    KickTune &t = L.tune;
+    int64_t ti = (int64_t)t.threads * t.ipt;
+    L.sorted = prec == QYM_KICK_MIXED && nb >= kSingleSortMin;
+    const int64_t align = L.sorted ? TILE : 1;
+    int64_t chunk = (nb + t.splits - 1) / t.splits;
+    chunk = (chunk + align - 1) / align * align;  // j-ranges start on tiles
+    t.splits = (int32_t)((nb + chunk - 1) / chunk);
+    L.chunk = (int32_t)chunk;
+    L.nitems = (int32_t)((nb + ti - 1) / ti * t.splits);
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     size_t o = 0;
-    L.off_pos = o; o = al(o + sizeof(float4) * rows);
-    L.off_lo = o; o = al(o + sizeof(float4) * rows);
-    L.off_items = o; o = al(o + sizeof(int4) * L.nitems);
-    L.off_slots = o; o = al(o + sizeof(int32_t) * L.nitems);
-    L.off_apart = o; o = al(o + sizeof(double) * 3 * rows * L.splits);
+    const int64_t packs = prec == QYM_KICK_MIXED ? rows : 0;
+    L.off_pos = o; o = al(o + sizeof(float4) * packs);
+    L.off_lo = o; o = al(o + sizeof(float4) * packs);
+    L.off_apart = o; o = al(o + sizeof(double) * 3 * rows * t.splits);
     L.off_heavy = o; o = al(o + sizeof(int32_t) * (QYM_HEAVY_CAP + 1));
-    L.sorted = prec == QYM_KICK_MIXED && nb >= kSingleSortMin;
     L.off_perm = L.off_inv = L.off_box = L.off_k0 = L.off_k1 = L.off_v0 = L.off_v1 = L.off_hist = 0;
     L.off_far = L.off_tile = 0;
     if (L.sorted) {
@@ -859,22 +948,6 @@ __global__ void k_pack_single(int64_t rows, const double *m, const double *q, do
     lo[pi] = make_float4(xl, yl, zl, 0.0f);
 }
 
-__global__ void k_items_single(int64_t rows, int32_t ti, int32_t splits, int4 *items,
-                               int32_t *slots, int32_t nitems, int32_t align) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nitems) return;
-    int64_t b0 = 1, b1 = rows, nb = rows - 1;
-    int64_t chunk = (nb + splits - 1) / splits;
-    chunk = (chunk + align - 1) / align * align;  // j-ranges start on tiles
-    int ib = idx / splits, sp = idx % splits;
-    int64_t i0 = b0 + (int64_t)ib * ti, i1 = i0 + ti < b1 ? i0 + ti : b1;
-    int64_t j0 = b0 + sp * chunk, j1 = j0 + chunk;
-    if (j0 > b1) j0 = b1;
-    if (j1 > b1) j1 = b1;
-    items[idx] = make_int4((int)i0, (int)i1, (int)j0, (int)j1);
-    slots[idx] = sp;
-}
-
 __global__ void k_sum_partials(int64_t rows, int32_t splits, const double *apart,
                                const int32_t *hl, const double *m, const double *q, double G,
                                double *a, const int32_t *inv) {
@@ -904,11 +977,10 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
     d.q = const_cast<double *>(q);
     d.pk_pos = (float4 *)(w + L.off_pos);
     d.pk_lo = (float4 *)(w + L.off_lo);
-    d.items = (int4 *)(w + L.off_items);
-    d.item_slot = (int32_t *)(w + L.off_slots);
     d.apart = (double *)(w + L.off_apart);
     d.nitems = L.nitems;
-    d.splits = L.splits;
+    d.splits = L.tune.splits;
+    d.item_chunk = L.chunk;
     int tb = 256;
     // heavy split (mixed kick only): threshold relative to the star mass m[0],
     // read on the device
@@ -933,25 +1005,19 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
         cudaError_t e = launch_sort_rows(rows, q, ss, d.perm, d.inv, st);
         if (e != cudaSuccess) return e;
     }
-    k_pack_single<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, m, q, G, hl, d.pk_pos,
-                                                                    d.pk_lo, d.inv);
-    k_items_single<<<(L.nitems + tb - 1) / tb, tb, 0, st>>>(rows, L.tune.threads * L.tune.ipt,
-                                                             L.splits, d.items, d.item_slot,
-                                                             L.nitems, L.sorted ? TILE : 1);
     cudaError_t e;
     if (prec == QYM_KICK_MIXED) {
+        k_pack_single<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, m, q, G, hl, d.pk_pos,
+                                                                        d.pk_lo, d.inv);
         e = launch_kick_tiles(d, prec, 0, G, L.tune.threads, L.tune.ipt, st);
     } else {
-        KickArgs ka;
-        ka.items = d.items; ka.slots = d.item_slot; ka.pos = d.pk_pos; ka.lo = d.pk_lo;
+        KickArgs ka{};
         ka.q = q; ka.m = m; ka.G = G; ka.apart = d.apart; ka.rows = rows;
-        ka.cand = nullptr; ka.max_cand = 0; ka.ncand = nullptr; ka.status = nullptr;
-        ka.fchunk = nullptr; ka.max_fchunk = 0; ka.nfchunk = nullptr; ka.far_tiles = 0;
-        ka.perm = nullptr; ka.far = nullptr; ka.tile = nullptr;
+        ka.splits = d.splits; ka.chunk = d.item_chunk;
         e = launch_f64<false, true>(ka, L.nitems, L.tune.threads, L.tune.ipt, st);
     }
     if (e != cudaSuccess) return e;
-    k_sum_partials<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, L.splits, d.apart, hl, m,
+    k_sum_partials<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, d.splits, d.apart, hl, m,
                                                                      q, G, a, d.inv);
     return cudaGetLastError();
 }

@@ -44,6 +44,7 @@ struct Dev {
     int4 *items = nullptr;
     int32_t *item_slot = nullptr;
     int32_t nitems = 0;
+    int32_t item_chunk = 0;       // items == NULL (one system): j rows per split
     // momentum reduction
     int4 *mchunks = nullptr;      // (row0, row1, sys, -) chunks of at most 1024 rows
     int32_t nmchunks = 0;
@@ -267,6 +268,7 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t,
                      int4 *items, int32_t *slots, int32_t *nitems, int32_t *splits_used,
                      int32_t max_items, int64_t i_lo = 0, int64_t i_hi = INT64_MAX,
                      int32_t align = 1);
+KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec);
 constexpr int kKickTile = 256;  // j rows per shared-memory tile of the kick
 int32_t kick_items_count(const int64_t *offsets, int32_t nsys, const KickTune &t,
                          int64_t i_lo = 0, int64_t i_hi = INT64_MAX);

@@ -37,3 +37,80 @@ def test_gradient_tiles(torch, n):
     d = np.abs(g.cpu().numpy().astype(np.float64) - go)
     assert np.all(d <= 2.0 ** -6 * gabs + 1e-7 * np.abs(go).max()), np.max(d / (gabs + 1e-300))
     assert abs(loss.item() - L) <= 1e-4 * L + 1e-7
+
+
+def _accel_ref(m, x, G):
+    """Accelerations in extended precision, and the sums of the terms' magnitudes."""
+    L = np.longdouble
+    xb, gm = x[1:].astype(L), L(G) * m[1:].astype(L)
+    a, mag = np.zeros(x.shape, L), np.zeros(x.shape, L)
+    for i in range(len(xb)):
+        d = xb - xb[i]
+        r2 = (d * d).sum(1)
+        with np.errstate(divide="ignore", invalid="ignore"):
+            s = np.where(r2 > 0, gm / (r2 * np.sqrt(r2)), L(0))
+        t = s[:, None] * d
+        a[1 + i], mag[1 + i] = t.sum(0), np.abs(t).sum(0)
+    return a, mag
+
+
+# (bodies, length unit, mass unit, kind)
+FP64_CASES = [
+    (1, 1.0, 1.0, "disk"), (2, 1.0, 1.0, "disk"), (16, 1.0, 1.0, "disk"), (129, 1.0, 1.0, "disk"),
+    (300, 1.5e11, 2e30 * 6.67e-11, "disk"),   # SI lengths, G folded into the masses
+    (300, 1e-30, 1e-30, "disk"),              # far from 1: scaled by powers of two
+    (300, 1e90, 1e40, "disk"),                # outside the scaled range: plain FP64
+    (300, 1.0, 1.0, "close"),                 # coincident, nearly coincident and far bodies
+    (300, 1.0, 1.0, "masses"),                # massless, tiny and large masses
+    (300, 1.0, 1.0, "flat"),                  # coplanar
+    (2200, 1.0, 1.0, "disk"),
+]
+
+
+@pytest.mark.parametrize("n,lu,mu,kind", FP64_CASES)
+def test_fp64_kick_edges(torch, n, lu, mu, kind):
+    """The FP64 kick, whose pairs are formed on the FP32 pipes, over sizes,
+    units, close pairs and masses, against extended precision. A pair's term
+    carries at most 2^-51 (two half-unit roundings of its weight, one of the
+    separation, one of the product), a sum of n of them n 2^-53 more."""
+    rng = np.random.default_rng(n + int(abs(np.log10(lu))))
+    x = np.concatenate([np.zeros((1, 3)), rng.normal(size=(n, 3)) * [10.0, 10.0, 0.1]])
+    m = np.concatenate([[1.0], 10.0 ** rng.uniform(-12, -3, n)])
+    if kind == "flat":
+        x[:, 2] = 0.0
+    if kind == "masses":
+        m[1::3] = 0.0
+        m[2] = 1e-40
+        m[3] = 1e3
+    if kind == "close":
+        x[2] = x[1]                        # coincident: no pull on each other
+        x[4] = x[3] + [1e-13, 0.0, 0.0]    # below the float form's range
+        x[6] = x[5] + [1e-6, -1e-7, 1e-9]
+        x[8] = x[7] * (1 + 2.0 ** -52)
+        x[9] *= 1e9
+        x[10] *= 1e-9
+    x, m = x * lu, m * mu
+    a = torch.empty((3, n + 1), dtype=torch.float64, device="cuda")
+    work = torch.empty(q.qym_accel_workspace_bytes(n + 1, q.QYM_KICK_FP64), dtype=torch.uint8, device="cuda")
+    q.qym_accel_dev(n + 1, torch.from_numpy(m).cuda(), torch.from_numpy(np.ascontiguousarray(x.T)).cuda(),
+                    a, 1.0, q.QYM_KICK_FP64, work)
+    ref, mag = _accel_ref(m, x, 1.0)
+    err = np.abs(a.cpu().numpy().T.astype(np.longdouble) - ref)
+    bound = (n + 4) * np.longdouble(2.0) ** -53 * mag + np.longdouble(1e-300)
+    assert np.all(err <= bound), float(np.max(err / bound))
+
+
+def test_fp64_kick_nonfinite(torch):
+    """A non-finite coordinate spreads as in plain FP64 arithmetic: NaN in
+    that component of the body and of every other one, nowhere else."""
+    n = 70
+    w = W.outer_disk(n - 4, seed=2)
+    for bad in (np.nan, np.inf):
+        x = w.q.copy()
+        x[9, 1] = bad
+        a = torch.empty((3, n + 1), dtype=torch.float64, device="cuda")
+        work = torch.empty(q.qym_accel_workspace_bytes(n + 1, q.QYM_KICK_FP64), dtype=torch.uint8, device="cuda")
+        q.qym_accel_dev(n + 1, torch.from_numpy(w.m).cuda(), torch.from_numpy(np.ascontiguousarray(x.T)).cuda(),
+                        a, 1.0, q.QYM_KICK_FP64, work)
+        a = a.cpu().numpy()
+        assert np.all(np.isnan(a[1, 1:])) and np.all(np.isfinite(a[[0, 2]]))
