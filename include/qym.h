@@ -462,8 +462,8 @@ qym_status qym_encounter_test_dev(int64_t rows, const double *q0, const double *
 
 /* Total energy of one system (Sec. 2, Eqs. 2-4), star at row 0, into device
  * double E[1]. `work` is caller-owned device scratch of
- * qym_energy_workspace_bytes(rows) bytes. Small work tables are staged from
- * the host, so this call waits for `stream` before returning. */
+ * qym_energy_workspace_bytes(rows) bytes. This call waits for `stream` before
+ * returning. */
 size_t qym_energy_workspace_bytes(int64_t rows);
 qym_status qym_energy_dev(int64_t rows, const double *m, const double *q, const double *v,
                           double G, double *E, void *work, size_t work_bytes, void *stream);

@@ -43,10 +43,10 @@ struct qym_ctx {
     void *arena = nullptr;
     KickTune tune;
     // energy
-    int4 *eitems = nullptr;
-    int32_t *eisys = nullptr, *eitem0 = nullptr;
+    EnergyPlan eplan;
+    int4 *eblocks = nullptr;
+    int32_t *eblock0 = nullptr;
     double *epart = nullptr, *E = nullptr;
-    int32_t neitems = 0;
     double *mt = nullptr;  // [nsys] total masses
     void *flush = nullptr; // L2 flush buffer (params.l2_flush_bytes)
     SetScratch ss;
@@ -297,10 +297,9 @@ static void carve_all(qym_ctx *c, Carver &k) {
     c->ss.size = k.take<int32_t>(R + 1);
     c->ss.fill = k.take<int32_t>(R + 1);
     c->ss.rc_bits = k.take<unsigned long long>(R + 1);
-    c->eitems = k.take<int4>(c->neitems);
-    c->eisys = k.take<int32_t>(c->neitems);
-    c->eitem0 = k.take<int32_t>(d.nsys + 1);
-    c->epart = k.take<double>(c->neitems);
+    c->eblocks = k.take<int4>(c->eplan.nblocks);
+    c->eblock0 = k.take<int32_t>(d.nsys + 1);
+    c->epart = k.take<double>(energy_partials(c->eplan));
     c->E = k.take<double>(d.nsys);
     c->mt = k.take<double>(d.nsys);
     c->mlp_w = k.take<float>(QYM_MLP_NW);
@@ -535,7 +534,7 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     d.max_log = params->max_log ? params->max_log : (int64_t)1 << 22;
     d.max_sets = (int32_t)R;
     d.max_members = (int32_t)R;
-    c->neitems = energy_items_host(offsets, nsys, nullptr, nullptr, nullptr);
+    c->eplan = energy_plan(offsets, nsys, nullptr, nullptr);
     // heavy bodies per system (mixed kick): m >= heavy_mass m0, at most
     // QYM_HEAVY_CAP of them, else the system keeps all bodies in FP32
     std::vector<int32_t> hrows, hstart(nsys + 1);
@@ -633,9 +632,11 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     int32_t ni = 0, spu = 0;
     kick_items_host(offsets, nsys, c->tune, items.data(), slots.data(), &ni, &spu, d.nitems, 0,
                     INT64_MAX, c->sort_rows ? kKickTile / 2 : 1);
-    std::vector<int4> eit(c->neitems);
-    std::vector<int32_t> eis(c->neitems), ei0(nsys + 1);
-    energy_items_host(offsets, nsys, eit.data(), eis.data(), ei0.data());
+    std::vector<int4> eblk(c->eplan.nblocks);
+    std::vector<int32_t> eb0(nsys + 1);
+    energy_plan(offsets, nsys, eblk.data(), eb0.data());
+    c->eplan.blocks = c->eblocks;
+    c->eplan.block0 = c->eblock0;
     CKI(cudaMemcpyAsync(d.offsets, offsets, sizeof(int64_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
     if (!c->h_wh_heavy.empty())
         CKI(cudaMemcpyAsync(c->wh_heavy, c->h_wh_heavy.data(), sizeof(int32_t) * c->h_wh_heavy.size(),
@@ -646,9 +647,8 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     CKI(cudaMemcpyAsync(d.item_slot, slots.data(), sizeof(int32_t) * d.nitems, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.mchunks, mch.data(), sizeof(int4) * d.nmchunks, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.sys_chunk0, sc0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
-    CKI(cudaMemcpyAsync(c->eitems, eit.data(), sizeof(int4) * c->neitems, cudaMemcpyHostToDevice, c->stream));
-    CKI(cudaMemcpyAsync(c->eisys, eis.data(), sizeof(int32_t) * c->neitems, cudaMemcpyHostToDevice, c->stream));
-    CKI(cudaMemcpyAsync(c->eitem0, ei0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
+    CKI(cudaMemcpyAsync(c->eblocks, eblk.data(), sizeof(int4) * eblk.size(), cudaMemcpyHostToDevice, c->stream));
+    CKI(cudaMemcpyAsync(c->eblock0, eb0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
     if (!hrows.empty())
         CKI(cudaMemcpyAsync(d.heavy_rows, hrows.data(), sizeof(int32_t) * hrows.size(), cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.heavy_start, hstart.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
@@ -1170,8 +1170,8 @@ extern "C" qym_status qym_get_order(qym_ctx *c, int32_t *order) {
 extern "C" qym_status qym_energy(qym_ctx *c, double *E) {
     if (!c || !E) FAIL(c, QYM_EINVAL, "qym_energy: NULL argument");
     Dev &d = c->d;
-    CK(c, launch_energy_items(c->neitems, c->eitems, c->eisys, c->eitem0, d.nsys, d.offsets, d.rows,
-                              d.m, d.q, d.v, c->p.G, c->epart, c->E, c->stream));
+    CK(c, launch_energy(c->eplan, d.nsys, d.offsets, d.rows, d.m, d.q, d.v, c->p.G, c->epart, c->E,
+                        c->stream));
     CK(c, cudaMemcpyAsync(E, c->E, sizeof(double) * d.nsys, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     return QYM_OK;
@@ -1637,10 +1637,8 @@ extern "C" qym_status qym_encounter_test_dev(int64_t rows, const double *q0, con
 
 extern "C" size_t qym_energy_workspace_bytes(int64_t rows) {
     if (rows < 2) return 0;
-    int64_t off[2] = {0, rows};
-    int32_t n = energy_items_host(off, 1, nullptr, nullptr, nullptr);
-    return al256(sizeof(int4) * n) + al256(sizeof(int32_t) * n) + al256(sizeof(int32_t) * 2) +
-           al256(sizeof(double) * n) + al256(sizeof(int64_t) * 2);
+    const int64_t off[2] = {0, rows};
+    return al256(sizeof(double) * energy_partials(energy_plan(off, 1, nullptr, nullptr)));
 }
 
 extern "C" qym_status qym_energy_dev(int64_t rows, const double *m, const double *q, const double *v,
@@ -1648,25 +1646,10 @@ extern "C" qym_status qym_energy_dev(int64_t rows, const double *m, const double
                                      void *stream) {
     if (rows < 2 || !m || !q || !v || !E || !work) FAIL(nullptr, QYM_EINVAL, "qym_energy_dev: bad argument");
     if (work_bytes < qym_energy_workspace_bytes(rows)) FAIL(nullptr, QYM_EINVAL, "qym_energy_dev: workspace too small");
-    int64_t off[2] = {0, rows};
-    int32_t n = energy_items_host(off, 1, nullptr, nullptr, nullptr);
-    std::vector<int4> it(n);
-    std::vector<int32_t> is(n), i0(2);
-    energy_items_host(off, 1, it.data(), is.data(), i0.data());
-    char *w = (char *)work;
-    int4 *d_it = (int4 *)w; w += al256(sizeof(int4) * n);
-    int32_t *d_is = (int32_t *)w; w += al256(sizeof(int32_t) * n);
-    int32_t *d_i0 = (int32_t *)w; w += al256(sizeof(int32_t) * 2);
-    double *d_part = (double *)w; w += al256(sizeof(double) * n);
-    int64_t *d_off = (int64_t *)w;
+    const int64_t off[2] = {0, rows};
     cudaStream_t st = (cudaStream_t)stream;
-    // the tables are staged through pageable memory; the copies complete
-    // before this call returns
-    CK(nullptr, cudaMemcpyAsync(d_it, it.data(), sizeof(int4) * n, cudaMemcpyHostToDevice, st));
-    CK(nullptr, cudaMemcpyAsync(d_is, is.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
-    CK(nullptr, cudaMemcpyAsync(d_i0, i0.data(), sizeof(int32_t) * 2, cudaMemcpyHostToDevice, st));
-    CK(nullptr, cudaMemcpyAsync(d_off, off, sizeof(int64_t) * 2, cudaMemcpyHostToDevice, st));
-    CK(nullptr, launch_energy_items(n, d_it, d_is, d_i0, 1, d_off, rows, m, q, v, G, d_part, E, st));
+    CK(nullptr, launch_energy(energy_plan(off, 1, nullptr, nullptr), 1, nullptr, rows, m, q, v, G,
+                              (double *)work, E, st));
     CK(nullptr, cudaStreamSynchronize(st));
     return QYM_OK;
 }

@@ -1,120 +1,195 @@
 // energy.cu -- total energy of each system (Sec. 2, Eqs. 2-4), FP64:
 //   E = |S|^2 / (2 m0) + sum_i [m_i v_i^2 / 2 - G m0 m_i / |Q_i|]
-//       - (1/2) sum_{i != j} G m_i m_j / |Q_i - Q_j|        (i, j bodies),
-// the pair sum taken over all ordered pairs in tiles (the paper's N^2
-// over-count) with the star mass restored for the star terms.
+//       - sum_{i < j} G m_i m_j / |Q_i - Q_j|        (i, j bodies),
+// each pair once (the paper's kernel takes both orders and halves the sum),
+// with the star mass restored for the star terms.
+//
+// The pair sum is bound by issue: a pair's separation, r^2 and G m / r run to
+// FP64 accuracy on the FP32 pipes (pair64.cuh, some 270 instructions), FP64 adds
+// the result (one instruction). A CTA takes 128 rows against a range of later
+// rows; the range's length (energy_plan) gives the GPU about 16 CTAs per SM
+// whatever the sizes, where one CTA per 256 rows against all rows left 16384
+// bodies on 64 of the 152 SMs with 15 FP64 instructions per ordered pair
+// (16.6 ms).
+#include <algorithm>
+
+#include "pair64.cuh"
 #include "qym_internal.cuh"
 
 namespace qym {
 
-constexpr int ETILE = 256;
+constexpr int ET = 128;  // rows of an i-block = threads of a CTA = rows of a j tile
 
-// one CTA per item (i0, i1, j0, j1) of one system; writes its partial of
-// sum_i [m v^2 / 2 - G m0 m / r - (1/2) m_i sum_j G m_j / r_ij]
-__global__ void __launch_bounds__(256) k_energy_items(const int4 *items, const int32_t *isys,
-                                                      const int64_t *offsets, int64_t R,
-                                                      const double *m, const double *q,
-                                                      const double *v, double G, double *part) {
-    __shared__ D4 s_q[ETILE];
-    __shared__ double red[8];
-    const int4 it = items[blockIdx.x];
-    const int64_t star = offsets[isys[blockIdx.x]];
-    const double m0 = m[star];
-    const int64_t i = it.x + threadIdx.x;
-    const bool act = i < it.y;
-    double xi = 0, yi = 0, zi = 0;
-    if (act) { xi = q[i]; yi = q[R + i]; zi = q[2 * R + i]; }
-    double phi = 0.0;
-    for (int jt = it.z; jt < it.w; jt += ETILE) {
-        int n = min(ETILE, it.w - jt);
-        __syncthreads();
-        for (int t = threadIdx.x; t < n; t += blockDim.x) {
-            int64_t j = jt + t;
-            s_q[t] = D4{q[j], q[R + j], q[2 * R + j], G * m[j]};
-        }
-        __syncthreads();
-        if (act) {
-            for (int t = 0; t < n; ++t) {
-                D4 p = s_q[t];
-                double dx = xi - p.x, dy = yi - p.y, dz = zi - p.z;
-                double r2 = dx * dx + dy * dy + dz * dz;
-                phi += (r2 > 0.0) ? p.w * rsqrt(r2) : 0.0;
-            }
-        }
-    }
-    double e = 0.0;
-    if (act) {
-        double mi = m[i];
-        double vx = v[i], vy = v[R + i], vz = v[2 * R + i];
-        double r = sqrt(xi * xi + yi * yi + zi * zi);
-        e = 0.5 * mi * (vx * vx + vy * vy + vz * vz) - G * m0 * mi / r - 0.5 * mi * phi;
-    }
-    e = warp_sum(e);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
-        part[blockIdx.x] = s;
-    }
+// G m / r of a pair in FP64, where the float form does not hold
+__device__ __noinline__ double potential_fp64(double dx, double dy, double dz, double gm) {
+    if ((__double_as_longlong(gm) << 1) == 0) return 0.0;  // a massless partner
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    return (r2 > 0.0) ? gm * rsqrt(r2) : 0.0;
 }
 
-// per system: fixed-order sum of its items' partials plus |S|^2 / (2 m0),
-// with S = sum m v computed here in fixed order as well
-__global__ void k_energy_final(int32_t nsys, const int64_t *offsets, const int32_t *item0,
-                               const double *part, const double *m, const double *v, int64_t R,
-                               double *E) {
-    int s = blockIdx.x;
-    if (s >= nsys) return;
-    int64_t lo = offsets[s], hi = offsets[s + 1];
-    double sx = 0.0, sy = 0.0, sz = 0.0;
-    for (int64_t r = lo + 1 + threadIdx.x; r < hi; r += blockDim.x) {
-        sx += m[r] * v[r];
-        sy += m[r] * v[R + r];
-        sz += m[r] * v[2 * R + r];
+// CTA (I, c): rows of i-block I against the rows j > i of its c-th range;
+// writes -sum_i m_i sum_j G m_j / r_ij, and for c = 0 adds the rows' kinetic
+// and star terms and writes their momentum to ps[I]
+__global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, const double *m,
+                                                     const double *q, const double *v, double G,
+                                                     double *pe, double *ps) {
+    __shared__ D4 s_q[ET];
+    __shared__ float4 s_h[ET], s_m[ET], s_l[ET];
+    __shared__ int s_hi[2][ET / 32];
+    __shared__ double red[4][ET / 32];
+    const int64_t I = blockIdx.x / pl.nranges;
+    const int c = (int)(blockIdx.x - I * pl.nranges);
+    // (first row, last row + 1, end of the system, its star row)
+    const int4 bk = pl.blocks ? pl.blocks[I]
+                              : make_int4((int)(1 + I * ET), (int)min(1 + (I + 1) * (int64_t)ET, R), (int)R, 0);
+    const int64_t jb = bk.x + (int64_t)c * pl.range;
+    if (jb >= bk.z) {
+        if (threadIdx.x == 0) pe[blockIdx.x] = 0.0;
+        return;
     }
-    __shared__ double sh[3][8];
-    sx = warp_sum(sx); sy = warp_sum(sy); sz = warp_sum(sz);
+    const int j0 = (int)jb, j1 = (int)min(jb + pl.range, (int64_t)bk.z);
+    const int i = bk.x + threadIdx.x;
+    const int r = min(i, bk.y - 1);  // an idle lane repeats the last row
+    const double xi = q[r], yi = q[R + r], zi = q[2 * R + r];
+    int hl = max(p64::hi_abs(xi), max(p64::hi_abs(yi), p64::hi_abs(zi)));
+    int hw = j0 + (int)threadIdx.x < j1 ? p64::hi_abs(G * m[j0 + threadIdx.x]) : 0;
+    hl = __reduce_max_sync(0xffffffffu, hl);
+    hw = __reduce_max_sync(0xffffffffu, hw);
     if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = sx; sh[1][threadIdx.x >> 5] = sy; sh[2][threadIdx.x >> 5] = sz;
+        s_hi[0][threadIdx.x >> 5] = hl;
+        s_hi[1][threadIdx.x >> 5] = hw;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double S[3] = {0, 0, 0};
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k)
-            for (int c = 0; c < 3; ++c) S[c] += sh[c][k];
-        double e = 0.0;
-        for (int k = item0[s]; k < item0[s + 1]; ++k) e += part[k];
-        E[s] = e + (S[0] * S[0] + S[1] * S[1] + S[2] * S[2]) / (2.0 * m[lo]);
+    for (int w = 0; w < ET / 32; ++w) {
+        hl = max(hl, s_hi[0][w]);
+        hw = max(hw, s_hi[1][w]);
+    }
+    const p64::Scale sc(hl, hw);
+    const uint64_t bias = sc.bias(1);
+    const p64::F3 px = p64::split3(xi * sc.len), py = p64::split3(yi * sc.len);
+    const p64::F3 pz = p64::split3(zi * sc.len);
+    double phi = 0.0;
+    for (int jt = j0; jt < j1; jt += ET) {
+        const int n = min(ET, j1 - jt);
+        __syncthreads();
+        if ((int)threadIdx.x < n) {
+            const int j = jt + threadIdx.x, t = threadIdx.x;
+            const D4 p{q[j], q[R + j], q[2 * R + j], G * m[j]};
+            const p64::F3 x = p64::split3(p.x * sc.len), y = p64::split3(p.y * sc.len);
+            const p64::F3 z = p64::split3(p.z * sc.len), g = p64::split3(p.w * sc.wt);
+            s_q[t] = p;
+            s_h[t] = make_float4(x.h, y.h, z.h, g.h);
+            s_m[t] = make_float4(x.m, y.m, z.m, g.m);
+            s_l[t] = make_float4(x.l, y.l, z.l, g.l);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int t = 0; t < n; ++t) {
+            const float4 H = s_h[t], M = s_m[t], L = s_l[t];
+            const p64::F3 r2 = p64::norm2(p64::diff(px, p64::F3{H.x, M.x, L.x}),
+                                          p64::diff(py, p64::F3{H.y, M.y, L.y}),
+                                          p64::diff(pz, p64::F3{H.z, M.z, L.z}));
+            double s;
+            const bool ok = p64::g_over_r(p64::F3{H.w, M.w, L.w}, r2, rsqrt_ftz(r2.h), bias, s) &&
+                            p64::r2_fits(r2.h) && p64::g_fits(H.w) && sc.ok;
+            const bool later = jt + t > i;
+            if (!ok && later) {
+                const D4 p = s_q[t];
+                s = potential_fp64(xi - p.x, yi - p.y, zi - p.z, p.w);
+            }
+            if (later) phi += s;
+        }
+    }
+    const bool act = i < bk.y;
+    double e[4] = {0.0, 0.0, 0.0, 0.0};
+    if (act) {
+        const double mi = m[i];
+        e[0] = -mi * phi;
+        if (c == 0) {
+            const double vx = v[i], vy = v[R + i], vz = v[2 * R + i];
+            const double d = sqrt(xi * xi + yi * yi + zi * zi);
+            e[0] += 0.5 * mi * (vx * vx + vy * vy + vz * vz) - G * m[bk.w] * mi / d;
+            e[1] = mi * vx;
+            e[2] = mi * vy;
+            e[3] = mi * vz;
+        }
+    }
+    const int nq = c == 0 ? 4 : 1;
+    for (int k = 0; k < nq; ++k) {
+        e[k] = warp_sum(e[k]);
+        if ((threadIdx.x & 31) == 0) red[k][threadIdx.x >> 5] = e[k];
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < nq) {
+        double s = 0.0;
+        for (int k = 0; k < ET / 32; ++k) s += red[threadIdx.x][k];
+        if (threadIdx.x == 0)
+            pe[blockIdx.x] = s;
+        else
+            ps[3 * I + threadIdx.x - 1] = s;
     }
 }
 
-// host: items of at most 256 i-rows against the whole system
-int32_t energy_items_host(const int64_t *offsets, int32_t nsys, int4 *items, int32_t *isys,
-                          int32_t *item0) {
+// per system (one CTA each): its CTAs' sums in a fixed order plus |S|^2 / (2 m0)
+__global__ void __launch_bounds__(256) k_energy_final(EnergyPlan pl, const int64_t *offsets,
+                                                      const double *m, const double *pe,
+                                                      const double *ps, double *E) {
+    const int s = blockIdx.x;
+    const int64_t b0 = pl.block0 ? pl.block0[s] : 0, b1 = pl.block0 ? pl.block0[s + 1] : pl.nblocks;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t k = b0 * pl.nranges + threadIdx.x; k < b1 * pl.nranges; k += blockDim.x) t[0] += pe[k];
+    for (int64_t k = b0 + threadIdx.x; k < b1; k += blockDim.x)
+        for (int c = 0; c < 3; ++c) t[1 + c] += ps[3 * k + c];
+    __shared__ double sh[4][8];
+    for (int c = 0; c < 4; ++c) {
+        t[c] = warp_sum(t[c]);
+        if ((threadIdx.x & 31) == 0) sh[c][threadIdx.x >> 5] = t[c];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 4; ++c) {
+            t[c] = 0.0;
+            for (int k = 0; k < 8; ++k) t[c] += sh[c][k];
+        }
+        E[s] = t[0] + (t[1] * t[1] + t[2] * t[2] + t[3] * t[3]) / (2.0 * m[offsets ? offsets[s] : 0]);
+    }
+}
+
+// host: i-blocks of at most 128 rows of each system (blocks and block0 may be
+// NULL: counted only) and the ranges' length: about 16 CTAs per SM over the
+// batch's pairs, ranges of 8 (a small system's walk is latency) to 4096 rows
+EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, int4 *blocks, int32_t *block0) {
+    EnergyPlan pl;
+    double pairs = 0.0;
+    int64_t nbmax = 0;
     int32_t n = 0;
     for (int32_t s = 0; s < nsys; ++s) {
-        if (item0) item0[s] = n;
-        int64_t b0 = offsets[s] + 1, b1 = offsets[s + 1];
-        for (int64_t i0 = b0; i0 < b1; i0 += 256) {
-            if (items) {
-                items[n] = make_int4((int)i0, (int)(i0 + 256 < b1 ? i0 + 256 : b1), (int)b0, (int)b1);
-                isys[n] = s;
-            }
+        if (block0) block0[s] = n;
+        const int64_t b0 = offsets[s] + 1, b1 = offsets[s + 1];
+        pairs += 0.5 * (double)(b1 - b0) * (double)(b1 - b0);
+        nbmax = std::max(nbmax, b1 - b0);
+        for (int64_t i0 = b0; i0 < b1; i0 += ET) {
+            if (blocks)
+                blocks[n] = make_int4((int)i0, (int)std::min<int64_t>(i0 + ET, b1), (int)b1, (int)offsets[s]);
             ++n;
         }
     }
-    if (item0) item0[nsys] = n;
-    return n;
+    if (block0) block0[nsys] = n;
+    const double want = pairs / (16.0 * 152.0 * ET);
+    pl.range = (int32_t)std::min(4096.0, std::max(8.0, 8.0 * (double)(int64_t)(want / 8.0 + 1.0)));
+    pl.nranges = (int32_t)((nbmax + pl.range - 1) / pl.range);
+    pl.nblocks = n;
+    return pl;
 }
 
-cudaError_t launch_energy_items(int32_t nitems, const int4 *items, const int32_t *isys,
-                                const int32_t *item0, int32_t nsys, const int64_t *offsets,
-                                int64_t R, const double *m, const double *q, const double *v,
-                                double G, double *part, double *E, cudaStream_t st) {
-    if (nitems > 0)
-        k_energy_items<<<nitems, 256, 0, st>>>(items, isys, offsets, R, m, q, v, G, part);
-    k_energy_final<<<nsys, 256, 0, st>>>(nsys, offsets, item0, part, m, v, R, E);
+int64_t energy_partials(const EnergyPlan &pl) { return (int64_t)pl.nblocks * (pl.nranges + 3); }
+
+cudaError_t launch_energy(const EnergyPlan &pl, int32_t nsys, const int64_t *offsets, int64_t R,
+                          const double *m, const double *q, const double *v, double G, double *part,
+                          double *E, cudaStream_t st) {
+    double *ps = part + (int64_t)pl.nblocks * pl.nranges;
+    k_energy_pairs<<<(unsigned)((int64_t)pl.nblocks * pl.nranges), ET, 0, st>>>(pl, R, m, q, v, G, part, ps);
+    k_energy_final<<<nsys, 256, 0, st>>>(pl, offsets, m, part, ps, E);
     return cudaGetLastError();
 }
 

@@ -355,11 +355,16 @@ cudaError_t launch_wh_blocks(const WholeArgs &w, int nblocks, cudaStream_t st);
 cudaError_t launch_wh_store(const WholeArgs &w, double *q1, double *v1, cudaStream_t st);
 
 // energy.cu
-int32_t energy_items_host(const int64_t *offsets, int32_t nsys, int4 *items, int32_t *isys,
-                          int32_t *item0);
-cudaError_t launch_energy_items(int32_t nitems, const int4 *items, const int32_t *isys,
-                                const int32_t *item0, int32_t nsys, const int64_t *offsets,
-                                int64_t R, const double *m, const double *q, const double *v,
-                                double G, double *part, double *E, cudaStream_t st);
+struct EnergyPlan {
+    const int4 *blocks = nullptr;     // i-blocks (device; NULL: one system of R rows)
+    const int32_t *block0 = nullptr;  // [nsys+1] first i-block of each system (NULL: one system)
+    int32_t nblocks = 0;
+    int32_t range = 0, nranges = 0;   // j rows per CTA, ranges per i-block
+};
+EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, int4 *blocks, int32_t *block0);
+int64_t energy_partials(const EnergyPlan &pl);  // doubles of `part`
+cudaError_t launch_energy(const EnergyPlan &pl, int32_t nsys, const int64_t *offsets, int64_t R,
+                          const double *m, const double *q, const double *v, double G, double *part,
+                          double *E, cudaStream_t st);
 
 }  // namespace qym

@@ -114,3 +114,47 @@ def test_fp64_kick_nonfinite(torch):
                         a, 1.0, q.QYM_KICK_FP64, work)
         a = a.cpu().numpy()
         assert np.all(np.isnan(a[1, 1:])) and np.all(np.isfinite(a[[0, 2]]))
+
+
+@pytest.mark.parametrize("sizes", [[1], [2, 1, 130], [128], [129, 7], [700, 300, 257]])
+@pytest.mark.parametrize("lu,mu", [(1.0, 1.0), (1.5e11, 2e30), (1e120, 1.0)])
+def test_energy_blocks(torch, sizes, lu, mu):
+    """Energy over system sizes at the edges of the 128-row blocks, in several
+    units (one outside the scaled float range), against extended precision:
+    n terms of at most 2^-51 each and a sum of n of them, relative to the sum
+    of the terms' magnitudes. Two bodies coincide (no pair term)."""
+    L = np.longdouble
+    rng = np.random.default_rng(sum(sizes))
+    ms, qs, vs, off = [], [], [], [0]
+    for n in sizes:
+        m = np.concatenate([[1.0], 10.0 ** rng.uniform(-10, -3, n)])
+        x = rng.normal(size=(n + 1, 3)) * [10, 10, 0.1]
+        v = rng.normal(size=(n + 1, 3)) * 0.3
+        x[0] = v[0] = 0.0
+        if n > 5:
+            m[4] = 0.0
+            x[2] = x[1]
+        ms.append(m * mu), qs.append(x * lu), vs.append(v * np.sqrt(mu / lu)), off.append(off[-1] + n + 1)
+    m, x, v = np.concatenate(ms), np.concatenate(qs), np.concatenate(vs)
+    sim = q.Simulation(m, x, v, np.array(off), coords=1, kick_prec=q.QYM_KICK_FP64, encounters=0)
+    E = sim.energy()
+    sim.close()
+    for s, n in enumerate(sizes):
+        ml, xl, vl = ms[s].astype(L), qs[s].astype(L), vs[s].astype(L)
+        mb, xb, vb = ml[1:], xl[1:], vl[1:]
+        S = (mb[:, None] * vb).sum(0)
+        kin = mb * (vb * vb).sum(1) / 2
+        star = ml[0] * mb / np.sqrt((xb * xb).sum(1))
+        pair = L(0)
+        for i in range(n):
+            r = np.sqrt(((xb[i + 1:] - xb[i]) ** 2).sum(1))
+            pair += (mb[i] * mb[i + 1:][r > 0] / r[r > 0]).sum()
+        ref = (S * S).sum() / (2 * ml[0]) + kin.sum() - star.sum() - pair
+        mag = (np.abs(mb[:, None] * vb).sum(0) ** 2).sum() / (2 * ml[0]) + kin.sum() + star.sum() + pair
+        assert abs(E[s] - ref) <= (n + 8) * L(2.0) ** -53 * mag, (s, float((E[s] - ref) / mag))
+        if len(sizes) == 1 or s == 0:
+            t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+            out = torch.empty(1, dtype=torch.float64, device="cuda")
+            work = torch.empty(q.qym_energy_workspace_bytes(n + 1), dtype=torch.uint8, device="cuda")
+            q.qym_energy_dev(n + 1, t(ms[s]), t(qs[s].T), t(vs[s].T), 1.0, out, work)
+            assert abs(out.item() - ref) <= (n + 8) * L(2.0) ** -53 * mag
