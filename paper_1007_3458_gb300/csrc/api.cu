@@ -392,6 +392,11 @@ __global__ void k_aos_from_soa(int64_t R, const double *soa, double *aos) {
     for (int c = 0; c < 3; ++c) aos[3 * r + c] = soa[c * R + r];
 }
 
+// partial-sum slots a context of R rows holds: up to 128, within ~0.5 GB
+static int64_t slots_cap(int64_t R) {
+    return std::min<int64_t>(128, std::max<int64_t>(4, ((int64_t)1 << 29) / (24 * R)));
+}
+
 // Launch shape of the kick for this batch
 static KickTune default_tune(const std::vector<int64_t> &off, int prec) {
     const int32_t nsys = (int32_t)off.size() - 1;
@@ -402,7 +407,7 @@ static KickTune default_tune(const std::vector<int64_t> &off, int prec) {
         ib += (nb + ti - 1) / ti;
         nbmax = std::max(nbmax, nb);
     }
-    return default_kick_tune(ib * ti, nbmax, prec);
+    return default_kick_tune(ib * ti, nbmax, prec, slots_cap(off[nsys]));
 }
 
 static qym_status upload_state(qym_ctx *c, const double *q, const double *v) {
@@ -505,9 +510,7 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
         big.threads = 128;
         big.ipt = 1;
         big.splits = 16;
-        // partial-sum slots: up to 128 for small batches, within ~0.5 GB
-        int64_t by_mem = ((int64_t)1 << 29) / (24 * R);
-        c->splits_cap = (int32_t)std::max<int64_t>(c->tune.splits, std::min<int64_t>(128, std::max<int64_t>(4, by_mem)));
+        c->splits_cap = (int32_t)std::max<int64_t>(c->tune.splits, slots_cap(R));
         big.splits = c->splits_cap;
         c->items_cap = std::max(kick_items_count(offsets, nsys, big), d.nitems);
         c->items_cap = std::max(c->items_cap, kick_items_count(offsets, nsys, c->tune));

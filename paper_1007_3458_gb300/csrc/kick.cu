@@ -527,11 +527,14 @@ __device__ __noinline__ double weight_fp64(double dx, double dy, double dz, doub
 }
 
 // The FP64 kick. The separations, r^2 and G m / r^3 of a pair are formed to FP64
-// accuracy on the FP32 pipes (pair64.cuh); the FP64 pipe, one warp instruction
-// per ~19 cycles and SM, keeps the separation and the sum of a pair's
-// acceleration, six instructions where the plain form has 22. Rows and partners
-// are split into three floats once per CTA and tile, scaled by powers of two;
-// pairs outside the float range take weight_fp64.
+// accuracy on the FP32 pipes (pair64.cuh, about 400 issue slots); beside them the
+// FP64 pipe, one warp instruction per ~19 cycles and SM, forms the separation
+// again and sums the pair's acceleration, six instructions where the plain form
+// has 22: 10240 bodies take 1.26 ms, 112 cycles of an SM per warp of pairs, both
+// pipes full (4.08 ms before; assembling the separation's doubles from the floats
+// instead of three FP64 subtractions, 1.34 ms). Rows and partners are split into
+// three floats once per CTA and tile, scaled by powers of two; pairs outside the
+// float range take plain FP64.
 template <int IPT, bool FLAG, bool FORCE>
 __global__ void __launch_bounds__(256) k_kick_fp64(KickArgs a) {
     __shared__ D4 s_q[TILE];
@@ -599,13 +602,13 @@ __global__ void __launch_bounds__(256) k_kick_fp64(KickArgs a) {
         for (int j = 0; j < n; ++j) {
             const D4 p = s_q[j];
             const float4 H = s_h[j], M = s_m[j], L = s_l[j];
-            const bool g_ok = sc.ok && p64::g_fits(H.w);
+            const bool g_ok = p64::g_fits(H.w);
 #pragma unroll
             for (int k = 0; k < IPT; ++k) {
                 const p64::F3 r2 = p64::norm2(p64::diff(px[k], p64::F3{H.x, M.x, L.x}),
                                               p64::diff(py[k], p64::F3{H.y, M.y, L.y}),
                                               p64::diff(pz[k], p64::F3{H.z, M.z, L.z}));
-                const bool fits = p64::r2_fits(r2.h);
+                const bool fits = sc.ok && p64::r2_fits(r2.h);
                 const double dx = xi[k] - p.x, dy = yi[k] - p.y, dz = zi[k] - p.z;
                 if (FORCE) {
                     double s;
@@ -618,7 +621,7 @@ __global__ void __launch_bounds__(256) k_kick_fp64(KickArgs a) {
                 }
                 if (FLAG) {
                     float r2f = __fadd_rn(r2.h, r2.m) * r2u;
-                    if (!(fits && r2_ok && sc.ok)) r2f = (float)(dx * dx + dy * dy + dz * dz);
+                    if (!(fits && r2_ok)) r2f = (float)(dx * dx + dy * dy + dz * dz);
                     if (r2f < rho[k] + s_rho[j]) {
                         int gj = jt + j;
                         if (gi[k] < gj) push_candidate(a, gi[k], gj);
@@ -692,22 +695,33 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t, in
 }
 
 // Default launch shape for i-blocks of nb bodies in all (nbmax in the largest
-// system). Mixed: about four CTAs per SM, at least a tile of j rows per split.
+// system), at most max_splits ranges per i-block.
+// Mixed: one or two rows per thread and j-ranges of one tile (one row, half a
+// tile and less for small systems, where a CTA's walk is the launch's length),
+// as long as the partial slots stay few: 64 a row, and about 12288 CTAs. Many
+// short CTAs even out the near and far tiles and the last wave: 16384 bodies
+// take 0.134 ms in 64 ranges, 0.150 in 16, 0.188 in 10 (four CTAs per SM);
+// 262144 bodies 26.9 ms in 12, 29.6 in one; 4096 bodies 20.5 us in 32, 1024
+// bodies 6.2 us in 32 (14.4 in 4).
 // FP64: as many CTAs as fit the GPU at once (eight of 128 threads per SM),
-// since a pair takes some 300 issue slots: 10240 bodies on 80 i-blocks fill
-// the chip with 15 splits; small systems take splits of at least 16 rows (a
-// 260-body kick is one warp's walk over its j-range: 185 us in one range, a
-// plain FP64 form, 7 us in 16).
-KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec) {
+// since a pair takes some 400 issue slots: 10240 bodies on 80 i-blocks fill
+// the chip with 15 splits; small systems take splits of at least 8 rows (a
+// 260-body kick is one warp's walk over its j-range: 185 us in one range in
+// plain FP64, 14 us in ranges of 16).
+KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t max_splits) {
     KickTune t;
     const bool mixed = prec == QYM_KICK_MIXED;
     t.threads = 128;
-    t.ipt = mixed ? 2 : 1;
+    t.ipt = mixed && iblocks_nb > 6144 ? 2 : 1;
     const int64_t ib = std::max<int64_t>(1, (iblocks_nb + t.threads * t.ipt - 1) / (t.threads * t.ipt));
-    const int64_t want = (mixed ? 4 : 8) * 152;
-    const int64_t sp = mixed ? (want + ib - 1) / ib : want / ib;
-    const int64_t maxsp = mixed ? (nbmax + 255) / 256 : nbmax / 16;
-    t.splits = (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min(sp, maxsp), 128));
+    int64_t sp;
+    if (mixed) {
+        const int64_t range = nbmax > 6144 ? 256 : (nbmax > 2048 ? 128 : 32);
+        sp = std::min<int64_t>({(nbmax + range - 1) / range, 12288 / ib, 64});
+    } else {
+        sp = std::min<int64_t>({8 * 152 / ib, nbmax / 8, 128});
+    }
+    t.splits = (int32_t)std::max<int64_t>(1, std::min(sp, max_splits));
     return t;
 }
 
@@ -856,7 +870,8 @@ constexpr int64_t kSingleSortMin = 2048;
 static SingleLayout single_layout(int64_t rows, int prec) {
     SingleLayout L;
     int64_t nb = rows - 1;
-    L.tune = default_kick_tune(nb, nb, prec);
+    // (the fixed scratch of qym_accel_dev_static holds about 2^17.6 row slots)
+    L.tune = default_kick_tune(nb, nb, prec, std::max<int64_t>(1, 200000 / rows));
     KickTune &t = L.tune;
     int64_t ti = (int64_t)t.threads * t.ipt;
     L.sorted = prec == QYM_KICK_MIXED && nb >= kSingleSortMin;
@@ -948,21 +963,31 @@ __global__ void k_pack_single(int64_t rows, const double *m, const double *q, do
     lo[pi] = make_float4(xl, yl, zl, 0.0f);
 }
 
-__global__ void k_sum_partials(int64_t rows, int32_t splits, const double *apart,
-                               const int32_t *hl, const double *m, const double *q, double G,
-                               double *a, const int32_t *inv) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
+// per row the sum of its slots and the heavy bodies' pull, SL threads a row
+// (thread group q of the CTA the slots and heavies q, q + SL, ...), the parts
+// added in a fixed tree
+constexpr int SL = 8;
+__global__ void __launch_bounds__(256) k_sum_partials(int64_t rows, int32_t splits, const double *apart,
+                                                      const int32_t *hl, const double *m, const double *q,
+                                                      double G, double *a, const int32_t *inv) {
+    constexpr int RB = 256 / SL;
+    __shared__ double sh[SL][3][RB];
+    const int t = threadIdx.x % RB, g = threadIdx.x / RB;
+    const int64_t i = (int64_t)blockIdx.x * RB + t;
     double s[3] = {0.0, 0.0, 0.0};
-    if (i > 0) {
+    if (i > 0 && i < rows) {
         const int64_t pi = inv ? inv[i] : i;  // the kick's order
-        for (int c = 0; c < 3; ++c)
-            for (int sp = 0; sp < splits; ++sp) s[c] += apart[((int64_t)sp * 3 + c) * rows + pi];
+        for (int sp = g; sp < splits; sp += SL)
+            for (int c = 0; c < 3; ++c) s[c] += apart[((int64_t)sp * 3 + c) * rows + pi];
         if (hl)
-            heavy_pull(hl, hl[QYM_HEAVY_CAP], i, q[i], q[rows + i], q[2 * rows + i], q, m, rows, G,
-                       s[0], s[1], s[2]);
+            heavy_pull(hl, g, SL, hl[QYM_HEAVY_CAP], i, q[i], q[rows + i], q[2 * rows + i], q, m, rows,
+                       G, s[0], s[1], s[2]);
     }
-    for (int c = 0; c < 3; ++c) a[c * rows + i] = s[c];
+    for (int c = 0; c < 3; ++c) sh[g][c][t] = s[c];
+    __syncthreads();
+    if (g >= 3 || i >= rows) return;
+    a[g * rows + i] = ((sh[0][g][t] + sh[1][g][t]) + (sh[2][g][t] + sh[3][g][t])) +
+                      ((sh[4][g][t] + sh[5][g][t]) + (sh[6][g][t] + sh[7][g][t]));
 }
 
 cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, double *a,
@@ -1017,7 +1042,7 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
         e = launch_f64<false, true>(ka, L.nitems, L.tune.threads, L.tune.ipt, st);
     }
     if (e != cudaSuccess) return e;
-    k_sum_partials<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, d.splits, d.apart, hl, m,
+    k_sum_partials<<<(unsigned)((rows + 256 / SL - 1) / (256 / SL)), 256, 0, st>>>(rows, d.splits, d.apart, hl, m,
                                                                      q, G, a, d.inv);
     return cudaGetLastError();
 }

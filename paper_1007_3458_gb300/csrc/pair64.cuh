@@ -44,6 +44,7 @@ __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ uint32_t bits(float a) { return __float_as_uint(a); }
 __device__ __forceinline__ float from_bits(uint32_t a) { return __uint_as_float(a); }
 __device__ __forceinline__ int32_t to_int(float a) { return __float2int_rn(a); }
+__device__ __forceinline__ uint64_t bits64(double a) { return (uint64_t)__double_as_longlong(a); }
 __device__ __forceinline__ double from_bits64(uint64_t a) { return __longlong_as_double((long long)a); }
 #else
 P64_HD float add(float a, float b) { return a + b; }
@@ -53,6 +54,7 @@ P64_HD float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 P64_HD uint32_t bits(float a) { uint32_t u; memcpy(&u, &a, 4); return u; }
 P64_HD float from_bits(uint32_t u) { float a; memcpy(&a, &u, 4); return a; }
 P64_HD int32_t to_int(float a) { return (int32_t)lrintf(a); }
+P64_HD uint64_t bits64(double a) { uint64_t u; memcpy(&u, &a, 8); return u; }
 P64_HD double from_bits64(uint64_t u) { double a; memcpy(&a, &u, 8); return a; }
 #endif
 
@@ -77,12 +79,28 @@ P64_HD void two_prod(float a, float b, float &p, float &e) {
     e = fma_(a, b, -p);
 }
 
+// x as h + m + l, exact for 2^-88 <= |x| < 2^128 (zero below, h infinite above
+// or NaN), by moving its bits: the leading 24 in place, the next 15 and the last
+// 14 under the exponents they stand for, each less its implicit one. No FP64
+// instruction (a conversion holds the FP64 pipe like an addition).
 P64_HD F3 split3(double x) {
+    const uint64_t u = bits64(x);
+    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+    const uint32_t e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+    const uint32_t a = ((((hi << 3) | (lo >> 29)) & 0x7fffffffu) ^ 0x40000000u) | sign;
+    const uint32_t b1 = (a & 0xff800000u) - (23u << 23), b2 = b1 - (15u << 23);
+    // rounded to nearest part by part: each stays under half the last place of
+    // the one before
     F3 r;
-    r.h = (float)x;
-    const double t = x - (double)r.h;
-    r.m = (float)t;
-    r.l = (float)(t - (double)r.m);
+    float t, v;
+    fast_two_sum(from_bits(a), sub(from_bits(b1 | ((lo >> 6) & 0x7fff00u)), from_bits(b1)), t, v);
+    two_sum(v, sub(from_bits(b2 | ((lo << 9) & 0x7ffe00u)), from_bits(b2)), v, r.l);
+    fast_two_sum(t, v, r.h, r.m);
+    if (e - (1023u - 88u) > 88u + 127u) {
+        const bool small = e < 1023u - 88u;
+        r.h = small ? 0.0f : from_bits(0x7f800000u | sign);
+        r.m = r.l = small ? 0.0f : r.h;
+    }
     return r;
 }
 
@@ -262,6 +280,37 @@ struct Scale {
     }
 };
 __device__ __forceinline__ int hi_abs(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+// x 2^-k by its exponent field: zero below the normal range, infinite above it;
+// infinities and NaN as they are
+__device__ __forceinline__ double scale2(double x, int k) {
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    if (e == 0x7ff) return x;
+    if (e == 0 || e - k <= 0) return 0.0;
+    if (e - k >= 0x7ff) return __hiloint2double(0x7ff00000, 0);
+    return __hiloint2double(hi - k * (1 << 20), __double2loint(x));
+}
+
+// the leading 24 bits of x 2^-k as a float, truncated (zero below FP32's normal
+// range, infinite above it)
+__device__ __forceinline__ float lead(double x, int k) {
+    const int hi = __double2hiint(x), field = (hi >> 20) & 0x7ff, e = field - k - 896;
+    const unsigned b = ((unsigned)hi << 3 | (unsigned)__double2loint(x) >> 29) & 0x7fffffu;
+    const unsigned f = field == 0 || e <= 0 ? 0u : (e >= 255 ? 0x7f800000u : ((unsigned)e << 23 | b));
+    return __uint_as_float(f | ((unsigned)hi & 0x80000000u));
+}
+
+// an upper bound of |(x, y, z)| within 1e-6, without an FP64 instruction (an
+// FP64 square root is ten); NaN or infinite for such inputs
+__device__ __forceinline__ float norm_up(double x, double y, double z) {
+    const int hm = max(hi_abs(x), max(hi_abs(y), hi_abs(z)));
+    if (hm >= 0x7ff00000) return (float)x + (float)y + (float)z;
+    const int k = (hm >> 20) - 1023;
+    const float a = lead(x, k), b = lead(y, k), c = lead(z, k);
+    const float n = sqrtf(fmaf(a, a, fmaf(b, b, c * c))) * (1.0f + 0x1p-21f);
+    if (k > 125) return INFINITY;
+    return k < -125 ? n * 0x1p-125f : n * __int_as_float((127 + k) << 23);
+}
 #endif
 
 }  // namespace p64

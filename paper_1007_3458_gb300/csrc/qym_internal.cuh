@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/qym.h"
+#include "pair64.cuh"
 
 namespace qym {
 
@@ -163,19 +164,41 @@ __device__ __forceinline__ void split_ds(double x, float &hi, float &lo) {
     lo = __double2float_rn(x - (double)hi);
 }
 
-// FP64 pull of the heavy bodies hs[0..nh) (ascending rows, i excluded) on
-// the body at (x, y, z): sum -G m_h (r_i - r_h) / |r_i - r_h|^3
-__device__ __forceinline__ void heavy_pull(const int32_t *hs, int nh, int64_t i, double x,
-                                           double y, double z, const double *q, const double *m,
-                                           int64_t R, double G, double &ax, double &ay,
-                                           double &az) {
-    for (int k = 0; k < nh; ++k) {
-        int64_t h = hs[k];
+// pull of the heavy bodies hs[k0], hs[k0 + step], ... below nh (ascending rows,
+// i excluded) on the body at (x, y, z): sum -G m_h (r_i - r_h) / |r_i - r_h|^3,
+// each pair to FP64 accuracy on the FP32 pipes (pair64.cuh), seven FP64
+// instructions instead of 25; lengths scaled by the body's own largest
+// coordinate, weights each by itself
+__device__ __forceinline__ void heavy_pull(const int32_t *hs, int k0, int step, int nh, int64_t i,
+                                           double x, double y, double z, const double *q,
+                                           const double *m, int64_t R, double G, double &ax,
+                                           double &ay, double &az) {
+    if (k0 >= nh) return;
+    const int hm = max(p64::hi_abs(x), max(p64::hi_abs(y), p64::hi_abs(z)));
+    const int kb = (hm >> 20) - 1023;
+    const bool kb_ok = kb >= -200 && kb <= 200;
+    const int kbs = kb_ok ? kb : 0;
+    const p64::F3 X = p64::split3(p64::scale2(x, kbs)), Y = p64::split3(p64::scale2(y, kbs));
+    const p64::F3 Z = p64::split3(p64::scale2(z, kbs));
+    for (int k = k0; k < nh; k += step) {
+        const int64_t h = hs[k];
         if (h == i) continue;
-        double dx = x - q[h], dy = y - q[R + h], dz = z - q[2 * R + h];
-        double r2 = dx * dx + dy * dy + dz * dz;
-        double ri = rsqrt(r2);
-        double s = G * m[h] * (ri * ri) * ri;
+        const double qx = q[h], qy = q[R + h], qz = q[2 * R + h], gm = G * m[h];
+        const int ka = (p64::hi_abs(gm) >> 20) - 1023;
+        const p64::F3 r2 = p64::norm2(p64::diff(X, p64::split3(p64::scale2(qx, kbs))),
+                                      p64::diff(Y, p64::split3(p64::scale2(qy, kbs))),
+                                      p64::diff(Z, p64::split3(p64::scale2(qz, kbs))));
+        const double dx = x - qx, dy = y - qy, dz = z - qz;
+        double s;
+        const bool ka_ok = ka >= -200 && ka <= 200;
+        const int kas = ka_ok ? ka : 0;
+        const bool ok = p64::g_over_r3(p64::split3(p64::scale2(gm, kas)), r2, rsqrt_ftz(r2.h),
+                                       (uint64_t)(int64_t)(kas - 3 * kbs) << 52, s);
+        if (!(ok && kb_ok && ka_ok && p64::r2_fits(r2.h))) {
+            const double d2 = dx * dx + dy * dy + dz * dz;
+            const double ri = rsqrt(d2);
+            s = gm * (ri * ri) * ri;
+        }
         ax -= s * dx;
         ay -= s * dy;
         az -= s * dz;
@@ -268,7 +291,7 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t,
                      int4 *items, int32_t *slots, int32_t *nitems, int32_t *splits_used,
                      int32_t max_items, int64_t i_lo = 0, int64_t i_hi = INT64_MAX,
                      int32_t align = 1);
-KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec);
+KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t max_splits);
 constexpr int kKickTile = 256;  // j rows per shared-memory tile of the kick
 int32_t kick_items_count(const int64_t *offsets, int32_t nsys, const KickTune &t,
                          int64_t i_lo = 0, int64_t i_hi = INT64_MAX);

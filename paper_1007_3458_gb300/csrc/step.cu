@@ -3,6 +3,8 @@
 // partial accelerations, updates velocities, records |a| and the Hill radii
 // used by the encounter test), Hill radii (Eq. 9), and the heliocentric <->
 // barycentric velocity conversion (Sec. 2).
+#include <cmath>
+
 #include "qym_internal.cuh"
 
 namespace qym {
@@ -81,7 +83,68 @@ struct DriftArgs {
     double kick_span;  // time of the kick(s) between this pack and the Kepler drift
     double a_allow;    // bound on |a| of that kick as a multiple of the last |a|
     int flag_next, hill_fixed;
+    float tau_f, span_f, a_E_f, a_allow_f;  // |tau|, |kick_span|, a_E, a_allow in FP32
 };
+
+// Crude reach of row r (Sec. 2.4), rho_i = F_i (R_i + |tau| (u_i + w_i)):
+//   R_i  a_E times a bound on this step's Hill radius
+//   u_i  speed relative to the local circular velocity Omega (z x Q)
+//   w_i  bound on the velocity change of the kick(s) before the Kepler
+//        drift: (tau/2) 1.01 |a| (the last kick was at the same
+//        separations), or with merged kicks tau 2 |a| (the last kick
+//        was a step earlier); the finisher checks the bound
+//   F_i  stretch for the Keplerian shear over one step
+// or with QYM_SEARCH_ESCAPE, the paper's crude sweep, a_E times the Hill radius
+// plus the distance covered at the escape velocity over the step. Returns
+// 2 rho^2: kernels test r^2 < c_i + c_j with c = 2 rho^2 >= ... a superset of
+// r < rho_i + rho_j, as (rho_i + rho_j)^2 <= 2 rho_i^2 + 2 rho_j^2; the factor
+// covers the FP32 rounding of r^2 (a few 1e-7 relative, also in the kick's
+// far-tile form). Out of line: only the escape mode and positions outside
+// FP32's range come here.
+__device__ __noinline__ float crude_reach_fp64(const Dev &d, const DriftArgs &a, int64_t r, double m0,
+                                               double qx, double qy, double qz, double vx, double vy,
+                                               double vz) {
+    const double mu = a.G * m0;
+    const double rH = a.hill_fixed ? d.rH_fixed[r] : hill(qx, qy, qz, d.hfac[r]);
+    const float rHb = round_up_f(rH * (1.0 + 1e-6));
+    d.rH_bound[r] = rHb;
+    const double rr = sqrt(qx * qx + qy * qy + qz * qz);
+    double rho;
+    if (d.escape_reach) {
+        rho = a.a_E * (double)rHb + fabs(a.tau) * sqrt(2.0 * mu / rr) + 1e-12 * rr;
+    } else {
+        double Om = sqrt(mu / (rr * rr * rr));
+        double ux = vx + Om * qy, uy = vy - Om * qx, uz = vz;
+        double u = sqrt(ux * ux + uy * uy + uz * uz);
+        double w = fabs(a.kick_span) * a.a_allow * (double)d.amag[r];
+        double sh = fmin(0.8, 2.5 * Om * fabs(a.tau));
+        double F = 2.0 / (1.0 - sh);
+        rho = F * (a.a_E * (double)rHb + fabs(a.tau) * (u + w)) + 1e-12 * rr;
+    }
+    return round_up_f(2.0 * rho * rho * (1.0 + 4e-6));
+}
+
+// The same reach in FP32, every term raised by its rounding: the positions are
+// within 2^-24 and the velocities within 2^-23 of the FP64 ones, Omega and the
+// products within 1e-6, so u is within 2e-6 (|v| + Omega r) and the rest within
+// 4e-6, relative; rho is raised by 1e-5. In FP64 the reach was two thirds of
+// this kernel's 107 FP64 instructions per row (217 us on 1.06e6 rows).
+__device__ __forceinline__ float crude_reach(const Dev &d, const DriftArgs &a, int64_t r, int sys,
+                                             float x, float y, float z, float r2, float vx, float vy,
+                                             float vz) {
+    const float rr = sqrtf(r2), mu = p64::lead(d.kmu[3 * sys], 0), tau = a.tau_f;
+    const float rHb = (a.hill_fixed ? p64::lead(d.rH_fixed[r], 0) : rr * p64::lead(d.hfac[r], 0)) *
+                      (1.0f + 4e-6f);
+    d.rH_bound[r] = rHb;
+    const float Om = sqrtf(mu / r2 / rr);
+    const float ux = fmaf(Om, y, vx), uy = fmaf(-Om, x, vy);
+    const float u = sqrtf(fmaf(ux, ux, fmaf(uy, uy, vz * vz))) +
+                    2e-6f * (fabsf(vx) + fabsf(vy) + fabsf(vz) + Om * rr);
+    const float w = a.span_f * a.a_allow_f * d.amag[r];
+    const float sh = fminf(0.8f, 2.5f * Om * tau);
+    const float rho = 2.0f / (1.0f - sh) * fmaf(a.a_E_f, rHb, tau * (u + w)) * (1.0f + 1e-5f);
+    return 2.0f * rho * rho;
+}
 
 // the systems whose shifts a CTA of k_drift_pack forms once (its rows span at
 // most this many systems; else every row forms its own)
@@ -133,53 +196,21 @@ __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
     }
     d.q[r] = qx; d.q[R + r] = qy; d.q[2 * R + r] = qz;
     if (a.vs != d.v) { d.v[r] = vx; d.v[R + r] = vy; d.v[2 * R + r] = vz; }
-    float xh, xl, yh, yl, zh, zl;
-    split_ds(qx, xh, xl);
-    split_ds(qy, yh, yl);
-    split_ds(qz, zh, zl);
+    // float pairs hi + lo of the position (its three-part split, rounded to two)
+    const p64::F3 sx = p64::split3(qx), sy = p64::split3(qy), sz = p64::split3(qz);
+    const float xh = sx.h, yh = sy.h, zh = sz.h;
+    const float xl = sx.m + sx.l, yl = sy.m + sy.l, zl = sz.m + sz.l;
     const double mm = d.m[r];
     float reach = 0.0f;
     if (a.flag_next && r != star) {
-        // crude reach rho_i = F_i (R_i + |tau| (u_i + w_i)):
-        //   R_i  a_E times a bound on this step's Hill radius
-        //   u_i  speed relative to the local circular velocity Omega (z x Q)
-        //   w_i  bound on the velocity change of the kick(s) before the Kepler
-        //        drift: (tau/2) 1.01 |a| (the last kick was at the same
-        //        separations), or with merged kicks tau 2 |a| (the last kick
-        //        was a step earlier); the finisher checks the bound
-        //   F_i  stretch for the Keplerian shear over one step
-        const double m0 = d.m[star];
-        const double mu = a.G * m0;
-        double rH;
-        if (a.hill_fixed) {
-            rH = d.rH_fixed[r];
-        } else {
-            rH = hill(qx, qy, qz, d.hfac[r]);  // positions do not change in the kick
-        }
-        if (a.flag_next == 2) d.rH[r] = rH;
-        float rHb = round_up_f(rH * (1.0 + 1e-6));
-        d.rH_bound[r] = rHb;
-        double rr = sqrt(qx * qx + qy * qy + qz * qz);
-        double rho;
-        if (d.escape_reach) {
-            // QYM_SEARCH_ESCAPE, the paper's crude sweep (Sec. 2.4): a_E times
-            // the Hill radius plus the distance covered at the escape
-            // velocity over the step
-            rho = a.a_E * (double)rHb + fabs(a.tau) * sqrt(2.0 * mu / rr) + 1e-12 * rr;
-        } else {
-            double Om = sqrt(mu / (rr * rr * rr));
-            double ux = vx + Om * qy, uy = vy - Om * qx, uz = vz;
-            double u = sqrt(ux * ux + uy * uy + uz * uz);
-            double w = fabs(a.kick_span) * a.a_allow * (double)d.amag[r];
-            double sh = fmin(0.8, 2.5 * Om * fabs(a.tau));
-            double F = 2.0 / (1.0 - sh);
-            rho = F * (a.a_E * (double)rHb + fabs(a.tau) * (u + w)) + 1e-12 * rr;
-        }
-        // kernels test r^2 < c_i + c_j with c = 2 rho^2 >= ... a superset of
-        // r < rho_i + rho_j, as (rho_i + rho_j)^2 <= 2 rho_i^2 + 2 rho_j^2;
-        // the factor covers the FP32 rounding of r^2 (a few 1e-7 relative,
-        // also in the kick's far-tile form)
-        reach = round_up_f(2.0 * rho * rho * (1.0 + 4e-6));
+        if (a.flag_next == 2)  // positions do not change in the kick
+            d.rH[r] = a.hill_fixed ? d.rH_fixed[r] : hill(qx, qy, qz, d.hfac[r]);
+        const float r2 = fmaf(xh, xh, fmaf(yh, yh, zh * zh));
+        if (!d.escape_reach && r2 > 1e-24f && r2 < 1e24f)
+            reach = crude_reach(d, a, r, sys, xh, yh, zh, r2, p64::lead(vx, 0), p64::lead(vy, 0),
+                                p64::lead(vz, 0));
+        else
+            reach = crude_reach_fp64(d, a, r, d.m[star], qx, qy, qz, vx, vy, vz);
     }
     // heavy bodies enter the FP32 tiles with zero mass (their pull is added
     // in FP64 by the finisher); they still take part in the encounter search
@@ -205,6 +236,10 @@ cudaError_t launch_drift_pack_from(const Dev &d, const double *qs, const double 
     a.G = G;
     a.flag_next = flag_next;
     a.hill_fixed = hill_fixed;
+    a.tau_f = (float)std::fabs(tau);
+    a.span_f = (float)std::fabs(kick_span);
+    a.a_E_f = (float)a_E;
+    a.a_allow_f = (float)a_allow;
     int tb = 256;
     k_drift_pack<<<(unsigned)((d.rows + tb - 1) / tb), tb, 0, st>>>(d, a);
     return cudaGetLastError();
@@ -226,43 +261,67 @@ struct FinishArgs {
     int skip_whole;     // v of systems flagged in d.wh_flag stays
 };
 
-constexpr int kFinLanes = 4;  // lanes that share one row's partial sums
-
+// L threads share one position's partial sums and heavy bodies: thread group q
+// of the CTA adds the slots q, q + L, ... and the heavies q, q + L, ... (loads
+// coalesced across positions, dependent FP64 adds in chains 1/L as long), the
+// groups' parts added as a fixed tree; the first group then does the rows' own
+// work in full warps. (An FP64 instruction costs the same for one active lane as
+// for 32: with the four parts on neighbouring lanes the row work ran on eight
+// lanes per warp, 492 us on 1.06e6 rows.)
+template <int L>
 __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
-    // kFinLanes lanes per position of the kick's order: lane q sums the slots
-    // q, q + 4, ... (loads coalesced across positions, dependent FP64 adds in
-    // chains a quarter as long), the four parts added in a fixed tree; lane 0
-    // then does the row's own work
-    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t pr = gt / kFinLanes;
-    const int q = (int)(gt % kFinLanes);
+    constexpr int RB = 256 / L;
+    const int t = threadIdx.x % RB, q = threadIdx.x / RB;
+    const int64_t pr = (int64_t)blockIdx.x * RB + t;
     const int64_t R = d.rows;
     double ax = 0.0, ay = 0.0, az = 0.0;
-    const int nslots = d.kick_cnt ? 1 : d.splits;  // the kick added its slots into slot 0
-    if (pr < R)
-        for (int s = q; s < nslots; s += kFinLanes) {
+    int64_t r = 0;
+    int sys = 0;
+    bool live = pr < R;
+    if (live) {
+        r = d.perm ? d.perm[pr] : pr;
+        sys = d.sys_of[r];
+        live = r != d.offsets[sys] &&  // the star
+               !(d.own_hi > 0 && (r < d.own_lo || r >= d.own_hi));  // another GPU's row
+    }
+    if (live) {
+        const int nslots = d.kick_cnt ? 1 : d.splits;  // the kick added its slots into slot 0
+        for (int s = q; s < nslots; s += L) {
             const double *p = d.apart + (int64_t)s * 3 * R;
             ax += p[pr];
             ay += p[R + pr];
             az += p[2 * R + pr];
         }
+        if (d.heavy_split) {
+            const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
+            heavy_pull(d.heavy_rows + h0, q, L, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q,
+                       d.m, R, a.G, ax, ay, az);
+        }
+    }
+    if (L > 1) {
+        __shared__ double sh[L > 1 ? L - 1 : 1][3][RB];
+        if (q > 0) {
+            sh[q - 1][0][t] = ax;
+            sh[q - 1][1][t] = ay;
+            sh[q - 1][2][t] = az;
+        }
+        __syncthreads();
+        if (q > 0) return;
+        double p[L > 1 ? L : 1][3];
+        p[0][0] = ax; p[0][1] = ay; p[0][2] = az;
 #pragma unroll
-    for (int o = 1; o < kFinLanes; o <<= 1) {
-        ax += __shfl_xor_sync(0xffffffffu, ax, o);
-        ay += __shfl_xor_sync(0xffffffffu, ay, o);
-        az += __shfl_xor_sync(0xffffffffu, az, o);
+        for (int k = 1; k < L; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) p[k][c] = sh[k - 1][c][t];
+#pragma unroll
+        for (int w = 1; w < L; w *= 2)
+#pragma unroll
+            for (int k = 0; k < L; k += 2 * w)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) p[k][c] += p[k + w][c];
+        ax = p[0][0]; ay = p[0][1]; az = p[0][2];
     }
-    if (pr >= R || q != 0) return;
-    const int64_t r = d.perm ? d.perm[pr] : pr;
-    if (d.own_hi > 0 && (r < d.own_lo || r >= d.own_hi)) return;  // another GPU's row
-    const int sys = d.sys_of[r];
-    const int64_t star = d.offsets[sys];
-    if (r == star) return;
-    if (d.heavy_split) {
-        int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
-        heavy_pull(d.heavy_rows + h0, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q, d.m, R,
-                   a.G, ax, ay, az);
-    }
+    if (!live) return;
     double vx = a.v[r], vy = a.v[R + r], vz = a.v[2 * R + r];
     if (!(a.skip_whole && d.wh_flag && d.wh_flag[sys])) {
         vx += a.dt * ax;
@@ -270,10 +329,10 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
         vz += a.dt * az;
         a.v[r] = vx; a.v[R + r] = vy; a.v[2 * R + r] = vz;
     }
-    float an = round_up_f(sqrt(ax * ax + ay * ay + az * az));
+    const float an = p64::norm_up(ax, ay, az);
     if (a.check) {
         if (d.vmax)  // the binned search's bound takes the largest |v| entering the drift
-            atomicMax(d.vmax + sys, __float_as_int(round_up_f(sqrt(vx * vx + vy * vy + vz * vz))));
+            atomicMax(d.vmax + sys, __float_as_int(p64::norm_up(vx, vy, vz)));
         double rH = a.hill_fixed ? d.rH_fixed[r] : hill(a.q[r], a.q[R + r], a.q[2 * R + r], d.hfac[r]);
         d.rH[r] = rH;
         // check 1 (the search fused into this kick): audit its reach
@@ -299,8 +358,15 @@ cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, doubl
     a.a_allow = (float)a_allow;
     a.check = check;
     a.hill_fixed = hill_fixed;
-    int tb = 256;
-    k_finish<<<(unsigned)((kFinLanes * d.rows + tb - 1) / tb), tb, 0, st>>>(d, a);
+    // groups of 4 or 8 threads a row where there are that many slots to add (8
+    // also halves the chain of a small system), one where there are few
+    const int nslots = d.kick_cnt ? 1 : d.splits;
+    if (nslots >= 16)
+        k_finish<8><<<(unsigned)((d.rows + 31) / 32), 256, 0, st>>>(d, a);
+    else if (nslots >= 4)
+        k_finish<4><<<(unsigned)((d.rows + 63) / 64), 256, 0, st>>>(d, a);
+    else
+        k_finish<1><<<(unsigned)((d.rows + 255) / 256), 256, 0, st>>>(d, a);
     return cudaGetLastError();
 }
 
