@@ -112,6 +112,7 @@ __device__ __forceinline__ void push_encounter(const Dev &d, int i, int j) {
 // rigorous test of the crude candidates: (d.q, d.v) hold the state entering
 // the Kepler drift, (d.q1, d.v1) the Kepler result
 __global__ void __launch_bounds__(256) k_refine(Dev d, double tau, double a_E) {
+    chain_wait();
     unsigned long long n = d.ctr[C_NCAND];
     if (n > (unsigned long long)d.max_cand) n = d.max_cand;
     const int64_t R = d.rows;
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(256) k_refine(Dev d, double tau, double a_E) {
 // exact re-search of rows whose crude bounds were exceeded: the row against
 // every other body of its system (one CTA per row)
 __global__ void __launch_bounds__(256) k_rescan(Dev d, double tau, double a_E) {
+    chain_wait();
     unsigned long long n = d.ctr[C_NRESCAN];
     if (n > (unsigned long long)d.rows) n = d.rows;
     const int64_t R = d.rows;
@@ -145,8 +147,8 @@ __global__ void __launch_bounds__(256) k_rescan(Dev d, double tau, double a_E) {
 }
 
 cudaError_t launch_refine(const Dev &d, double tau, double a_E, cudaStream_t st) {
-    k_refine<<<2 * 152, 256, 0, st>>>(d, tau, a_E);
-    k_rescan<<<152, 256, 0, st>>>(d, tau, a_E);
+    launch_chain(k_refine, 2 * 152, 256, 0, st, d, tau, a_E);
+    launch_chain(k_rescan, 152, 256, 0, st, d, tau, a_E);
     return cudaGetLastError();
 }
 
@@ -171,6 +173,7 @@ __device__ __forceinline__ int uf_find(int *uf, int x, int &guard) {
 }
 
 __global__ void k_uf_hook(Dev d) {
+    chain_wait();
     unsigned long long n = d.ctr[C_NENC];
     if (n > (unsigned long long)d.max_enc) n = d.max_enc;
     int *uf = d.uf;
@@ -193,6 +196,7 @@ __global__ void k_uf_hook(Dev d) {
 
 // per-block counts of roots, for an ordered numbering of the sets
 __global__ void __launch_bounds__(1024) k_uf_count(Dev d, int32_t *blk) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int isroot = 0;
     if (r < d.rows) {
@@ -205,6 +209,7 @@ __global__ void __launch_bounds__(1024) k_uf_count(Dev d, int32_t *blk) {
 
 // exclusive scan of the block counts (one CTA)
 __global__ void __launch_bounds__(1024) k_scan_blocks(Dev d, int32_t *blk, int nblk) {
+    chain_wait();
     __shared__ int32_t part[1024];
     int per = (nblk + 1023) / 1024;
     int b0 = threadIdx.x * per;
@@ -230,6 +235,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(Dev d, int32_t *blk, int n
 // number the roots in row order: sid[root] = set index; members are counted
 __global__ void __launch_bounds__(1024) k_uf_number(Dev d, const int32_t *blk, int32_t *sid,
                                                     int32_t *size) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int isroot = 0;
     if (r < d.rows) isroot = (d.uf[r] == (int)r);
@@ -262,6 +268,7 @@ __global__ void __launch_bounds__(1024) k_uf_number(Dev d, const int32_t *blk, i
 // previous step)
 __global__ void __launch_bounds__(256) k_uf_members(Dev d, const int32_t *sid, int32_t *size,
                                                     unsigned long long *rc_bits, double a_H) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= d.rows) return;
     int p = d.uf[r];
@@ -280,6 +287,7 @@ __global__ void __launch_bounds__(256) k_uf_members(Dev d, const int32_t *sid, i
 // set_start = exclusive scan of set sizes (one CTA); the fill counters reset
 __global__ void __launch_bounds__(1024) k_scan_sets(Dev d, int32_t *size, int32_t *fill,
                                                     unsigned long long *rc_bits) {
+    chain_wait();
     __shared__ int32_t part[1024];
     int n = (int)d.ctr[C_NSETS];
     if (n > d.max_sets) n = d.max_sets;
@@ -322,8 +330,10 @@ __global__ void __launch_bounds__(1024) k_scan_sets(Dev d, int32_t *size, int32_
 }
 
 __global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int32_t *fill) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= d.rows) return;
+    d.hcost[r] = 0;  // k_uf_members has read the last step's; this step's sets write theirs
     int p = d.uf[r];
     if (p < 0) return;
     int guard = 0;
@@ -336,15 +346,15 @@ __global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int
 
 cudaError_t launch_sets_impl(const Dev &d, double a_H, const SetScratch &s, cudaStream_t st) {
     int nblk = (int)((d.rows + 1023) / 1024);
-    k_uf_hook<<<152, 256, 0, st>>>(d);
-    k_uf_count<<<nblk, 1024, 0, st>>>(d, s.blk);
-    k_scan_blocks<<<1, 1024, 0, st>>>(d, s.blk, nblk);
-    k_uf_number<<<nblk, 1024, 0, st>>>(d, s.blk, s.sid, s.size);
+    launch_chain(k_uf_hook, 152, 256, 0, st, d);
+    launch_chain(k_uf_count, nblk, 1024, 0, st, d, s.blk);
+    launch_chain(k_scan_blocks, 1, 1024, 0, st, d, s.blk, nblk);
+    launch_chain(k_uf_number, nblk, 1024, 0, st, d, s.blk, s.sid, s.size);
     int tb = 256;
     unsigned g = (unsigned)((d.rows + tb - 1) / tb);
-    k_uf_members<<<g, tb, 0, st>>>(d, s.sid, s.size, s.rc_bits, a_H);
-    k_scan_sets<<<1, 1024, 0, st>>>(d, s.size, s.fill, s.rc_bits);
-    k_uf_place<<<g, tb, 0, st>>>(d, s.sid, s.fill);
+    launch_chain(k_uf_members, g, tb, 0, st, d, s.sid, s.size, s.rc_bits, a_H);
+    launch_chain(k_scan_sets, 1, 1024, 0, st, d, s.size, s.fill, s.rc_bits);
+    launch_chain(k_uf_place, g, tb, 0, st, d, s.sid, s.fill);
     return cudaGetLastError();
 }
 

@@ -33,6 +33,7 @@ __device__ __noinline__ double potential_fp64(double dx, double dy, double dz, d
 __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, const double *m,
                                                      const double *q, const double *v, double G,
                                                      double *pe, double *ps) {
+    chain_wait();
     __shared__ D4 s_q[ET];
     __shared__ float4 s_h[ET], s_m[ET], s_l[ET];
     __shared__ int s_hi[2][ET / 32];
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, c
 __global__ void __launch_bounds__(256) k_energy_final(EnergyPlan pl, const int64_t *offsets,
                                                       const double *m, const double *pe,
                                                       const double *ps, double *E) {
+    chain_wait();
     const int s = blockIdx.x;
     const int64_t b0 = pl.block0 ? pl.block0[s] : 0, b1 = pl.block0 ? pl.block0[s + 1] : pl.nblocks;
     double t[4] = {0.0, 0.0, 0.0, 0.0};
@@ -188,8 +190,8 @@ cudaError_t launch_energy(const EnergyPlan &pl, int32_t nsys, const int64_t *off
                           const double *m, const double *q, const double *v, double G, double *part,
                           double *E, cudaStream_t st) {
     double *ps = part + (int64_t)pl.nblocks * pl.nranges;
-    k_energy_pairs<<<(unsigned)((int64_t)pl.nblocks * pl.nranges), ET, 0, st>>>(pl, R, m, q, v, G, part, ps);
-    k_energy_final<<<nsys, 256, 0, st>>>(pl, offsets, m, part, ps, E);
+    launch_chain(k_energy_pairs, (unsigned)((int64_t)pl.nblocks * pl.nranges), ET, 0, st, pl, R, m, q, v, G, part, ps);
+    launch_chain(k_energy_final, nsys, 256, 0, st, pl, offsets, m, part, ps, E);
     return cudaGetLastError();
 }
 

@@ -1065,6 +1065,7 @@ constexpr int kPlanCap = 4096;
 // integrates only the sets whose lowest row is its own: sets are numbered in
 // the order of their lowest rows, so those are the index range [s_lo, s_hi).
 __global__ void __launch_bounds__(1024) k_hermite_plan(Dev d, int ncl) {
+    chain_wait();
     __shared__ unsigned long long key[kPlanCap];
     __shared__ int wsum[32];
     __shared__ int s_range[2];
@@ -1175,6 +1176,7 @@ __global__ void __launch_bounds__(1024) k_hermite_plan(Dev d, int ncl) {
 // the order of a counter, so CTAs freed early take more.
 template <int CLT>
 __global__ void __cluster_dims__(CLT, 1, 1) __launch_bounds__(HTHREADS, 2) k_hermite(Dev d, HermArgs h) {
+    chain_wait();
     static_assert(CLT == 2 || CLT == 4 || CLT == 8, "a cluster is 2, 4 or 8 CTAs");
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
@@ -1196,6 +1198,7 @@ __global__ void __cluster_dims__(CLT, 1, 1) __launch_bounds__(HTHREADS, 2) k_her
 // integrated only its own sets, the other sets' members get their states and
 // costs from the GPUs that did
 __global__ void k_uf_clear_members(Dev d) {
+    chain_wait();
     const unsigned long long n = min(d.ctr[C_NMEM], (unsigned long long)d.max_members);
     for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (unsigned long long)gridDim.x * blockDim.x)
@@ -1240,20 +1243,17 @@ cudaError_t launch_hermite(const Dev &d, const qym_params &p, double tau, cudaSt
     const int grid = (cls == 2 ? 1 : 2) * 152;  // CTAs per SM x SMs
     static_assert(2 * 152 / 4 <= kHermMaxClusters && 152 / 2 <= kHermMaxClusters,
                   "more clusters than plan entries");
-    k_hermite_plan<<<1, 1024, 0, st>>>(d, grid / cls);
+    launch_chain(k_hermite_plan, 1, 1024, 0, st, d, grid / cls);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // the plan has read the previous step's costs; this step's sets write theirs
-    e = cudaMemsetAsync(d.hcost, 0, sizeof(int32_t) * (size_t)d.rows, st);
-    if (e != cudaSuccess) return e;
     switch (cls) {
-    case 2: k_hermite<2><<<grid, HTHREADS, kHermSmem, st>>>(d, h); break;
-    case 4: k_hermite<4><<<grid, HTHREADS, kHermSmem, st>>>(d, h); break;
-    default: k_hermite<8><<<grid, HTHREADS, kHermSmem, st>>>(d, h); break;
+    case 2: launch_chain(k_hermite<2>, grid, HTHREADS, kHermSmem, st, d, h); break;
+    case 4: launch_chain(k_hermite<4>, grid, HTHREADS, kHermSmem, st, d, h); break;
+    default: launch_chain(k_hermite<8>, grid, HTHREADS, kHermSmem, st, d, h); break;
     }
     e = cudaGetLastError();
     if (e != cudaSuccess || d.own_hi == 0) return e;
-    k_uf_clear_members<<<152, 256, 0, st>>>(d);
+    launch_chain(k_uf_clear_members, 152, 256, 0, st, d);
     return cudaGetLastError();
 }
 

@@ -124,6 +124,7 @@ __device__ __forceinline__ int newton_f32(const KepEq &eq, double lo, double hi,
 
 template <bool MLP>
 __global__ void __launch_bounds__(256) k_kepler(KeplerArgs a) {
+    chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int iters = 0;
     const bool act = k < a.n;
@@ -350,9 +351,9 @@ cudaError_t launch_kepler(const KeplerArgs &a, cudaStream_t st) {
     int threads = 256;
     int64_t blocks = (a.n + threads - 1) / threads;
     if (a.guess == QYM_GUESS_MLP && a.mlp_w)
-        k_kepler<true><<<(unsigned)blocks, threads, 0, st>>>(a);
+        launch_chain(k_kepler<true>, (unsigned)blocks, threads, 0, st, a);
     else
-        k_kepler<false><<<(unsigned)blocks, threads, 0, st>>>(a);
+        launch_chain(k_kepler<false>, (unsigned)blocks, threads, 0, st, a);
     return cudaGetLastError();
 }
 

@@ -301,6 +301,7 @@ __device__ __forceinline__ void push_flag(const KickArgs &a, int i, int j0, int 
 // FORCE = false: the crude search alone (no partial sums written)
 template <int IPT, bool FLAG, bool FORCE>
 __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
+    chain_wait();
     __shared__ float4 s_a[TILE / 2], s_b[TILE / 2], s_c[TILE / 2], s_d[TILE / 2];
     __shared__ float4 s_fa[TILE / 2], s_fb[TILE / 2];
     const JPairs sp{s_a, s_b, s_c, s_d};
@@ -477,6 +478,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
 // candidates are rows. The last CTA to finish resets the entry counter for
 // the next search kick.
 __global__ void __launch_bounds__(256) k_flag_chunks(KickArgs a, unsigned long long *done) {
+    chain_wait();
     unsigned long long n = *(volatile unsigned long long *)a.nfchunk;
     if (n > (unsigned long long)a.max_fchunk) n = a.max_fchunk;
     const int lane = threadIdx.x & 31;
@@ -537,6 +539,7 @@ __device__ __noinline__ double weight_fp64(double dx, double dy, double dz, doub
 // float range take plain FP64.
 template <int IPT, bool FLAG, bool FORCE>
 __global__ void __launch_bounds__(256) k_kick_fp64(KickArgs a) {
+    chain_wait();
     __shared__ D4 s_q[TILE];
     __shared__ float4 s_h[TILE], s_m[TILE], s_l[TILE];  // (x, y, z, G m) in three parts
     __shared__ float s_rho[TILE];
@@ -729,9 +732,9 @@ template <bool FLAG, bool FORCE>
 static cudaError_t launch_mixed(const KickArgs &a, int nitems, int threads, int ipt,
                                 cudaStream_t st) {
     switch (ipt) {
-    case 1: k_kick_mixed<1, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
-    case 2: k_kick_mixed<2, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
-    case 4: k_kick_mixed<4, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
+    case 1: launch_chain(k_kick_mixed<1, FLAG, FORCE>, nitems, threads, 0, st, a); break;
+    case 2: launch_chain(k_kick_mixed<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
+    case 4: launch_chain(k_kick_mixed<4, FLAG, FORCE>, nitems, threads, 0, st, a); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -741,9 +744,9 @@ template <bool FLAG, bool FORCE>
 static cudaError_t launch_f64(const KickArgs &a, int nitems, int threads, int ipt,
                               cudaStream_t st) {
     switch (ipt) {
-    case 1: k_kick_fp64<1, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
-    case 2: k_kick_fp64<2, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
-    default: k_kick_fp64<2, FLAG, FORCE><<<nitems, threads, 0, st>>>(a); break;
+    case 1: launch_chain(k_kick_fp64<1, FLAG, FORCE>, nitems, threads, 0, st, a); break;
+    case 2: launch_chain(k_kick_fp64<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
+    default: launch_chain(k_kick_fp64<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
     }
     return cudaGetLastError();
 }
@@ -756,6 +759,7 @@ static cudaError_t launch_f64(const KickArgs &a, int nitems, int threads, int ip
 // x_hi - c, then x_lo added), beside its G m.
 __global__ void __launch_bounds__(TILE) k_tile_prep(int64_t npos, const float4 *pos,
                                                     const float4 *lo, float4 *far, float4 *tile) {
+    chain_wait();
     __shared__ float s_m[TILE / 32][7];
     __shared__ float s_c[3];
     const int64_t p = 1 + (int64_t)blockIdx.x * TILE + threadIdx.x;
@@ -830,7 +834,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     a.chunk = d.item_chunk;
     if (a.far_tiles) {
         const int64_t ntiles = (d.rows - 1 + TILE - 1) / TILE;
-        k_tile_prep<<<(unsigned)ntiles, TILE, 0, st>>>(d.rows, d.pk_pos, d.pk_lo, d.far, d.tile);
+        launch_chain(k_tile_prep, (unsigned)ntiles, TILE, 0, st, d.rows, d.pk_pos, d.pk_lo, d.far, d.tile);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -846,7 +850,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
         int64_t blocks = (d.rows + 63) / 64;
         if (blocks > 4 * 152) blocks = 4 * 152;
         if (blocks < 1) blocks = 1;
-        k_flag_chunks<<<(int)blocks, 256, 0, st>>>(a, d.ctr + C_FCDONE);
+        launch_chain(k_flag_chunks, (int)blocks, 256, 0, st, a, d.ctr + C_FCDONE);
         return cudaGetLastError();
     }
     if (flag == KICK_FORCE) return launch_f64<false, true>(a, d.nitems, threads, ipt, st);
@@ -916,6 +920,7 @@ size_t accel_single_workspace(int64_t rows, int prec) {
 // bodies past the cap stay in the FP32 tiles
 __global__ void __launch_bounds__(1024) k_heavy_thr_single(int64_t rows, const double *m,
                                                            double heavy_mass, int32_t *hl) {
+    chain_wait();
     // same compaction as k_heavy_single with the threshold taken from m[0]
     __shared__ int base;
     __shared__ int wsum[32];
@@ -946,6 +951,7 @@ __global__ void __launch_bounds__(1024) k_heavy_thr_single(int64_t rows, const d
 
 __global__ void k_pack_single(int64_t rows, const double *m, const double *q, double G,
                               const int32_t *hl, float4 *pos, float4 *lo, const int32_t *inv) {
+    chain_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows) return;
     const int64_t pi = inv ? inv[i] : i;  // the kick's order
@@ -970,6 +976,7 @@ constexpr int SL = 8;
 __global__ void __launch_bounds__(256) k_sum_partials(int64_t rows, int32_t splits, const double *apart,
                                                       const int32_t *hl, const double *m, const double *q,
                                                       double G, double *a, const int32_t *inv) {
+    chain_wait();
     constexpr int RB = 256 / SL;
     __shared__ double sh[SL][3][RB];
     const int t = threadIdx.x % RB, g = threadIdx.x / RB;
@@ -1012,7 +1019,7 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
     int32_t *hl = nullptr;
     if (prec == QYM_KICK_MIXED && heavy_mass > 0.0) {
         hl = (int32_t *)(w + L.off_heavy);
-        k_heavy_thr_single<<<1, 1024, 0, st>>>(rows, m, heavy_mass, hl);
+        launch_chain(k_heavy_thr_single, 1, 1024, 0, st, rows, m, heavy_mass, hl);
     }
     if (L.sorted) {
         // the bodies in Morton order, as the step's kick holds them
@@ -1032,7 +1039,7 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
     }
     cudaError_t e;
     if (prec == QYM_KICK_MIXED) {
-        k_pack_single<<<(unsigned)((rows + tb - 1) / tb), tb, 0, st>>>(rows, m, q, G, hl, d.pk_pos,
+        launch_chain(k_pack_single, (unsigned)((rows + tb - 1) / tb), tb, 0, st, rows, m, q, G, hl, d.pk_pos,
                                                                         d.pk_lo, d.inv);
         e = launch_kick_tiles(d, prec, 0, G, L.tune.threads, L.tune.ipt, st);
     } else {
@@ -1042,7 +1049,7 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
         e = launch_f64<false, true>(ka, L.nitems, L.tune.threads, L.tune.ipt, st);
     }
     if (e != cudaSuccess) return e;
-    k_sum_partials<<<(unsigned)((rows + 256 / SL - 1) / (256 / SL)), 256, 0, st>>>(rows, d.splits, d.apart, hl, m,
+    launch_chain(k_sum_partials, (unsigned)((rows + 256 / SL - 1) / (256 / SL)), 256, 0, st, rows, d.splits, d.apart, hl, m,
                                                                      q, G, a, d.inv);
     return cudaGetLastError();
 }

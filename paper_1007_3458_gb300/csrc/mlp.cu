@@ -33,6 +33,7 @@ constexpr int NRED = 448;    // column sums: W1 (4 x 64), b1, b2, W3
 __global__ void __launch_bounds__(256) k_mlp_forward(int64_t n, const float *__restrict__ w,
                                                      const float *__restrict__ u,
                                                      float *__restrict__ y) {
+    chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float uu[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (k < n) {
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
                                                     const float *__restrict__ rows, int64_t n,
                                                     float inv_n, float *__restrict__ part,
                                                     float *__restrict__ lpart) {
+    chain_wait();
     __shared__ __align__(16) __nv_bfloat16 s_w2[64 * LDT];             // bf16 W2[j][k]
     __shared__ __align__(16) uint32_t s_t[2][16 * GWARPS * LDT / 2];   // h1, dL/dp2 [row][col]
     __shared__ __align__(16) float s_w1[256];                          // bf16-rounded W1
@@ -368,6 +370,7 @@ __global__ void __launch_bounds__(RT) k_mlp_reduce(const float *__restrict__ par
                                                    float *__restrict__ v, int adam, float lr,
                                                    float beta1, float beta2, float eps, float bc1,
                                                    float bc2) {
+    chain_wait();
     constexpr int SL = RT / 32;
     __shared__ float s_hi[SL][32], s_lo[SL][32];
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
@@ -417,7 +420,7 @@ size_t mlp_workspace_bytes() { return (size_t)MAXBLK * NW * sizeof(float) + MAXB
 cudaError_t launch_mlp_forward(int64_t n, const float *w, const float *u, float *y, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const int64_t blocks = (n + 255) / 256;
-    k_mlp_forward<<<(unsigned)blocks, 256, 0, st>>>(n, w, u, y);
+    launch_chain(k_mlp_forward, (unsigned)blocks, 256, 0, st, n, w, u, y);
     return cudaGetLastError();
 }
 
@@ -427,7 +430,7 @@ static cudaError_t grad_partials(int64_t n, const float *w, const float *rows, v
     nblk = (int)(tiles < GRID ? tiles : GRID);
     float *part = static_cast<float *>(work);
     float *lpart = part + (size_t)MAXBLK * NW;
-    k_mlp_grad<<<nblk, GT, 0, st>>>(w, rows, n, 1.0f / (float)n, part, lpart);
+    launch_chain(k_mlp_grad, nblk, GT, 0, st, w, rows, n, 1.0f / (float)n, part, lpart);
     return cudaGetLastError();
 }
 
@@ -438,7 +441,7 @@ cudaError_t launch_mlp_grad(int64_t n, const float *w, const float *rows, float 
     if (e != cudaSuccess) return e;
     float *part = static_cast<float *>(work);
     float *lpart = part + (size_t)MAXBLK * NW;
-    k_mlp_reduce<<<(NW + 31) / 32, RT, 0, st>>>(part, nblk, lpart, 1.0f / (float)n, grad, loss,
+    launch_chain(k_mlp_reduce, (NW + 31) / 32, RT, 0, st, part, nblk, lpart, 1.0f / (float)n, grad, loss,
                                                    nullptr, nullptr, nullptr, 0, 0.f, 0.f, 0.f, 0.f,
                                                    1.f, 1.f);
     return cudaGetLastError();
@@ -453,7 +456,7 @@ cudaError_t launch_mlp_adam(float *w, float *m, float *v, const float *grad, int
                             float beta1, float beta2, float eps, cudaStream_t st) {
     float bc1, bc2;
     bias_corr(t, beta1, beta2, bc1, bc2);
-    k_mlp_reduce<<<(NW + 31) / 32, RT, 0, st>>>(grad, 1, nullptr, 0.f, nullptr, nullptr, w, m, v,
+    launch_chain(k_mlp_reduce, (NW + 31) / 32, RT, 0, st, grad, 1, nullptr, 0.f, nullptr, nullptr, w, m, v,
                                                    1, lr, beta1, beta2, eps, bc1, bc2);
     return cudaGetLastError();
 }
@@ -477,7 +480,7 @@ cudaError_t launch_mlp_train(float *w, float *m, float *v, int64_t t0, const flo
                            0.5 * ((double)lr - (double)lr_final) * (1.0 + std::cos(kPi * (double)s / (double)S));
         float bc1, bc2;
         bias_corr(t0 + s + 1, beta1, beta2, bc1, bc2);
-        k_mlp_reduce<<<(NW + 31) / 32, RT, 0, st>>>(part, nblk, lpart, 1.0f / (float)len, nullptr,
+        launch_chain(k_mlp_reduce, (NW + 31) / 32, RT, 0, st, part, nblk, lpart, 1.0f / (float)len, nullptr,
                                                        losses ? losses + s : nullptr, w, m, v, 1,
                                                        (float)lrs, beta1, beta2, eps, bc1, bc2);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/qym.h"
@@ -209,6 +210,32 @@ __device__ __forceinline__ void heavy_pull(const int32_t *hs, int k0, int step, 
 void set_thread_error(const std::string &msg);
 
 // ---------------------------------------------------------------- launches
+// Launches in a chain: each kernel may be set up while the one before it in
+// the stream still runs (programmatic dependent launch) and waits for it, and
+// for the visibility of all it wrote, in chain_wait(), its first statement. The
+// kernels of a small step are a few microseconds each, so the ~1 us a launch
+// otherwise takes between them counts. chain_wait() first lets the next kernel
+// be set up in turn; a kernel's end still implies the end of every one before.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         A &&...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 // Each returns cudaSuccess or the launch error. All work goes on `st`.
 
 // kepler.cu

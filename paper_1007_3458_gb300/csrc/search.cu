@@ -81,6 +81,7 @@ __device__ __forceinline__ int fbits(float f) {
 __device__ __forceinline__ float fvalue(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 __global__ void __launch_bounds__(256) k_search_prep(Dev d, SearchArgs s) {
+    chain_wait();
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t p = gt >> 2;           // position
     const int k = (int)(gt & 3);         // axis (3: idle)
@@ -249,6 +250,7 @@ __device__ __forceinline__ bool cubic_may_flag(const float *oi0, const float *oi
 
 // tile pairs of a system whose boxes overlap, appended to the active list
 __global__ void __launch_bounds__(256) k_search_tilepairs(Dev d, SearchArgs s) {
+    chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool hit = false;
     int2 tp = make_int2(0, 0);
@@ -271,6 +273,7 @@ __global__ void __launch_bounds__(256) k_search_tilepairs(Dev d, SearchArgs s) {
 // one CTA per overlapping tile pair (I, J): tile J staged in shared memory
 // relative to a point of tile I, each thread one body of I against all of J
 __global__ void __launch_bounds__(kSTile) k_search_pairs(Dev d, SearchArgs s) {
+    chain_wait();
     __shared__ float4 j_lo[kSTile], j_hi[kSTile];
     __shared__ float j_o0[kSTile][3], j_o1[kSTile][3], j_v0[kSTile][3], j_v1[kSTile][3];
     __shared__ float j_thr[kSTile];
@@ -342,9 +345,9 @@ cudaError_t launch_binned_search(const Dev &d, const SearchArgs &s0, double tau,
     s.tau = tau;
     s.a_E = a_E;
     if (s.ntiles <= 0) return cudaSuccess;
-    k_search_prep<<<(unsigned)((4 * d.rows + 255) / 256), 256, 0, st>>>(d, s);
-    k_search_tilepairs<<<(unsigned)((s.ntpairs + 255) / 256), 256, 0, st>>>(d, s);
-    k_search_pairs<<<4 * 152, kSTile, 0, st>>>(d, s);
+    launch_chain(k_search_prep, (unsigned)((4 * d.rows + 255) / 256), 256, 0, st, d, s);
+    launch_chain(k_search_tilepairs, (unsigned)((s.ntpairs + 255) / 256), 256, 0, st, d, s);
+    launch_chain(k_search_pairs, 4 * 152, kSTile, 0, st, d, s);
     return cudaGetLastError();
 }
 

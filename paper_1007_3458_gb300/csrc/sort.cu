@@ -35,10 +35,12 @@ __device__ __forceinline__ int fkey(float f) {
 __device__ __forceinline__ float kfloat(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 __global__ void k_sort_box_init(int *box) {
+    chain_wait();
     if (threadIdx.x < 6) box[threadIdx.x] = 0x7fffffff;
 }
 
 __global__ void __launch_bounds__(256) k_sort_box(int64_t rows, const double *q, int *box) {
+    chain_wait();
     float m[6] = {3e38f, 3e38f, 3e38f, 3e38f, 3e38f, 3e38f};
     for (int64_t r = 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
          r += (int64_t)gridDim.x * blockDim.x) {
@@ -83,6 +85,7 @@ __device__ __forceinline__ uint32_t morton_code(int64_t rows, const double *q, i
 }
 __global__ void __launch_bounds__(256) k_sort_keys(int64_t rows, const double *q, const int *box,
                                                     uint32_t *keys, int32_t *vals) {
+    chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // body k = row k + 1
     if (k >= rows - 1) return;
     const int64_t r = k + 1;
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(256) k_sort_keys(int64_t rows, const double *q
 // digit counts of each block: hist[digit * nblk + block]
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(int64_t n, const uint32_t *keys,
                                                             int shift, uint32_t *hist, int nblk) {
+    chain_wait();
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -107,6 +111,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(int64_t n, const uin
 
 // exclusive scan of the m = 256 * nblk counts (one CTA)
 __global__ void __launch_bounds__(1024) k_sort_scan(uint32_t *hist, int m) {
+    chain_wait();
     __shared__ uint32_t part[1024];
     const int per = (m + 1023) / 1024;
     const int b0 = threadIdx.x * per;
@@ -135,6 +140,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(int64_t n, const 
                                                                const int32_t *vin, uint32_t *kout,
                                                                int32_t *vout, int shift,
                                                                const uint32_t *hist, int nblk) {
+    chain_wait();
     constexpr int NW = kSortThreads / 32;
     __shared__ uint32_t run[256];
     __shared__ uint32_t wc[NW][256];
@@ -170,6 +176,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(int64_t n, const 
 // position p (1 .. rows-1) holds row perm[p]; inv[perm[p]] = p; row 0 stays
 __global__ void __launch_bounds__(256) k_sort_perm(int64_t rows, const int32_t *vals,
                                                     int32_t *perm, int32_t *inv) {
+    chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k == 0) {
         perm[0] = 0;
@@ -187,19 +194,19 @@ cudaError_t launch_sort_rows(int64_t rows, const double *q, const SortScratch &s
     if (n < 1) return cudaSuccess;
     const int nblk = (int)sort_blocks(n);
     const unsigned g = (unsigned)((n + 255) / 256);
-    k_sort_box_init<<<1, 32, 0, st>>>(s.box);
-    k_sort_box<<<(unsigned)std::min<int64_t>(g, 4 * 152), 256, 0, st>>>(rows, q, s.box);
-    k_sort_keys<<<g, 256, 0, st>>>(rows, q, s.box, s.k0, s.v0);
+    launch_chain(k_sort_box_init, 1, 32, 0, st, s.box);
+    launch_chain(k_sort_box, (unsigned)std::min<int64_t>(g, 4 * 152), 256, 0, st, rows, q, s.box);
+    launch_chain(k_sort_keys, g, 256, 0, st, rows, q, s.box, s.k0, s.v0);
     uint32_t *ka = s.k0, *kb = s.k1;
     int32_t *va = s.v0, *vb = s.v1;
     for (int shift = 0; shift < 32; shift += 8) {
-        k_sort_hist<<<nblk, kSortThreads, 0, st>>>(n, ka, shift, s.hist, nblk);
-        k_sort_scan<<<1, 1024, 0, st>>>(s.hist, 256 * nblk);
-        k_sort_scatter<<<nblk, kSortThreads, 0, st>>>(n, ka, va, kb, vb, shift, s.hist, nblk);
+        launch_chain(k_sort_hist, nblk, kSortThreads, 0, st, n, ka, shift, s.hist, nblk);
+        launch_chain(k_sort_scan, 1, 1024, 0, st, s.hist, 256 * nblk);
+        launch_chain(k_sort_scatter, nblk, kSortThreads, 0, st, n, ka, va, kb, vb, shift, s.hist, nblk);
         std::swap(ka, kb);
         std::swap(va, vb);
     }
-    k_sort_perm<<<g, 256, 0, st>>>(rows, va, perm, inv);
+    launch_chain(k_sort_perm, g, 256, 0, st, rows, va, perm, inv);
     return cudaGetLastError();
 }
 

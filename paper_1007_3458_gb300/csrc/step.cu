@@ -13,6 +13,7 @@ namespace qym {
 // chunk partial sums of m_i v_i (bodies only), deterministic tree order
 // (a chunk lies in one system, ch.z: its star row is known per chunk)
 __global__ void __launch_bounds__(256) k_mom_chunks(Dev d) {
+    chain_wait();
     const int4 ch = d.mchunks[blockIdx.x];
     const int64_t star = d.offsets[ch.z];
     double sx = 0.0, sy = 0.0, sz = 0.0;
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) k_mom_chunks(Dev d) {
 // adds the chunks l, l + 32, ... in order, then a fixed shuffle tree (the
 // loads of a long system's chunk list overlap instead of following one another)
 __global__ void k_mom_final(Dev d) {
+    chain_wait();
     const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (s >= d.nsys) return;
@@ -54,8 +56,8 @@ __global__ void k_mom_final(Dev d) {
 }
 
 cudaError_t launch_momentum(const Dev &d, cudaStream_t st) {
-    k_mom_chunks<<<d.nmchunks, 256, 0, st>>>(d);
-    k_mom_final<<<(unsigned)((32 * (int64_t)d.nsys + 127) / 128), 128, 0, st>>>(d);
+    launch_chain(k_mom_chunks, d.nmchunks, 256, 0, st, d);
+    launch_chain(k_mom_final, (unsigned)((32 * (int64_t)d.nsys + 127) / 128), 128, 0, st, d);
     return cudaGetLastError();
 }
 
@@ -151,6 +153,7 @@ __device__ __forceinline__ float crude_reach(const Dev &d, const DriftArgs &a, i
 constexpr int kDriftSys = 8;
 
 __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
+    chain_wait();
     // The shifts (h S_k) / m0 of the CTA's systems, the same quotients every
     // row would form: FP64 divisions cost ~385 cycles and ~8 FP64-pipe
     // instructions here, six per row otherwise.
@@ -241,7 +244,7 @@ cudaError_t launch_drift_pack_from(const Dev &d, const double *qs, const double 
     a.a_E_f = (float)a_E;
     a.a_allow_f = (float)a_allow;
     int tb = 256;
-    k_drift_pack<<<(unsigned)((d.rows + tb - 1) / tb), tb, 0, st>>>(d, a);
+    launch_chain(k_drift_pack, (unsigned)((d.rows + tb - 1) / tb), tb, 0, st, d, a);
     return cudaGetLastError();
 }
 
@@ -270,6 +273,7 @@ struct FinishArgs {
 // lanes per warp, 492 us on 1.06e6 rows.)
 template <int L>
 __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
+    chain_wait();
     constexpr int RB = 256 / L;
     const int t = threadIdx.x % RB, q = threadIdx.x / RB;
     const int64_t pr = (int64_t)blockIdx.x * RB + t;
@@ -362,16 +366,17 @@ cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, doubl
     // also halves the chain of a small system), one where there are few
     const int nslots = d.kick_cnt ? 1 : d.splits;
     if (nslots >= 16)
-        k_finish<8><<<(unsigned)((d.rows + 31) / 32), 256, 0, st>>>(d, a);
+        launch_chain(k_finish<8>, (unsigned)((d.rows + 31) / 32), 256, 0, st, d, a);
     else if (nslots >= 4)
-        k_finish<4><<<(unsigned)((d.rows + 63) / 64), 256, 0, st>>>(d, a);
+        launch_chain(k_finish<4>, (unsigned)((d.rows + 63) / 64), 256, 0, st, d, a);
     else
-        k_finish<1><<<(unsigned)((d.rows + 255) / 256), 256, 0, st>>>(d, a);
+        launch_chain(k_finish<1>, (unsigned)((d.rows + 255) / 256), 256, 0, st, d, a);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- Hill radii at init
 __global__ void k_hill_init(Dev d, double G) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= d.rows) return;
     const int64_t R = d.rows;
@@ -382,7 +387,7 @@ __global__ void k_hill_init(Dev d, double G) {
 
 cudaError_t launch_hill_init(const Dev &d, double G, cudaStream_t st) {
     int tb = 256;
-    k_hill_init<<<(unsigned)((d.rows + tb - 1) / tb), tb, 0, st>>>(d, G);
+    launch_chain(k_hill_init, (unsigned)((d.rows + tb - 1) / tb), tb, 0, st, d, G);
     return cudaGetLastError();
 }
 
@@ -393,6 +398,7 @@ cudaError_t launch_hill_init(const Dev &d, double G, cudaStream_t st) {
 // Needs d.S = sum m v of the input velocities and, for the forward direction,
 // the total body mass per system in mt.
 __global__ void k_mass_total(Dev d, double *mt) {
+    chain_wait();
     int s = blockIdx.x;
     int64_t lo = d.offsets[s], hi = d.offsets[s + 1];
     double t = 0.0;
@@ -409,6 +415,7 @@ __global__ void k_mass_total(Dev d, double *mt) {
 }
 
 __global__ void k_to_dh(Dev d, int inverse, const double *mt, double *vout) {
+    chain_wait();
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= d.rows) return;
     const int64_t R = d.rows;
@@ -428,10 +435,10 @@ cudaError_t launch_to_dh_impl(const Dev &d, int inverse, double *vout, double *m
     cudaError_t e = launch_momentum(d, st);
     if (e != cudaSuccess) return e;
     if (!inverse) {
-        k_mass_total<<<d.nsys, 256, 0, st>>>(d, mt_scratch);
+        launch_chain(k_mass_total, d.nsys, 256, 0, st, d, mt_scratch);
     }
     int tb = 256;
-    k_to_dh<<<(unsigned)((d.rows + tb - 1) / tb), tb, 0, st>>>(d, inverse, mt_scratch, vout);
+    launch_chain(k_to_dh, (unsigned)((d.rows + tb - 1) / tb), tb, 0, st, d, inverse, mt_scratch, vout);
     return cudaGetLastError();
 }
 
