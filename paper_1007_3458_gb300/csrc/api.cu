@@ -1078,7 +1078,7 @@ extern "C" qym_status qym_step(qym_ctx *c, double tau, int64_t nsteps) {
         if ((e = cudaMemsetAsync(d.status, 0, sizeof(int32_t), st))) return e;
         if (sort) {
             if ((e = launch_sort_rows(d.rows, d.q, c->sortw, d.perm, d.inv, st))) return e;
-            c->launches += 16;
+            c->launches += sort_launches(d.rows);
         }
         if ((e = launch_momentum(d, st))) return e;
         if ((e = launch_drift_pack_from(d, d.q, d.v, 0.0, 0.5 * tau, tau, p.a_E, p.G,
@@ -1114,7 +1114,7 @@ extern "C" qym_status qym_step(qym_ctx *c, double tau, int64_t nsteps) {
                                          fused_search(c), p.hill_fixed, st,
                                          p.merge_kicks ? tau : 0.5 * tau,
                                          p.merge_kicks ? 2.0 : 1.01));
-            c->launches += 17;
+            c->launches += sort_launches(d.rows) + 1;
         }
         if (graphs && (interior >= 2 || c->g_step.exec)) CK(c, replay(c, c->g_step, tau, one));
         else CK(c, one());

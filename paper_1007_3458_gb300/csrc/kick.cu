@@ -756,19 +756,12 @@ static cudaError_t launch_f64(const KickArgs &a, int nitems, int threads, int ip
 // middle, a radius R >= max |Q_j - c| (rounded up, with room for the lo parts
 // and the rounding of c), the largest crude-search reach c_j of its bodies
 // (tile[1].w), and each body's offset o_j = Q_j - c, rounded once (two-sum of
-// x_hi - c, then x_lo added), beside its G m.
-__global__ void __launch_bounds__(TILE) k_tile_prep(int64_t npos, const float4 *pos,
-                                                    const float4 *lo, float4 *far, float4 *tile) {
-    chain_wait();
+// x_hi - c, then x_lo added), beside its G m. One CTA of TILE threads per tile;
+// (P, L): the packs of position p of this thread.
+__device__ __forceinline__ void tile_prep(bool act, int64_t p, const float4 &P, const float4 &L,
+                                          float4 *far, float4 *tile) {
     __shared__ float s_m[TILE / 32][7];
     __shared__ float s_c[3];
-    const int64_t p = 1 + (int64_t)blockIdx.x * TILE + threadIdx.x;
-    const bool act = p < npos;
-    float4 P = make_float4(0.f, 0.f, 0.f, 0.f), L = P;
-    if (act) {
-        P = pos[p];
-        L = lo[p];
-    }
     // (m[6]: minus the largest search reach c of the tile's bodies)
     float m[7] = {act ? P.x : 3e38f, act ? P.y : 3e38f, act ? P.z : 3e38f,
                   act ? -P.x : 3e38f, act ? -P.y : 3e38f, act ? -P.z : 3e38f,
@@ -805,6 +798,19 @@ __global__ void __launch_bounds__(TILE) k_tile_prep(int64_t npos, const float4 *
                              ds_add(P.z, -s_c[2], L.z), P.w);
 }
 
+__global__ void __launch_bounds__(TILE) k_tile_prep(int64_t npos, const float4 *pos,
+                                                    const float4 *lo, float4 *far, float4 *tile) {
+    chain_wait();
+    const int64_t p = 1 + (int64_t)blockIdx.x * TILE + threadIdx.x;
+    const bool act = p < npos;
+    float4 P = make_float4(0.f, 0.f, 0.f, 0.f), L = P;
+    if (act) {
+        P = pos[p];
+        L = lo[p];
+    }
+    tile_prep(act, p, P, L, far, tile);
+}
+
 cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int threads, int ipt,
                               cudaStream_t st) {
     if (d.nitems <= 0) return cudaSuccess;
@@ -832,7 +838,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     a.blk_cnt = d.kick_cnt;
     a.splits = d.splits;
     a.chunk = d.item_chunk;
-    if (a.far_tiles) {
+    if (a.far_tiles && !d.tiles_ready) {
         const int64_t ntiles = (d.rows - 1 + TILE - 1) / TILE;
         launch_chain(k_tile_prep, (unsigned)ntiles, TILE, 0, st, d.rows, d.pk_pos, d.pk_lo, d.far, d.tile);
         cudaError_t e = cudaGetLastError();
@@ -874,8 +880,9 @@ constexpr int64_t kSingleSortMin = 2048;
 static SingleLayout single_layout(int64_t rows, int prec) {
     SingleLayout L;
     int64_t nb = rows - 1;
-    // (the fixed scratch of qym_accel_dev_static holds about 2^17.6 row slots)
-    L.tune = default_kick_tune(nb, nb, prec, std::max<int64_t>(1, 200000 / rows));
+    // slots that fit the fixed scratch of qym_accel_dev_static beside 60 bytes a
+    // row of packs, order and tiles; beyond its sizes, 16
+    L.tune = default_kick_tune(nb, nb, prec, rows <= QYM_STATIC_MAX_ROWS ? (((8 << 20) - (1 << 17)) / rows - 60) / 24 : 16);
     KickTune &t = L.tune;
     int64_t ti = (int64_t)t.threads * t.ipt;
     L.sorted = prec == QYM_KICK_MIXED && nb >= kSingleSortMin;
@@ -890,22 +897,27 @@ static SingleLayout single_layout(int64_t rows, int prec) {
     const int64_t packs = prec == QYM_KICK_MIXED ? rows : 0;
     L.off_pos = o; o = al(o + sizeof(float4) * packs);
     L.off_lo = o; o = al(o + sizeof(float4) * packs);
-    L.off_apart = o; o = al(o + sizeof(double) * 3 * rows * t.splits);
     L.off_heavy = o; o = al(o + sizeof(int32_t) * (QYM_HEAVY_CAP + 1));
     L.off_perm = L.off_inv = L.off_box = L.off_k0 = L.off_k1 = L.off_v0 = L.off_v1 = L.off_hist = 0;
     L.off_far = L.off_tile = 0;
     if (L.sorted) {
         L.off_perm = o; o = al(o + sizeof(int32_t) * rows);
         L.off_inv = o; o = al(o + sizeof(int32_t) * rows);
+        L.off_far = o; o = al(o + sizeof(float4) * rows);
+        L.off_tile = o; o = al(o + sizeof(float4) * 3 * (size_t)((rows - 1 + TILE - 1) / TILE));
+    }
+    // the partial slots, over the sort's scratch (dead by then)
+    L.off_apart = o;
+    size_t end = al(o + sizeof(double) * 3 * rows * t.splits);
+    if (L.sorted) {
         L.off_box = o; o = al(o + sizeof(int) * 8);
         L.off_k0 = o; o = al(o + sizeof(uint32_t) * rows);
         L.off_k1 = o; o = al(o + sizeof(uint32_t) * rows);
         L.off_v0 = o; o = al(o + sizeof(int32_t) * rows);
         L.off_v1 = o; o = al(o + sizeof(int32_t) * rows);
         L.off_hist = o; o = al(o + sizeof(uint32_t) * 256 * (size_t)sort_blocks(rows));
-        L.off_far = o; o = al(o + sizeof(float4) * rows);
-        L.off_tile = o; o = al(o + sizeof(float4) * 3 * (size_t)((rows - 1 + TILE - 1) / TILE));
     }
+    o = std::max(o, end);
     L.total = o;
     return L;
 }
@@ -915,58 +927,48 @@ size_t accel_single_workspace(int64_t rows, int prec) {
     return single_layout(rows, prec).total;
 }
 
-// heavy list of one system: the first QYM_HEAVY_CAP bodies (ascending rows)
-// with m >= heavy_mass * m[0]; hl[QYM_HEAVY_CAP] receives their count, and the
-// bodies past the cap stay in the FP32 tiles
-__global__ void __launch_bounds__(1024) k_heavy_thr_single(int64_t rows, const double *m,
-                                                           double heavy_mass, int32_t *hl) {
-    chain_wait();
-    // same compaction as k_heavy_single with the threshold taken from m[0]
-    __shared__ int base;
-    __shared__ int wsum[32];
-    const double thr = heavy_mass * m[0];
-    if (threadIdx.x == 0) base = 0;
-    __syncthreads();
-    for (int64_t r0 = 1; r0 < rows; r0 += blockDim.x) {
-        int64_t r = r0 + threadIdx.x;
-        int hv = (r < rows && m[r] >= thr) ? 1 : 0;
-        unsigned b = __ballot_sync(0xffffffffu, hv);
-        int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        if (lane == 0) wsum[w] = __popc(b);
-        __syncthreads();
-        int before = 0;
-        for (int k = 0; k < w; ++k) before += wsum[k];
-        int pos = base + before + __popc(b & ((1u << lane) - 1u));
-        if (hv && pos < QYM_HEAVY_CAP) hl[pos] = (int32_t)r;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int t = 0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += wsum[k];
-            base += t;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) hl[QYM_HEAVY_CAP] = base < QYM_HEAVY_CAP ? base : QYM_HEAVY_CAP;
+// the packs of row r: its position as hi + lo floats and its G m (zero for a
+// heavy body in the list; the list is ascending, so bodies past a full one are
+// those beyond its last row)
+__device__ __forceinline__ void pack_row(int64_t rows, int64_t r, const double *m, const double *q,
+                                         double G, const int32_t *hl, double thr, float4 &P, float4 &L) {
+    const p64::F3 x = p64::split3(q[r]), y = p64::split3(q[rows + r]), z = p64::split3(q[2 * rows + r]);
+    const double mr = m[r];
+    float gm = (float)(G * mr);
+    if (hl && mass_reaches(mr, thr) && (hl[QYM_HEAVY_CAP] < QYM_HEAVY_CAP || r <= hl[QYM_HEAVY_CAP - 1])) gm = 0.0f;
+    P = make_float4(x.h, y.h, z.h, gm);
+    L = make_float4(x.m + x.l, y.m + y.l, z.m + z.l, 0.0f);
 }
 
-__global__ void k_pack_single(int64_t rows, const double *m, const double *q, double G,
-                              const int32_t *hl, float4 *pos, float4 *lo, const int32_t *inv) {
+// packs and tile data of a sorted system, by position: one CTA per tile
+__global__ void __launch_bounds__(TILE) k_pack_tiles(int64_t rows, const double *m, const double *q,
+                                                     double G, double heavy_mass, const int32_t *hl,
+                                                     const int32_t *perm, float4 *pos, float4 *lo,
+                                                     float4 *far, float4 *tile) {
     chain_wait();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    const int64_t pi = inv ? inv[i] : i;  // the kick's order
-    float xh, xl, yh, yl, zh, zl;
-    split_ds(q[i], xh, xl);
-    split_ds(q[rows + i], yh, yl);
-    split_ds(q[2 * rows + i], zh, zl);
-    float gm = (float)(G * m[i]);
-    if (hl) {
-        int nh = hl[QYM_HEAVY_CAP];
-        for (int k = 0; k < nh; ++k)
-            if (hl[k] == (int32_t)i) gm = 0.0f;
+    const int64_t p = 1 + (int64_t)blockIdx.x * TILE + threadIdx.x;
+    const bool act = p < rows;
+    float4 P = make_float4(0.f, 0.f, 0.f, 0.f), L = P;
+    if (act) {
+        pack_row(rows, perm[p], m, q, G, hl, heavy_mass * m[0], P, L);
+        pos[p] = P;
+        lo[p] = L;
     }
-    pos[pi] = make_float4(xh, yh, zh, gm);
-    lo[pi] = make_float4(xl, yl, zl, 0.0f);
+    tile_prep(act, p, P, L, far, tile);
+}
+
+// heavy list and packs of a small system in row order, one CTA
+__global__ void __launch_bounds__(1024) k_pack_small(int64_t rows, const double *m, const double *q,
+                                                     double G, double heavy_mass, int32_t *hl,
+                                                     float4 *pos, float4 *lo) {
+    chain_wait();
+    __shared__ int s[33];
+    if (hl) {
+        heavy_list(rows, m, heavy_mass, hl, s);
+        __syncthreads();  // (the list is read back below by the CTA that wrote it)
+    }
+    for (int64_t r = threadIdx.x; r < rows; r += blockDim.x)
+        pack_row(rows, r, m, q, G, hl, heavy_mass * m[0], pos[r], lo[r]);
 }
 
 // per row the sum of its slots and the heavy bodies' pull, SL threads a row
@@ -1013,34 +1015,32 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
     d.nitems = L.nitems;
     d.splits = L.tune.splits;
     d.item_chunk = L.chunk;
-    int tb = 256;
     // heavy split (mixed kick only): threshold relative to the star mass m[0],
     // read on the device
-    int32_t *hl = nullptr;
-    if (prec == QYM_KICK_MIXED && heavy_mass > 0.0) {
-        hl = (int32_t *)(w + L.off_heavy);
-        launch_chain(k_heavy_thr_single, 1, 1024, 0, st, rows, m, heavy_mass, hl);
-    }
-    if (L.sorted) {
-        // the bodies in Morton order, as the step's kick holds them
-        d.perm = (int32_t *)(w + L.off_perm);
-        d.inv = (int32_t *)(w + L.off_inv);
-        d.far = (float4 *)(w + L.off_far);
-        d.tile = (float4 *)(w + L.off_tile);
-        SortScratch ss;
-        ss.box = (int *)(w + L.off_box);
-        ss.k0 = (uint32_t *)(w + L.off_k0);
-        ss.k1 = (uint32_t *)(w + L.off_k1);
-        ss.v0 = (int32_t *)(w + L.off_v0);
-        ss.v1 = (int32_t *)(w + L.off_v1);
-        ss.hist = (uint32_t *)(w + L.off_hist);
-        cudaError_t e = launch_sort_rows(rows, q, ss, d.perm, d.inv, st);
-        if (e != cudaSuccess) return e;
-    }
+    int32_t *hl = prec == QYM_KICK_MIXED && heavy_mass > 0.0 ? (int32_t *)(w + L.off_heavy) : nullptr;
     cudaError_t e;
     if (prec == QYM_KICK_MIXED) {
-        launch_chain(k_pack_single, (unsigned)((rows + tb - 1) / tb), tb, 0, st, rows, m, q, G, hl, d.pk_pos,
-                                                                        d.pk_lo, d.inv);
+        if (L.sorted) {
+            // the bodies in Morton order, as the step's kick holds them
+            d.perm = (int32_t *)(w + L.off_perm);
+            d.inv = (int32_t *)(w + L.off_inv);
+            d.far = (float4 *)(w + L.off_far);
+            d.tile = (float4 *)(w + L.off_tile);
+            d.tiles_ready = 1;
+            SortScratch ss;
+            ss.box = (int *)(w + L.off_box);
+            ss.k0 = (uint32_t *)(w + L.off_k0);
+            ss.k1 = (uint32_t *)(w + L.off_k1);
+            ss.v0 = (int32_t *)(w + L.off_v0);
+            ss.v1 = (int32_t *)(w + L.off_v1);
+            ss.hist = (uint32_t *)(w + L.off_hist);
+            if ((e = launch_sort_rows(rows, q, ss, d.perm, d.inv, st, m, heavy_mass, hl)) != cudaSuccess)
+                return e;
+            launch_chain(k_pack_tiles, (unsigned)((rows - 1 + TILE - 1) / TILE), TILE, 0, st, rows, m, q,
+                         G, heavy_mass, hl, d.perm, d.pk_pos, d.pk_lo, d.far, d.tile);
+        } else {
+            launch_chain(k_pack_small, 1, 1024, 0, st, rows, m, q, G, heavy_mass, hl, d.pk_pos, d.pk_lo);
+        }
         e = launch_kick_tiles(d, prec, 0, G, L.tune.threads, L.tune.ipt, st);
     } else {
         KickArgs ka{};

@@ -300,6 +300,16 @@ __device__ __forceinline__ float lead(double x, int k) {
     return __uint_as_float(f | ((unsigned)hi & 0x80000000u));
 }
 
+// x rounded to the nearest float, by its bits where the result is normal
+__device__ __forceinline__ float to_float(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7ff) - 896;
+    if (e <= 0 || e >= 254) return (float)x;  // (the conversion holds the FP64 pipe)
+    const unsigned b = ((unsigned)e << 23) | ((hi << 3 | lo >> 29) & 0x7fffffu);
+    const unsigned rest = (lo << 3) | (b & 1u);  // above half, or at half with an odd b
+    return __uint_as_float((b + (rest > 0x80000000u ? 1u : 0u)) | (hi & 0x80000000u));
+}
+
 // an upper bound of |(x, y, z)| within 1e-6, without an FP64 instruction (an
 // FP64 square root is ten); NaN or infinite for such inputs
 __device__ __forceinline__ float norm_up(double x, double y, double z) {

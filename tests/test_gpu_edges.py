@@ -158,3 +158,54 @@ def test_energy_blocks(torch, sizes, lu, mu):
             work = torch.empty(q.qym_energy_workspace_bytes(n + 1), dtype=torch.uint8, device="cuda")
             q.qym_energy_dev(n + 1, t(ms[s]), t(qs[s].T), t(vs[s].T), 1.0, out, work)
             assert abs(out.item() - ref) <= (n + 8) * L(2.0) ** -53 * mag
+
+
+@pytest.mark.parametrize("n", [2048, 8192, 8193, 16385, 32769, 65536, 65537])
+def test_order_sizes(torch, n):
+    """The Morton order at the edges of the one-cluster sort (words per thread
+    1, 2, 4, 8) and just past it, with a third of the bodies at one point
+    (equal codes keep row order): the host's (code, row) order."""
+    from test_gpu_order import _host_order
+    w = W.outer_disk(n - 4, 1e-10, seed=n)
+    x = w.q.copy()
+    x[5:5 + n // 3] = x[5]
+    sim = q.Simulation(w.m, x, w.v, w.offsets, encounters=0)
+    assert np.array_equal(sim.order(), _host_order(sim.state()[0]))
+    sim.close()
+
+
+@pytest.mark.parametrize("n,heavies", [(1, 1), (2, 0), (33, 2), (257, 4), (700, 300), (2047, 4), (2048, 4),
+                                       (2305, 0), (6145, 256), (9000, 300)])
+def test_mixed_accel_sizes(torch, n, heavies):
+    """The mixed kick over one-CTA packs, tile packs, launch shapes and heavy
+    lists (none, full, and longer than the 256 bodies it holds), with the
+    caller's and the fixed scratch. A pair carries a few 2^-22 (separation,
+    reciprocal square root cubed, products) and a sum of 64 pairs in FP32 at
+    most 2^-18 of its terms' magnitudes; heavy bodies in the list are exact."""
+    rng = np.random.default_rng(n)
+    w = W.outer_disk(max(n - 4, 0), 1e-9, seed=3)
+    x, m = w.q[:n + 1].copy(), w.m[:n + 1].copy()
+    m[1:] = 10.0 ** rng.uniform(-11, -8, n)
+    m[1 + rng.permutation(n)[:heavies]] = 10.0 ** rng.uniform(-6, -3, heavies)
+    md, xd = torch.from_numpy(m).cuda(), torch.from_numpy(np.ascontiguousarray(x.T)).cuda()
+    a, b = (torch.empty((3, n + 1), dtype=torch.float64, device="cuda") for _ in range(2))
+    work = torch.empty(q.qym_accel_workspace_bytes(n + 1, q.QYM_KICK_MIXED), dtype=torch.uint8, device="cuda")
+    q.qym_accel_dev(n + 1, md, xd, a, 1.0, q.QYM_KICK_MIXED, work)
+    q.qym_accel_dev_static(n + 1, md, xd, b, 1.0, q.QYM_KICK_MIXED)
+    assert torch.equal(a, b)
+    ref, mag = _accel_ref(m, x, 1.0) if n <= 700 else _accel_ref64(torch, m, x)
+    err = np.abs(a.cpu().numpy().T - np.asarray(ref, dtype=np.float64))
+    assert np.all(err <= 2.0 ** -18 * np.asarray(mag, dtype=np.float64)), float((err / (mag + 1e-300)).max())
+
+
+def _accel_ref64(torch, m, x):
+    xb, gm = torch.from_numpy(x[1:]).cuda(), torch.from_numpy(m[1:]).cuda()
+    a, mag = np.zeros(x.shape), np.zeros(x.shape)
+    for i in range(0, len(xb), 512):
+        d = xb[None] - xb[i:i + 512, None]
+        r2 = (d * d).sum(-1)
+        s = torch.where(r2 > 0, gm / (r2 * r2.sqrt()), torch.zeros_like(r2))
+        t = s[..., None] * d
+        a[1 + i:1 + i + 512] = t.sum(1).cpu().numpy()
+        mag[1 + i:1 + i + 512] = t.abs().sum(1).cpu().numpy()
+    return a, mag
