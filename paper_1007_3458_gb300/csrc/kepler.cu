@@ -2,9 +2,20 @@
 // star (Sec. 2 and the Appendix: f and g functions, Stumpff C and S, the
 // universal Kepler equation F(x) = 0 solved by Laguerre's method, n = 5).
 //
-// One thread per body, FP64 throughout. Structure-of-arrays loads are
-// coalesced; q0, v0 are kept and the result goes to separate buffers because
-// the encounter test needs both ends of the step (Sec. 2.3 item 4).
+// One thread per body, the state and the solve in FP64. Structure-of-arrays
+// loads are coalesced; q0, v0 are kept and the result goes to separate buffers
+// because the encounter test needs both ends of the step (Sec. 2.3 item 4).
+//
+// The kernel is bound by the FP64 pipe: one warp instruction per ~19 cycles and
+// SM, whatever the number of active lanes. So (1) only arithmetic on the state
+// goes there: comparisons, scalings by powers of two and conversions work on the
+// bits, the residual's scale and (until it matters) the root's bracket are FP32
+// with the margins stated at each, square roots and reciprocals take one step from FP32
+// (pair64.cuh); (2) F' and F'' are formed only where a step follows; (3) a warp
+// iterates while at least kPackBelow of its lanes do, then the CTA's unfinished
+// bodies are packed into full warps (some 5% of bodies need another evaluation,
+// that is four of five warps). 1,048,576 test particles with NEWTON32: 369 FP64
+// warp instructions per warp before.
 //
 // With the learned guess (MLP = true) each warp first evaluates the guess
 // network for its 32 bodies on the tensor cores (mlp.cuh); the iteration then
@@ -28,15 +39,16 @@ namespace qym {
 // S are NaN, which the iteration treats as a point beyond the root.
 __device__ __forceinline__ void stumpff(double y, double &C, double &S) {
     int k = 0;
-    if (!(fabs(y) < 1.0)) {
+    const int hi = p64::hi_abs(y);
+    if (hi >= 0x3ff00000) {
         // |y| in [2^e, 2^(e+1)): k = floor(e/2) + 1 puts y / 4^k in [1/4, 1)
-        const int e = ((__double2hiint(y) >> 20) & 0x7ff) - 1023;
+        const int e = (hi >> 20) - 1023;
         k = e / 2 + 1;
         if (k > 64) {
             C = S = __longlong_as_double(0x7ff8000000000000ll);
             return;
         }
-        y *= __hiloint2double((1023 - 2 * k) << 20, 0);
+        y = p64::mul_pow2(y, -2 * k);
     }
     // 1/(2n+2)! and 1/(2n+3)! for n = 0..8, alternating signs
     C = 1.0 / 2.0 + y * (-1.0 / 24.0 + y * (1.0 / 720.0 + y * (-1.0 / 40320.0 +
@@ -47,22 +59,31 @@ __device__ __forceinline__ void stumpff(double y, double &C, double &S) {
         y * (-1.0 / 355687428096000.0 + y * (1.0 / 121645100408832000.0))))))));
     for (int i = 0; i < k; ++i) {
         const double c1 = fma(-y, S, 1.0);
-        S = 0.25 * fma(c1, C, S);
-        C = 0.5 * c1 * c1;
-        y *= 4.0;
+        S = p64::mul_pow2(fma(c1, C, S), -2);
+        C = p64::mul_pow2(c1 * c1, -1);
+        y = p64::mul_pow2(y, 2);
     }
 }
 
 // F, F', F'' of the universal Kepler equation (Appendix), sig = r0.v0/sqrt(mu)
 struct KepEq {
     double sqmu_dt, r0, sig, alpha, b;  // b = 1 - r0 alpha
-    __device__ __forceinline__ void eval(double x, double &F, double &Fp, double &Fpp,
-                                         double &C, double &S) const {
-        double x2 = x * x;
-        double y = alpha * x2;
-        stumpff(y, C, S);
-        double oyS = 1.0 - y * S;
-        F = sig * x2 * C + b * x2 * x * S + r0 * x - sqmu_dt;
+    // F at x with C, S; sc: the sum of F's terms' magnitudes in FP32 (within
+    // 1e-6; NaN or out of FP32's range where a term is)
+    __device__ __forceinline__ double value(double x, double &C, double &S, float &sc) const {
+        const double x2 = x * x;
+        stumpff(alpha * x2, C, S);
+        const double t1 = sig * x2, t2 = b * x2 * x;
+        sc = fabsf(p64::lead(sqmu_dt, 0)) + fabsf(p64::lead(t1, 0) * p64::lead(C, 0)) +
+             fabsf(p64::lead(t2, 0) * p64::lead(S, 0)) + p64::lead(r0, 0) * fabsf(p64::lead(x, 0));
+        return t1 * C + t2 * S + r0 * x - sqmu_dt;
+    }
+    __device__ __forceinline__ double scale(double x, double C, double S) const {
+        const double x2 = x * x;
+        return fabs(sqmu_dt) + fabs(sig * x2 * C) + fabs(b * x2 * x * S) + r0 * fabs(x);
+    }
+    __device__ __forceinline__ void slopes(double x, double C, double S, double &Fp, double &Fpp) const {
+        const double x2 = x * x, y = alpha * x2, oyS = 1.0 - y * S;
         Fp = sig * x * oyS + b * x2 * C + r0;
         Fpp = sig * (1.0 - y * C) + b * x * oyS;
     }
@@ -91,6 +112,110 @@ __device__ __forceinline__ void stumpff_f32(float y, float &C, float &S) {
     }
 }
 
+// The iteration of one body between two evaluations of F
+struct KepIter {
+    double x, lo, hi;      // the point to evaluate next; the root's bracket
+    bool rough;            // its outer bound is the FP32 one (kep_bracket), then
+    float inside;          // a magnitude below the FP64 form's
+    double dx_old;         // last step
+    double x_prev, res_prev;  // settle: the point the last step started from, its relative residual
+    double C, S;           // Stumpff values of the last evaluation
+    int it, iters;         // evaluations of this pass; iterations counted in all
+    bool settle;           // the last step was at the rounding level
+    bool conv, cs_at_x;    // C, S hold the Stumpff values at the final x
+};
+
+// Root bracket: F(0) = -sqrt(mu) dt and F' = r >= r_p (periapsis distance), so
+// the root lies between 0 and the outer bound sqrt(mu) dt / r_p; for an unbound
+// orbit also |x| <= 700 / sqrt(-alpha), past which C and S overflow. Widened by
+// 1e-12 for the rounding of r_p = p / (1 + e).
+__device__ __noinline__ void kep_outer_exact(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                             double &lo, double &hi) {
+    const int64_t ld = a.ld;
+    const double qx = a.q0[r], qy = a.q0[ld + r], qz = a.q0[2 * ld + r];
+    const double vx = a.v0[r], vy = a.v0[ld + r], vz = a.v0[2 * ld + r];
+    const double hx = qy * vz - qz * vy, hy = qz * vx - qx * vz, hz = qx * vy - qy * vx;
+    const double p = (hx * hx + hy * hy + hz * hz) * imu;
+    const double ecc = sqrt(fmax(0.0, 1.0 - p * eq.alpha));
+    lo = -INFINITY;
+    hi = INFINITY;
+    if (p > 0.0) {
+        const double xb = eq.sqmu_dt * (1.0 + ecc) / p * (1.0 + 1e-12);
+        if (a.dt >= 0.0) { lo = 0.0; hi = xb; } else { lo = xb; hi = 0.0; }
+    }
+    if (eq.alpha < 0.0) {
+        // rsqrt within 2 ulp: the bound is widened by 1e-12
+        const double xm = 700.0 * (1.0 + 1e-12) * rsqrt(-eq.alpha);
+        if (a.dt >= 0.0) { lo = fmax(lo, 0.0); hi = fmin(hi, xm); }
+        else { lo = fmax(lo, -xm); hi = fmin(hi, 0.0); }
+    }
+}
+
+// The outer bound of an iteration by the FP64 form, where a decision may depend
+// on it (`rough` says that neither bound there has been replaced by a point)
+__device__ __forceinline__ void kep_refine_bracket(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                                   KepIter &s) {
+    if (!s.rough) return;
+    double lo, hi;
+    kep_outer_exact(a, r, imu, eq, lo, hi);
+    if (a.dt >= 0.0) s.hi = hi; else s.lo = lo;
+    s.rough = false;
+}
+
+// whether x, reached by a step dx of 2^-10 or more, may lie beyond the FP64 form's
+// outer bound (the rough one is at or above it, s.inside below)
+__device__ __forceinline__ bool kep_near_outer(const KepIter &s, double x, double dx) {
+    return !(fabsf(p64::lead(x, 0)) <= s.inside) && p64::abs_bits(dx) > p64::abs_bits(x) - (10ll << 52);
+}
+
+// The bracket of a bound orbit in FP32: the angular momentum is within 1e-6 |q||v|
+// of the FP64 one, so where it is above |q||v| / 4, p is within 1e-5, and the bound
+// is known from both sides: within 0.4% for e below 0.01, 1e-4 and less above 0.1.
+// The upper side serves until a step of 2^-10 or more may end beyond the FP64 bound
+// or would be bisected, which is rare; then the FP64 form takes its place and the
+// decision is that form's. (A smaller step that ends a hair beyond the FP64 bound, on
+// a near-circular orbit, is kept where that form would bisect.) Other orbits take the
+// FP64 form at once.
+__device__ __forceinline__ void kep_bracket(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                            double qx, double qy, double qz, double vx, double vy,
+                                            double vz, double r0sq, double vv, KepIter &s) {
+    const float x = p64::lead(qx, 0), y = p64::lead(qy, 0), z = p64::lead(qz, 0);
+    const float u = p64::lead(vx, 0), v = p64::lead(vy, 0), w = p64::lead(vz, 0);
+    const float hx = y * w - z * v, hy = z * u - x * w, hz = x * v - y * u;
+    const float h2 = fmaf(hx, hx, fmaf(hy, hy, hz * hz));
+    const float qv = p64::lead(r0sq, 0) * p64::lead(vv, 0), al = p64::lead(eq.alpha, 0);
+    const float p = h2 * p64::lead(imu, 0), pa = p * al, num = p64::lead(eq.sqmu_dt, 0);
+    s.rough = false;
+    if (al > 0.0f && h2 > 0x1p-4f * qv && h2 > 1e-25f && qv < 1e30f && p > 1e-25f && p < 1e25f &&
+        pa < 1e20f && fabsf(num) > 1e-15f && fabsf(num) < 1e10f) {
+        // e = sqrt(1 - p alpha), raised by the error of p alpha
+        const float E = 1.0f - pa, xp = num / p;
+        const float b = xp * (1.0f + sqrtf(fmaxf(0.0f, E) + 1.2e-5f)) * (1.0f + 2e-5f);
+        s.inside = fabsf(xp) * (1.0f + sqrtf(fmaxf(0.0f, E - 1.2e-5f))) * (1.0f - 2e-5f);
+        s.rough = fabsf(b) < 1e37f && fabsf(b) > 1e-35f;
+        const double xb = p64::to_double(b);
+        s.lo = a.dt >= 0.0 ? 0.0 : xb;
+        s.hi = a.dt >= 0.0 ? xb : 0.0;
+    }
+    if (!s.rough) kep_outer_exact(a, r, imu, eq, s.lo, s.hi);
+}
+
+// standard: x is the standard guess sqrt(mu) dt / r0, inside the bracket as r0 >= r_p
+__device__ __forceinline__ void kep_start(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                          KepIter &s, double x, bool standard) {
+    if (s.rough && !standard &&
+        !(p64::finite_bits(x) && !kep_near_outer(s, x, x) && (x >= 0.0) == (a.dt >= 0.0)))
+        kep_refine_bracket(a, r, imu, eq, s);
+    s.x = x;
+    if (!s.rough && p64::finite_bits(s.lo) && p64::finite_bits(s.hi) && !(x >= s.lo && x <= s.hi))
+        s.x = 0.5 * (s.lo + s.hi);
+    s.dx_old = INFINITY;
+    s.settle = s.conv = s.cs_at_x = false;
+    s.x_prev = s.x;
+    s.res_prev = INFINITY;
+    s.it = 0;
+}
+
 // QYM_SOLVER_NEWTON32: Newton's method on F in FP32 from x while it stays in
 // the bracket [lo, hi] (at most 12 steps), until a step falls below 1e-5 |x|;
 // x then holds the FP32 root (relative error about 1e-7, more where F's terms
@@ -98,11 +223,12 @@ __device__ __forceinline__ void stumpff_f32(float y, float &C, float &S) {
 // residual test. Returns
 // the FP32 steps taken, and leaves x unchanged (0 steps counted) when the FP32
 // form fails (a step leaves the bracket, F or F' is not finite).
-__device__ __forceinline__ int newton_f32(const KepEq &eq, double lo, double hi, double &x) {
-    const float sq = (float)eq.sqmu_dt, r0 = (float)eq.r0, sig = (float)eq.sig;
-    const float al = (float)eq.alpha, b = (float)eq.b;
-    const float lof = (float)lo, hif = (float)hi;
-    float xf = (float)x;
+__device__ __forceinline__ int newton_f32(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                          KepIter &s, double &x) {
+    const float sq = p64::to_float(eq.sqmu_dt), r0 = p64::to_float(eq.r0), sig = p64::to_float(eq.sig);
+    const float al = p64::to_float(eq.alpha), b = p64::to_float(eq.b);
+    float lof = p64::to_float(s.lo), hif = p64::to_float(s.hi);
+    float xf = p64::to_float(x);
     for (int it = 0; it < 12; ++it) {
         const float x2 = xf * xf, y = al * x2;
         float C, S;
@@ -112,45 +238,166 @@ __device__ __forceinline__ int newton_f32(const KepEq &eq, double lo, double hi,
         if (!isfinite(F) || !(Fp > 0.0f) || !isfinite(Fp)) return 0;
         const float dx = F / Fp;
         const float xn = xf - dx;
+        if (s.rough && !(fabsf(xn) <= s.inside || fabsf(dx) < 0x1p-10f * fabsf(xn))) {
+            kep_refine_bracket(a, r, imu, eq, s);
+            lof = p64::to_float(s.lo);
+            hif = p64::to_float(s.hi);
+        }
         if (!(xn >= lof && xn <= hif)) return 0;
         xf = xn;
         if (fabsf(dx) <= 1e-5f * fabsf(xf)) {
-            x = (double)xf;
+            x = fabsf(xf) >= 1.1754944e-38f ? p64::to_double(xf) : (double)xf;
             return it + 1;
         }
     }
     return 0;
 }
 
-template <bool MLP>
-__global__ void __launch_bounds__(256) k_kepler(KeplerArgs a) {
+// One evaluation and the step from it; true when the iteration has ended
+// (converged, or max_iter evaluations made)
+__device__ __forceinline__ bool kep_iterate(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                            bool laguerre, KepIter &s) {
+    if (s.it >= a.max_iter) return true;
+    ++s.it;
+    ++s.iters;
+    const double x = s.x;
+    float sc;
+    const double F = eq.value(x, s.C, s.S, sc);
+    const bool F_ok = p64::finite_bits(F);
+    double scale = 0.0;
+    if (F_ok) {
+        // |F| <= 1e-14 sum |terms|, in FP32 where its range holds (the factor
+        // covers the FP32 sum, so no residual above 1e-14 passes)
+        bool small;
+        if (sc > 1e-18f && sc < 1e30f) {
+            small = fabsf(p64::lead(F, 0)) <= 1e-14f * (1.0f - 4e-6f) * sc;
+        } else {
+            scale = eq.scale(x, s.C, s.S);
+            small = fabs(F) <= 1e-14 * scale;
+        }
+        if (small) {
+            --s.iters;
+            s.conv = s.cs_at_x = true;
+            return true;
+        }
+        if (s.settle) {
+            // evaluated after a rounding-level step and still above 1e-14: the
+            // better of the last two points is the root
+            if (scale == 0.0) scale = eq.scale(x, s.C, s.S);
+            --s.iters;
+            s.conv = true;
+            if (fabs(F) / scale <= s.res_prev) s.cs_at_x = true; else s.x = s.x_prev;
+            return true;
+        }
+    }
+    double Fp = 0.0, Fpp = 0.0;
+    if (F_ok) eq.slopes(x, s.C, s.S, Fp, Fpp);
+    if (!F_ok || !p64::finite_bits(Fp) || !p64::finite_bits(Fpp)) {
+        if (x > 0.0) s.hi = x; else s.lo = x;
+        if ((x > 0.0) == (a.dt >= 0.0)) s.rough = false;
+        kep_refine_bracket(a, r, imu, eq, s);
+        s.x = 0.5 * (s.lo + s.hi);
+        return false;
+    }
+    if (F < 0.0) s.lo = x; else s.hi = x;
+    if ((F < 0.0) == (a.dt < 0.0)) s.rough = false;  // the outer bound is a point now
+    double dx;
+    const double iFp = Fp > 0.0 ? p64::rcp(Fp) : 1.0 / Fp;
+    if (laguerre) {
+        // Laguerre, n = 5: dx = n F / (F' + sgn(F') sqrt|(n-1)^2 F'^2 - n(n-1) F F''|),
+        // with F' taken out of the root so that F'^2 never overflows:
+        // dx = rf 5 / (1 + sqrt|16 - 20 z|), rf = F / F', z = rf F'' / F'.
+        // Near the root (|z| < 1e-6) the factor is its series
+        // 1 + z / 2 + 13 z^2 / 32 (next term 0.38 z^3 < 4e-19): the same
+        // step to rounding without the square root and the division
+        const double rf = F * iFp, z = rf * (Fpp * iFp);
+        if (p64::hi_abs(z) < 0x3eb0c6f7) {  // 1e-6
+            dx = rf * fma(z, fma(13.0 / 32.0, z, 0.5), 1.0);
+        } else {
+            const double w = fabs(16.0 - 20.0 * z);
+            const double rt = p64::mid_range(w) ? w * p64::rsqrt_mid(w) : sqrt(w);
+            dx = 5.0 * rf * p64::rcp(1.0 + rt);
+        }
+    } else {
+        dx = F * iFp;
+    }
+    double xn = x - dx;
+    // bisect when the step is not finite, leaves the bracket, or fails
+    // to halve the previous step (slow approach along exp(sqrt(-alpha) x))
+    if (s.rough && (!p64::finite_bits(dx) || kep_near_outer(s, xn, dx) ||
+                    p64::abs_bits(dx) > p64::abs_bits(s.dx_old) - (1ll << 52) ||
+                    p64::order_bits(xn) < p64::order_bits(s.lo) || p64::order_bits(xn) > p64::order_bits(s.hi)))
+        kep_refine_bracket(a, r, imu, eq, s);
+    const bool have_br = p64::finite_bits(s.lo) && p64::finite_bits(s.hi);
+    if (have_br) {
+        const long long xo = p64::order_bits(xn);
+        if (!p64::finite_bits(dx) || xo < p64::order_bits(s.lo) || xo > p64::order_bits(s.hi) ||
+            p64::abs_bits(dx) > p64::abs_bits(s.dx_old) - (1ll << 52)) {
+            xn = 0.5 * (s.lo + s.hi);
+            dx = x - xn;
+        }
+    }
+    s.dx_old = dx;
+    const long long small = p64::abs_bits(xn) - (50ll << 52);  // 2^-50 |xn|
+    const double wd = s.hi - s.lo;
+    if (p64::abs_bits(dx) <= small || p64::abs_bits(dx) == 0 ||
+        (have_br && (p64::abs_bits(wd) <= small || p64::abs_bits(wd) == 0 || __double2hiint(wd) < 0))) {
+        s.settle = true;
+        s.x_prev = x;
+        s.res_prev = fabs(F) / eq.scale(x, s.C, s.S);
+    }
+    s.x = xn;
+    return false;
+}
+
+constexpr int kPackBelow = 12;  // lanes still iterating below which a warp's bodies are packed
+
+// an unfinished body on its way to another thread of the CTA
+struct KepPacked {
+    KepEq eq;
+    KepIter s;
+    int64_t r;
+    double imu;
+};
+
+template <bool MLP, int T>
+__global__ void __launch_bounds__(T) k_kepler(KeplerArgs a) {
     chain_wait();
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int iters = 0;
+    __shared__ KepPacked s_body[T];
+    __shared__ int s_list[T];
+    __shared__ int s_n;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_n = 0;
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + tid;
     const bool act = k < a.n;
     const int64_t r = act ? (a.rows ? a.rows[k] : a.row0 + k) : 0;
     const int64_t ld = a.ld;
     double qx = 0.0, qy = 0.0, qz = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;
-    // mu = G m0 with sqrt(mu) and 1/mu, formed once per system on the host
+    // sqrt(mu) and 1/mu of mu = G m0, formed once per system on the host
     // (correctly rounded, as sqrt and the division here would give them)
-    double mu = 1.0, sqmu = 1.0, imu = 1.0;
+    double sqmu = 1.0, imu = 1.0;
     if (act) {
         qx = a.q0[r]; qy = a.q0[ld + r]; qz = a.q0[2 * ld + r];
         vx = a.v0[r]; vy = a.v0[ld + r]; vz = a.v0[2 * ld + r];
         if (a.kmu) {
             const double *km = a.kmu + 3 * (int64_t)a.sys_of[r];
-            mu = km[0]; sqmu = km[1]; imu = km[2];
+            sqmu = km[1]; imu = km[2];
         } else {
-            mu = a.mu; sqmu = a.sqmu; imu = a.imu;
+            sqmu = a.sqmu; imu = a.imu;
         }
     }
     const double dt = a.dt;
-    const double r0 = sqrt(qx * qx + qy * qy + qz * qz);
-    const bool feat = act && r0 > 0.0 && dt != 0.0;
+    const double r0sq = qx * qx + qy * qy + qz * qz;
+    double ir0 = 0.0;
+    const double r0 = p64::sqrt_rcp(r0sq, ir0);
+    const bool body = act && !(r0 == 0.0);
+    const double vv = vx * vx + vy * vy + vz * vz;
+    const double rv = qx * vx + qy * vy + qz * vz;
     float u[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     double sigma = 0.0;
     bool bound = false;  // in the learned guess's domain
-    if (feat && (MLP || a.log)) bound = mlp::features(qx, qy, qz, vx, vy, vz, r0, mu, dt, u, sigma);
+    if (act && r0 > 0.0 && dt != 0.0 && (MLP || a.log))
+        bound = mlp::features(rv, vv, r0, ir0, sqmu, imu, dt, u, sigma);
     double x_mlp = 0.0;
     bool have_mlp = false;
     if (MLP) {
@@ -159,202 +406,138 @@ __global__ void __launch_bounds__(256) k_kepler(KeplerArgs a) {
         mlp::normalise(a.mlp_w, u, fn);
         const float y = mlp::warp_forward(a.mlp_w, fn);
         const float tn = a.mlp_w[mlp::OM] + a.mlp_w[mlp::OSD] * y;
-        x_mlp = sqmu * dt / r0 * (1.0 + sigma * (double)tn);
+        x_mlp = sqmu * dt * ir0 * (1.0 + sigma * (double)tn);
         have_mlp = bound && isfinite(x_mlp);
     }
-    if (act) {
-        if (r0 == 0.0) {
-            // a star row (held at Q = v = 0): stays at the origin
-            a.q1[r] = 0.0; a.q1[ld + r] = 0.0; a.q1[2 * ld + r] = 0.0;
-            a.v1[r] = 0.0; a.v1[ld + r] = 0.0; a.v1[2 * ld + r] = 0.0;
-            if (a.x_out) a.x_out[k] = 0.0;
-            if (a.x0_out) a.x0_out[k] = 0.0;
-            if (a.iters) a.iters[k] = 0;
-            goto done;
-        }
-        {
-        double vv = vx * vx + vy * vy + vz * vz;
-        // the FP64 pipe bounds this kernel: divisions by mu, sqrt(mu) and r0
-        // become products with reciprocals formed once (within an ulp of the
-        // quotients)
-        const double ir0 = 1.0 / r0, isqmu = sqmu * imu;
-        KepEq eq;
+    // the FP64 pipe bounds this kernel: divisions by mu, sqrt(mu) and r0
+    // become products with reciprocals formed once (within an ulp of the
+    // quotients)
+    const double isqmu = sqmu * imu;
+    KepEq eq;
+    KepIter s;
+    s.iters = 0;
+    bool laguerre = a.solver != QYM_SOLVER_NEWTON;
+    bool busy = body;
+    if (body) {
         eq.sqmu_dt = sqmu * dt;
         eq.r0 = r0;
         eq.alpha = 2.0 * ir0 - vv * imu;
-        eq.sig = (qx * vx + qy * vy + qz * vz) * isqmu;
+        eq.sig = rv * isqmu;
         eq.b = 1.0 - r0 * eq.alpha;
         double x;
-        if (a.guess == QYM_GUESS_R0)
-            x = r0;
-        else if (MLP && have_mlp)
-            x = x_mlp;
-        else
+        const bool standard = a.guess != QYM_GUESS_R0 && !(MLP && have_mlp);
+        if (standard)
             x = eq.sqmu_dt * ir0;
+        else
+            x = a.guess == QYM_GUESS_R0 ? r0 : x_mlp;
         if (a.x0_out) a.x0_out[k] = x;
-        int solver = a.solver;
-        bool conv = false;
-        bool cs_at_x = false;  // C, S hold the Stumpff values at the final x
-        double C = 0.5, S = 1.0 / 6.0;
-        // Root bracket: F(0) = -sqrt(mu) dt and F' = r >= r_p (periapsis
-        // distance), so the root lies between 0 and sqrt(mu) dt / r_p; for an
-        // unbound orbit also |x| <= 700 / sqrt(-alpha), past which C and S
-        // overflow. Widened by 1e-12 for the rounding of r_p = p / (1 + e).
-        double lo = -INFINITY, hi = INFINITY;
-        {
-            double hx = qy * vz - qz * vy, hy = qz * vx - qx * vz, hz = qx * vy - qy * vx;
-            double p = (hx * hx + hy * hy + hz * hz) * imu;
-            double ecc = sqrt(fmax(0.0, 1.0 - p * eq.alpha));
-            if (p > 0.0) {
-                double xb = eq.sqmu_dt * (1.0 + ecc) / p * (1.0 + 1e-12);
-                if (dt >= 0.0) { lo = 0.0; hi = xb; } else { lo = xb; hi = 0.0; }
-            }
-            if (eq.alpha < 0.0) {
-                // rsqrt within 2 ulp: the bound is widened by 1e-12
-                double xm = 700.0 * (1.0 + 1e-12) * rsqrt(-eq.alpha);
-                if (dt >= 0.0) { lo = fmax(lo, 0.0); hi = fmin(hi, xm); }
-                else { lo = fmax(lo, -xm); hi = fmin(hi, 0.0); }
-            }
+        kep_bracket(a, r, imu, eq, qx, qy, qz, vx, vy, vz, r0sq, vv, s);
+        // FP32 Newton steps first, then the FP64 iteration in Laguerre's
+        // form: from the FP32 root (about 1e-7) one cubic step reaches
+        // the rounding level, so the evaluation after it meets the
+        // residual test
+        if (a.solver == QYM_SOLVER_NEWTON32) s.iters = newton_f32(a, r, imu, eq, s, x);
+        kep_start(a, r, imu, eq, s, x, standard && s.iters == 0);
+    }
+    // (a warp below the threshold from the start iterates once all the same)
+    do {
+        if (busy) busy = !kep_iterate(a, r, imu, eq, laguerre, s);
+    } while (__popc(__ballot_sync(0xffffffffu, busy)) >= kPackBelow);
+    __syncthreads();  // s_n = 0
+    int slot = -1;
+    if (busy) {
+        slot = atomicAdd(&s_n, 1);
+        s_list[slot] = tid;
+        s_body[tid].eq = eq;
+        s_body[tid].s = s;
+        s_body[tid].r = r;
+        s_body[tid].imu = imu;
+    }
+    __syncthreads();
+    if (tid < s_n) {
+        KepPacked &b = s_body[s_list[tid]];
+        const KepEq e = b.eq;
+        KepIter t = b.s;
+        while (!kep_iterate(a, b.r, b.imu, e, laguerre, t)) {}
+        b.s = t;
+    }
+    __syncthreads();
+    if (body) {
+        if (slot >= 0) s = s_body[tid].s;
+        // learned guess only: Laguerre from the standard guess if the iteration
+        // from it did not converge
+        if (MLP && !s.conv) {
+            s.rough = false;
+            kep_outer_exact(a, r, imu, eq, s.lo, s.hi);
+            kep_start(a, r, imu, eq, s, eq.sqmu_dt * ir0, true);
+            while (!kep_iterate(a, r, imu, eq, true, s)) {}
         }
-        const double lo0 = lo, hi0 = hi;
-        if (solver == QYM_SOLVER_NEWTON32) {
-            // FP32 Newton steps first, then the FP64 iteration in Laguerre's
-            // form: from the FP32 root (about 1e-7) one cubic step reaches
-            // the rounding level, so the evaluation after it meets the
-            // residual test
-            iters += newton_f32(eq, lo, hi, x);
-            solver = QYM_SOLVER_LAGUERRE;
-        }
-        // two passes at most: the requested start, then (learned guess only)
-        // Laguerre from the standard guess if the first did not converge
-        for (int pass = 0; pass < 2 && !conv; ++pass) {
-            if (pass == 1) {
-                if (!MLP) break;
-                x = eq.sqmu_dt * ir0;
-                solver = QYM_SOLVER_LAGUERRE;
-                lo = lo0;
-                hi = hi0;
-            }
-            const bool have_br = isfinite(lo) && isfinite(hi);
-            if (!(x >= lo && x <= hi) && have_br) x = 0.5 * (lo + hi);
-            double dx_old = INFINITY;
-            // after a step at the rounding level: the point it started from
-            // and its relative residual
-            bool settle = false;
-            double x_prev = x, res_prev = INFINITY;
-            for (int it = 0; it < a.max_iter; ++it) {
-                double F, Fp, Fpp;
-                eq.eval(x, F, Fp, Fpp, C, S);
-                ++iters;
-                if (!isfinite(F) || !isfinite(Fp) || !isfinite(Fpp)) {
-                    if (x > 0.0) hi = x; else lo = x;
-                    x = 0.5 * (lo + hi);
-                    continue;
-                }
-                if (F < 0.0) lo = x; else hi = x;
-                // residual against the rounding floor of F: the sum of |terms|
-                double x2 = x * x;
-                double scale = fabs(eq.sqmu_dt) + fabs(eq.sig * x2 * C) +
-                               fabs(eq.b * x2 * x * S) + r0 * fabs(x);
-                if (fabs(F) <= 1e-14 * scale) { --iters; conv = true; cs_at_x = true; break; }
-                if (settle) {
-                    // evaluated after a rounding-level step and still above
-                    // 1e-14: the better of the last two points is the root
-                    --iters;
-                    conv = true;
-                    if (fabs(F) / scale <= res_prev) cs_at_x = true; else x = x_prev;
-                    break;
-                }
-                double dx;
-                if (solver == QYM_SOLVER_LAGUERRE) {
-                    // Laguerre, n = 5: dx = n F / (F' + sgn(F') sqrt|(n-1)^2 F'^2 - n(n-1) F F''|),
-                    // with F' taken out of the root so that F'^2 never overflows:
-                    // dx = rf 5 / (1 + sqrt|16 - 20 z|), rf = F / F', z = rf F'' / F'.
-                    // Near the root (|z| < 1e-6) the factor is its series
-                    // 1 + z / 2 + 13 z^2 / 32 (next term 0.38 z^3 < 4e-19): the same
-                    // step to rounding without the square root and the division
-                    const double iFp = 1.0 / Fp, rf = F * iFp, z = rf * (Fpp * iFp);
-                    if (fabs(z) < 1e-6)
-                        dx = rf * fma(z, fma(13.0 / 32.0, z, 0.5), 1.0);
-                    else
-                        dx = 5.0 * rf / (1.0 + sqrt(fabs(16.0 - 20.0 * z)));
-                } else {
-                    dx = F / Fp;
-                }
-                double xn = x - dx;
-                // bisect when the step is not finite, leaves the bracket, or fails
-                // to halve the previous step (slow approach along exp(sqrt(-alpha) x))
-                if (isfinite(lo) && isfinite(hi) &&
-                    (!isfinite(dx) || !(xn >= lo && xn <= hi) || fabs(dx) > 0.5 * fabs(dx_old))) {
-                    xn = 0.5 * (lo + hi);
-                    dx = x - xn;
-                }
-                dx_old = dx;
-                if (fabs(dx) <= 0x1p-50 * fabs(xn) ||
-                    (isfinite(lo) && isfinite(hi) && hi - lo <= 0x1p-50 * fabs(xn))) {
-                    settle = true;
-                    x_prev = x;
-                    res_prev = fabs(F) / scale;
-                }
-                x = xn;
-            }
-        }
+        const double x = s.x;
         // f and g functions at the root (Appendix); r before fdot, gdot. The
         // last evaluation left C, S at this x unless the iteration kept the
         // point before it, or ran out of iterations after a step
-        double x2 = x * x;
-        double y = eq.alpha * x2;
-        if (!cs_at_x) stumpff(y, C, S);
-        double f = 1.0 - x2 * C * ir0;
-        double g = dt - x2 * x * S * isqmu;
-        double nx = f * qx + g * vx, ny = f * qy + g * vy, nz = f * qz + g * vz;
-        double irr = 1.0 / sqrt(nx * nx + ny * ny + nz * nz);
-        double fd = sqmu * x * (y * S - 1.0) * irr * ir0;
-        double gd = 1.0 - x2 * C * irr;
-        double ux = fd * qx + gd * vx, uy = fd * qy + gd * vy, uz = fd * qz + gd * vz;
+        const double x2 = x * x, y = eq.alpha * x2;
+        double C = s.C, S = s.S;
+        if (!s.cs_at_x) stumpff(y, C, S);
+        const double x2C = x2 * C;
+        const double f = 1.0 - x2C * ir0;
+        const double g = dt - x2 * x * S * isqmu;
+        const double nx = f * qx + g * vx, ny = f * qy + g * vy, nz = f * qz + g * vz;
+        const double irr = p64::rsqrt64(nx * nx + ny * ny + nz * nz);
+        const double fd = sqmu * x * (y * S - 1.0) * irr * ir0;
+        const double gd = 1.0 - x2C * irr;
+        const double ux = fd * qx + gd * vx, uy = fd * qy + gd * vy, uz = fd * qz + gd * vz;
         a.q1[r] = nx; a.q1[ld + r] = ny; a.q1[2 * ld + r] = nz;
         a.v1[r] = ux; a.v1[ld + r] = uy; a.v1[2 * ld + r] = uz;
         if (a.x_out) a.x_out[k] = x;
-        if (a.iters) a.iters[k] = iters;
+        if (a.iters) a.iters[k] = s.iters;
         if (a.log && bound) {
             // training row of this solve: slot (steps logged so far) * n + k
             const int64_t base = a.log_step ? (int64_t)(*a.log_base + *a.log_step) * a.n : 0;
-            const int64_t slot = base + k;
-            if (slot < a.log_cap) {
+            const int64_t row_i = base + k;
+            if (row_i < a.log_cap) {
                 const double t = (x * r0 / eq.sqmu_dt - 1.0) / sigma;
-                float *row = a.log + 5 * slot;
+                float *row = a.log + 5 * row_i;
                 row[0] = u[0]; row[1] = u[1]; row[2] = u[2]; row[3] = u[3];
                 row[4] = (float)t;
             }
         }
         if (a.status) {
             int bits = 0;
-            if (!conv) bits |= QYM_ST_KEPLER_NOCONV;
-            if (!(isfinite(nx) && isfinite(ny) && isfinite(nz) && isfinite(ux) && isfinite(uy) &&
-                  isfinite(uz)))
+            if (!s.conv) bits |= QYM_ST_KEPLER_NOCONV;
+            if (!(p64::finite_bits(nx) && p64::finite_bits(ny) && p64::finite_bits(nz) &&
+                  p64::finite_bits(ux) && p64::finite_bits(uy) && p64::finite_bits(uz)))
                 bits |= QYM_ST_NAN;
             if (bits) atomicOr(a.status, bits);
         }
-        }
+    } else if (act) {
+        // a star row (held at Q = v = 0): stays at the origin
+        a.q1[r] = 0.0; a.q1[ld + r] = 0.0; a.q1[2 * ld + r] = 0.0;
+        a.v1[r] = 0.0; a.v1[ld + r] = 0.0; a.v1[2 * ld + r] = 0.0;
+        if (a.x_out) a.x_out[k] = 0.0;
+        if (a.x0_out) a.x0_out[k] = 0.0;
+        if (a.iters) a.iters[k] = 0;
     }
-done:
     if (a.iter_sum) {
-        unsigned long long s = (unsigned long long)iters;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0 && s) atomicAdd(a.iter_sum, s);
+        const unsigned sum = __reduce_add_sync(0xffffffffu, body ? (unsigned)s.iters : 0u);
+        if ((tid & 31) == 0 && sum) atomicAdd(a.iter_sum, (unsigned long long)sum);
     }
+}
+
+template <bool MLP>
+static cudaError_t launch_kepler_t(const KeplerArgs &a, cudaStream_t st) {
+    // A warp issues an FP64 instruction every 64 cycles, an SM one every 19: the
+    // fewest bodies spread best as two warps a CTA, one or two CTAs on every SM
+    // (16384 test particles 64 us in CTAs of 256, on 64 of the SMs); large inputs
+    // pack their unfinished bodies over eight warps.
+    if (a.n <= 4 * 64 * 152)
+        return launch_chain(k_kepler<MLP, 64>, (unsigned)((a.n + 63) / 64), 64, 0, st, a);
+    return launch_chain(k_kepler<MLP, 256>, (unsigned)((a.n + 255) / 256), 256, 0, st, a);
 }
 
 cudaError_t launch_kepler(const KeplerArgs &a, cudaStream_t st) {
     if (a.n <= 0) return cudaSuccess;
-    int threads = 256;
-    int64_t blocks = (a.n + threads - 1) / threads;
-    if (a.guess == QYM_GUESS_MLP && a.mlp_w)
-        launch_chain(k_kepler<true>, (unsigned)blocks, threads, 0, st, a);
-    else
-        launch_chain(k_kepler<false>, (unsigned)blocks, threads, 0, st, a);
-    return cudaGetLastError();
+    return a.guess == QYM_GUESS_MLP && a.mlp_w ? launch_kepler_t<true>(a, st) : launch_kepler_t<false>(a, st);
 }
 
 }  // namespace qym

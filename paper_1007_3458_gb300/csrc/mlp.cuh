@@ -182,26 +182,26 @@ __device__ __forceinline__ float warp_forward(const float *__restrict__ w, const
     return mine;
 }
 
-// Raw features u1..u4 of a body (q, v) about a star of parameter mu for a
-// step dt (r0 = |q| > 0, dt != 0), and sigma = s / (1 + s) with
+// Raw features u1..u4 of a body with rv = q.v, v2 = |v|^2 about a star of
+// parameter mu for a step dt (r0 = |q| > 0, dt != 0), and sigma = s / (1 + s) with
 // s = |dt| sqrt(mu / r0^3):
 //   u1 = q.v / sqrt(mu r0), u2 = r0 |v|^2 / mu, u3 = ln s,
 //   u4 = dt sqrt(mu alpha^3) / (2 pi) for alpha = 2/r0 - |v|^2/mu > 0, else 0.
 // Returns whether the orbit is bound (alpha > 0): the domain of the learned
 // guess (there |u1| < sqrt 2 and u2 < 2; unbound states, such as bodies deep
 // in a planet's well during an encounter, keep the standard guess).
-__device__ __forceinline__ bool features(double qx, double qy, double qz, double vx, double vy,
-                                         double vz, double r0, double mu, double dt,
-                                         float (&u)[4], double &sigma) {
-    const double v2 = vx * vx + vy * vy + vz * vz;
-    const double rv = qx * vx + qy * vy + qz * vz;
-    const double alpha = 2.0 / r0 - v2 / mu;
-    const double s = fabs(dt) * sqrt(mu / (r0 * r0 * r0));
-    u[0] = (float)(rv / sqrt(mu * r0));
-    u[1] = (float)(r0 * v2 / mu);
+// (ir0, imu: 1/r0 and 1/mu; sqmu: sqrt(mu). Products with reciprocals and
+// reciprocal roots, within a few ulp of the quotients, rounded to float)
+__device__ __forceinline__ bool features(double rv, double v2, double r0, double ir0, double sqmu,
+                                         double imu, double dt, float (&u)[4], double &sigma) {
+    const double alpha = 2.0 * ir0 - v2 * imu, irt = p64::rsqrt64(r0);
+    const double s = fabs(dt) * sqmu * ir0 * irt;
+    u[0] = (float)(rv * (sqmu * imu) * irt);
+    u[1] = (float)(r0 * v2 * imu);
     u[2] = (float)log(s);
-    u[3] = alpha > 0.0 ? (float)(dt * sqrt(mu * alpha * alpha * alpha) / (2.0 * kPi)) : 0.0f;
-    sigma = s / (1.0 + s);
+    double irta;
+    u[3] = alpha > 0.0 ? (float)(dt * sqmu * alpha * p64::sqrt_rcp(alpha, irta) * (0.5 / kPi)) : 0.0f;
+    sigma = s * p64::rcp(1.0 + s);
     return alpha > 0.0;
 }
 

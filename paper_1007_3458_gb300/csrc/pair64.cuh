@@ -300,6 +300,69 @@ __device__ __forceinline__ float lead(double x, int k) {
     return __uint_as_float(f | ((unsigned)hi & 0x80000000u));
 }
 
+// |x| as an integer that orders like it
+__device__ __forceinline__ long long abs_bits(double x) {
+    return __double_as_longlong(x) & 0x7fffffffffffffffll;
+}
+// any finite or infinite double as an integer that orders like it (-0 below +0)
+__device__ __forceinline__ long long order_bits(double x) {
+    const long long u = __double_as_longlong(x);
+    return u ^ ((u >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool finite_bits(double x) { return hi_abs(x) < 0x7ff00000; }
+// x 2^k by its exponent field, for a normal result; zero, infinities and NaN (and
+// denormals) stay as they are
+__device__ __forceinline__ double mul_pow2(double x, int k) {
+    return (unsigned)(hi_abs(x) - 0x00100000) >= 0x7fe00000u ? x : __hiloint2double(__double2hiint(x) + k * (1 << 20), __double2loint(x));
+}
+// a normal float as a double
+__device__ __forceinline__ double to_double(float x) {
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// Reciprocal, reciprocal square root and square root of a positive normal x by
+// one third-order step from the FP32 approximation (Householder's method: the
+// binomial series in the residual e = 1 - x y or 1 - x y^2, |e| < 2^-20, to e^2;
+// the next term is below 2^-61), within an ulp: three to eight FP64 instructions
+// where the library's correctly rounded forms take ten and more. Outside the
+// exponents [-1000, 1000] the library forms.
+__device__ __forceinline__ bool mid_range(double x) {
+    const int hi = __double2hiint(x);
+    return hi > (23 << 20) && hi < (2023 << 20);
+}
+__device__ __forceinline__ double rcp(double x) {
+    if (!mid_range(x)) return 1.0 / x;
+    const int k = (__double2hiint(x) >> 20) - 1023;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(lead(x, k)));
+    const double y = mul_pow2(to_double(r), -k);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt_mid(double x) {
+    const int k = ((__double2hiint(x) >> 20) - 1023) & ~1;  // even
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(lead(x, k)));
+    const double y = mul_pow2(to_double(r), -(k >> 1));
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) { return mid_range(x) ? rsqrt_mid(x) : rsqrt(x); }
+// square root (the correction s + y (x - s^2) / 2 rounds it correctly but for
+// rare ties, Markstein) with its reciprocal
+__device__ __forceinline__ double sqrt_rcp(double x, double &ir) {
+    if (!mid_range(x)) {
+        const double r = sqrt(x);
+        ir = 1.0 / r;
+        return r;
+    }
+    const double y = rsqrt_mid(x), s = x * y;
+    const double r = fma(mul_pow2(y, -1), fma(-s, s, x), s);
+    ir = fma(y, fma(-r, y, 1.0), y);
+    return r;
+}
+
 // x rounded to the nearest float, by its bits where the result is normal
 __device__ __forceinline__ float to_float(double x) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);

@@ -258,11 +258,13 @@ void set_thread_error(const std::string &msg);
 // the stream still runs (programmatic dependent launch) and waits for it, and
 // for the visibility of all it wrote, in chain_wait(), its first statement. The
 // kernels of a small step are a few microseconds each, so the ~1 us a launch
-// otherwise takes between them counts. chain_wait() first lets the next kernel
-// be set up in turn; a kernel's end still implies the end of every one before.
+// otherwise takes between them counts. Only then does it let the next kernel be
+// set up: allowed before the wait, the kernels of a chain pile up on the SMs, and
+// a later one finds room on a few of them only (a drift of 16384 bodies took 65
+// us instead of 41).
 __device__ __forceinline__ void chain_wait() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <class... P, class... A>
 cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
