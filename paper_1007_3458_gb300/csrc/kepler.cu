@@ -129,26 +129,35 @@ struct KepIter {
 // the root lies between 0 and the outer bound sqrt(mu) dt / r_p; for an unbound
 // orbit also |x| <= 700 / sqrt(-alpha), past which C and S overflow. Widened by
 // 1e-12 for the rounding of r_p = p / (1 + e).
-__device__ __noinline__ void kep_outer_exact(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
-                                             double &lo, double &hi) {
-    const int64_t ld = a.ld;
-    const double qx = a.q0[r], qy = a.q0[ld + r], qz = a.q0[2 * ld + r];
-    const double vx = a.v0[r], vy = a.v0[ld + r], vz = a.v0[2 * ld + r];
+// Returns the outer bound (of dt's sign; infinite where there is none). Out of
+// line, by value: the body's iteration stays in registers.
+__device__ __noinline__ double kep_outer_exact(const double *q, const double *v, int64_t ld, double imu,
+                                               double alpha, double sqmu_dt, bool forward) {
+    const double qx = q[0], qy = q[ld], qz = q[2 * ld];
+    const double vx = v[0], vy = v[ld], vz = v[2 * ld];
     const double hx = qy * vz - qz * vy, hy = qz * vx - qx * vz, hz = qx * vy - qy * vx;
     const double p = (hx * hx + hy * hy + hz * hz) * imu;
-    const double ecc = sqrt(fmax(0.0, 1.0 - p * eq.alpha));
-    lo = -INFINITY;
-    hi = INFINITY;
-    if (p > 0.0) {
-        const double xb = eq.sqmu_dt * (1.0 + ecc) / p * (1.0 + 1e-12);
-        if (a.dt >= 0.0) { lo = 0.0; hi = xb; } else { lo = xb; hi = 0.0; }
-    }
-    if (eq.alpha < 0.0) {
+    const double ecc = sqrt(fmax(0.0, 1.0 - p * alpha));
+    double out = forward ? INFINITY : -INFINITY;
+    if (p > 0.0) out = sqmu_dt * (1.0 + ecc) / p * (1.0 + 1e-12);
+    if (alpha < 0.0) {
         // rsqrt within 2 ulp: the bound is widened by 1e-12
-        const double xm = 700.0 * (1.0 + 1e-12) * rsqrt(-eq.alpha);
-        if (a.dt >= 0.0) { lo = fmax(lo, 0.0); hi = fmin(hi, xm); }
-        else { lo = fmax(lo, -xm); hi = fmin(hi, 0.0); }
+        const double xm = 700.0 * (1.0 + 1e-12) * rsqrt(-alpha);
+        out = forward ? fmin(out, xm) : fmax(out, -xm);
     }
+    return out;
+}
+
+// both bounds by the FP64 form
+__device__ __forceinline__ void kep_exact_bracket(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
+                                                  KepIter &s) {
+    const bool forward = a.dt >= 0.0;
+    const double out = kep_outer_exact(a.q0 + r, a.v0 + r, a.ld, imu, eq.alpha, eq.sqmu_dt, forward);
+    // (a radial bound orbit has no outer bound, and then no inner one either)
+    const double in = p64::finite_bits(out) || out != out ? 0.0 : -out;
+    s.lo = forward ? in : out;
+    s.hi = forward ? out : in;
+    s.rough = false;
 }
 
 // The outer bound of an iteration by the FP64 form, where a decision may depend
@@ -156,9 +165,9 @@ __device__ __noinline__ void kep_outer_exact(const KeplerArgs &a, int64_t r, dou
 __device__ __forceinline__ void kep_refine_bracket(const KeplerArgs &a, int64_t r, double imu, const KepEq &eq,
                                                    KepIter &s) {
     if (!s.rough) return;
-    double lo, hi;
-    kep_outer_exact(a, r, imu, eq, lo, hi);
-    if (a.dt >= 0.0) s.hi = hi; else s.lo = lo;
+    const bool forward = a.dt >= 0.0;
+    const double out = kep_outer_exact(a.q0 + r, a.v0 + r, a.ld, imu, eq.alpha, eq.sqmu_dt, forward);
+    if (forward) s.hi = out; else s.lo = out;
     s.rough = false;
 }
 
@@ -197,7 +206,7 @@ __device__ __forceinline__ void kep_bracket(const KeplerArgs &a, int64_t r, doub
         s.lo = a.dt >= 0.0 ? 0.0 : xb;
         s.hi = a.dt >= 0.0 ? xb : 0.0;
     }
-    if (!s.rough) kep_outer_exact(a, r, imu, eq, s.lo, s.hi);
+    if (!s.rough) kep_exact_bracket(a, r, imu, eq, s);
 }
 
 // standard: x is the standard guess sqrt(mu) dt / r0, inside the bracket as r0 >= r_p
@@ -361,7 +370,7 @@ struct KepPacked {
 };
 
 template <bool MLP, int T>
-__global__ void __launch_bounds__(T) k_kepler(KeplerArgs a) {
+__global__ void __launch_bounds__(T, 512 / T) k_kepler(const __grid_constant__ KeplerArgs a) {
     chain_wait();
     __shared__ KepPacked s_body[T];
     __shared__ int s_list[T];
@@ -467,8 +476,7 @@ __global__ void __launch_bounds__(T) k_kepler(KeplerArgs a) {
         // learned guess only: Laguerre from the standard guess if the iteration
         // from it did not converge
         if (MLP && !s.conv) {
-            s.rough = false;
-            kep_outer_exact(a, r, imu, eq, s.lo, s.hi);
+            kep_exact_bracket(a, r, imu, eq, s);
             kep_start(a, r, imu, eq, s, eq.sqmu_dt * ir0, true);
             while (!kep_iterate(a, r, imu, eq, true, s)) {}
         }
