@@ -209,3 +209,35 @@ def _accel_ref64(torch, m, x):
         a[1 + i:1 + i + 512] = t.sum(1).cpu().numpy()
         mag[1 + i:1 + i + 512] = t.abs().sum(1).cpu().numpy()
     return a, mag
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 4 * 64 * 152, 4 * 64 * 152 + 1])
+@pytest.mark.parametrize("e", [0.0, 0.003, 0.5, 0.97])
+def test_kepler_sizes_and_brackets(torch, n, e):
+    """E_Kep at the edges of its CTA sizes, on orbits whose root lies at its
+    bracket's end (circular), inside it, and beyond the FP32 bracket's domain
+    (nearly radial), forwards and backwards: the orbits' elements propagated
+    (the mean anomaly advanced). A point that meets the 1e-14 residual is off in
+    phase by that per orbit covered, and by 1/(1 - e) of it near pericentre (as
+    test_kepler_matches_oracle)."""
+    rng = np.random.default_rng(n)
+    k = min(n, 2000)
+    a = 10.0 ** rng.uniform(-0.3, 1.7, k)
+    ang = [rng.uniform(0, np.pi, k)] + [rng.uniform(0, 2 * np.pi, k) for _ in range(3)]
+    orbit = lambda M: W.elements_to_cartesian(1.0, a, np.full(k, e), *ang[:3], M)
+    qq, vv = (np.resize(x, (n, 3)) for x in orbit(ang[3]))
+    q0, v0 = (torch.from_numpy(np.ascontiguousarray(x.T)).cuda() for x in (qq, vv))
+    q1, v1 = torch.empty_like(q0), torch.empty_like(v0)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for dt in (W.TAU_A5, -0.3):
+        r1, u1 = orbit(ang[3] + dt / a ** 1.5)
+        scale = (1.0 + abs(dt) / (2 * np.pi * a ** 1.5)) / (1.0 - e)
+        for solver in (q.QYM_SOLVER_LAGUERRE, q.QYM_SOLVER_NEWTON32):
+            q.qym_kepler_drift_dev(n, q0, v0, q1, v1, 1.0, dt, solver, status=st)
+            for got, ref in ((q1, r1), (v1, u1)):
+                g = got.cpu().numpy().T
+                d = np.linalg.norm(g[:k] - ref, axis=1) / np.linalg.norm(ref, axis=1)
+                assert np.all(d <= 1e-12 * scale), float((d / scale).max())
+                if n > k:  # copies of the same bodies, in other lanes and CTAs
+                    assert np.abs(g - np.resize(g[:k], g.shape)).max() <= 1e-12 * np.abs(g).max() * scale.max()
+    assert st.item() == 0
