@@ -17,6 +17,7 @@
 // is returned as a double. The FP32 arithmetic runs on Blackwell's packed
 // FP32x2 instructions, two j rows per instruction.
 #include <algorithm>
+#include <type_traits>
 
 #include "pair64.cuh"
 #include "qym_internal.cuh"
@@ -189,8 +190,10 @@ struct JPairs {
 // with a smaller minimum is recorded and re-tested exactly by k_flag_chunks.
 // In a chunk of the diagonal tile the row's own j (r^2 = 0) is left out of
 // the minimum. Without FORCE only the search runs (the same separations and
-// r^2).
-template <int IPT, bool FLAG, bool DIAG, bool FORCE>
+// r^2). With UNI every j has the same G m, which the caller multiplies the sums
+// by: one product a pair less on the FMA pipe that bounds the kick (planetesimals
+// of one mass fill nearly every window; heavy bodies are summed elsewhere).
+template <int IPT, bool FLAG, bool DIAG, bool FORCE, bool UNI>
 __device__ __forceinline__ void mixed_chunk(const JPairs &s, int p0, int p1, int jt,
                                             const int (&gi)[IPT],
                                             const float2 (&nxh)[IPT], const float2 (&nyh)[IPT],
@@ -213,7 +216,7 @@ __device__ __forceinline__ void mixed_chunk(const JPairs &s, int p0, int p1, int
             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             if (FORCE) {
                 const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                float2 sm = __fmul2_rn(__fmul2_rn(gm, ri), __fmul2_rn(ri, ri));
+                float2 sm = __fmul2_rn(UNI ? ri : __fmul2_rn(gm, ri), __fmul2_rn(ri, ri));
                 if (DIAG) {
                     sm.x = (r2.x > 0.0f) ? sm.x : 0.0f;
                     sm.y = (r2.y > 0.0f) ? sm.y : 0.0f;
@@ -246,7 +249,7 @@ struct JFar {
     float4 *a, *b, *d;  // d: the near layout's fourth float4, for -c0, -c1
 };
 
-template <int IPT, bool FLAG, bool FORCE>
+template <int IPT, bool FLAG, bool FORCE, bool UNI>
 __device__ __forceinline__ void far_chunk(const JFar &s, int p0, int p1, const float2 (&dxi)[IPT],
                                           const float2 (&dyi)[IPT], const float2 (&dzi)[IPT],
                                           float2 (&fx)[IPT], float2 (&fy)[IPT], float2 (&fz)[IPT],
@@ -269,7 +272,7 @@ __device__ __forceinline__ void far_chunk(const JFar &s, int p0, int p1, const f
             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             if (FORCE) {
                 const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                const float2 sm = __fmul2_rn(__fmul2_rn(gm, ri), __fmul2_rn(ri, ri));
+                const float2 sm = __fmul2_rn(UNI ? ri : __fmul2_rn(gm, ri), __fmul2_rn(ri, ri));
                 fx[k] = __ffma2_rn(sm, dx, fx[k]);
                 fy[k] = __ffma2_rn(sm, dy, fy[k]);
                 fz[k] = __ffma2_rn(sm, dz, fz[k]);
@@ -376,6 +379,10 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         // which layouts this CTA's warps need
         const bool any_far = __syncthreads_or(far);
         const bool any_near = __syncthreads_or(!far);
+        // one G m for the whole window (and not zero, so that the pad and a
+        // massless body are never taken for it)
+        const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
+        bool same = gm0 > 0.0f;
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
             const int j0 = jt + 2 * t;
             const bool two = 2 * t + 1 < n;
@@ -388,6 +395,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     l1 = a.lo[j0 + 1];
                 }
                 s_a[t] = make_float4(p0.x, p1.x, p0.y, p1.y);
+                same = same && p0.w == gm0 && (!two || p1.w == gm0);
                 s_b[t] = make_float4(p0.z, p1.z, p0.w, p1.w);
                 s_c[t] = make_float4(l0.x, l1.x, l0.y, l1.y);
                 s_d[t] = make_float4(l0.z, l1.z, -l0.w, -l1.w);
@@ -401,11 +409,13 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     c1 = a.lo[j0 + 1].w;
                 }
                 s_fa[t] = make_float4(f0.x, f1.x, f0.y, f1.y);
+                same = same && f0.w == gm0 && (!two || f1.w == gm0);
                 s_fb[t] = make_float4(f0.z, f1.z, f0.w, f1.w);
                 if (FLAG && !any_near) s_d[t] = make_float4(0.f, 0.f, -a.lo[j0].w, -c1);
             }
         }
-        __syncthreads();
+        const bool uni = FORCE ? __syncthreads_and(same) : (__syncthreads(), false);
+        const float gw = uni ? gm0 : 1.0f;
         if (far) {
             // d_i = c - Q_i = (c - x_hi) - x_lo rounded once, duplicated for
             // the packed form
@@ -428,26 +438,30 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                 fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
                 mind[k] = 3.0e38f;
             }
-            if (far && quiet)
-                far_chunk<IPT, false, FORCE>(sf, c, ce, dxi, dyi, dzi, fx, fy, fz, mind);
-            else if (far)
-                far_chunk<IPT, FLAG, FORCE>(sf, c, ce, dxi, dyi, dzi, fx, fy, fz, mind);
-            else if (quiet)
-                mixed_chunk<IPT, false, false, FORCE>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl,
-                                                      nzl, fx, fy, fz, mind);
-            else if (diag)
-                mixed_chunk<IPT, FLAG, true, FORCE>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl, nzl,
-                                                    fx, fy, fz, mind);
-            else
-                mixed_chunk<IPT, FLAG, false, FORCE>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl, nzl,
-                                                     fx, fy, fz, mind);
+            const auto run = [&](auto u) {
+                constexpr bool U = decltype(u)::value;
+                if (far && quiet)
+                    far_chunk<IPT, false, FORCE, U>(sf, c, ce, dxi, dyi, dzi, fx, fy, fz, mind);
+                else if (far)
+                    far_chunk<IPT, FLAG, FORCE, U>(sf, c, ce, dxi, dyi, dzi, fx, fy, fz, mind);
+                else if (quiet)
+                    mixed_chunk<IPT, false, false, FORCE, U>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl,
+                                                             nyl, nzl, fx, fy, fz, mind);
+                else if (diag)
+                    mixed_chunk<IPT, FLAG, true, FORCE, U>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl,
+                                                           nzl, fx, fy, fz, mind);
+                else
+                    mixed_chunk<IPT, FLAG, false, FORCE, U>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl,
+                                                            nzl, fx, fy, fz, mind);
+            };
+            if (FORCE && uni) run(std::integral_constant<bool, FORCE>{}); else run(std::false_type{});
 #pragma unroll
             for (int k = 0; k < IPT; ++k) {
                 if (FORCE) {
                     float s, e;
-                    two_sum(ahx[k], fx[k].x + fx[k].y, s, e); ahx[k] = s; alx[k] += e;
-                    two_sum(ahy[k], fy[k].x + fy[k].y, s, e); ahy[k] = s; aly[k] += e;
-                    two_sum(ahz[k], fz[k].x + fz[k].y, s, e); ahz[k] = s; alz[k] += e;
+                    two_sum(ahx[k], gw * (fx[k].x + fx[k].y), s, e); ahx[k] = s; alx[k] += e;
+                    two_sum(ahy[k], gw * (fy[k].x + fy[k].y), s, e); ahy[k] = s; aly[k] += e;
+                    two_sum(ahz[k], gw * (fz[k].x + fz[k].y), s, e); ahz[k] = s; alz[k] += e;
                 }
                 // only partners j > i become candidates, so a chunk wholly at or
                 // below the row needs no record
