@@ -58,6 +58,10 @@ struct qym_ctx {
     qym_stats stats;
     std::string err;
     int32_t status_bits = 0;
+    // pair-symmetric kick: its shape (G = 0: none for this context) and units;
+    // in use while d.sym.G > 0, a launch shape set by hand takes its place
+    SymShape sym;
+    std::vector<int4> sym_items;
     int32_t items_cap = 0, splits_cap = 0;  // sizes of the item and partial buffers
     int32_t *kick_cnt = nullptr;            // per i-block arrival counters of the kick
     int64_t n_heavy = 0;    // heavy bodies over all systems
@@ -179,6 +183,8 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // bodies from which a single system's kick holds them in Morton order
 constexpr int64_t kSortMinBodies = 2048;
+// bodies from which the mixed kick of one system forms each pair once (kick.cu)
+constexpr int64_t kSymMinBodies = 8192;
 // bodies from which QYM_SEARCH_AUTO takes the binned search for one system
 constexpr int64_t kBinnedMinBodies = 65536;
 // steps between re-sorts inside one qym_step call (bodies drift apart slowly;
@@ -199,6 +205,7 @@ struct Carver {
 };
 
 static void choose_slot_sums(qym_ctx *c);
+static void use_sym(qym_ctx *c, bool on);
 
 // the captured steps, dropped whenever what they hold by value changes (the
 // launch shape, the log and snapshot pointers, tau)
@@ -263,7 +270,8 @@ static void carve_all(qym_ctx *c, Carver &k) {
     d.pk_lo = k.take<float4>(R);
     d.amag = k.take<float>(R);
     d.rH_bound = k.take<float>(R);
-    d.apart = k.take<double>((size_t)3 * R * c->splits_cap);
+    d.apart = k.take<double>((size_t)3 * R * std::max(c->splits_cap, c->sym.splits));
+    d.sym_items = k.take<int4>(c->sym_items.size());
     d.items = k.take<int4>(c->items_cap);
     d.item_slot = k.take<int32_t>(c->items_cap);
     c->kick_cnt = k.take<int32_t>(c->items_cap);  // zero with the arena
@@ -581,6 +589,11 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     // one system of at least two tiles' worth of bodies, mixed kick: the kick
     // holds the bodies in Morton order (sort.cu)
     c->sort_rows = nsys == 1 && params->kick_prec == QYM_KICK_MIXED && R - 1 >= kSortMinBodies;
+    // the kick with each pair formed once, where its partial slots fit 2 GB
+    if (c->sort_rows && R - 1 >= kSymMinBodies) {
+        c->sym = sym_shape(R - 1, ((int64_t)2 << 30) / (24 * R));
+        if (c->sym.G > 0) sym_items_host(R - 1, c->sym, c->sym_items);
+    }
     // measured on one GB300 (same trajectories, so the same encounter work):
     // 16384-body disk 1.40 ms per step binned against 1.33 fused, the
     // 512-system ensemble 23.6 against 20.3 ms, the 262144-body disk 64.9
@@ -608,6 +621,7 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     Carver real{(char *)c->arena, 0, false};
     carve_all(c, real);
     choose_slot_sums(c);
+    use_sym(c, true);
     if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaFree(c->arena);
         delete c;
@@ -650,6 +664,9 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     CKI(cudaMemcpyAsync(d.m, m, sizeof(double) * R, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.items, items.data(), sizeof(int4) * d.nitems, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.item_slot, slots.data(), sizeof(int32_t) * d.nitems, cudaMemcpyHostToDevice, c->stream));
+    if (!c->sym_items.empty())
+        CKI(cudaMemcpyAsync(d.sym_items, c->sym_items.data(), sizeof(int4) * c->sym_items.size(),
+                            cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.mchunks, mch.data(), sizeof(int4) * d.nmchunks, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.sys_chunk0, sc0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(c->eblocks, eblk.data(), sizeof(int4) * eblk.size(), cudaMemcpyHostToDevice, c->stream));
@@ -677,8 +694,7 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     qym_status st = upload_state(c, q, v);
     if (st != QYM_OK) return bail(st);
     std::memset(&c->stats, 0, sizeof(c->stats));
-    c->stats.kick_tile_i = c->tune.threads * c->tune.ipt;
-    c->stats.kick_tile_splits = c->tune.splits;
+    use_sym(c, true);
     *out = c;
     return QYM_OK;
 }
@@ -1027,8 +1043,7 @@ static qym_status collect(qym_ctx *c, int64_t nsteps) {
     s.status_bits = status;
     s.launches = c->launches;
     s.hermite_steps_max = (int64_t)ctr[C_MAX_HSET];
-    s.kick_tile_i = c->tune.threads * c->tune.ipt;
-    s.kick_tile_splits = c->tune.splits;
+    use_sym(c, d.sym.G > 0);  // (the launch shape's counters)
     s.whole_steps = (int32_t)c->wh_steps;
     s.hermite_steps += c->wh_hsteps;
     s.hermite_steps_max = std::max<int64_t>(s.hermite_steps_max, c->wh_hmax);
@@ -1809,6 +1824,15 @@ static void choose_slot_sums(qym_ctx *c) {
     d.kick_cnt = 24 * d.rows * (int64_t)d.splits > kSlotSumInKickBytes ? c->kick_cnt : nullptr;
 }
 
+// the pair-symmetric kick on (where the context has one) or off
+static void use_sym(qym_ctx *c, bool on) {
+    Dev &d = c->d;
+    d.sym = on && d.own_hi == 0 ? c->sym : SymShape();
+    d.sym_nitems = d.sym.G > 0 ? (int32_t)c->sym_items.size() : 0;
+    c->stats.kick_tile_i = d.sym.G > 0 ? kSymBlock : c->tune.threads * c->tune.ipt;
+    c->stats.kick_tile_splits = d.sym.G > 0 ? d.sym.splits : c->tune.splits;
+}
+
 // rebuild the work items for a launch shape (device buffers sized for the
 // largest item count and split count seen so far are reused when they fit)
 static qym_status apply_tune(qym_ctx *c, const KickTune &t) {
@@ -1830,6 +1854,7 @@ static qym_status apply_tune(qym_ctx *c, const KickTune &t) {
     d.splits = t.splits;
     choose_slot_sums(c);
     c->tune = t;
+    use_sym(c, false);
     drop_graphs(c);  // the captured steps hold the old shape
     return QYM_OK;
 }
@@ -1848,8 +1873,6 @@ extern "C" qym_status qym_set_kick_shape(qym_ctx *c, int32_t threads, int32_t ip
     t.splits = splits;
     qym_status s = apply_tune(c, t);
     if (s != QYM_OK) return s;
-    c->stats.kick_tile_i = threads * ipt;
-    c->stats.kick_tile_splits = splits;
     return QYM_OK;
 }
 
@@ -1871,6 +1894,13 @@ extern "C" qym_status qym_autotune(qym_ctx *c) {
             }
     KickTune best = c->tune;
     double best_ms = 1e30;
+    bool sym = false;
+    if (c->sym.G > 0 && c->d.own_hi == 0) {  // the pair-symmetric kick first
+        use_sym(c, true);
+        qym_status s = time_kick_shape(c, fused_search(c), 3, best, &best_ms, true);
+        if (s != QYM_OK) return s;
+        sym = true;
+    }
     for (const KickTune &t : cands) {
         qym_status s = apply_tune(c, t);
         if (s != QYM_OK) return s;
@@ -1879,12 +1909,11 @@ extern "C" qym_status qym_autotune(qym_ctx *c) {
         // kick's tail but give the finisher more partial slots to add
         s = time_kick_shape(c, fused_search(c), 3, t, &ms, true);
         if (s != QYM_OK) return s;
-        if (ms < best_ms) { best_ms = ms; best = t; }
+        if (ms < best_ms) { best_ms = ms; best = t; sym = false; }
     }
     qym_status s = apply_tune(c, best);
     if (s != QYM_OK) return s;
-    c->stats.kick_tile_i = best.threads * best.ipt;
-    c->stats.kick_tile_splits = best.splits;
+    use_sym(c, sym);
     c->amag_valid = false;
     return QYM_OK;
 }

@@ -18,6 +18,7 @@
 // FP32x2 instructions, two j rows per instruction.
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "pair64.cuh"
 #include "qym_internal.cuh"
@@ -53,6 +54,7 @@ struct KickArgs {
     const int32_t *perm;    // row of each position of the packs (NULL: row order)
     const float4 *far;      // (o_x, o_y, o_z, G m): offset from the tile's reference point
     const float4 *tile;     // per tile: (c_x, c_y, c_z, R), box min (x, y, z, -), box max
+    SymShape sym;           // pair-symmetric form (k_kick_sym)
     int32_t *blk_cnt = nullptr;  // arrivals per i-block (NULL: each slot stays for the finisher)
     int32_t splits = 1;          // items (slots) per i-block
 };
@@ -484,6 +486,342 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
     if (a.blk_cnt) sum_block_slots<IPT>(a, gi, it.x, it.y);
 }
 
+// ---------------------------------------------------------------- pairs once
+// The mixed kick of one system in Morton order with each pair formed once: the
+// separation, r^2 and r^-3 serve both bodies (Newton's third law), 14 FMA-pipe
+// instructions a far pair of equal masses instead of 2 x 11, which is what bounds
+// the kick.
+//
+// An i-block is 512 consecutive positions, four per thread, a warp's 128
+// consecutive ones (compact along the Morton curve, so that more windows are far
+// from all of them). Windows of 256 positions past the block stream through shared
+// memory as in k_kick_mixed; the block's own two tiles take that kernel's
+// one-sided form. For the j side each lane starts at a different j pair of a
+// 64-body chunk and holds the pair's sums, which move on with the pair from lane
+// to lane (six shuffles a step, against twelve passes of shared memory for a
+// read-modify-write there), so after 32 steps lane l holds the sums of pair l over
+// the warp's 128 rows: added per step as sums of four, 32 in a row, as the i side
+// adds its own. The warps' sums are added in FP64.
+//
+// Work unit: G consecutive i-blocks against a range of rh half tiles (the part
+// past each block). Rows get one slot of partial sums per range from their own
+// block, and one per group of earlier i-blocks from the j side, added up in the
+// group's order by the unit that owns the slot. sym_slots (qym_internal.cuh)
+// gives a row's valid slots.
+constexpr int SYM_T = 128, SYM_R = 4, SYM_BLK = SYM_T * SYM_R, SYM_W = SYM_T / 32;
+static_assert(SYM_BLK == kSymBlock, "i-block of the pair-symmetric kick");
+
+struct SymShared {
+    float4 a[TILE / 2], b[TILE / 2], c[TILE / 2], d[TILE / 2];  // near layout (JPairs)
+    float4 fa[TILE / 2], fb[TILE / 2];                           // far layout (JFar)
+    float4 ip[SYM_BLK], il[SYM_BLK];                             // the i-block's packs
+    float acc[6][SYM_BLK];                                       // i sums, two-sum pairs (hi, lo)
+    float4 jxy[SYM_W][TILE / 2];                                 // j sums of a warp (x0, x1, y0, y1)
+    float2 jz[SYM_W][TILE / 2];
+};
+
+// One chunk of 32 j pairs from p0 against the four rows of a thread. FAR: (ix, iy,
+// iz) are the rows' d_i = c - Q_i; else -Q_i (hi) with (lx, ly, lz) -Q_i (lo).
+// UNI: one G m for the rows and one for the window, multiplied in by the caller.
+// Leaves in (jx, jy, jz) the j sums of pair p0 + lane, sign flipped.
+template <bool FLAG, bool FORCE, bool UNI, bool FAR>
+__device__ __forceinline__ void sym_chunk(const SymShared &S, int p0, const float2 (&ix)[SYM_R],
+                                          const float2 (&iy)[SYM_R], const float2 (&iz)[SYM_R],
+                                          const float2 (&lx)[SYM_R], const float2 (&ly)[SYM_R],
+                                          const float2 (&lz)[SYM_R], const float (&gi)[SYM_R],
+                                          float2 (&fx)[SYM_R], float2 (&fy)[SYM_R], float2 (&fz)[SYM_R],
+                                          float (&mind)[SYM_R], float2 &jx, float2 &jy, float2 &jz) {
+    const int lane = threadIdx.x & 31, next = (lane + 1) & 31;
+    jx = jy = jz = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+    for (int s = 0; s < 32; ++s) {
+        const int p = p0 + ((lane + s) & 31);
+        float4 A, B, C, D;
+        if (FAR) {
+            A = S.fa[p];
+            B = S.fb[p];
+            if (FLAG) D = S.d[p];
+        } else {
+            A = S.a[p];
+            B = S.b[p];
+            C = S.c[p];
+            D = S.d[p];
+        }
+        const float2 x = make_float2(A.x, A.y), y = make_float2(A.z, A.w);
+        const float2 z = make_float2(B.x, B.y), gm = make_float2(B.z, B.w);
+        float2 tx, ty, tz;
+#pragma unroll
+        for (int k = 0; k < SYM_R; ++k) {
+            float2 dx = __fadd2_rn(x, ix[k]), dy = __fadd2_rn(y, iy[k]), dz = __fadd2_rn(z, iz[k]);
+            if (!FAR) {
+                dx = __fadd2_rn(dx, __fadd2_rn(make_float2(C.x, C.y), lx[k]));
+                dy = __fadd2_rn(dy, __fadd2_rn(make_float2(C.z, C.w), ly[k]));
+                dz = __fadd2_rn(dz, __fadd2_rn(make_float2(D.x, D.y), lz[k]));
+            }
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            if (FORCE) {
+                const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+                const float2 r3 = __fmul2_rn(ri, __fmul2_rn(ri, ri));
+                const float2 si = UNI ? r3 : __fmul2_rn(gm, r3);
+                const float2 sj = UNI ? r3 : __fmul2_rn(make_float2(gi[k], gi[k]), r3);
+                fx[k] = __ffma2_rn(si, dx, fx[k]);
+                fy[k] = __ffma2_rn(si, dy, fy[k]);
+                fz[k] = __ffma2_rn(si, dz, fz[k]);
+                tx = k ? __ffma2_rn(sj, dx, tx) : __fmul2_rn(sj, dx);
+                ty = k ? __ffma2_rn(sj, dy, ty) : __fmul2_rn(sj, dy);
+                tz = k ? __ffma2_rn(sj, dz, tz) : __fmul2_rn(sj, dz);
+            }
+            if (FLAG) {
+                const float2 t = __fadd2_rn(r2, make_float2(D.z, D.w));
+                mind[k] = fmin3(mind[k], t.x, t.y);
+            }
+        }
+        if (FORCE) {
+            jx = __fadd2_rn(jx, tx);
+            jy = __fadd2_rn(jy, ty);
+            jz = __fadd2_rn(jz, tz);
+            // the next step takes the pair the lane above has just had
+            jx.x = __shfl_sync(0xffffffffu, jx.x, next);
+            jx.y = __shfl_sync(0xffffffffu, jx.y, next);
+            jy.x = __shfl_sync(0xffffffffu, jy.x, next);
+            jy.y = __shfl_sync(0xffffffffu, jy.y, next);
+            jz.x = __shfl_sync(0xffffffffu, jz.x, next);
+            jz.y = __shfl_sync(0xffffffffu, jz.y, next);
+        }
+    }
+}
+
+template <bool FLAG, bool FORCE>
+__global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
+    chain_wait();
+    extern __shared__ __align__(16) unsigned char g_symsmem[];
+    SymShared &S = *reinterpret_cast<SymShared *>(g_symsmem);
+    const JPairs sp{S.a, S.b, S.c, S.d};
+    const int4 u = a.items[blockIdx.x];  // i-blocks [x, y), half tiles [z, w)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int npos = (int)a.rows;
+    const int64_t rows = a.rows;
+    const int i_of = warp * 32 * SYM_R + lane;  // row k of this thread: block start + i_of + 32 k
+    for (int blk = u.x; blk < u.y; ++blk) {
+        const int i_lo = 1 + blk * SYM_BLK, i_hi = i_lo + SYM_BLK;
+        const int h0 = max(u.z, 4 * blk);  // from the block's own half tiles on
+        if (h0 >= u.w) continue;
+        int gi[SYM_R];
+        float rho[SYM_R], gmi[SYM_R];
+        bool i_same = true;
+        const float gi0 = a.pos[i_lo].w;
+        __syncthreads();  // the packs of the block before are no longer read
+#pragma unroll
+        for (int k = 0; k < SYM_R; ++k) {
+            const int o = i_of + 32 * k, i = i_lo + o;
+            gi[k] = i;
+            // idle row: parked far away so its arithmetic stays finite
+            float4 p = make_float4(1e18f, 1e18f, 1e18f, 0.0f), l = make_float4(0.f, 0.f, 0.f, -1e30f);
+            if (i < npos) {
+                p = a.pos[i];
+                l = a.lo[i];
+            }
+            i_same = i_same && p.w == gi0;
+            rho[k] = l.w;
+            gmi[k] = p.w;
+            S.ip[o] = p;
+            S.il[o] = l;
+#pragma unroll
+            for (int c = 0; c < 6; ++c) S.acc[c][o] = 0.0f;
+        }
+        const bool i_uni = __syncthreads_and(i_same) && gi0 > 0.0f;
+        for (int jt = 1 + h0 * (TILE / 2), n = 0; jt < npos && jt < 1 + u.w * (TILE / 2); jt += n) {
+            // windows to the end of the tile, the range or the system
+            n = min(min(1 + ((jt - 1) / TILE + 1) * TILE, 1 + u.w * (TILE / 2)), npos) - jt;
+            const int np = (n + 1) >> 1;
+            const bool diag = jt < i_hi;
+            bool far = false, quiet = false;
+            float4 m0 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!diag) {
+                const float4 *tm = a.tile + 3 * ((jt - 1) / TILE);
+                m0 = tm[0];
+                const float4 m1 = tm[1], m2 = tm[2];
+                bool mine = true, calm = true;
+#pragma unroll
+                for (int k = 0; k < SYM_R; ++k) {
+                    const float4 P = S.ip[i_of + 32 * k];
+                    const float ex = fmaxf(fmaxf(m1.x - P.x, P.x - m2.x), 0.0f);
+                    const float ey = fmaxf(fmaxf(m1.y - P.y, P.y - m2.y), 0.0f);
+                    const float ez = fmaxf(fmaxf(m1.z - P.z, P.z - m2.z), 0.0f);
+                    const float d2 = ex * ex + ey * ey + ez * ez;
+                    mine = mine && (d2 >= 1.02f * m0.w * m0.w);
+                    if (FLAG)
+                        calm = calm && (d2 >= 1.03f * (rho[k] + m1.w) +
+                                                  1e-9f * (P.x * P.x + P.y * P.y + P.z * P.z));
+                }
+                far = __all_sync(0xffffffffu, mine);
+                if (FLAG) quiet = __all_sync(0xffffffffu, calm);
+            }
+            const bool any_far = __syncthreads_or(far);
+            const bool any_near = __syncthreads_or(!far);
+            const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
+            bool same = gm0 > 0.0f;
+            // (padded to whole chunks of 32 pairs with massless bodies far from everything)
+            for (int t = tid; t < ((np + 31) & ~31); t += SYM_T) {
+                const int j0 = jt + 2 * t;
+                const bool one = 2 * t < n, two = 2 * t + 1 < n;
+                const float4 pad = make_float4(2e18f, 2e18f, 2e18f, 0.0f);
+                const float4 pad_l = make_float4(0.f, 0.f, 0.f, -1e30f);
+                const float4 l0 = one && (any_near || FLAG) ? a.lo[j0] : pad_l;
+                const float4 l1 = two && (any_near || FLAG) ? a.lo[j0 + 1] : pad_l;
+                if (any_near) {
+                    const float4 p0 = one ? a.pos[j0] : pad, p1 = two ? a.pos[j0 + 1] : pad;
+                    same = same && (!one || p0.w == gm0) && (!two || p1.w == gm0);
+                    S.a[t] = make_float4(p0.x, p1.x, p0.y, p1.y);
+                    S.b[t] = make_float4(p0.z, p1.z, p0.w, p1.w);
+                    S.c[t] = make_float4(l0.x, l1.x, l0.y, l1.y);
+                }
+                S.d[t] = make_float4(l0.z, l1.z, -l0.w, -l1.w);
+                if (any_far) {
+                    const float4 f0 = one ? a.far[j0] : pad, f1 = two ? a.far[j0 + 1] : pad;
+                    same = same && (!one || f0.w == gm0) && (!two || f1.w == gm0);
+                    S.fa[t] = make_float4(f0.x, f1.x, f0.y, f1.y);
+                    S.fb[t] = make_float4(f0.z, f1.z, f0.w, f1.w);
+                }
+            }
+            const bool j_uni = FORCE ? __syncthreads_and(same) : (__syncthreads(), false);
+            const bool uni = j_uni && i_uni && !diag;
+            const float gw = uni ? gm0 : 1.0f, gv = uni ? -gi0 : -1.0f;
+            float2 ix[SYM_R], iy[SYM_R], iz[SYM_R], lx[SYM_R], ly[SYM_R], lz[SYM_R];
+#pragma unroll
+            for (int k = 0; k < SYM_R; ++k) {
+                const float4 P = S.ip[i_of + 32 * k], L = S.il[i_of + 32 * k];
+                // far: d_i = c - Q_i = (c - x_hi) - x_lo rounded once
+                const float x = far ? ds_add(m0.x, -P.x, -L.x) : -P.x;
+                const float y = far ? ds_add(m0.y, -P.y, -L.y) : -P.y;
+                const float z = far ? ds_add(m0.z, -P.z, -L.z) : -P.z;
+                ix[k] = make_float2(x, x);
+                iy[k] = make_float2(y, y);
+                iz[k] = make_float2(z, z);
+                lx[k] = make_float2(-L.x, -L.x);
+                ly[k] = make_float2(-L.y, -L.y);
+                lz[k] = make_float2(-L.z, -L.z);
+            }
+            for (int c = 0; c < np; c += 32) {
+                float2 fx[SYM_R], fy[SYM_R], fz[SYM_R], jx, jy, jz;
+                float mind[SYM_R];
+#pragma unroll
+                for (int k = 0; k < SYM_R; ++k) {
+                    fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
+                    mind[k] = 3.0e38f;
+                }
+                if (diag) {
+                    mixed_chunk<SYM_R, FLAG, true, FORCE, false>(sp, c, min(c + 32, np), jt, gi, ix, iy, iz,
+                                                                 lx, ly, lz, fx, fy, fz, mind);
+                } else {
+                    const auto run = [&](auto U, auto F, auto Q) {
+                        sym_chunk<FLAG && decltype(Q)::value, FORCE, decltype(U)::value, decltype(F)::value>(
+                            S, c, ix, iy, iz, lx, ly, lz, gmi, fx, fy, fz, mind, jx, jy, jz);
+                    };
+                    using T1 = std::true_type;
+                    using T0 = std::false_type;
+                    if (far && (quiet || !FLAG)) {
+                        if (uni) run(T1{}, T1{}, T0{}); else run(T0{}, T1{}, T0{});
+                    } else if (far) {
+                        run(T0{}, T1{}, T1{});
+                    } else if (quiet || !FLAG) {
+                        if (uni) run(T1{}, T0{}, T0{}); else run(T0{}, T0{}, T0{});
+                    } else {
+                        run(T0{}, T0{}, T1{});
+                    }
+                    if (FORCE) {
+                        const float v = (FLAG && !quiet) ? -1.0f : gv;
+                        S.jxy[warp][c + lane] = make_float4(v * jx.x, v * jx.y, v * jy.x, v * jy.y);
+                        S.jz[warp][c + lane] = make_float2(v * jz.x, v * jz.y);
+                    }
+                }
+                const float g = (FLAG && !quiet) ? 1.0f : gw;
+#pragma unroll
+                for (int k = 0; k < SYM_R; ++k) {
+                    const int o = i_of + 32 * k;
+                    if (FORCE) {
+                        float s, e;
+                        two_sum(S.acc[0][o], g * (fx[k].x + fx[k].y), s, e); S.acc[0][o] = s; S.acc[3][o] += e;
+                        two_sum(S.acc[1][o], g * (fy[k].x + fy[k].y), s, e); S.acc[1][o] = s; S.acc[4][o] += e;
+                        two_sum(S.acc[2][o], g * (fz[k].x + fz[k].y), s, e); S.acc[2][o] = s; S.acc[5][o] += e;
+                    }
+                    // only partners j > i become candidates
+                    const int j1 = jt + min(2 * c + 64, n);
+                    if (FLAG && mind[k] < rho[k] && j1 - 1 > gi[k]) push_flag(a, gi[k], jt + 2 * c, j1);
+                }
+            }
+            __syncthreads();  // the window is no longer read; every warp's j sums are there
+            if (FORCE && !diag) {
+                // slot of the group's j sums: the group's first block stores, the others add
+                double *const out = a.apart + (int64_t)(a.sym.nc + blk / a.sym.G) * 3 * rows + jt;
+                const bool first = blk == u.x;
+                for (int t = tid; t < np; t += SYM_T) {
+                    const bool two = 2 * t + 1 < n;
+                    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                    for (int w = 0; w < SYM_W; ++w) {
+                        const float4 xy = S.jxy[w][t];
+                        const float2 z = S.jz[w][t];
+                        v[0] += (double)xy.x; v[1] += (double)xy.y; v[2] += (double)xy.z;
+                        v[3] += (double)xy.w; v[4] += (double)z.x; v[5] += (double)z.y;
+                    }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        double *const o = out + c * rows + 2 * t;
+                        o[0] = first ? v[2 * c] : o[0] + v[2 * c];
+                        if (two) o[1] = first ? v[2 * c + 1] : o[1] + v[2 * c + 1];
+                    }
+                }
+            }
+        }
+        if (FORCE) {
+            double *const out = a.apart + (int64_t)(u.z / a.sym.rh) * 3 * rows;
+#pragma unroll
+            for (int k = 0; k < SYM_R; ++k) {
+                const int o = i_of + 32 * k;
+                if (gi[k] < npos) {
+                    out[gi[k]] = (double)S.acc[0][o] + (double)S.acc[3][o];
+                    out[rows + gi[k]] = (double)S.acc[1][o] + (double)S.acc[4][o];
+                    out[2 * rows + gi[k]] = (double)S.acc[2][o] + (double)S.acc[5][o];
+                }
+            }
+        }
+    }
+}
+
+// Units of the pair-symmetric kick of nb bodies with at most max_slots slots a
+// row: about 2000 (four CTAs on each SM, several waves), ranges and groups of the
+// same length where the slots allow; G = 0 where they do not.
+SymShape sym_shape(int64_t nb, int64_t max_slots) {
+    SymShape y;
+    const int64_t nblk = (nb + SYM_BLK - 1) / SYM_BLK, nhalf = (nb + TILE / 2 - 1) / (TILE / 2);
+    y.G = (int32_t)std::max<int64_t>(1, (nblk + 63) / 64);
+    const int64_t ng = (nblk + y.G - 1) / y.G;
+    const int64_t want = std::min<int64_t>(128, std::max<int64_t>(64, 4096 / ng));
+    y.rh = (int32_t)std::max<int64_t>(1, (nhalf + want - 1) / want);
+    y.nc = (int32_t)((nhalf + y.rh - 1) / y.rh);
+    y.splits = (int32_t)(y.nc + ng);
+    if (y.splits > max_slots) y.G = 0;
+    return y;
+}
+
+void sym_items_host(int64_t nb, const SymShape &y, std::vector<int4> &items) {
+    const int64_t nblk = (nb + SYM_BLK - 1) / SYM_BLK;
+    items.clear();
+    for (int64_t b = 0; b < nblk; b += y.G)
+        for (int64_t c = 4 * b / y.rh; c < y.nc; ++c)
+            items.push_back(make_int4((int)b, (int)std::min<int64_t>(b + y.G, nblk), (int)(c * y.rh),
+                                      (int)((c + 1) * y.rh)));
+}
+
+template <bool FLAG, bool FORCE>
+static cudaError_t launch_sym(const KickArgs &a, int nitems, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(k_kick_sym<FLAG, FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(SymShared));
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_kick_sym<FLAG, FORCE>, nitems, SYM_T, sizeof(SymShared), st, a);
+}
+
 // Exact test of the flagged chunks, one warp per entry, lane l on the j rows
 // j0 + l and j0 + 32 + l: candidates (i, j), i < j, with r^2 < c_i + c_j, the
 // separation formed from the same split positions in the same order as the
@@ -861,10 +1199,19 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     if (flag != KICK_FORCE && flag != KICK_SEARCH && flag != KICK_SEARCH_ONLY)
         return cudaErrorInvalidValue;
     if (prec == QYM_KICK_MIXED) {
-        if (flag == KICK_FORCE) return launch_mixed<false, true>(a, d.nitems, threads, ipt, st);
+        const bool sym = d.sym.G > 0;
+        if (sym) {
+            a.items = d.sym_items;
+            a.sym = d.sym;
+        }
+        if (flag == KICK_FORCE)
+            return sym ? launch_sym<false, true>(a, d.sym_nitems, st)
+                       : launch_mixed<false, true>(a, d.nitems, threads, ipt, st);
         cudaError_t e = flag == KICK_SEARCH
-                            ? launch_mixed<true, true>(a, d.nitems, threads, ipt, st)
-                            : launch_mixed<true, false>(a, d.nitems, threads, ipt, st);
+                            ? (sym ? launch_sym<true, true>(a, d.sym_nitems, st)
+                                   : launch_mixed<true, true>(a, d.nitems, threads, ipt, st))
+                            : (sym ? launch_sym<true, false>(a, d.sym_nitems, st)
+                                   : launch_mixed<true, false>(a, d.nitems, threads, ipt, st));
         if (e) return e;
         // about one entry per row (its own chunk) plus the close pairs
         int64_t blocks = (d.rows + 63) / 64;

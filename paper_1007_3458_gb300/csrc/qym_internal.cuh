@@ -17,6 +17,15 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kHermMaxClusters = 160;  // entries of Dev::hcl (2 x 152 CTAs in clusters of 2 or more)
 
 // ---------------------------------------------------------------- layout
+// Units and partial slots of the pair-symmetric mixed kick (kick.cu): groups of G
+// i-blocks of kSymBlock positions against ranges of rh half tiles (128
+// positions); G = 0: not in use. A row's slots: one per range from its own block,
+// then one per group of earlier i-blocks.
+constexpr int kSymBlock = 512;
+struct SymShape {
+    int32_t G = 0, rh = 0, nc = 0, splits = 0;  // nc ranges; splits slots in all
+};
+
 // Device state of a context. Rows of all systems are concatenated; each
 // system's star sits at its first row with Q = v = 0. Positions and
 // velocities are float64 structure-of-arrays [3][rows].
@@ -37,6 +46,9 @@ struct Dev {
     float *rH_bound = nullptr;    // [rows] Hill radius bound used by the crude test
     double *apart = nullptr;      // [splits][3][rows] kick partial accelerations
     int32_t splits = 1;
+    SymShape sym;                 // pair-symmetric kick (one system in Morton order)
+    int4 *sym_items = nullptr;    // its units: i-blocks [x, y), half tiles [z, w)
+    int32_t sym_nitems = 0;
     int32_t *kick_cnt = nullptr;  // arrivals per i-block: with it the kick's last CTA of
                                   // each i-block adds the slots into slot 0 (kick.cu)
     int32_t *wh_flag = nullptr;   // [nsys] 1: this step of the system is integrated whole
@@ -253,6 +265,20 @@ __device__ __forceinline__ void heavy_list(int64_t rows, const double *m, double
 // the calling thread's context-free error message (qym_last_error(NULL))
 void set_thread_error(const std::string &msg);
 
+// The valid slots of position pr under the pair-symmetric kick, k = 0 .. n - 1:
+// the ranges that reach its own i-block b or lie past it, then the groups that
+// start before b
+struct SymSlots {
+    int c0, n1, n;
+    __device__ __forceinline__ SymSlots(const SymShape &y, int64_t pr) {
+        const int b = pr > 0 ? (int)((pr - 1) / kSymBlock) : 0;
+        c0 = 4 * b / y.rh;
+        n1 = y.nc - c0;
+        n = n1 + (b + y.G - 1) / y.G;
+    }
+    __device__ __forceinline__ int slot(int k, int nc) const { return k < n1 ? c0 + k : nc + k - n1; }
+};
+
 // ---------------------------------------------------------------- launches
 // Launches in a chain: each kernel may be set up while the one before it in
 // the stream still runs (programmatic dependent launch) and waits for it, and
@@ -365,6 +391,8 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t,
                      int32_t max_items, int64_t i_lo = 0, int64_t i_hi = INT64_MAX,
                      int32_t align = 1);
 KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t max_splits);
+SymShape sym_shape(int64_t nb, int64_t max_slots);
+void sym_items_host(int64_t nb, const SymShape &y, std::vector<int4> &items);
 constexpr int kKickTile = 256;  // j rows per shared-memory tile of the kick
 int32_t kick_items_count(const int64_t *offsets, int32_t nsys, const KickTune &t,
                          int64_t i_lo = 0, int64_t i_hi = INT64_MAX);

@@ -289,12 +289,23 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
                !(d.own_hi > 0 && (r < d.own_lo || r >= d.own_hi));  // another GPU's row
     }
     if (live) {
-        const int nslots = d.kick_cnt ? 1 : d.splits;  // the kick added its slots into slot 0
-        for (int s = q; s < nslots; s += L) {
-            const double *p = d.apart + (int64_t)s * 3 * R;
-            ax += p[pr];
-            ay += p[R + pr];
-            az += p[2 * R + pr];
+        if (d.sym.G > 0) {
+            const SymSlots y(d.sym, pr);
+#pragma unroll 4
+            for (int k = q; k < y.n; k += L) {
+                const double *p = d.apart + (int64_t)y.slot(k, d.sym.nc) * 3 * R;
+                ax += p[pr];
+                ay += p[R + pr];
+                az += p[2 * R + pr];
+            }
+        } else {
+            const int nslots = d.kick_cnt ? 1 : d.splits;  // the kick added its slots into slot 0
+            for (int s = q; s < nslots; s += L) {
+                const double *p = d.apart + (int64_t)s * 3 * R;
+                ax += p[pr];
+                ay += p[R + pr];
+                az += p[2 * R + pr];
+            }
         }
         if (d.heavy_split) {
             const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
@@ -364,7 +375,7 @@ cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, doubl
     a.hill_fixed = hill_fixed;
     // groups of 4 or 8 threads a row where there are that many slots to add (8
     // also halves the chain of a small system), one where there are few
-    const int nslots = d.kick_cnt ? 1 : d.splits;
+    const int nslots = d.sym.G > 0 ? d.sym.splits : (d.kick_cnt ? 1 : d.splits);
     if (nslots >= 16)
         launch_chain(k_finish<8>, (unsigned)((d.rows + 31) / 32), 256, 0, st, d, a);
     else if (nslots >= 4)
