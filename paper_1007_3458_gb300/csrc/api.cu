@@ -725,23 +725,12 @@ __global__ void k_step_begin(unsigned long long *ctr, int32_t *vmax, int32_t nsy
     if (vmax)  // the binned search's largest |v| per system, raised by the first finisher
         for (int32_t s = threadIdx.x; s < nsys; s += blockDim.x) vmax[s] = 0;
     for (int64_t k = threadIdx.x; k < ntb; k += blockDim.x) tbits[k] = 0x7fffffff;  // tile boxes
-    if (threadIdx.x) return;
-    ctr[C_NCAND] = 0;
-    ctr[C_NACTIVE] = 0;
-    ctr[C_NENC] = 0;
-    ctr[C_NRESCAN] = 0;
-    ctr[C_NSETS] = 0;
-    ctr[C_HSMALL] = 0;
-    ctr[C_NFCHUNK] = 0;
-    ctr[C_FCDONE] = 0;
+    if (threadIdx.x == 0) step_counters_begin(ctr);
 }
 
 __global__ void k_step_end(unsigned long long *ctr, int64_t max_cand, int64_t max_enc) {
     chain_wait();
-    ctr[C_SUM_CAND] += ctr[C_NCAND];
-    ctr[C_SUM_ENC] += ctr[C_NENC];
-    ctr[C_SUM_RESCAN] += ctr[C_NRESCAN];
-    ctr[C_STEP] += 1;
+    step_counters_end(ctr);
 }
 
 // one step whose opening drift has been applied: ends with the closing drift
@@ -897,7 +886,9 @@ static cudaError_t enqueue_step(qym_ctx *c, double tau, bool last, bool fresh = 
     if (c->flush) {
         if ((e = cudaMemsetAsync(c->flush, c->launches & 0xff, (size_t)p.l2_flush_bytes, st))) return e;
     }
-    launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, c->binned ? 6 * (int64_t)c->nstiles : 0);
+    // (the call's opening or the drift before this step has cleared the counters)
+    if (c->binned)
+        launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, 6 * (int64_t)c->nstiles);
     const int fz = fused_search(c);
     // the velocities entering the first kick, for a whole-system Hermite
     if (p.whole_hermite &&
@@ -937,14 +928,13 @@ static cudaError_t enqueue_step(qym_ctx *c, double tau, bool last, bool fresh = 
                                   p.whole_hermite)))
         return e;
     // item 10 (and item 1 of the next step): drift tau/2 with S = sum m v
-    if ((e = launch_momentum(d, st))) return e;
+    if ((e = launch_momentum(d, st, true))) return e;
     if ((e = launch_drift_pack_from(d, d.q, d.v, 0.5 * tau, last ? 0.0 : 0.5 * tau, tau, p.a_E,
-                                    p.G, (!last) && fz, p.hill_fixed, st, 0.5 * tau)))
+                                    p.G, (!last) && fz, p.hill_fixed, st, 0.5 * tau, 1.01, 1, 1)))
         return e;
-    launch_chain(k_step_end, 1, 1, 0, st, d.ctr, d.max_cand, d.max_enc);
-    // begin, kick [+ chunk re-test], finish, Kepler, [refine 2, sets 7, Hermite plan, Hermite],
-    // pack, kick, finish, momentum 2, drift, end
-    c->launches += 12 + (enc ? 11 : 0) + search_retest(p, fz);
+    // kick [+ chunk re-test], finish, Kepler, [refine, sets, Hermite plan, Hermite], pack, kick,
+    // finish, momentum [1 or 2], drift
+    c->launches += 7 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 3 + sets_launches(d.rows) : 0) + search_retest(p, fz);
     return cudaGetLastError();
 }
 
@@ -956,8 +946,10 @@ static cudaError_t enqueue_opening_kick(qym_ctx *c, double tau, bool fresh) {
     const qym_params &p = c->p;
     cudaStream_t st = c->stream;
     cudaError_t e;
-    launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, c->binned ? 6 * (int64_t)c->nstiles : 0);
-    c->launches += 1;
+    if (c->binned) {
+        launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, 6 * (int64_t)c->nstiles);
+        c->launches += 1;
+    }
     const int fz = fused_search(c);
     if (fz && fresh) return enqueue_fresh_search_kick(c, 0.5 * tau);
     if ((e = launch_kick_tiles(d, p.kick_prec, fz, p.G, c->tune.threads, c->tune.ipt, st)))
@@ -991,35 +983,35 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
         if ((e = launch_sets_impl(d, p.a_H, c->ss, st))) return e;
         if ((e = launch_hermite(d, p, tau, st))) return e;
     }
-    launch_chain(k_step_end, 1, 1, 0, st, d.ctr, d.max_cand, d.max_enc);
     // (q1, v1) -> (q, v)
     if ((e = launch_drift_pack_from(d, d.q1, d.v1, 0.0, 0.0, tau, p.a_E, p.G, 0, p.hill_fixed, st,
                                     0.5 * tau)))
         return e;
     if (!last) {
-        launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, c->binned ? 6 * (int64_t)c->nstiles : 0);
-        if ((e = launch_momentum(d, st))) return e;
+        if ((e = launch_momentum(d, st, true))) return e;
         // the last kick was a step earlier: its |a| bounds this one's only
         // loosely, so the crude reach allows twice it (and the finisher checks)
         if ((e = launch_drift_pack_from(d, d.q, d.v, 0.5 * tau, 0.5 * tau, tau, p.a_E, p.G, fz,
-                                        p.hill_fixed, st, tau, 2.0)))
+                                        p.hill_fixed, st, tau, 2.0, 1, 1)))
             return e;
+        if (c->binned)
+            launch_chain(k_step_begin, 1, 256, 0, st, d.ctr, d.vmax, d.nsys, c->sarg.tbox_bits, 6 * (int64_t)c->nstiles);
         if ((e = launch_kick_tiles(d, p.kick_prec, fz, p.G, c->tune.threads, c->tune.ipt, st))) return e;
         if ((e = launch_kick_finish_v(d, d.v, d.q, tau, p.G, enc ? (fz ? 1 : 2) : 0, p.hill_fixed,
                                       st, 2.0)))
             return e;
-        // Kepler, [refine 2, sets 7, Hermite plan, Hermite], end, copy, begin, momentum 2, drift, kick
+        // Kepler, [refine, sets, Hermite plan, Hermite], copy, momentum [1 or 2], drift, kick
         // [+ chunk re-test], finish
-        c->launches += 9 + (enc ? 11 : 0) + search_retest(p, fz);
+        c->launches += 5 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 3 + sets_launches(d.rows) : 0) + search_retest(p, fz);
     } else {
         if ((e = launch_kick_tiles(d, p.kick_prec, 0, p.G, c->tune.threads, c->tune.ipt, st))) return e;
         if ((e = launch_kick_finish_v(d, d.v, d.q, 0.5 * tau, p.G, 0, p.hill_fixed, st))) return e;
-        if ((e = launch_momentum(d, st))) return e;
+        if ((e = launch_momentum(d, st, true))) return e;
         if ((e = launch_drift_pack_from(d, d.q, d.v, 0.5 * tau, 0.0, tau, p.a_E, p.G, 0,
-                                        p.hill_fixed, st, 0.5 * tau)))
+                                        p.hill_fixed, st, 0.5 * tau, 1.01, 1, 1)))
             return e;
-        // Kepler, [refine 2, sets 7, Hermite plan, Hermite], end, copy, kick, finish, momentum 2, drift
-        c->launches += 8 + (enc ? 11 : 0);
+        // Kepler, [refine, sets, Hermite plan, Hermite], copy, kick, finish, momentum [1 or 2], drift
+        c->launches += 5 + momentum_launches(d, true) + (enc ? 3 + sets_launches(d.rows) : 0);
     }
     return cudaGetLastError();
 }
@@ -1095,11 +1087,11 @@ extern "C" qym_status qym_step(qym_ctx *c, double tau, int64_t nsteps) {
             if ((e = launch_sort_rows(d.rows, d.q, c->sortw, d.perm, d.inv, st))) return e;
             c->launches += sort_launches(d.rows);
         }
-        if ((e = launch_momentum(d, st))) return e;
+        if ((e = launch_momentum(d, st, true))) return e;
         if ((e = launch_drift_pack_from(d, d.q, d.v, 0.0, 0.5 * tau, tau, p.a_E, p.G,
                                         fused_search(c) && !fresh, p.hill_fixed, st, 0.5 * tau)))
             return e;
-        c->launches += 3;
+        c->launches += 1 + momentum_launches(d, true);
         return cudaSuccess;
     };
     CK(c, fresh ? opening() : replay(c, c->g_open[sort ? 1 : 0], tau, opening));

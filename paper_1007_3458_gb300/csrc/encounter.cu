@@ -110,29 +110,28 @@ __device__ __forceinline__ void push_encounter(const Dev &d, int i, int j) {
 }
 
 // rigorous test of the crude candidates: (d.q, d.v) hold the state entering
-// the Kepler drift, (d.q1, d.v1) the Kepler result
+// the Kepler drift, (d.q1, d.v1) the Kepler result; and, on the CTAs past
+// kRefineCtas, the exact re-search of rows whose crude bounds were exceeded: the
+// row against every other body of its system (one CTA per row; nearly always none)
+constexpr int kRefineCtas = 2 * 152;
 __global__ void __launch_bounds__(256) k_refine(Dev d, double tau, double a_E) {
     chain_wait();
-    unsigned long long n = d.ctr[C_NCAND];
-    if (n > (unsigned long long)d.max_cand) n = d.max_cand;
     const int64_t R = d.rows;
-    for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (unsigned long long)gridDim.x * blockDim.x) {
-        int2 p = d.cand[k];
-        double thr2;
-        double dm = pair_test(d.q, d.v, d.q1, d.v1, d.rH, R, p.x, p.y, tau, a_E, thr2);
-        if (dm < thr2) push_encounter(d, p.x, p.y);
+    if (blockIdx.x < kRefineCtas) {
+        unsigned long long n = d.ctr[C_NCAND];
+        if (n > (unsigned long long)d.max_cand) n = d.max_cand;
+        for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+             k += (unsigned long long)kRefineCtas * blockDim.x) {
+            int2 p = d.cand[k];
+            double thr2;
+            double dm = pair_test(d.q, d.v, d.q1, d.v1, d.rH, R, p.x, p.y, tau, a_E, thr2);
+            if (dm < thr2) push_encounter(d, p.x, p.y);
+        }
+        return;
     }
-}
-
-// exact re-search of rows whose crude bounds were exceeded: the row against
-// every other body of its system (one CTA per row)
-__global__ void __launch_bounds__(256) k_rescan(Dev d, double tau, double a_E) {
-    chain_wait();
     unsigned long long n = d.ctr[C_NRESCAN];
     if (n > (unsigned long long)d.rows) n = d.rows;
-    const int64_t R = d.rows;
-    for (unsigned long long b = blockIdx.x; b < n; b += gridDim.x) {
+    for (unsigned long long b = blockIdx.x - kRefineCtas; b < n; b += gridDim.x - kRefineCtas) {
         int64_t i = d.rescan[b];
         int sys = d.sys_of[i];
         int64_t lo = d.offsets[sys] + 1, hi = d.offsets[sys + 1];
@@ -147,9 +146,7 @@ __global__ void __launch_bounds__(256) k_rescan(Dev d, double tau, double a_E) {
 }
 
 cudaError_t launch_refine(const Dev &d, double tau, double a_E, cudaStream_t st) {
-    launch_chain(k_refine, 2 * 152, 256, 0, st, d, tau, a_E);
-    launch_chain(k_rescan, 152, 256, 0, st, d, tau, a_E);
-    return cudaGetLastError();
+    return launch_chain(k_refine, kRefineCtas + 152, 256, 0, st, d, tau, a_E);
 }
 
 // ---------------------------------------------------------------- sets
@@ -172,26 +169,29 @@ __device__ __forceinline__ int uf_find(int *uf, int x, int &guard) {
     return x;
 }
 
+// join the sets of a pair
+__device__ __forceinline__ void uf_hook(const Dev &d, int2 p) {
+    int *uf = d.uf;
+    atomicCAS(uf + p.x, -1, p.x);
+    atomicCAS(uf + p.y, -1, p.y);
+    int guard = 0;
+    while (guard < UF_CAP) {
+        int a = uf_find(uf, p.x, guard), b = uf_find(uf, p.y, guard);
+        if (a == b) break;
+        if (a > b) { int t = a; a = b; b = t; }
+        if (atomicCAS(uf + b, b, a) == b) break;
+        ++guard;
+    }
+    if (guard >= UF_CAP) atomicOr(d.status, QYM_ST_UF_CAP);
+}
+
 __global__ void k_uf_hook(Dev d) {
     chain_wait();
     unsigned long long n = d.ctr[C_NENC];
     if (n > (unsigned long long)d.max_enc) n = d.max_enc;
-    int *uf = d.uf;
     for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (unsigned long long)gridDim.x * blockDim.x) {
-        int2 p = d.enc[k];
-        atomicCAS(uf + p.x, -1, p.x);
-        atomicCAS(uf + p.y, -1, p.y);
-        int guard = 0;
-        while (guard < UF_CAP) {
-            int a = uf_find(uf, p.x, guard), b = uf_find(uf, p.y, guard);
-            if (a == b) break;
-            if (a > b) { int t = a; a = b; b = t; }
-            if (atomicCAS(uf + b, b, a) == b) break;
-            ++guard;
-        }
-        if (guard >= UF_CAP) atomicOr(d.status, QYM_ST_UF_CAP);
-    }
+         k += (unsigned long long)gridDim.x * blockDim.x)
+        uf_hook(d, d.enc[k]);
 }
 
 // per-block counts of roots, for an ordered numbering of the sets
@@ -262,17 +262,11 @@ __global__ void __launch_bounds__(1024) k_uf_number(Dev d, const int32_t *blk, i
     }
 }
 
-// each member finds its root (compressing the path), adds itself to its set
-// size, raises the set's r_crit (a_H times the largest Hill radius) and the
-// set's predicted Hermite cost (the block steps of the member's set in the
-// previous step)
-__global__ void __launch_bounds__(256) k_uf_members(Dev d, const int32_t *sid, int32_t *size,
-                                                    unsigned long long *rc_bits, double a_H) {
-    chain_wait();
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= d.rows) return;
-    int p = d.uf[r];
-    if (p < 0) return;
+// each member finds its root, adds itself to its set size, raises the set's
+// r_crit (a_H times the largest Hill radius) and the set's predicted Hermite cost
+// (the block steps of the member's set in the previous step)
+__device__ __forceinline__ void uf_member(const Dev &d, int64_t r, const int32_t *sid, int32_t *size,
+                                          unsigned long long *rc_bits, double a_H) {
     int guard = 0;
     int root = uf_find(d.uf, (int)r, guard);
     int s = sid[root];
@@ -284,17 +278,24 @@ __global__ void __launch_bounds__(256) k_uf_members(Dev d, const int32_t *sid, i
     if (hc > 0) atomicMax(d.hsetcost + s, hc);
 }
 
-// set_start = exclusive scan of set sizes (one CTA); the fill counters reset
-__global__ void __launch_bounds__(1024) k_scan_sets(Dev d, int32_t *size, int32_t *fill,
-                                                    unsigned long long *rc_bits) {
+__global__ void __launch_bounds__(256) k_uf_members(Dev d, const int32_t *sid, int32_t *size,
+                                                    unsigned long long *rc_bits, double a_H) {
     chain_wait();
+    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < d.rows && d.uf[r] >= 0) uf_member(d, r, sid, size, rc_bits, a_H);
+}
+
+// set_start = exclusive scan of set sizes (one CTA); the fill counters reset
+// (sizes and r_crit come from atomics: read past L1, for callers that raised
+// them in the same kernel)
+__device__ __forceinline__ void scan_sets(const Dev &d, int n, const int32_t *size, int32_t *fill,
+                                          unsigned long long *rc_bits) {
     __shared__ int32_t part[1024];
-    int n = (int)d.ctr[C_NSETS];
     if (n > d.max_sets) n = d.max_sets;
     int per = (n + 1023) / 1024;
     int b0 = threadIdx.x * per;
     int s = 0;
-    for (int b = b0; b < b0 + per && b < n; ++b) s += size[b];
+    for (int b = b0; b < b0 + per && b < n; ++b) s += __ldcg(size + b);
     part[threadIdx.x] = s;
     __syncthreads();
     for (int off = 1; off < 1024; off <<= 1) {
@@ -307,10 +308,10 @@ __global__ void __launch_bounds__(1024) k_scan_sets(Dev d, int32_t *size, int32_
     int mx = 0;
     for (int b = b0; b < b0 + per && b < n; ++b) {
         d.set_start[b] = run;
-        run += size[b];
-        mx = max(mx, size[b]);
+        run += __ldcg(size + b);
+        mx = max(mx, __ldcg(size + b));
         fill[b] = 0;
-        d.rcrit[b] = __longlong_as_double((long long)rc_bits[b]);
+        d.rcrit[b] = __longlong_as_double((long long)__ldcg(rc_bits + b));
         rc_bits[b] = 0ull;
     }
     // largest set
@@ -329,13 +330,13 @@ __global__ void __launch_bounds__(1024) k_scan_sets(Dev d, int32_t *size, int32_
     }
 }
 
-__global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int32_t *fill) {
+__global__ void __launch_bounds__(1024) k_scan_sets(Dev d, const int32_t *size, int32_t *fill,
+                                                    unsigned long long *rc_bits) {
     chain_wait();
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= d.rows) return;
-    d.hcost[r] = 0;  // k_uf_members has read the last step's; this step's sets write theirs
-    int p = d.uf[r];
-    if (p < 0) return;
+    scan_sets(d, (int)d.ctr[C_NSETS], size, fill, rc_bits);
+}
+
+__device__ __forceinline__ void uf_place(const Dev &d, int64_t r, const int32_t *sid, int32_t *fill) {
     int guard = 0;
     int root = uf_find(d.uf, (int)r, guard);
     int s = sid[root];
@@ -344,7 +345,89 @@ __global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int
     if (pos < d.max_members) d.set_mem[pos] = (int32_t)r;
 }
 
+__global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int32_t *fill) {
+    chain_wait();
+    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= d.rows) return;
+    d.hcost[r] = 0;  // uf_member has read the last step's; this step's sets write theirs
+    if (d.uf[r] >= 0) uf_place(d, r, sid, fill);
+}
+
+// The whole set builder in one CTA for up to kSetsOneRows rows: the seven kernels
+// below are a few microseconds of latency each (22 us a step, 10 us here for 260
+// rows; at 16384 rows the one CTA's rounds take 3 us longer than the seven), while
+// the pairs of a step are few. A thread takes the rows tid, tid + 1024, ...: whether they are
+// members and roots stays in two bit masks; the roots' counts per (round, warp) are
+// numbered by one scan of 1024 entries.
+constexpr int kSetsRounds = 8;
+constexpr int64_t kSetsOneRows = kSetsRounds * 1024;
+__global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a_H) {
+    chain_wait();
+    __shared__ int s_cnt[32][32], s_warp[32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int rows = (int)d.rows, rounds = (rows + 1023) >> 10;
+    const unsigned long long n = min(d.ctr[C_NENC], (unsigned long long)d.max_enc);
+    for (unsigned long long k = tid; k < n; k += 1024) uf_hook(d, d.enc[k]);
+    __syncthreads();
+    unsigned member = 0, root = 0;
+#pragma unroll
+    for (int it = 0; it < kSetsRounds; ++it) {
+        const int r = it * 1024 + tid;
+        if (r >= rows) break;
+        const int p = n ? __ldcg(d.uf + r) : -1;
+        if (p >= 0) member |= 1u << it;
+        if (p == r) root |= 1u << it;
+    }
+    if (w >= kSetsRounds) s_cnt[w][lane] = 0;
+    for (int it = 0; it < kSetsRounds; ++it) {
+        const unsigned b = __ballot_sync(0xffffffffu, (root >> it) & 1u);
+        if (lane == 0) s_cnt[it][w] = __popc(b);
+    }
+    __syncthreads();
+    // exclusive scan of the 1024 counts in row order
+    const int c = s_cnt[w][lane];
+    int inc = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_warp[w] = inc;
+    __syncthreads();
+    const int ws = s_warp[lane];
+    const int nsets = __reduce_add_sync(0xffffffffu, ws);
+    s_cnt[w][lane] = __reduce_add_sync(0xffffffffu, lane < w ? ws : 0) + inc - c;
+    __syncthreads();
+    for (int it = 0; it < rounds; ++it) {
+        const bool mine = (root >> it) & 1u;
+        const unsigned b = __ballot_sync(0xffffffffu, mine);
+        if (mine) {
+            const int k = s_cnt[it][w] + __popc(b & ((1u << lane) - 1u));
+            s.sid[it * 1024 + tid] = k;
+            s.size[k] = 0;
+            if (k < d.max_sets) d.set_root[k] = it * 1024 + tid;
+        }
+    }
+    if (tid == 0) d.ctr[C_NSETS] = (unsigned long long)nsets;
+    __threadfence();  // the cleared sizes before the members' atomics on them
+    __syncthreads();
+    for (unsigned m = member; m; m &= m - 1)
+        uf_member(d, (int64_t)(__ffs(m) - 1) * 1024 + tid, s.sid, s.size, s.rc_bits, a_H);
+    __syncthreads();
+    scan_sets(d, nsets, s.size, s.fill, s.rc_bits);
+    __threadfence();
+    __syncthreads();
+    for (int it = 0; it < rounds; ++it) {
+        const int r = it * 1024 + tid;
+        if (r < rows) d.hcost[r] = 0;
+    }
+    for (unsigned m = member; m; m &= m - 1)
+        uf_place(d, (int64_t)(__ffs(m) - 1) * 1024 + tid, s.sid, s.fill);
+}
+
+int sets_launches(int64_t rows) { return rows <= kSetsOneRows ? 1 : 7; }
+
 cudaError_t launch_sets_impl(const Dev &d, double a_H, const SetScratch &s, cudaStream_t st) {
+    if (d.rows <= kSetsOneRows) return launch_chain(k_sets_one, 1, 1024, 0, st, d, s, a_H);
     int nblk = (int)((d.rows + 1023) / 1024);
     launch_chain(k_uf_hook, 152, 256, 0, st, d);
     launch_chain(k_uf_count, nblk, 1024, 0, st, d, s.blk);

@@ -142,6 +142,24 @@ enum Ctr : int {
     C_COUNT
 };
 
+// a step's counters join the call's; the next step's start from zero
+__device__ __forceinline__ void step_counters_end(unsigned long long *ctr) {
+    ctr[C_SUM_CAND] += ctr[C_NCAND];
+    ctr[C_SUM_ENC] += ctr[C_NENC];
+    ctr[C_SUM_RESCAN] += ctr[C_NRESCAN];
+    ctr[C_STEP] += 1;
+}
+__device__ __forceinline__ void step_counters_begin(unsigned long long *ctr) {
+    ctr[C_NCAND] = 0;
+    ctr[C_NACTIVE] = 0;
+    ctr[C_NENC] = 0;
+    ctr[C_NRESCAN] = 0;
+    ctr[C_NSETS] = 0;
+    ctr[C_HSMALL] = 0;
+    ctr[C_NFCHUNK] = 0;
+    ctr[C_FCDONE] = 0;
+}
+
 // ---------------------------------------------------------------- helpers
 // one MUFU instruction; inputs here are squared separations, never denormal
 __device__ __forceinline__ float rsqrt_ftz(float x) {
@@ -349,13 +367,19 @@ cudaError_t launch_mlp_train(float *w, float *m, float *v, int64_t t0, const flo
                              void *work, cudaStream_t st);
 
 // step kernels (step.cu)
-cudaError_t launch_momentum(const Dev &d, cudaStream_t st);
+// sum m v per system into d.S; for_drift: only for the drift that follows, which
+// adds a small system's chunks itself (one launch less)
+cudaError_t launch_momentum(const Dev &d, cudaStream_t st, bool for_drift = false);
+int momentum_launches(const Dev &d, bool for_drift);
 // kick_span: the time of the kick(s) between this pack and the Kepler drift
-// (tau/2, or tau when two half kicks are merged); it sizes the crude reach
+// (tau/2, or tau when two half kicks are merged); it sizes the crude reach.
+// ctr_end, ctr_begin: also count the step that ends with this drift, and clear
+// the counters of the step that begins after it
 cudaError_t launch_drift_pack_from(const Dev &d, const double *qs, const double *vs,
                                    double h_close, double h_open, double tau, double a_E,
                                    double G, int flag_next, int hill_fixed, cudaStream_t st,
-                                   double kick_span, double a_allow = 1.01);
+                                   double kick_span, double a_allow = 1.01, int ctr_end = 0,
+                                   int ctr_begin = 0);
 // a_allow: the bound on |a| / |a of the last kick| that the crude reach of the
 // preceding pack assumed (checked when check != 0)
 // skip_whole: leave v of the systems flagged in d.wh_flag (their step was
@@ -439,6 +463,7 @@ struct SetScratch {
 };
 cudaError_t launch_refine(const Dev &d, double tau, double a_E, cudaStream_t st);
 cudaError_t launch_sets_impl(const Dev &d, double a_H, const SetScratch &s, cudaStream_t st);
+int sets_launches(int64_t rows);  // kernels launch_sets_impl enqueues
 cudaError_t launch_pair_test(int64_t rows, const double *q0, const double *v0, const double *q1,
                              const double *v1, const double *rH, double tau, double a_E,
                              int64_t npairs, const int32_t *pairs, double *d2, int32_t *flag,

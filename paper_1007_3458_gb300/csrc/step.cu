@@ -55,8 +55,14 @@ __global__ void k_mom_final(Dev d) {
     if (lane < 3) d.S[3 * s + lane] = lane == 0 ? t[0] : (lane == 1 ? t[1] : t[2]);
 }
 
-cudaError_t launch_momentum(const Dev &d, cudaStream_t st) {
+// one system of few chunks: the drift adds them itself
+static bool drift_sums(const Dev &d) { return d.nsys == 1 && d.nmchunks <= 64; }
+
+int momentum_launches(const Dev &d, bool for_drift) { return for_drift && drift_sums(d) ? 1 : 2; }
+
+cudaError_t launch_momentum(const Dev &d, cudaStream_t st, bool for_drift) {
     launch_chain(k_mom_chunks, d.nmchunks, 256, 0, st, d);
+    if (for_drift && drift_sums(d)) return cudaGetLastError();
     launch_chain(k_mom_final, (unsigned)((32 * (int64_t)d.nsys + 127) / 128), 128, 0, st, d);
     return cudaGetLastError();
 }
@@ -85,6 +91,8 @@ struct DriftArgs {
     double kick_span;  // time of the kick(s) between this pack and the Kepler drift
     double a_allow;    // bound on |a| of that kick as a multiple of the last |a|
     int flag_next, hill_fixed;
+    int ctr_end, ctr_begin;  // count the step that ends here, clear the next step's counters
+    int sum_chunks;          // S of the one system from its momentum chunks, here
     float tau_f, span_f, a_E_f, a_allow_f;  // |tau|, |kick_span|, a_E, a_allow in FP32
 };
 
@@ -162,10 +170,26 @@ __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
     const int64_t rb = (int64_t)blockIdx.x * blockDim.x;
     const int s_lo = d.sys_of[rb], s_hi = d.sys_of[min(rb + (int64_t)blockDim.x, R) - 1];
     const bool cached = s_hi - s_lo < kDriftSys;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (a.ctr_end) step_counters_end(d.ctr);
+        if (a.ctr_begin) step_counters_begin(d.ctr);
+    }
+    __shared__ double sh_S[3];
+    if (a.sum_chunks) {
+        // k_mom_final's sum, in its order, by every CTA for itself
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (w < 3) {
+            double t = 0.0;
+            for (int c = lane; c < d.nmchunks; c += 32) t += d.mpart[3 * c + w];
+            t = warp_sum(t);
+            if (lane == 0) sh_S[w] = t;
+        }
+        __syncthreads();
+    }
     if (cached && threadIdx.x < 6 * (s_hi - s_lo + 1)) {
         const int ss = s_lo + threadIdx.x / 6, k = threadIdx.x % 6;
         const double h = k < 3 ? a.h_close : a.h_open;
-        sh_shift[threadIdx.x / 6][k] = h * d.S[3 * ss + k % 3] / d.m[d.offsets[ss]];
+        sh_shift[threadIdx.x / 6][k] = h * (a.sum_chunks ? sh_S[k % 3] : d.S[3 * ss + k % 3]) / d.m[d.offsets[ss]];
     }
     __syncthreads();
     int64_t r = rb + threadIdx.x;
@@ -226,8 +250,11 @@ __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
 cudaError_t launch_drift_pack_from(const Dev &d, const double *qs, const double *vs,
                                    double h_close, double h_open, double tau, double a_E,
                                    double G, int flag_next, int hill_fixed, cudaStream_t st,
-                                   double kick_span, double a_allow) {
+                                   double kick_span, double a_allow, int ctr_end, int ctr_begin) {
     DriftArgs a;
+    a.ctr_end = ctr_end;
+    a.ctr_begin = ctr_begin;
+    a.sum_chunks = (h_close != 0.0 || h_open != 0.0) && drift_sums(d);
     a.qs = qs;
     a.vs = vs;
     a.h_close = h_close;

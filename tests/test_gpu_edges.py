@@ -241,3 +241,57 @@ def test_kepler_sizes_and_brackets(torch, n, e):
                 if n > k:  # copies of the same bodies, in other lanes and CTAs
                     assert np.abs(g - np.resize(g[:k], g.shape)).max() <= 1e-12 * np.abs(g).max() * scale.max()
     assert st.item() == 0
+
+
+@pytest.mark.parametrize("n", [40, 1000, 1100, 8191, 8192, 9000])
+def test_sets_sizes(torch, n):
+    """The set builder in one CTA (up to 8192 rows) and in its seven kernels,
+    on a disk crowded around a planet (large sets, many pairs): after a step the
+    records' connected components are the sets counted, the largest of them the
+    largest set, and a rerun on a fresh context gives the same bits."""
+    import networkx as nx
+    w = W.outer_disk(n - 4, 1e-9, seed=n, a_lo=9.0, a_hi=10.0 if n < 2000 else 40.0)
+    out = []
+    for _ in range(2):
+        sim = q.Simulation(w.m, w.q, w.v, w.offsets, eps_H=w.eps_H)
+        sim.step(0.2 * w.tau, 1)
+        out.append((*sim.state(), sim.encounters(), sim.stats()))
+        sim.close()
+    (q0, v0, rec, st), (q1, v1, rec1, _) = out
+    g = nx.Graph(list(map(tuple, rec[:, 1:])))
+    comps = [len(c) for c in nx.connected_components(g)]
+    assert len(rec) > 0 and st["sets"] == len(comps) and st["max_set"] == max(comps)
+    assert np.array_equal(rec, rec1) and np.array_equal(q0, q1) and np.array_equal(v0, v1)
+
+
+@pytest.mark.parametrize("n", [8192, 8705, 16385, 33000])
+@pytest.mark.parametrize("equal", [True, False])
+def test_pairs_once(torch, n, equal):
+    """One kick with each pair formed once against the one-sided form (a launch
+    shape set by hand) and the FP64 kick, bodies of one mass and of several, a
+    ragged last block: the velocity change of a kick within 2^-18 of the sum of
+    the pulls' magnitudes of the FP64 one (as test_mixed_accel_sizes; here by
+    the largest pull of any body), and the two FP32 forms' errors alike."""
+    w = W.outer_disk(n - 4, 1e-10, seed=n)
+    m = w.m.copy()
+    if not equal:
+        m[5:] *= 10.0 ** np.random.default_rng(n).uniform(-1, 1, n - 4)
+    tau = 1e-3
+    dv = []
+    for prec, shape in ((q.QYM_KICK_FP64, None), (q.QYM_KICK_MIXED, None), (q.QYM_KICK_MIXED, (128, 2, 16))):
+        # no heavy split: every pull goes through the FP32 pairs
+        sim = q.Simulation(m, w.q, np.zeros_like(w.v), w.offsets, kick_prec=prec, encounters=0, heavy_mass=0.0,
+                           coords=1, G=1e-6)
+        if prec == q.QYM_KICK_MIXED:
+            assert sim.stats()["kick_tile_i"] == 512
+        if shape:
+            q.qym_set_kick_shape(sim.ctx, *shape)
+            assert sim.stats()["kick_tile_i"] == 256
+        sim.step(tau, 1)
+        dv.append(sim.state()[1])
+        sim.close()
+    a = [np.linalg.norm(x - dv[0], axis=1) for x in dv[1:]]
+    big = np.linalg.norm(dv[0], axis=1).max()
+    assert big > 0 and max(x.max() for x in a) <= 2.0 ** -18 * big
+    rms = [np.sqrt((x ** 2).mean()) for x in a]
+    assert rms[0] <= 1.5 * rms[1] + 1e-16 * big, (rms, big)
