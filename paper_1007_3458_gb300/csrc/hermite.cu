@@ -339,21 +339,39 @@ __device__ __forceinline__ float to_float_scaled(double v, int s) {
 // FP64 evaluation needs dt_c within ~1e-7 of a level boundary.
 // level_from: that level from the criterion's inputs as floats f[c * ACH]
 // (stride ACH): a (3), j g (3), a2 g^2 (3), a3 g^3 (3)
+// (square roots and the division by the approximate instructions, within 2^-22:
+// the criterion is latency between the corrector and the next block step)
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ int level_from(const float *f, int lv, float eta, float T2) {
     float q[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         const float x = f[(3 * g) * ACH], y = f[(3 * g + 1) * ACH], z = f[(3 * g + 2) * ACH];
-        q[g] = sqrtf(fmaf(x, x, fmaf(y, y, z * z)));
+        q[g] = sqrt_approx(fmaf(x, x, fmaf(y, y, z * z)));
     }
     const float num = eta * fmaf(q[0], q[2], q[1] * q[1]);
     const float den = fmaf(q[1], q[3], q[2] * q[2]);
     if (!(den > 0.0f)) return 0;
     if (!(num > 0.0f)) return KMAX;
-    const float r = num / den;
+    const float r = __fdividef(num, den);
     if (!(r < INFINITY)) return 0;
+    // r = fr 2^er, T2 = ft 2^et with fr, ft in [1/2, 1)
     int er, et;
-    const float fr = frexpf(r, &er), ft = frexpf(T2, &et);
+    float fr, ft;
+    const int br = __float_as_int(r), bt = __float_as_int(T2);
+    if (br >= 0x00800000 && bt >= 0x00800000) {
+        er = br >> 23;
+        et = bt >> 23;
+        fr = __int_as_float((br & 0x7fffff) | 0x3f000000);
+        ft = __int_as_float((bt & 0x7fffff) | 0x3f000000);
+    } else {
+        fr = frexpf(r, &er);
+        ft = frexpf(T2, &et);
+    }
     const int dd = er - et;
     const int m = (dd & 1) ? (dd - 1) >> 1 : ((ft <= fr) ? dd >> 1 : (dd >> 1) - 1);
     const int k = lv - m;
@@ -506,9 +524,9 @@ __shared__ int g_na;
 // after the barrier that follows. The end times stay in registers
 // between the two passes; the minimum (below 2^49) is taken as the minimum of
 // the high words, then of the low words among the lanes that hold it.
-__device__ __forceinline__ void next_block(const int32_t *lev, const long long *ti, int32_t *act,
-                                           int n) {
-    constexpr int NI = HCAP / 32;
+template <int NI>
+__device__ __forceinline__ void next_block_of(const int32_t *lev, const long long *ti, int32_t *act,
+                                              int n) {
     const int wl = threadIdx.x & 31;
     long long te[NI];
     long long t = LLONG_MAX;
@@ -535,6 +553,15 @@ __device__ __forceinline__ void next_block(const int32_t *lev, const long long *
         g_tn = t;
         g_na = na;
     }
+}
+
+// (most sets have at most 64 members: two rounds instead of ten)
+__device__ __forceinline__ void next_block(const int32_t *lev, const long long *ti, int32_t *act,
+                                           int n) {
+    if (n <= 64)
+        next_block_of<2>(lev, ti, act, n);
+    else
+        next_block_of<HCAP / 32>(lev, ti, act, n);
 }
 
 // Copy the member range [lo, hi) of arrays a..: from CTA `r` of the cluster
@@ -955,7 +982,11 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 }
                 __syncthreads();
             }
-            // corrector, one warp per coordinate (the same in every CTA)
+            // corrector, one warp per coordinate (the same in every CTA), in two
+            // parts: the derivatives first, which warp 3 waits for to set the new
+            // levels and find the next block time, then positions and
+            // velocities beside it (levels and next block took 1700 of a
+            // block step's 12000 cycles after the whole corrector)
             if (warp < 3) {
                 const int c = warp;
                 double *xa = c == 0 ? S.x : (c == 1 ? S.y : S.z);
@@ -964,37 +995,57 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 double *ja = c == 0 ? S.jx : (c == 1 ? S.jy : S.jz);
                 const double *ea = c == 0 ? S.ex : (c == 1 ? S.ey : S.ez);
                 const double *fa = c == 0 ? S.eu : (c == 1 ? S.ev : S.ew);
-                for (int sl = wl; sl < nc; sl += 32) {
+                constexpr int LS = KMAX + 1, NS = ACH / 32;
+                int kk[NS], lvs[NS];
+                double A2[NS], A3[NS], A1[NS], J1[NS];
+#pragma unroll
+                for (int q = 0; q < NS; ++q) {
+                    const int sl = wl + 32 * q;
+                    kk[q] = -1;
+                    if (sl >= nc) continue;
                     const int k = S.act[a0 + sl];
                     const int lv = S.lev[k];
                     const double *L = S.lvt + lv;
-                    constexpr int LS = KMAX + 1;
                     const double a1c = S.a1s[c * ACH + sl], j1c = S.a1s[(3 + c) * ACH + sl];
                     const double d = aa[k] - a1c, j0c = ja[k];
                     const double a2 =
                         fma(L[LV_A2D * LS], d, fma(L[LV_A2J0 * LS], j0c, L[LV_A2J1 * LS] * j1c));
                     const double a3 = fma(L[LV_A3D * LS], d, L[LV_A3J * LS] * (j0c + j1c));
-                    const double xn = fma(L[LV_H4 * LS], a2, fma(L[LV_H5 * LS], a3, ea[k]));
-                    const double un = fma(L[LV_H3 * LS], a2, fma(L[LV_H4 * LS], a3, fa[k]));
-                    xa[k] = xn;
-                    ua[k] = un;
-                    aa[k] = a1c;
-                    ja[k] = j1c;
-                    S.f[c * HCAP + k] = to_float_scaled(xn, 0);
-                    S.f[(3 + c) * HCAP + k] = to_float_scaled(un, 0);
-                    S.f[(6 + c) * HCAP + k] = to_float_scaled(a1c, 0);
-                    S.f[(9 + c) * HCAP + k] = to_float_scaled(j1c, 0);
                     const double a2e = fma(L[LV_H * LS], a3, a2);  // a2 at the end of the step
                     S.cf[c * ACH + sl] = to_float_scaled(a1c, 0);
                     S.cf[(3 + c) * ACH + sl] = to_float_scaled(j1c, -lv);
                     S.cf[(6 + c) * ACH + sl] = to_float_scaled(a2e, -2 * lv);
                     S.cf[(9 + c) * ACH + sl] = to_float_scaled(a3, -3 * lv);
+                    kk[q] = k;
+                    lvs[q] = lv;
+                    A2[q] = a2;
+                    A3[q] = a3;
+                    A1[q] = a1c;
+                    J1[q] = j1c;
                 }
-            }
-            __syncthreads();
-            // new time and level by the Aarseth criterion (FP32 on scaled
-            // inputs); a larger step only by one level and on a commensurate time
-            if (warp == 3) {
+                __syncwarp();
+                asm volatile("bar.arrive 5, 128;" ::: "memory");
+                // (the members' levels and the active list are warp 3's from here)
+#pragma unroll
+                for (int q = 0; q < NS; ++q) {
+                    const int k = kk[q];
+                    if (k < 0) continue;
+                    const double *L = S.lvt + lvs[q];
+                    const double xn = fma(L[LV_H4 * LS], A2[q], fma(L[LV_H5 * LS], A3[q], ea[k]));
+                    const double un = fma(L[LV_H3 * LS], A2[q], fma(L[LV_H4 * LS], A3[q], fa[k]));
+                    xa[k] = xn;
+                    ua[k] = un;
+                    aa[k] = A1[q];
+                    ja[k] = J1[q];
+                    S.f[c * HCAP + k] = to_float_scaled(xn, 0);
+                    S.f[(3 + c) * HCAP + k] = to_float_scaled(un, 0);
+                    S.f[(6 + c) * HCAP + k] = to_float_scaled(A1[q], 0);
+                    S.f[(9 + c) * HCAP + k] = to_float_scaled(J1[q], 0);
+                }
+            } else if (warp == 3) {
+                // new time and level by the Aarseth criterion (FP32 on scaled
+                // inputs); a larger step only by one level and on a commensurate time
+                asm volatile("bar.sync 5, 128;" ::: "memory");
                 for (int sl = wl; sl < nc; sl += 32) {
                     const int k = S.act[a0 + sl];
                     const int lv = S.lev[k];
@@ -1006,7 +1057,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     S.lev[k] = kn;
                     S.ti[k] = tn;
                 }
+                __syncwarp();
             }
+            if (a0 + ACH < na) __syncthreads();  // the next round's sums and derivatives
         }
         // every thread read (tn, na) before the barriers above; the active
         // list is no longer read in this block step
