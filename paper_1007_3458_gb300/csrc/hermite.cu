@@ -36,42 +36,62 @@ namespace cg = cooperative_groups;
 constexpr int HCAP = 320;       // members per set held in shared memory
 constexpr int HTHREADS = 256;
 
+// Comparisons by the bits of a double: an FP64 comparison holds the warp like an
+// addition. y <= 0, y >= 1 and y > 1/2 of the transition's argument (finite), and
+// a >= b for a, b >= 0 (false where a is NaN)
+__device__ __forceinline__ bool y_at_most_0(double y) {
+    return __double_as_longlong(y) <= 0;
+}
+__device__ __forceinline__ bool y_at_least_1(double y) {
+    return (unsigned)(__double2hiint(y) - 0x3ff00000) <= 0x40000000u;  // (not NaN)
+}
+__device__ __forceinline__ bool y_above_half(double y) {
+    return __double_as_longlong(y) > 0x3fe0000000000000ll;
+}
+__device__ __forceinline__ bool at_least(double a, double b) {
+    const long long ua = __double_as_longlong(a);
+    return ua >= __double_as_longlong(b) && ua <= 0x7ff0000000000000ll;
+}
+
 // sin and cos of (pi/2) y for y in [0, 1]: y > 1/2 is folded onto 1 - y
 // (sin and cos swap), so the argument w = (pi/2) y' stays in [0, pi/4], where
 // the Taylor series of sin to w^15 and of cos to w^16 leave truncation errors
 // below 7e-17 and 3e-18 (the next terms, w^17/17! and w^18/18!, at pi/4).
 struct HalfPi {
-    double w, x, x2, x4;  // w = (pi/2) y', y' = y or 1 - y; x = w^2, x^2, x^4
-    bool fold;            // y' = 1 - y: sin and cos swap
+    double w, x;  // w = (pi/2) y', y' = y or 1 - y; x = w^2
+    bool fold;    // y' = 1 - y: sin and cos swap
 };
 __device__ __forceinline__ HalfPi half_pi_arg(double y) {
     HalfPi a;
-    a.fold = y > 0.5;
+    a.fold = y_above_half(y);
     a.w = 1.5707963267948966 * (a.fold ? 1.0 - y : y);
     a.x = a.w * a.w;
-    a.x2 = a.x * a.x;
-    a.x4 = a.x2 * a.x2;
     return a;
 }
-// both polynomials in x = w^2 by Estrin's scheme (dependent depth 4-5
-// instead of 8-9: FP64 operations have long latency on this GPU)
+// both polynomials in x = w^2 by Horner's scheme: a warp issues an FP64
+// instruction every 64 cycles, dependent or not, so the fewest instructions are
+// the fastest (Estrin's scheme takes two and three more)
 // sin w = w (1 - x/3! + x^2/5! - ... - x^7/15!)
 __device__ __forceinline__ double sin_w(const HalfPi &a) {
-    const double s01 = fma(-1.0 / 6.0, a.x, 1.0);
-    const double s23 = fma(-1.0 / 5040.0, a.x, 1.0 / 120.0);
-    const double s45 = fma(-1.0 / 39916800.0, a.x, 1.0 / 362880.0);
-    const double s67 = fma(-1.0 / 1307674368000.0, a.x, 1.0 / 6227020800.0);
-    const double ps = fma(fma(s67, a.x2, s45), a.x4, fma(s23, a.x2, s01));
-    return a.w * ps;
+    double p = fma(-1.0 / 1307674368000.0, a.x, 1.0 / 6227020800.0);
+    p = fma(p, a.x, -1.0 / 39916800.0);
+    p = fma(p, a.x, 1.0 / 362880.0);
+    p = fma(p, a.x, -1.0 / 5040.0);
+    p = fma(p, a.x, 1.0 / 120.0);
+    p = fma(p, a.x, -1.0 / 6.0);
+    p = fma(p, a.x, 1.0);
+    return a.w * p;
 }
 // cos w = 1 - x/2! + x^2/4! - ... + x^8/16!
 __device__ __forceinline__ double cos_w(const HalfPi &a) {
-    const double c01 = fma(-0.5, a.x, 1.0);
-    const double c23 = fma(-1.0 / 720.0, a.x, 1.0 / 24.0);
-    const double c45 = fma(-1.0 / 3628800.0, a.x, 1.0 / 40320.0);
-    const double c67 = fma(-1.0 / 87178291200.0, a.x, 1.0 / 479001600.0);
-    const double c8 = (1.0 / 20922789888000.0) * (a.x4 * a.x4);
-    return fma(fma(c67, a.x2, c45), a.x4, fma(c23, a.x2, c01)) + c8;
+    double p = fma(1.0 / 20922789888000.0, a.x, -1.0 / 87178291200.0);
+    p = fma(p, a.x, 1.0 / 479001600.0);
+    p = fma(p, a.x, -1.0 / 3628800.0);
+    p = fma(p, a.x, 1.0 / 40320.0);
+    p = fma(p, a.x, -1.0 / 720.0);
+    p = fma(p, a.x, 1.0 / 24.0);
+    p = fma(p, a.x, -0.5);
+    return fma(p, a.x, 1.0);
 }
 __device__ __forceinline__ void sincos_half_pi(double y, double &sn, double &cs) {
     const HalfPi a = half_pi_arg(y);
@@ -98,9 +118,9 @@ __device__ __forceinline__ double trans_y(double s, const TransC &tc) { return f
 __device__ __forceinline__ void transition(double s, const TransC &tc, double &K, double &Kp,
                                            double &Kpp) {
     const double y = trans_y(s, tc);
-    if (y <= 0.0) {
+    if (y_at_most_0(y)) {
         K = 0.0; Kp = 0.0; Kpp = 0.0;
-    } else if (y >= 1.0) {
+    } else if (y_at_least_1(y)) {
         K = 1.0; Kp = 0.0; Kpp = 0.0;
     } else {
         double sn, cs;
@@ -254,7 +274,7 @@ __device__ void kcorr_part(const HermSmem &S, int lo, int hi, int k, int l0, int
         if (l == k) continue;
         double qx = S.ex[k] - S.ex[l], qy = S.ey[k] - S.ey[l], qz = S.ez[k] - S.ez[l];
         double q2 = qx * qx + qy * qy + qz * qz;
-        if (q2 >= tc.rc2) continue;  // K = 1 beyond r_crit: no (1-K) part
+        if (at_least(q2, tc.rc2)) continue;  // K = 1 beyond r_crit: no (1-K) part
         const double qi = rsqrt(q2);
         const double q = q2 * qi;
         double K, Kp, Kpp;
@@ -289,7 +309,7 @@ __device__ void herm_part(const HermSmem &S, int lo, int hi, int k, int l0, int 
         if (l == k) continue;
         double qx = xk - S.ex[l], qy = yk - S.ey[l], qz = zk - S.ez[l];
         double q2 = qx * qx + qy * qy + qz * qz + eps2;
-        if (q2 >= tc.rc2) continue;  // K = 1, K' = K'' = 0: no force, no jerk
+        if (at_least(q2, tc.rc2)) continue;  // K = 1, K' = K'' = 0: no force, no jerk
         double px = uk - S.eu[l], py = vk - S.ev[l], pz = wk - S.ew[l];
         const double qi = rsqrt(q2);
         const double qi2 = qi * qi;
@@ -488,7 +508,7 @@ __device__ __forceinline__ void herm_item(const HermSmem &S, int k, int item, in
     const int l = mlo + item;
     const double qx = xk - S.ex[l], qy = yk - S.ey[l], qz = zk - S.ez[l];
     const double q2 = pair_q2(qx, qy, qz, eps2);
-    if (q2 >= tc.rc2) return;  // K = 1, K' = K'' = 0: no force, no jerk
+    if (at_least(q2, tc.rc2)) return;  // K = 1, K' = K'' = 0: no force, no jerk
     const double px = uk - S.eu[l], py = vk - S.ev[l], pz = wk - S.ew[l];
     const double qi = rsqrt(q2);
     const double qi2 = qi * qi;
@@ -863,13 +883,13 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                             qy = S.ey[k] - S.ey[l];
                             qz = S.ez[k] - S.ez[l];
                             const double q2 = pair_q2(qx, qy, qz, h.eps2);
-                            valid = q2 < tc.rc2;  // beyond r_crit: no force, no jerk
+                            valid = !at_least(q2, tc.rc2);  // beyond r_crit: no force, no jerk
                             if (valid) {
                                 const double qi = rsqrt(q2);
                                 qi2 = qi * qi;
                                 sq = q2 * qi;
                                 y = trans_y(sq, tc);
-                                if (y > 0.0 && y < 1.0) {
+                                if (!y_at_most_0(y) && !y_at_least_1(y)) {
                                     const HalfPi arg = half_pi_arg(y);
                                     fold = arg.fold;
                                     mine = role == 0 ? sin_w(arg) : cos_w(arg);
@@ -891,9 +911,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                         pair_bar(warp >> 1);
                         if (valid) {
                             double K = 0.0, Kp = 0.0, Kpp = 0.0;
-                            if (y >= 1.0) {
+                            if (y_at_least_1(y)) {
                                 K = 1.0;
-                            } else if (y > 0.0) {
+                            } else if (!y_at_most_0(y)) {
                                 const double sw = role == 0 ? mine : xs[vl];
                                 const double pc = role == 1 ? mine : xs[2 * 96 + vl];
                                 const double sn = fold ? pc : sw, cs = fold ? sw : pc;
@@ -952,18 +972,14 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                         if (live && g < CLT) cl.map_shared_rank(rbb, g)[(rank * 6 + c) * RSL + sl] = v;
                     }
                     cl.sync();
-                    for (int pi = tid; pi < 6 * cnt; pi += HTHREADS) {
+                    // pairwise tree over CLT lanes: rank r with rank r + w, halving w
+                    for (int t0 = warp * 32; t0 < 6 * cnt * CLT; t0 += HTHREADS) {
+                        const int t = t0 + wl, pi = t / CLT, r = t % CLT;
                         const int sl = pi / 6, c = pi - 6 * sl;
-                        double pv[CLT];
+                        double v = pi < 6 * cnt ? rbb[(r * 6 + c) * RSL + sl] : 0.0;
 #pragma unroll
-                        for (int r = 0; r < CLT; ++r) pv[r] = rbb[(r * 6 + c) * RSL + sl];
-                        // pairwise tree: rank r with rank r + w, halving w
-#pragma unroll
-                        for (int w = CLT / 2; w >= 1; w >>= 1) {
-#pragma unroll
-                            for (int r = 0; r < w; ++r) pv[r] += pv[r + w];
-                        }
-                        S.a1s[c * ACH + s0 + sl] = pv[0];
+                        for (int w = CLT / 2; w >= 1; w >>= 1) v += __shfl_xor_sync(0xffffffffu, v, w);
+                        if (pi < 6 * cnt && r == 0) S.a1s[c * ACH + s0 + sl] = v;
                     }
                     buf ^= 1;
                 } else {
