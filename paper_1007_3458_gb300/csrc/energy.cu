@@ -4,9 +4,9 @@
 // each pair once (the paper's kernel takes both orders and halves the sum),
 // with the star mass restored for the star terms.
 //
-// The pair sum is bound by issue: a pair's separation, r^2 and G m / r run to
-// FP64 accuracy on the FP32 pipes (pair64.cuh, some 270 instructions), FP64 adds
-// the result (one instruction). A CTA takes 128 rows against a range of later
+// The pair sum is bound by issue: a pair's separation, r^2 and 1 / r run to
+// FP64 accuracy on the FP32 pipes (pair64.cuh), FP64 multiplies by G m and adds
+// (one instruction). A CTA takes 128 rows against a range of later
 // rows; the range's length (energy_plan) gives the GPU about 16 CTAs per SM
 // whatever the sizes, where one CTA per 256 rows against all rows left 16384
 // bodies on 64 of the 152 SMs with 15 FP64 instructions per ordered pair
@@ -20,11 +20,10 @@ namespace qym {
 
 constexpr int ET = 128;  // rows of an i-block = threads of a CTA = rows of a j tile
 
-// G m / r of a pair in FP64, where the float form does not hold
-__device__ __noinline__ double potential_fp64(double dx, double dy, double dz, double gm) {
-    if ((__double_as_longlong(gm) << 1) == 0) return 0.0;  // a massless partner
+// 1 / r of a pair in FP64, where the float form does not hold (0 for r = 0)
+__device__ __noinline__ double inv_r_fp64(double dx, double dy, double dz) {
     const double r2 = dx * dx + dy * dy + dz * dz;
-    return (r2 > 0.0) ? gm * rsqrt(r2) : 0.0;
+    return (r2 > 0.0) ? rsqrt(r2) : 0.0;
 }
 
 // CTA (I, c): rows of i-block I against the rows j > i of its c-th range;
@@ -35,8 +34,9 @@ __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, c
                                                      double *pe, double *ps) {
     chain_wait();
     __shared__ D4 s_q[ET];
-    __shared__ float4 s_h[ET], s_m[ET], s_l[ET];
-    __shared__ int s_hi[2][ET / 32];
+    __shared__ float4 s_a[ET], s_b[ET];  // (x, y, z) in three parts: x.h y.h z.h x.m, y.m z.m x.l y.l
+    __shared__ float s_c[ET];            // z.l
+    __shared__ int s_hi[ET / 32];
     __shared__ double red[4][ET / 32];
     const int64_t I = blockIdx.x / pl.nranges;
     const int c = (int)(blockIdx.x - I * pl.nranges);
@@ -52,20 +52,11 @@ __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, c
     const int i = bk.x + threadIdx.x;
     const int r = min(i, bk.y - 1);  // an idle lane repeats the last row
     const double xi = q[r], yi = q[R + r], zi = q[2 * R + r];
-    int hl = max(p64::hi_abs(xi), max(p64::hi_abs(yi), p64::hi_abs(zi)));
-    int hw = j0 + (int)threadIdx.x < j1 ? p64::hi_abs(G * m[j0 + threadIdx.x]) : 0;
-    hl = __reduce_max_sync(0xffffffffu, hl);
-    hw = __reduce_max_sync(0xffffffffu, hw);
-    if ((threadIdx.x & 31) == 0) {
-        s_hi[0][threadIdx.x >> 5] = hl;
-        s_hi[1][threadIdx.x >> 5] = hw;
-    }
+    int hl = __reduce_max_sync(0xffffffffu, max(p64::hi_abs(xi), max(p64::hi_abs(yi), p64::hi_abs(zi))));
+    if ((threadIdx.x & 31) == 0) s_hi[threadIdx.x >> 5] = hl;
     __syncthreads();
-    for (int w = 0; w < ET / 32; ++w) {
-        hl = max(hl, s_hi[0][w]);
-        hw = max(hw, s_hi[1][w]);
-    }
-    const p64::Scale sc(hl, hw);
+    for (int w = 0; w < ET / 32; ++w) hl = max(hl, s_hi[w]);
+    const p64::Scale sc(hl, 0x3ff00000);
     const uint64_t bias = sc.bias(1);
     const p64::F3 px = p64::split3(xi * sc.len), py = p64::split3(yi * sc.len);
     const p64::F3 pz = p64::split3(zi * sc.len);
@@ -77,28 +68,26 @@ __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, c
             const int j = jt + threadIdx.x, t = threadIdx.x;
             const D4 p{q[j], q[R + j], q[2 * R + j], G * m[j]};
             const p64::F3 x = p64::split3(p.x * sc.len), y = p64::split3(p.y * sc.len);
-            const p64::F3 z = p64::split3(p.z * sc.len), g = p64::split3(p.w * sc.wt);
+            const p64::F3 z = p64::split3(p.z * sc.len);
             s_q[t] = p;
-            s_h[t] = make_float4(x.h, y.h, z.h, g.h);
-            s_m[t] = make_float4(x.m, y.m, z.m, g.m);
-            s_l[t] = make_float4(x.l, y.l, z.l, g.l);
+            s_a[t] = make_float4(x.h, y.h, z.h, x.m);
+            s_b[t] = make_float4(y.m, z.m, x.l, y.l);
+            s_c[t] = z.l;
         }
         __syncthreads();
-#pragma unroll 1
+#pragma unroll 2
         for (int t = 0; t < n; ++t) {
-            const float4 H = s_h[t], M = s_m[t], L = s_l[t];
-            const p64::F3 r2 = p64::norm2(p64::diff(px, p64::F3{H.x, M.x, L.x}),
-                                          p64::diff(py, p64::F3{H.y, M.y, L.y}),
-                                          p64::diff(pz, p64::F3{H.z, M.z, L.z}));
-            double s;
-            const bool ok = p64::g_over_r(p64::F3{H.w, M.w, L.w}, r2, rsqrt_ftz(r2.h), bias, s) &&
-                            p64::r2_fits(r2.h) && p64::g_fits(H.w) && sc.ok;
+            const float4 A = s_a[t], B = s_b[t];
+            const p64::F3 r2 = p64::norm2(p64::diff(px, p64::F3{A.x, A.w, B.z}),
+                                          p64::diff(py, p64::F3{A.y, B.x, B.w}),
+                                          p64::diff(pz, p64::F3{A.z, B.y, s_c[t]}));
+            double y = p64::inv_r(r2, rsqrt_ftz(r2.h), bias);
             const bool later = jt + t > i;
-            if (!ok && later) {
+            if (later && !(sc.ok && p64::r2_fits(r2.h))) {
                 const D4 p = s_q[t];
-                s = potential_fp64(xi - p.x, yi - p.y, zi - p.z, p.w);
+                y = inv_r_fp64(xi - p.x, yi - p.y, zi - p.z);
             }
-            if (later) phi += s;
+            if (later) phi = fma(s_q[t].w, y, phi);
         }
     }
     const bool act = i < bk.y;

@@ -240,22 +240,15 @@ P64_HD bool g_over_r3(const F3 &g, const F3 &r2, float y0, uint64_t bias, double
     return s.h >= kMinResult;
 }
 
-// out = g / r 2^k; false where it is below kMinResult
-P64_HD bool g_over_r(const F3 &g, const F3 &r2, float y0, uint64_t bias, double &out) {
+// 1 / r 2^k (bias: k << 52) as a double
+P64_HD double inv_r(const F3 &r2, float y0, uint64_t bias) {
     const Residual R = residual(r2, y0);
     // (1 - e)^(-1/2) = 1 + e / 2 + 3/8 e^2
     const float C0 = mul(0.5f, R.E0);
     const float C1 = fma_(mul(0.375f, R.E0), R.E0, mul(0.5f, R.E1));
-    float p, pe, q, qe, k1, k2, z0, z0e, z, ze;
-    two_prod(g.h, y0, p, pe);
-    two_prod(g.m, y0, q, qe);
-    two_sum(pe, q, k1, k2);
-    two_prod(p, C0, z0, z0e);
-    two_sum(z0, k1, z, ze);
-    const float lo = add(fma_(p, C1, fma_(k1, C0, z0e)),
-                         add(fma_(g.l, y0, add(qe, k2)), ze));
-    out = to_double(p, z, lo, bias);
-    return p >= kMinResult;
+    float z, ze;
+    two_prod(y0, C0, z, ze);
+    return to_double(y0, z, fma_(y0, C1, ze), bias);
 }
 
 #ifdef __CUDACC__
