@@ -173,12 +173,16 @@ constexpr int RSL = 16;    // members per force round on a cluster (receive buff
 
 constexpr int KMAX = 48;
 
-// corrector constants of a level's step h (signed), rows of HermSmem::lvt:
-// a2 = (-6 d - h (4 j0 + 2 j1)) / h^2 = A2D d + A2J0 j0 + A2J1 j1,
-// a3 = (12 d + 6 h (j0 + j1)) / h^3 = A3D d + A3J (j0 + j1),
-// x1 = x_p + h^4/24 a2 + h^5/120 a3, v1 = v_p + h^3/6 a2 + h^4/24 a3,
-// and a2 at the end of the step, a2 + h a3 (d = a0 - a1)
-enum LvConst : int { LV_H = 0, LV_A2D, LV_A2J0, LV_A2J1, LV_A3D, LV_A3J, LV_H4, LV_H5, LV_H3, LV_N };
+// Constants of a level's step h (signed), rows of HermSmem::lvt. With d = a0 - a1
+// the corrector and the step criterion are linear in (d, j0, j1):
+//   x1  = x_p - 3/20 h^2 d - h^3 (7/60 j0 + 1/30 j1)
+//   v1  = v_p - 1/2 h d - h^2 (5/12 j0 + 1/12 j1)
+//   a2e = 6 d / h^2 + (2 j0 + 4 j1) / h     (a2 at the end of the step)
+//   a3  = 12 d / h^3 + 6 (j0 + j1) / h^2
+// (x_p + h^4/24 a2 + h^5/120 a3 and v_p + h^3/6 a2 + h^4/24 a3 written out). Form f's
+// factors of d, j0, j1 are the rows 3 f, 3 f + 1, 3 f + 2; a3's last two are one row.
+enum LvForm : int { LF_X = 0, LF_V, LF_A2, LF_A3 };
+constexpr int LV_N = 11;
 
 struct HermSmem {
     double *ex, *ey, *ez, *eu, *ev, *ew;      // evaluation point of every member
@@ -197,7 +201,7 @@ struct HermSmem {
     int32_t *act;                             // members whose step ends now
     int32_t *ids;
     int32_t *need;                            // member needed in FP64 at this block time
-    int32_t *nl;                              // per coordinate warp: those members [3][HCAP]
+    int32_t *nl;                              // those members [HCAP], 2 HCAP spare
                                               // (need and nl also hold the two-warp force's
                                               // exchange slots, [2][3][96] doubles)
 };
@@ -398,20 +402,32 @@ __device__ __forceinline__ int level_from(const float *f, int lv, float eta, flo
     return k < 0 ? 0 : (k > KMAX ? KMAX : k);
 }
 
-// component c of member k predicted from its own time to tn
-__device__ __forceinline__ void predict_c(const HermSmem &S, int k, int c, long long tn,
+// a time in ticks (below 2^52) times a factor, in one FP64 operation: the bits of
+// 2^52 + dt are dt's under the exponent, and the product with f less 2^52 f is rounded
+// once, as (double)dt * f is
+__device__ __forceinline__ double ticks_times(long long dt, double f) {
+    return fma(__longlong_as_double(0x4330000000000000ll | dt), f, f * -0x1p52);
+}
+// v / 2 from the bits (v / 2 normal), else by the multiplication
+__device__ __forceinline__ double half_of(double v) {
+    const int hi = __double2hiint(v);
+    if ((hi & 0x7fe00000) == 0) return 0.5 * v;
+    return __hiloint2double(hi - 0x00100000, __double2loint(v));
+}
+// Coordinate c of member k predicted from its own time to tn: the position
+// x + h (u + h/2 (a + h/3 j)) or the velocity u + h (a + h/2 j). stick3 = stick / 3
+__device__ __forceinline__ void predict_x(const HermSmem &S, int k, int c, long long tn,
+                                          double stick, double stick3) {
+    const long long dt = tn - S.ti[k];
+    const int o = c * HCAP + k;
+    const double h3 = ticks_times(dt, stick3), hs = ticks_times(dt, stick);
+    S.ex[o] = fma(hs, fma(half_of(hs), fma(h3, S.jx[o], S.ax[o]), S.u[o]), S.x[o]);
+}
+__device__ __forceinline__ void predict_v(const HermSmem &S, int k, int c, long long tn,
                                           double stick) {
-    const double hs = (double)(tn - S.ti[k]) * stick;
-    const double h6 = hs * (1.0 / 6.0);
-    double *x = c == 0 ? S.x : (c == 1 ? S.y : S.z);
-    double *u = c == 0 ? S.u : (c == 1 ? S.v : S.w);
-    double *a = c == 0 ? S.ax : (c == 1 ? S.ay : S.az);
-    double *j = c == 0 ? S.jx : (c == 1 ? S.jy : S.jz);
-    double *ex = c == 0 ? S.ex : (c == 1 ? S.ey : S.ez);
-    double *eu = c == 0 ? S.eu : (c == 1 ? S.ev : S.ew);
-    const double ak = a[k], jk = j[k], uk = u[k];
-    ex[k] = x[k] + hs * (uk + hs * (0.5 * ak + h6 * jk));
-    eu[k] = uk + hs * (ak + 0.5 * hs * jk);
+    const int o = c * HCAP + k;
+    const double hs = ticks_times(tn - S.ti[k], stick);
+    S.eu[o] = fma(hs, fma(half_of(hs), S.jx[o], S.ax[o]), S.u[o]);
 }
 
 // FP32 copies of member k's state (truncated: within 2^-23 of the FP64
@@ -422,8 +438,8 @@ __device__ __forceinline__ void store_f32(const HermSmem &S, int k) {
     for (int q = 0; q < 12; ++q) S.f[q * HCAP + k] = to_float_scaled(src[q][k], 0);
 }
 
-// Member k's position predicted to tn in FP32 from the copies, by the same
-// Horner form as the FP64 predictor, and a bound pd on its distance from the
+// Member k's position predicted to tn in FP32 from the copies, by the
+// Horner form x + h (u + h (a/2 + (h/6) j)), and a bound pd on its distance from the
 // FP64 prediction. Each input is within 2^-23 of its FP64 value (hs within
 // 3 2^-24), and each of the three fmaf roundings adds 2^-24 relative to the
 // magnitude of what it rounds, so every term of the polynomial is within
@@ -538,6 +554,7 @@ struct HermArgs {
 __shared__ int g_next_small;
 __shared__ long long g_tn;
 __shared__ int g_na;
+__shared__ int g_nneed;  // members of the FP32-screened list
 
 // Next block time (the earliest end of a member's step) and the members whose
 // step ends then, in member order, by one warp; every thread reads (tn, na)
@@ -735,10 +752,11 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     // one warp per (member, component) for the sums.
     const int warp = tid >> 5, wl = tid & 31;
     const double stick = sgn * tick;
-    const double T2d = T * T, T3 = T2d * T, T4 = T3 * T;
+    const double T2d = T * T, T3 = T2d * T;
     const double iT2 = inv_T * inv_T, iT3 = iT2 * inv_T;
     const float T2f = (float)T2d, etaf = (float)h.eta;
     const float stickf = (float)stick;
+    const double stick3 = stick / 3.0;
     const float rcf = __double2float_ru(d.rcrit[set] * (1.0 + 0x1p-20));
     const int npart = mhi - mlo;
     // the largest range of the cluster: every CTA derives its lane layout and
@@ -751,45 +769,49 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     for (int k = tid; k < n; k += blockDim.x) store_f32(S, k);
     for (int lv = tid; lv <= KMAX; lv += blockDim.x) {
         double *L = S.lvt + lv;
+        constexpr int LS = KMAX + 1;
         const double ih = sgn * inv_T * pow2d(lv), ih2 = iT2 * pow2d(2 * lv);
-        L[LV_H * (KMAX + 1)] = sgn * T * pow2d(-lv);
-        L[LV_A2D * (KMAX + 1)] = -6.0 * ih2;
-        L[LV_A2J0 * (KMAX + 1)] = -4.0 * ih;
-        L[LV_A2J1 * (KMAX + 1)] = -2.0 * ih;
-        L[LV_A3D * (KMAX + 1)] = 12.0 * (sgn * iT3 * pow2d(3 * lv));
-        L[LV_A3J * (KMAX + 1)] = 6.0 * ih2;
-        L[LV_H4 * (KMAX + 1)] = (T4 * pow2d(-4 * lv)) * (1.0 / 24.0);
-        L[LV_H5 * (KMAX + 1)] = (sgn * T4 * T * pow2d(-5 * lv)) * (1.0 / 120.0);
-        L[LV_H3 * (KMAX + 1)] = (sgn * T3 * pow2d(-3 * lv)) * (1.0 / 6.0);
+        const double h = sgn * T * pow2d(-lv), h2 = T2d * pow2d(-2 * lv);
+        const double h3 = sgn * T3 * pow2d(-3 * lv);
+        L[(3 * LF_X) * LS] = h2 * (-3.0 / 20.0);
+        L[(3 * LF_X + 1) * LS] = h3 * (-7.0 / 60.0);
+        L[(3 * LF_X + 2) * LS] = h3 * (-1.0 / 30.0);
+        L[(3 * LF_V) * LS] = h * -0.5;
+        L[(3 * LF_V + 1) * LS] = h2 * (-5.0 / 12.0);
+        L[(3 * LF_V + 2) * LS] = h2 * (-1.0 / 12.0);
+        L[(3 * LF_A2) * LS] = 6.0 * ih2;
+        L[(3 * LF_A2 + 1) * LS] = 2.0 * ih;
+        L[(3 * LF_A2 + 2) * LS] = 4.0 * ih;
+        L[(3 * LF_A3) * LS] = 12.0 * (sgn * iT3 * pow2d(3 * lv));
+        L[(3 * LF_A3 + 1) * LS] = 6.0 * ih2;
     }
     const bool with_star = rank == 0;
     int64_t steps = 0;
     bool capped = false;
     int buf = 0;
-    // the first block time; later ones are found by warp 3 right after it sets
+    // the first block time; later ones are found by warp 6 right after it sets
     // the new levels (it wrote every value the scan reads), so one barrier per
     // block step publishes them
-    if (warp == 3) next_block(S.lev, S.ti, S.act, n);
+    if (warp == 6) next_block(S.lev, S.ti, S.act, n);
+    // chunk of 32 prediction items this warp takes first: positions (even) and
+    // velocities (odd) on all four sub-partitions
+    const int pq0 = warp ^ (warp >> 2);
     for (;;) {
         __syncthreads();
         const long long tn = g_tn;
         if (tn > TT) break;  // every member has reached tau
         if (steps >= h.max_steps) { capped = true; break; }
         const int na = g_na;
-        // Predict this CTA's partners and the active members to tn. Up to two
-        // warps' worth, FP64 passes over them all (one warp per coordinate);
-        // above that the FP32 prediction first rules out the partners that are
-        // surely beyond r_crit of every active member.
+        // Predict this CTA's partners and the active members to tn: items
+        // (member, coordinate), 32 to a warp, positions and velocities in chunks of
+        // their own, so that a few members cost one warp's five FP64 instructions
+        // instead of eleven on each of three warps. Up to F32MIN members FP64 passes
+        // over them all; above that the FP32 prediction first rules out the partners
+        // that are surely beyond r_crit of every active member.
         const bool f32 = npmax + na > F32MIN;
-        if (!f32) {
-            if (warp < 3) {
-                for (int i = wl; i < npart + na; i += 32) {
-                    int k = mlo + i;
-                    if (i >= npart) k = S.act[i - npart];
-                    if (i < npart || k < mlo || k >= mhi) predict_c(S, k, warp, tn, stick);
-                }
-            }
-        } else {
+        const int32_t *list = nullptr;
+        int np = npart + na;
+        if (f32) {
             for (int k = tid; k < n; k += HTHREADS) S.need[k] = 0;
             for (int i = tid; i < npart + na; i += HTHREADS) {
                 int k = mlo + i;
@@ -809,21 +831,39 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 if (l != k && maybe_near(S, k, l, rcf)) S.need[l] = 1;
             }
             __syncthreads();
-            // their FP64 prediction, one warp per coordinate, each warp listing
-            // them in member order for itself
-            if (warp < 3) {
-                int32_t *nl = S.nl + warp * HCAP;
+            // listed in member order by one warp
+            if (warp == 0) {
                 int nn = 0;
                 for (int k0 = 0; k0 < n; k0 += 32) {
                     const int k = k0 + wl;
                     const bool f = k < n && S.need[k] != 0;
                     const unsigned b = __ballot_sync(0xffffffffu, f);
-                    if (f) nl[nn + __popc(b & ((1u << wl) - 1u))] = k;
+                    if (f) S.nl[nn + __popc(b & ((1u << wl) - 1u))] = k;
                     nn += __popc(b);
                 }
-                __syncwarp();
-                for (int i = wl; i < nn; i += 32) predict_c(S, nl[i], warp, tn, stick);
+                if (wl == 0) g_nneed = nn;
             }
+            __syncthreads();
+            list = S.nl;
+            np = g_nneed;
+        }
+        for (int pq = pq0; (pq >> 1) * 32 < 3 * np; pq += HTHREADS / 32) {
+            const int it = (pq >> 1) * 32 + wl, i = it / 3, c = it - 3 * i;
+            if (i >= np) continue;
+            int k;
+            if (f32) {
+                k = list[i];
+            } else {
+                k = mlo + i;
+                if (i >= npart) {
+                    k = S.act[i - npart];
+                    if (k >= mlo && k < mhi) continue;
+                }
+            }
+            if (pq & 1)
+                predict_v(S, k, c, tn, stick);
+            else
+                predict_x(S, k, c, tn, stick, stick3);
         }
         __syncthreads();
         for (int a0 = 0; a0 < na; a0 += ACH) {
@@ -998,70 +1038,67 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 }
                 __syncthreads();
             }
-            // corrector, one warp per coordinate (the same in every CTA), in two
-            // parts: the derivatives first, which warp 3 waits for to set the new
-            // levels and find the next block time, then positions and
-            // velocities beside it (levels and next block took 1700 of a
-            // block step's 12000 cycles after the whole corrector)
-            if (warp < 3) {
-                const int c = warp;
-                double *xa = c == 0 ? S.x : (c == 1 ? S.y : S.z);
-                double *ua = c == 0 ? S.u : (c == 1 ? S.v : S.w);
-                double *aa = c == 0 ? S.ax : (c == 1 ? S.ay : S.az);
-                double *ja = c == 0 ? S.jx : (c == 1 ? S.jy : S.jz);
-                const double *ea = c == 0 ? S.ex : (c == 1 ? S.ey : S.ez);
-                const double *fa = c == 0 ? S.eu : (c == 1 ? S.ev : S.ew);
-                constexpr int LS = KMAX + 1, NS = ACH / 32;
-                int kk[NS], lvs[NS];
-                double A2[NS], A3[NS], A1[NS], J1[NS];
-#pragma unroll
-                for (int q = 0; q < NS; ++q) {
-                    const int sl = wl + 32 * q;
-                    kk[q] = -1;
-                    if (sl >= nc) continue;
-                    const int k = S.act[a0 + sl];
+            // Corrector and step criterion (the same in every CTA): items (member,
+            // coordinate), 32 to a warp, and each of the four linear forms on a warp of
+            // its own sub-partition, four FP64 instructions deep; warps 4 and 5 bring
+            // the new acceleration and jerk. Warp 6 sets the new levels when the
+            // criterion's inputs are there, and finds the next block time.
+            // (One warp per coordinate with a2 and a3 first took eight instructions to
+            // the criterion and twelve to the state.)
+            constexpr int LS = KMAX + 1;
+            if (warp < 4) {
+                const int f = warp;
+                const double *cd = S.lvt + 3 * f * LS;
+                const double *c1 = cd + (f == LF_A3 ? LS : 2 * LS);
+                for (int it = wl; it < 3 * nc; it += 32) {
+                    const int sl = it / 3, c = it - 3 * sl;
+                    const int k = S.act[a0 + sl], o = c * HCAP + k;
                     const int lv = S.lev[k];
-                    const double *L = S.lvt + lv;
-                    const double a1c = S.a1s[c * ACH + sl], j1c = S.a1s[(3 + c) * ACH + sl];
-                    const double d = aa[k] - a1c, j0c = ja[k];
-                    const double a2 =
-                        fma(L[LV_A2D * LS], d, fma(L[LV_A2J0 * LS], j0c, L[LV_A2J1 * LS] * j1c));
-                    const double a3 = fma(L[LV_A3D * LS], d, L[LV_A3J * LS] * (j0c + j1c));
-                    const double a2e = fma(L[LV_H * LS], a3, a2);  // a2 at the end of the step
-                    S.cf[c * ACH + sl] = to_float_scaled(a1c, 0);
-                    S.cf[(3 + c) * ACH + sl] = to_float_scaled(j1c, -lv);
-                    S.cf[(6 + c) * ACH + sl] = to_float_scaled(a2e, -2 * lv);
-                    S.cf[(9 + c) * ACH + sl] = to_float_scaled(a3, -3 * lv);
-                    kk[q] = k;
-                    lvs[q] = lv;
-                    A2[q] = a2;
-                    A3[q] = a3;
-                    A1[q] = a1c;
-                    J1[q] = j1c;
+                    const double d = S.ax[o] - S.a1s[c * ACH + sl];
+                    const double base = f == LF_X ? S.ex[o] : (f == LF_V ? S.eu[o] : 0.0);
+                    const double r = fma(
+                        cd[lv], d,
+                        fma(cd[LS + lv], S.jx[o], fma(c1[lv], S.a1s[(3 + c) * ACH + sl], base)));
+                    if (f < LF_A2) {
+                        S.x[3 * f * HCAP + o] = r;
+                        S.f[3 * f * HCAP + o] = to_float_scaled(r, 0);
+                    } else {
+                        S.cf[(3 * f + c) * ACH + sl] = to_float_scaled(r, -f * lv);
+                    }
                 }
                 __syncwarp();
-                asm volatile("bar.arrive 5, 128;" ::: "memory");
-                // (the members' levels and the active list are warp 3's from here)
+                asm volatile("bar.arrive 5, 224;" ::: "memory");
+                // (levels, active list, a and adot are not read by these warps any more)
+            } else if (warp < 6) {
+                const int f = warp - 4;  // 0: a, 1: adot
+                constexpr int NS = 3 * ACH / 32;
+                int oo[NS];
+                float fv[NS];
 #pragma unroll
                 for (int q = 0; q < NS; ++q) {
-                    const int k = kk[q];
-                    if (k < 0) continue;
-                    const double *L = S.lvt + lvs[q];
-                    const double xn = fma(L[LV_H4 * LS], A2[q], fma(L[LV_H5 * LS], A3[q], ea[k]));
-                    const double un = fma(L[LV_H3 * LS], A2[q], fma(L[LV_H4 * LS], A3[q], fa[k]));
-                    xa[k] = xn;
-                    ua[k] = un;
-                    aa[k] = A1[q];
-                    ja[k] = J1[q];
-                    S.f[c * HCAP + k] = to_float_scaled(xn, 0);
-                    S.f[(3 + c) * HCAP + k] = to_float_scaled(un, 0);
-                    S.f[(6 + c) * HCAP + k] = to_float_scaled(A1[q], 0);
-                    S.f[(9 + c) * HCAP + k] = to_float_scaled(J1[q], 0);
+                    const int it = q * 32 + wl, sl = it / 3, c = it - 3 * sl;
+                    oo[q] = -1;
+                    if (it >= 3 * nc) continue;
+                    const int k = S.act[a0 + sl];
+                    const double r = S.a1s[(3 * f + c) * ACH + sl];
+                    oo[q] = c * HCAP + k;
+                    fv[q] = to_float_scaled(r, 0);
+                    S.cf[(3 * f + c) * ACH + sl] = to_float_scaled(r, -f * S.lev[k]);
                 }
-            } else if (warp == 3) {
+                __syncwarp();
+                asm volatile("bar.sync 5, 224;" ::: "memory");
+                double *to = S.ax + 3 * f * HCAP;
+#pragma unroll
+                for (int q = 0; q < NS; ++q) {
+                    if (oo[q] < 0) continue;
+                    const int it = q * 32 + wl, sl = it / 3, c = it - 3 * sl;
+                    to[oo[q]] = S.a1s[(3 * f + c) * ACH + sl];
+                    S.f[(6 + 3 * f) * HCAP + oo[q]] = fv[q];
+                }
+            } else if (warp == 6) {
                 // new time and level by the Aarseth criterion (FP32 on scaled
                 // inputs); a larger step only by one level and on a commensurate time
-                asm volatile("bar.sync 5, 128;" ::: "memory");
+                asm volatile("bar.sync 5, 224;" ::: "memory");
                 for (int sl = wl; sl < nc; sl += 32) {
                     const int k = S.act[a0 + sl];
                     const int lv = S.lev[k];
@@ -1079,7 +1116,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         }
         // every thread read (tn, na) before the barriers above; the active
         // list is no longer read in this block step
-        if (warp == 3) next_block(S.lev, S.ti, S.act, n);
+        if (warp == 6) next_block(S.lev, S.ti, S.act, n);
         ++steps;
     }
     // peers may still read this CTA's partial sums of the last round
