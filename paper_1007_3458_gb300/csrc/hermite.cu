@@ -198,10 +198,11 @@ struct HermSmem {
     float *px, *py, *pz, *pd;                 // FP32 prediction and its error bound
     float *cf;                                // step criterion inputs [12][ACH]
     int32_t *lev;                             // member level: step = tau 2^-lev
-    int32_t *act;                             // members whose step ends now
+    uint16_t *act;                            // members whose step ends now, and at the next
+                                              // block time [2][HCAP]
     int32_t *ids;
     int32_t *need;                            // member needed in FP64 at this block time
-    int32_t *nl;                              // those members [HCAP], 2 HCAP spare
+    int32_t *nl;                              // those members [HCAP], 2 HCAP - 64 spare
                                               // (need and nl also hold the two-warp force's
                                               // exchange slots, [2][3][96] doubles)
 };
@@ -227,7 +228,7 @@ __device__ __forceinline__ HermSmem carve(void *base) {
     s.cf = fp; fp += 12 * ACH;
     int32_t *ip = (int32_t *)fp;
     s.lev = ip; ip += HCAP;
-    s.act = ip; ip += HCAP;
+    s.act = (uint16_t *)ip; ip += HCAP;
     s.ids = ip; ip += HCAP;
     s.need = ip; ip += HCAP;
     s.nl = ip;
@@ -235,11 +236,12 @@ __device__ __forceinline__ HermSmem carve(void *base) {
 }
 constexpr size_t kHermSmem =
     sizeof(double) * (HCAP * 20 + 6 * HTHREADS + 2 * CLMAX * 6 * RSL + 6 * ACH + LV_N * (KMAX + 1)) +
-    sizeof(float) * (16 * HCAP + 12 * ACH) + sizeof(int32_t) * HCAP * 7;
-static_assert(2 * 3 * 96 * sizeof(double) <= 4 * HCAP * sizeof(int32_t),
+    sizeof(float) * (16 * HCAP + 12 * ACH) + sizeof(int32_t) * (HCAP * 7 - 64);
+static_assert(2 * 3 * 96 * sizeof(double) <= (4 * HCAP - 64) * sizeof(int32_t),
               "the two-warp force's exchange slots overlay need and nl");
-// two CTAs per SM (228 KB of shared memory, 1 KB of it per CTA reserved)
-static_assert(2 * (kHermSmem + 1024) <= 228 * 1024, "Hermite shared memory above two CTAs per SM");
+// two CTAs per SM (228 KB of shared memory, 1 KB of it per CTA reserved, 128 bytes
+// for the variables below)
+static_assert(2 * (kHermSmem + 128 + 1024) <= 228 * 1024, "Hermite shared memory above two CTAs per SM");
 
 // smallest k with T 2^-k <= dt_c, in [0, KMAX]: with T = fT 2^eT and
 // dt_c = fd 2^ed (fT, fd in [1/2, 1)), T 2^-k <= dt_c exactly when
@@ -370,7 +372,13 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ int level_from(const float *f, int lv, float eta, float T2) {
+// T^2 split for level_from: T2 = ft 2^et, ft in [1/2, 1)
+struct T2Split {
+    int et;
+    float ft;
+    __device__ __forceinline__ explicit T2Split(float T2) { ft = frexpf(T2, &et); }
+};
+__device__ __forceinline__ int level_from(const float *f, int lv, float eta, const T2Split &T2) {
     float q[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
@@ -379,34 +387,29 @@ __device__ __forceinline__ int level_from(const float *f, int lv, float eta, flo
     }
     const float num = eta * fmaf(q[0], q[2], q[1] * q[1]);
     const float den = fmaf(q[1], q[3], q[2] * q[2]);
-    if (!(den > 0.0f)) return 0;
-    if (!(num > 0.0f)) return KMAX;
     const float r = __fdividef(num, den);
-    if (!(r < INFINITY)) return 0;
-    // r = fr 2^er, T2 = ft 2^et with fr, ft in [1/2, 1)
-    int er, et;
-    float fr, ft;
-    const int br = __float_as_int(r), bt = __float_as_int(T2);
-    if (br >= 0x00800000 && bt >= 0x00800000) {
-        er = br >> 23;
-        et = bt >> 23;
-        fr = __int_as_float((br & 0x7fffff) | 0x3f000000);
-        ft = __int_as_float((bt & 0x7fffff) | 0x3f000000);
-    } else {
-        fr = frexpf(r, &er);
-        ft = frexpf(T2, &et);
-    }
-    const int dd = er - et;
-    const int m = (dd & 1) ? (dd - 1) >> 1 : ((ft <= fr) ? dd >> 1 : (dd >> 1) - 1);
-    const int k = lv - m;
-    return k < 0 ? 0 : (k > KMAX ? KMAX : k);
+    // r = fr 2^er with fr in [1/2, 1)
+    const int br = __float_as_int(r);
+    int er = (br >> 23) - 126;
+    float fr = __int_as_float((br & 0x7fffff) | 0x3f000000);
+    if (br < 0x00800000) fr = frexpf(r, &er);
+    const int dd = er - T2.et;
+    const int m = (dd & 1) ? (dd - 1) >> 1 : ((T2.ft <= fr) ? dd >> 1 : (dd >> 1) - 1);
+    int k = min(max(lv - m, 0), KMAX);
+    if (!(r < INFINITY)) k = 0;
+    if (!(num > 0.0f)) k = KMAX;
+    return den > 0.0f ? k : 0;
 }
 
-// a time in ticks (below 2^52) times a factor, in one FP64 operation: the bits of
+// A time in ticks (below 2^52) times a factor f in one FP64 operation: the bits of
 // 2^52 + dt are dt's under the exponent, and the product with f less 2^52 f is rounded
-// once, as (double)dt * f is
-__device__ __forceinline__ double ticks_times(long long dt, double f) {
-    return fma(__longlong_as_double(0x4330000000000000ll | dt), f, f * -0x1p52);
+// once, as (double)dt * f is. (b = -2^52 f, exact.)
+struct TickF {
+    double f, b;
+    __device__ __forceinline__ explicit TickF(double v) : f(v), b(v * -0x1p52) {}
+};
+__device__ __forceinline__ double ticks_times(long long dt, const TickF &s) {
+    return fma(__longlong_as_double(0x4330000000000000ll | dt), s.f, s.b);
 }
 // v / 2 from the bits (v / 2 normal), else by the multiplication
 __device__ __forceinline__ double half_of(double v) {
@@ -417,14 +420,14 @@ __device__ __forceinline__ double half_of(double v) {
 // Coordinate c of member k predicted from its own time to tn: the position
 // x + h (u + h/2 (a + h/3 j)) or the velocity u + h (a + h/2 j). stick3 = stick / 3
 __device__ __forceinline__ void predict_x(const HermSmem &S, int k, int c, long long tn,
-                                          double stick, double stick3) {
+                                          const TickF &stick, const TickF &stick3) {
     const long long dt = tn - S.ti[k];
     const int o = c * HCAP + k;
     const double h3 = ticks_times(dt, stick3), hs = ticks_times(dt, stick);
     S.ex[o] = fma(hs, fma(half_of(hs), fma(h3, S.jx[o], S.ax[o]), S.u[o]), S.x[o]);
 }
 __device__ __forceinline__ void predict_v(const HermSmem &S, int k, int c, long long tn,
-                                          double stick) {
+                                          const TickF &stick) {
     const int o = c * HCAP + k;
     const double hs = ticks_times(tn - S.ti[k], stick);
     S.eu[o] = fma(hs, fma(half_of(hs), S.jx[o], S.ax[o]), S.u[o]);
@@ -461,6 +464,32 @@ __device__ __forceinline__ void predict_f32(const HermSmem &S, int k, long long 
     }
     S.pd[k] = fmaf(m, 0x1p-18f, 1e-30f);
 }
+
+// One item (active slot, coordinate) of the corrector's linear form f: everything but
+// the new acceleration and jerk, read while those are on their way.
+struct CorrItem {
+    double cd, c0, c1, a, j, base;
+    int o, s, lv;  // coordinate and member, coordinate and slot, the member's level
+    __device__ __forceinline__ void fetch(const HermSmem &S, int f, const uint16_t *act, int it) {
+        constexpr int LS = KMAX + 1;
+        const int sl = it / 3, c = it - 3 * sl;
+        const int k = act[sl];
+        o = c * HCAP + k;
+        s = c * ACH + sl;
+        lv = S.lev[k];
+        const double *L = S.lvt + 3 * f * LS + lv;
+        cd = L[0];
+        c0 = L[LS];
+        c1 = f == LF_A3 ? c0 : L[2 * LS];
+        a = S.ax[o];
+        j = S.jx[o];
+        base = f < LF_A2 ? S.ex[3 * f * HCAP + o] : 0.0;
+    }
+    __device__ __forceinline__ double value(const HermSmem &S) const {
+        const double d = a - S.a1s[s], j1 = S.a1s[3 * ACH + s];
+        return fma(cd, d, fma(c0, j, fma(c1, j1, base)));
+    }
+};
 
 // false only when members k and l, both predicted in FP32 to the same time,
 // are surely farther apart than r_crit in their FP64 predictions: then the
@@ -546,6 +575,50 @@ __device__ __forceinline__ void pair_bar(int p) {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + p) : "memory");
 }
 
+// A cluster's exchange of force sums: every CTA stores its sums into the others'
+// receive buffers by st.async, which counts the bytes on the receiver's mbarrier
+// (g_rbar, one per receive buffer; a phase ends when the bytes of all CTAs' sums,
+// announced by one thread, are there). A cluster barrier instead waits for the
+// stores' round trip and then for the barrier's own.
+__shared__ __align__(8) unsigned long long g_rbar[2];
+__device__ __forceinline__ unsigned smem_addr(const void *p) {
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void rbar_init() {
+    for (int b = 0; b < 2; ++b)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&g_rbar[b])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void rbar_expect(int b, int bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&g_rbar[b])),
+                 "r"(bytes)
+                 : "memory");
+}
+// v into CTA r's copy of *p, counted on its g_rbar[b]
+__device__ __forceinline__ void rbar_send(double *p, double v, int r, int b) {
+    unsigned pa, ba;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(pa) : "r"(smem_addr(p)), "r"(r));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ba) : "r"(smem_addr(&g_rbar[b])), "r"(r));
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(pa),
+                 "l"(__double_as_longlong(v)), "r"(ba)
+                 : "memory");
+}
+// waits for the phase of the given parity; false when it does not end in a second or so
+__device__ __forceinline__ bool rbar_wait(int b, int parity) {
+    for (int i = 0; i < (1 << 20); ++i) {
+        unsigned done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(smem_addr(&g_rbar[b])), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
 struct HermArgs {
     double G, eps2, eta, eta_s, tau;
     int64_t max_steps;
@@ -556,14 +629,18 @@ __shared__ long long g_tn;
 __shared__ int g_na;
 __shared__ int g_nneed;  // members of the FP32-screened list
 
-// Next block time (the earliest end of a member's step) and the members whose
-// step ends then, in member order, by one warp; every thread reads (tn, na)
-// after the barrier that follows. The end times stay in registers
-// between the two passes; the minimum (below 2^49) is taken as the minimum of
-// the high words, then of the low words among the lanes that hold it.
+// The earliest end of a member's step later than `after`, and the members whose step
+// ends then, listed in member order in act, by one warp (LLONG_MAX and none when no
+// step ends later). The end times stay in registers between the two passes; the
+// minimum (below 2^49) is taken as the minimum of the high words, then of the low
+// words among the lanes that hold it.
+struct Block {
+    long long t;
+    int na;
+};
 template <int NI>
-__device__ __forceinline__ void next_block_of(const int32_t *lev, const long long *ti, int32_t *act,
-                                              int n) {
+__device__ __forceinline__ Block next_block_of(const int32_t *lev, const long long *ti,
+                                               uint16_t *act, int n, long long after) {
     const int wl = threadIdx.x & 31;
     long long te[NI];
     long long t = LLONG_MAX;
@@ -571,34 +648,32 @@ __device__ __forceinline__ void next_block_of(const int32_t *lev, const long lon
     for (int q = 0; q < NI; ++q) {
         const int k = q * 32 + wl;
         te[q] = (k < n) ? ti[k] + (1ll << (KMAX - lev[k])) : LLONG_MAX;
+        if (te[q] <= after) te[q] = LLONG_MAX;
         t = min(t, te[q]);
     }
     const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(t >> 32));
     const unsigned lo =
         __reduce_min_sync(0xffffffffu, (unsigned)(t >> 32) == hi ? (unsigned)t : 0xffffffffu);
-    t = (long long)(((unsigned long long)hi << 32) | lo);
-    int na = 0;
+    Block b;
+    b.t = (long long)(((unsigned long long)hi << 32) | lo);
+    b.na = 0;
+    if (b.t == LLONG_MAX) return b;
 #pragma unroll
     for (int q = 0; q < NI; ++q) {
         if (q * 32 >= n) break;
-        const bool f = te[q] == t;
-        const unsigned b = __ballot_sync(0xffffffffu, f);
-        if (f) act[na + __popc(b & ((1u << wl) - 1u))] = q * 32 + wl;
-        na += __popc(b);
+        const bool f = te[q] == b.t;
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (f) act[b.na + __popc(m & ((1u << wl) - 1u))] = (uint16_t)(q * 32 + wl);
+        b.na += __popc(m);
     }
-    if (wl == 0) {
-        g_tn = t;
-        g_na = na;
-    }
+    return b;
 }
 
 // (most sets have at most 64 members: two rounds instead of ten)
-__device__ __forceinline__ void next_block(const int32_t *lev, const long long *ti, int32_t *act,
-                                           int n) {
-    if (n <= 64)
-        next_block_of<2>(lev, ti, act, n);
-    else
-        next_block_of<HCAP / 32>(lev, ti, act, n);
+__device__ __forceinline__ Block next_block(const int32_t *lev, const long long *ti,
+                                            uint16_t *act, int n, long long after) {
+    return n <= 64 ? next_block_of<2>(lev, ti, act, n, after)
+                   : next_block_of<HCAP / 32>(lev, ti, act, n, after);
 }
 
 // Copy the member range [lo, hi) of arrays a..: from CTA `r` of the cluster
@@ -644,6 +719,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             for (int k = tid; k < n; k += blockDim.x) d.uf[d.set_mem[st + k]] = -1;
         return;
     }
+    // (the first cluster barrier below comes before the first exchange; a cluster
+    // integrates one set)
+    if (COOP && tid == 0) rbar_init();
     // this CTA's member range (COOP) or all members
     const int mlo = n * rank / cs, mhi = n * (rank + 1) / cs;
     const int P = lanes_per_member(mhi - mlo, n);
@@ -754,15 +832,24 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const double stick = sgn * tick;
     const double T2d = T * T, T3 = T2d * T;
     const double iT2 = inv_T * inv_T, iT3 = iT2 * inv_T;
-    const float T2f = (float)T2d, etaf = (float)h.eta;
+    const T2Split T2s((float)T2d);
+    const float etaf = (float)h.eta;
     const float stickf = (float)stick;
-    const double stick3 = stick / 3.0;
+    const TickF tick1(stick), tick3(stick / 3.0);
     const float rcf = __double2float_ru(d.rcrit[set] * (1.0 + 0x1p-20));
     const int npart = mhi - mlo;
     // the largest range of the cluster: every CTA derives its lane layout and
     // its round count from it, so all CTAs pass the same cluster barriers and
     // lay out their partial sums alike
     const int npmax = (n + cs - 1) / cs;
+    // lanes per active member of the pair forces, LA = 2^las, and the members of a
+    // round in either form (constants of the set: a division in every block step is
+    // latency on its only chain)
+    int las = 0;
+    while ((1 << las) < npmax && las < 6) ++las;
+    const int LA = 1 << las;
+    const int NU = min(COOP ? RSL : 32, (HTHREADS - 32) >> las);
+    const int NP = min(COOP ? RSL : 32, 96 >> las);
     // FP32 copies of the start-up state; the corrector's constants per level
     // (products with powers of two, so the table holds the same values)
     __syncthreads();
@@ -787,12 +874,20 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     }
     const bool with_star = rank == 0;
     int64_t steps = 0;
-    bool capped = false;
-    int buf = 0;
-    // the first block time; later ones are found by warp 6 right after it sets
-    // the new levels (it wrote every value the scan reads), so one barrier per
-    // block step publishes them
-    if (warp == 6) next_block(S.lev, S.ti, S.act, n);
+    bool capped = false, lost = false;
+    int buf = 0, par = 0;  // receive buffer and its barrier's parity
+    // The first block time. Later ones are found by warp 6, which writes every level
+    // and time: over the members that do not move now while the other warps evaluate
+    // the forces, and over those that do right after it sets their levels; one barrier
+    // per block step publishes them. (One scan of all members after the levels took
+    // 550 of a block step's 10000 cycles.)
+    if (warp == 6) {
+        const Block b = next_block(S.lev, S.ti, S.act, n, -1);
+        if (wl == 0) {
+            g_tn = b.t;
+            g_na = b.na;
+        }
+    }
     // chunk of 32 prediction items this warp takes first: positions (even) and
     // velocities (odd) on all four sub-partitions
     const int pq0 = warp ^ (warp >> 2);
@@ -802,6 +897,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         if (tn > TT) break;  // every member has reached tau
         if (steps >= h.max_steps) { capped = true; break; }
         const int na = g_na;
+        const uint16_t *act = S.act + (steps & 1) * HCAP;
         // Predict this CTA's partners and the active members to tn: items
         // (member, coordinate), 32 to a warp, positions and velocities in chunks of
         // their own, so that a few members cost one warp's five FP64 instructions
@@ -816,7 +912,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             for (int i = tid; i < npart + na; i += HTHREADS) {
                 int k = mlo + i;
                 if (i >= npart) {
-                    k = S.act[i - npart];
+                    k = act[i - npart];
                     if (k >= mlo && k < mhi) continue;
                 }
                 predict_f32(S, k, tn, stickf);
@@ -824,10 +920,10 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             __syncthreads();
             // members needed in FP64: the active ones and the partners that
             // maybe_near does not rule out for some active member
-            for (int i = tid; i < na; i += HTHREADS) S.need[S.act[i]] = 1;
+            for (int i = tid; i < na; i += HTHREADS) S.need[act[i]] = 1;
             for (int p = tid; p < na * npart; p += HTHREADS) {
                 const int ia = p / npart, l = mlo + (p - ia * npart);
-                const int k = S.act[ia];
+                const int k = act[ia];
                 if (l != k && maybe_near(S, k, l, rcf)) S.need[l] = 1;
             }
             __syncthreads();
@@ -856,22 +952,25 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             } else {
                 k = mlo + i;
                 if (i >= npart) {
-                    k = S.act[i - npart];
+                    k = act[i - npart];
                     if (k >= mlo && k < mhi) continue;
                 }
             }
             if (pq & 1)
-                predict_v(S, k, c, tn, stick);
+                predict_v(S, k, c, tn, tick1);
             else
-                predict_x(S, k, c, tn, stick, stick3);
+                predict_x(S, k, c, tn, tick1, tick3);
         }
         __syncthreads();
+        uint16_t *nact = S.act + (~steps & 1) * HCAP;
+        Block nb;       // (warp 6)
+        int lmax = -1;  // (warp 6) the deepest new level, and
+        int mk = 0;     // the lane's member when at most 32 move
+        if (warp == 6) nb = next_block(S.lev, S.ti, nact, n, tn);
         for (int a0 = 0; a0 < na; a0 += ACH) {
             const int nc = min(ACH, na - a0);
             // pair items on warps 0-6 (LA lanes per member), the star's pull
             // (rank 0) on warp 7, so neither path diverges inside a warp
-            int LA = 1;
-            while (LA < npmax && LA < 64) LA <<= 1;
             // slots per round (warp 7 holds one star per slot; on a cluster at
             // most RSL, the receive buffer's width). When the round's members
             // fit three warps' worth of lanes, each pair item runs on two warps
@@ -879,32 +978,32 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // q . p and the acceleration, the odd warp cos and the jerk, which
             // shortens each warp's FP64 instruction stream by about a third.
             // Either way every partial is the same sum in the same order.
-            const int NG = min(COOP ? RSL : 32, (HTHREADS - 32) / LA);
-            const bool paired = nc <= min(COOP ? RSL : 32, 96 / LA);
-            const int NR = paired ? nc : NG;
+            const bool paired = nc <= NP;
+            const int NR = paired ? nc : NU;
+            CorrItem item;  // (warps 0-3)
             for (int s0 = 0; s0 < nc; s0 += NR) {
                 const int cnt = min(NR, nc - s0);
                 double *prb = S.pr;
                 if (!paired) {
                     double aj[6] = {0, 0, 0, 0, 0, 0};
                     if (warp < 7) {
-                        const int slot = s0 + tid / LA, la = tid % LA;
+                        const int slot = s0 + (tid >> las), la = tid & (LA - 1);
                         if (slot < s0 + cnt) {
-                            const int k = S.act[a0 + slot];
+                            const int k = act[a0 + slot];
                             for (int it = la; it < npart; it += LA)
                                 herm_item(S, k, it, mlo, npart, false, gm0, tc, h.eps2, f32, rcf, aj);
                         }
                     } else if (with_star && wl < cnt) {
-                        herm_item(S, S.act[a0 + s0 + wl], npart, mlo, npart, true, gm0, tc, h.eps2,
+                        herm_item(S, act[a0 + s0 + wl], npart, mlo, npart, true, gm0, tc, h.eps2,
                                   f32, rcf, aj);
                     }
 #pragma unroll
                     for (int c = 0; c < 6; ++c) prb[c * HTHREADS + tid] = aj[c];
                 } else if (warp < 6) {
                     const int role = warp & 1, vl = (warp >> 1) * 32 + wl;
-                    const int slot = vl / LA, la = vl - slot * LA;
+                    const int slot = vl >> las, la = vl & (LA - 1);
                     const bool sv = slot < cnt;
-                    const int k = sv ? S.act[a0 + slot] : 0;
+                    const int k = sv ? act[a0 + slot] : 0;
                     // exchange slots [2][3][96] (sin, q . p, cos): the FP32
                     // pass's lists, which are idle until the next block time
                     double *xch = reinterpret_cast<double *>(S.need);
@@ -981,7 +1080,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 } else if (warp == 7) {
                     double aj[6] = {0, 0, 0, 0, 0, 0};
                     if (with_star && wl < cnt)
-                        herm_item(S, S.act[a0 + s0 + wl], npart, mlo, npart, true, gm0, tc, h.eps2,
+                        herm_item(S, act[a0 + s0 + wl], npart, mlo, npart, true, gm0, tc, h.eps2,
                                   f32, rcf, aj);
 #pragma unroll
                     for (int c = 0; c < 6; ++c) prb[c * HTHREADS + tid] = aj[c];
@@ -989,29 +1088,33 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 if (COOP) {
                     // This CTA's part of every (member, component): its LA lanes
                     // summed by a group of eight lanes in a fixed order (plus the
-                    // star's pull on rank 0), stored by lane g into CTA g's
-                    // receive buffer under this rank; after the cluster barrier
-                    // every CTA adds the CTAs' parts in rank order. Receive
-                    // buffers are double-buffered: a CTA stores into this one
-                    // again only after the next round's cluster barrier, which
-                    // every CTA passes after reading it.
+                    // star's pull on rank 0), sent by lane g into CTA g's
+                    // receive buffer under this rank; when all CTAs' parts are
+                    // there every CTA adds them in rank order. Receive buffers
+                    // are double-buffered: a CTA sends into this one again only
+                    // when it has the next round's parts of every CTA, which
+                    // that CTA sends after it has read this one (and announced
+                    // this round's bytes).
                     __syncthreads();
+                    if (tid == HTHREADS - 1) rbar_expect(buf, CLT * 6 * cnt * (int)sizeof(double));
                     double *rbb = S.rb + buf * (CLT * 6 * RSL);
                     const int g = wl & 7;
                     for (int pi0 = warp * 4; pi0 < 6 * cnt; pi0 += HTHREADS / 8) {
                         const int pi = pi0 + (wl >> 3);
                         const bool live = pi < 6 * cnt;
                         const int sl = pi / 6, c = pi - 6 * sl;
-                        double v = 0.0;
+                        const double *col = prb + c * HTHREADS + (sl << las);
+                        double v = live && g < LA ? col[g] : 0.0;
                         if (live)
-                            for (int m = g; m < LA; m += 8) v += prb[c * HTHREADS + sl * LA + m];
+                            for (int m = g + 8; m < LA; m += 8) v += col[m];
                         v += __shfl_xor_sync(0xffffffffu, v, 1);
                         v += __shfl_xor_sync(0xffffffffu, v, 2);
                         v += __shfl_xor_sync(0xffffffffu, v, 4);
                         if (live && with_star) v += prb[c * HTHREADS + 224 + sl];
-                        if (live && g < CLT) cl.map_shared_rank(rbb, g)[(rank * 6 + c) * RSL + sl] = v;
+                        if (live && g < CLT) rbar_send(rbb + (rank * 6 + c) * RSL + sl, v, g, buf);
                     }
-                    cl.sync();
+                    if (warp < 4 && wl < 3 * nc) item.fetch(S, warp, act + a0, wl);
+                    if (!rbar_wait(buf, par)) lost = true;
                     // pairwise tree over CLT lanes: rank r with rank r + w, halving w
                     for (int t0 = warp * 32; t0 < 6 * cnt * CLT; t0 += HTHREADS) {
                         const int t = t0 + wl, pi = t / CLT, r = t % CLT;
@@ -1021,16 +1124,18 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                         for (int w = CLT / 2; w >= 1; w >>= 1) v += __shfl_xor_sync(0xffffffffu, v, w);
                         if (pi < 6 * cnt && r == 0) S.a1s[c * ACH + s0 + sl] = v;
                     }
+                    par ^= buf;
                     buf ^= 1;
                 } else {
+                    if (warp < 4 && wl < 3 * nc) item.fetch(S, warp, act + a0, wl);
                     __syncthreads();
                     // sums over the LA lanes of each (member, component), one
                     // warp each, in a fixed order
                     for (int pi = warp; pi < 6 * cnt; pi += HTHREADS / 32) {
                         const int sl = pi / 6, c = pi - 6 * sl;
-                        const double *col = prb + c * HTHREADS + sl * LA;
-                        double v = 0.0;
-                        for (int m = wl; m < LA; m += 32) v += col[m];
+                        const double *col = prb + c * HTHREADS + (sl << las);
+                        double v = wl < LA ? col[wl] : 0.0;
+                        for (int m = wl + 32; m < LA; m += 32) v += col[m];
                         for (int off = (LA < 32 ? LA : 32) >> 1; off > 0; off >>= 1)
                             v += __shfl_xor_sync(0xffffffffu, v, off);
                         if (wl == 0) S.a1s[c * ACH + s0 + sl] = v + prb[c * HTHREADS + 224 + sl];
@@ -1045,25 +1150,16 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // criterion's inputs are there, and finds the next block time.
             // (One warp per coordinate with a2 and a3 first took eight instructions to
             // the criterion and twelve to the state.)
-            constexpr int LS = KMAX + 1;
             if (warp < 4) {
                 const int f = warp;
-                const double *cd = S.lvt + 3 * f * LS;
-                const double *c1 = cd + (f == LF_A3 ? LS : 2 * LS);
                 for (int it = wl; it < 3 * nc; it += 32) {
-                    const int sl = it / 3, c = it - 3 * sl;
-                    const int k = S.act[a0 + sl], o = c * HCAP + k;
-                    const int lv = S.lev[k];
-                    const double d = S.ax[o] - S.a1s[c * ACH + sl];
-                    const double base = f == LF_X ? S.ex[o] : (f == LF_V ? S.eu[o] : 0.0);
-                    const double r = fma(
-                        cd[lv], d,
-                        fma(cd[LS + lv], S.jx[o], fma(c1[lv], S.a1s[(3 + c) * ACH + sl], base)));
+                    if (it >= 32) item.fetch(S, f, act + a0, it);
+                    const double r = item.value(S);
                     if (f < LF_A2) {
-                        S.x[3 * f * HCAP + o] = r;
-                        S.f[3 * f * HCAP + o] = to_float_scaled(r, 0);
+                        S.x[3 * f * HCAP + item.o] = r;
+                        S.f[3 * f * HCAP + item.o] = to_float_scaled(r, 0);
                     } else {
-                        S.cf[(3 * f + c) * ACH + sl] = to_float_scaled(r, -f * lv);
+                        S.cf[3 * f * ACH + item.s] = to_float_scaled(r, -f * item.lv);
                     }
                 }
                 __syncwarp();
@@ -1079,7 +1175,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     const int it = q * 32 + wl, sl = it / 3, c = it - 3 * sl;
                     oo[q] = -1;
                     if (it >= 3 * nc) continue;
-                    const int k = S.act[a0 + sl];
+                    const int k = act[a0 + sl];
                     const double r = S.a1s[(3 * f + c) * ACH + sl];
                     oo[q] = c * HCAP + k;
                     fv[q] = to_float_scaled(r, 0);
@@ -1098,30 +1194,60 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             } else if (warp == 6) {
                 // new time and level by the Aarseth criterion (FP32 on scaled
                 // inputs); a larger step only by one level and on a commensurate time
+                // (what does not wait for the inputs is read before they are there)
+                int k = wl < nc ? act[a0 + wl] : 0;
+                int lv = S.lev[k];
+                bool up = (tn & ((1ll << (KMAX + 1 - lv)) - 1)) == 0;
                 asm volatile("bar.sync 5, 224;" ::: "memory");
                 for (int sl = wl; sl < nc; sl += 32) {
-                    const int k = S.act[a0 + sl];
-                    const int lv = S.lev[k];
-                    int kn = level_from(S.cf + sl, lv, etaf, T2f);
-                    if (kn < lv) {
-                        const int up1 = lv - 1;
-                        kn = (tn & ((1ll << (KMAX - up1)) - 1)) == 0 ? up1 : lv;
+                    if (sl >= 32) {
+                        k = act[a0 + sl];
+                        lv = S.lev[k];
+                        up = (tn & ((1ll << (KMAX + 1 - lv)) - 1)) == 0;
                     }
+                    int kn = level_from(S.cf + sl, lv, etaf, T2s);
+                    if (kn < lv) kn = up ? lv - 1 : lv;
                     S.lev[k] = kn;
                     S.ti[k] = tn;
+                    lmax = max(lmax, kn);
                 }
-                __syncwarp();
+                mk = k;
             }
             if (a0 + ACH < na) __syncthreads();  // the next round's sums and derivatives
         }
-        // every thread read (tn, na) before the barriers above; the active
-        // list is no longer read in this block step
-        if (warp == 6) next_block(S.lev, S.ti, S.act, n);
+        // the next block time: the earliest of the others' and of the members that
+        // moved now, the ends of whose steps are their levels' (every thread read
+        // (tn, na) before the barriers above)
+        if (warp == 6) {
+            const int deep = __reduce_max_sync(0xffffffffu, lmax);
+            const long long tm = tn + (1ll << (KMAX - deep));
+            const long long t = min(tm, nb.t);
+            int nn = nb.t == t ? nb.na : 0;
+            if (tm == t && na <= 32) {
+                const bool f = lmax == deep;
+                const unsigned m = __ballot_sync(0xffffffffu, f);
+                if (f) nact[nn + __popc(m & ((1u << wl) - 1u))] = (uint16_t)mk;
+                nn += __popc(m);
+            } else if (tm == t) {
+                __syncwarp();
+                for (int b0 = 0; b0 < na; b0 += 32) {
+                    const int k = b0 + wl < na ? act[b0 + wl] : -1;
+                    const bool f = k >= 0 && S.lev[k] == deep;
+                    const unsigned m = __ballot_sync(0xffffffffu, f);
+                    if (f) nact[nn + __popc(m & ((1u << wl) - 1u))] = (uint16_t)k;
+                    nn += __popc(m);
+                }
+            }
+            if (wl == 0) {
+                g_tn = lost ? LLONG_MAX : t;  // (ends the set)
+                g_na = nn;
+            }
+        }
         ++steps;
     }
     // peers may still read this CTA's partial sums of the last round
     if (COOP) cl.sync(); else __syncthreads();
-    if (capped && tid == 0 && rank == 0) atomicOr(d.status, QYM_ST_HERMITE_CAP);
+    if ((capped && tid == 0 && rank == 0) || lost) atomicOr(d.status, QYM_ST_HERMITE_CAP);
     // item 7: pre-remove the (1-K) part of the coming kick at q1 (own members)
     for (int k = tid; k < n; k += blockDim.x) {
         S.ex[k] = S.x[k]; S.ey[k] = S.y[k]; S.ez[k] = S.z[k];
