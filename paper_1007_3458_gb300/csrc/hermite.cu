@@ -266,6 +266,7 @@ __device__ __forceinline__ int lanes_per_member(int n, int partners) {
 }
 
 __device__ __forceinline__ void group_sum(double *v, int cnt, int P) {
+    #pragma unroll 1
     for (int off = P >> 1; off > 0; off >>= 1)
         for (int c = 0; c < cnt; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], off);
 }
@@ -276,6 +277,7 @@ __device__ __forceinline__ void group_sum(double *v, int cnt, int P) {
 __device__ void kcorr_part(const HermSmem &S, int lo, int hi, int k, int l0, int P,
                            const TransC &tc, double *c) {
     c[0] = c[1] = c[2] = 0.0;
+    #pragma unroll 1
     for (int l = lo + l0; l < hi; l += P) {
         if (l == k) continue;
         double qx = S.ex[k] - S.ex[l], qy = S.ey[k] - S.ey[l], qz = S.ez[k] - S.ez[l];
@@ -311,6 +313,7 @@ __device__ void herm_part(const HermSmem &S, int lo, int hi, int k, int l0, int 
         aj[0] = c * xk; aj[1] = c * yk; aj[2] = c * zk;
         aj[3] = c * (uk - t * xk); aj[4] = c * (vk - t * yk); aj[5] = c * (wk - t * zk);
     }
+    #pragma unroll 1
     for (int l = lo + l0; l < hi; l += P) {
         if (l == k) continue;
         double qx = xk - S.ex[l], qy = yk - S.ey[l], qz = zk - S.ez[l];
@@ -605,6 +608,7 @@ __device__ __forceinline__ void rbar_send(double *p, double v, int r, int b) {
 }
 // waits for the phase of the given parity; false when it does not end in a second or so
 __device__ __forceinline__ bool rbar_wait(int b, int parity) {
+    #pragma unroll 1
     for (int i = 0; i < (1 << 20); ++i) {
         unsigned done;
         asm volatile(
@@ -631,26 +635,24 @@ __shared__ int g_nneed;  // members of the FP32-screened list
 
 // The earliest end of a member's step later than `after`, and the members whose step
 // ends then, listed in member order in act, by one warp (LLONG_MAX and none when no
-// step ends later). The end times stay in registers between the two passes; the
-// minimum (below 2^49) is taken as the minimum of the high words, then of the low
-// words among the lanes that hold it.
+// step ends later). The minimum (below 2^49) is taken as the minimum of the high words,
+// then of the low words among the lanes that hold it.
 struct Block {
     long long t;
     int na;
 };
-template <int NI>
-__device__ __forceinline__ Block next_block_of(const int32_t *lev, const long long *ti,
-                                               uint16_t *act, int n, long long after) {
+__device__ __forceinline__ long long step_end(const int32_t *lev, const long long *ti, int k,
+                                              int n, long long after) {
+    const long long te = k < n ? ti[k] + (1ll << (KMAX - lev[k])) : LLONG_MAX;
+    return te > after ? te : LLONG_MAX;
+}
+__device__ __forceinline__ Block next_block(const int32_t *lev, const long long *ti,
+                                            uint16_t *act, int n, long long after) {
     const int wl = threadIdx.x & 31;
-    long long te[NI];
-    long long t = LLONG_MAX;
-#pragma unroll
-    for (int q = 0; q < NI; ++q) {
-        const int k = q * 32 + wl;
-        te[q] = (k < n) ? ti[k] + (1ll << (KMAX - lev[k])) : LLONG_MAX;
-        if (te[q] <= after) te[q] = LLONG_MAX;
-        t = min(t, te[q]);
-    }
+    const long long t0 = step_end(lev, ti, wl, n, after);
+    long long t = t0;
+#pragma unroll 1
+    for (int k = 32 + wl; k - wl < n; k += 32) t = min(t, step_end(lev, ti, k, n, after));
     const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(t >> 32));
     const unsigned lo =
         __reduce_min_sync(0xffffffffu, (unsigned)(t >> 32) == hi ? (unsigned)t : 0xffffffffu);
@@ -658,30 +660,26 @@ __device__ __forceinline__ Block next_block_of(const int32_t *lev, const long lo
     b.t = (long long)(((unsigned long long)hi << 32) | lo);
     b.na = 0;
     if (b.t == LLONG_MAX) return b;
-#pragma unroll
-    for (int q = 0; q < NI; ++q) {
-        if (q * 32 >= n) break;
-        const bool f = te[q] == b.t;
-        const unsigned m = __ballot_sync(0xffffffffu, f);
-        if (f) act[b.na + __popc(m & ((1u << wl) - 1u))] = (uint16_t)(q * 32 + wl);
+    t = t0;
+#pragma unroll 1
+    for (int k = wl;;) {
+        const unsigned m = __ballot_sync(0xffffffffu, t == b.t);
+        if (t == b.t) act[b.na + __popc(m & ((1u << wl) - 1u))] = (uint16_t)k;
         b.na += __popc(m);
+        k += 32;
+        if (k - wl >= n) return b;
+        t = step_end(lev, ti, k, n, after);
     }
-    return b;
-}
-
-// (most sets have at most 64 members: two rounds instead of ten)
-__device__ __forceinline__ Block next_block(const int32_t *lev, const long long *ti,
-                                            uint16_t *act, int n, long long after) {
-    return n <= 64 ? next_block_of<2>(lev, ti, act, n, after)
-                   : next_block_of<HCAP / 32>(lev, ti, act, n, after);
 }
 
 // Copy the member range [lo, hi) of arrays a..: from CTA `r` of the cluster
 // into this CTA's shared memory.
 __device__ __forceinline__ void pull_range(cg::cluster_group &cl, const HermSmem &S, int r,
                                            int lo, int hi, double *const *arrs, int narr) {
+    #pragma unroll 1
     for (int q = 0; q < narr; ++q) {
         const double *src = cl.map_shared_rank(arrs[q], r);
+        #pragma unroll 1
         for (int k = lo + threadIdx.x; k < hi; k += blockDim.x) arrs[q][k] = src[k];
     }
 }
@@ -708,6 +706,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     if (n > HCAP || st + n > d.max_members) {
         if (tid == 0 && rank == 0) atomicOr(d.status, QYM_ST_SET_OVERFLOW);
         if (rank == 0)
+            #pragma unroll 1
             for (int k = tid; k < n && st + k < d.max_members; k += blockDim.x)
                 d.uf[d.set_mem[st + k]] = -1;
         return;
@@ -716,6 +715,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     // members only leave the union-find
     if (d.wh_flag && d.wh_flag[d.sys_of[d.set_mem[st]]]) {
         if (rank == 0)
+            #pragma unroll 1
             for (int k = tid; k < n; k += blockDim.x) d.uf[d.set_mem[st + k]] = -1;
         return;
     }
@@ -729,6 +729,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const int grp = tid / P, lane = tid % P;
     // members in ascending row order (rank sort)
     __syncthreads();
+    #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) S.ids[k] = d.set_mem[st + k];
     __syncthreads();
     int myid[HCAP / HTHREADS], myrank[HCAP / HTHREADS];
@@ -737,6 +738,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         myid[c] = k < n ? S.ids[k] : 0;
         int rk = 0;
         if (k < n)
+            #pragma unroll 1
             for (int l = 0; l < n; ++l) rk += S.ids[l] < myid[c];
         myrank[c] = rk;
     }
@@ -751,6 +753,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const TransC tc(d.rcrit[set]);
     const double tau = h.tau;
     // state entering the Kepler drift (after the first kick)
+    #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) {
         int64_t r = S.ids[k];
         S.ex[k] = S.x[k] = d.q[r];
@@ -763,6 +766,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     }
     __syncthreads();
     // item 5: remove the (1-K) part of the first kick (own members)
+    #pragma unroll 1
     for (int k0 = mlo; k0 < mhi; k0 += NG) {
         int k = k0 + grp;
         double c[3] = {0.0, 0.0, 0.0};
@@ -777,12 +781,14 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     if (COOP) {
         cl.sync();
         double *const arr[3] = {S.u, S.v, S.w};
+        #pragma unroll 1
         for (int r = 0; r < cs; ++r)
             if (r != rank) pull_range(cl, S, r, n * r / cs, n * (r + 1) / cs, arr, 3);
         cl.sync();
     } else {
         __syncthreads();
     }
+    #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) {
         S.eu[k] = S.u[k]; S.ev[k] = S.v[k]; S.ew[k] = S.w[k];
     }
@@ -793,6 +799,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const long long TT = 1ll << KMAX;
     const double tick = T / (double)TT;
     const double inv_T = 1.0 / T;
+    #pragma unroll 1
     for (int k0 = mlo; k0 < mhi; k0 += NG) {
         int k = k0 + grp;
         double aj[6] = {0, 0, 0, 0, 0, 0};
@@ -810,11 +817,13 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     if (COOP) {
         cl.sync();
         double *const arr[6] = {S.ax, S.ay, S.az, S.jx, S.jy, S.jz};
+        #pragma unroll 1
         for (int r = 0; r < cs; ++r) {
             if (r == rank) continue;
             const int lo = n * r / cs, hi = n * (r + 1) / cs;
             pull_range(cl, S, r, lo, hi, arr, 6);
             const int32_t *pl = cl.map_shared_rank(S.lev, r);
+            #pragma unroll 1
             for (int k = lo + tid; k < hi; k += blockDim.x) {
                 S.lev[k] = pl[k];
                 S.ti[k] = 0;
@@ -853,7 +862,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     // FP32 copies of the start-up state; the corrector's constants per level
     // (products with powers of two, so the table holds the same values)
     __syncthreads();
+    #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) store_f32(S, k);
+    #pragma unroll 1
     for (int lv = tid; lv <= KMAX; lv += blockDim.x) {
         double *L = S.lvt + lv;
         constexpr int LS = KMAX + 1;
@@ -908,7 +919,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         const int32_t *list = nullptr;
         int np = npart + na;
         if (f32) {
+            #pragma unroll 1
             for (int k = tid; k < n; k += HTHREADS) S.need[k] = 0;
+            #pragma unroll 1
             for (int i = tid; i < npart + na; i += HTHREADS) {
                 int k = mlo + i;
                 if (i >= npart) {
@@ -920,7 +933,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             __syncthreads();
             // members needed in FP64: the active ones and the partners that
             // maybe_near does not rule out for some active member
+            #pragma unroll 1
             for (int i = tid; i < na; i += HTHREADS) S.need[act[i]] = 1;
+            #pragma unroll 1
             for (int p = tid; p < na * npart; p += HTHREADS) {
                 const int ia = p / npart, l = mlo + (p - ia * npart);
                 const int k = act[ia];
@@ -930,6 +945,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // listed in member order by one warp
             if (warp == 0) {
                 int nn = 0;
+                #pragma unroll 1
                 for (int k0 = 0; k0 < n; k0 += 32) {
                     const int k = k0 + wl;
                     const bool f = k < n && S.need[k] != 0;
@@ -943,6 +959,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             list = S.nl;
             np = g_nneed;
         }
+        #pragma unroll 1
         for (int pq = pq0; (pq >> 1) * 32 < 3 * np; pq += HTHREADS / 32) {
             const int it = (pq >> 1) * 32 + wl, i = it / 3, c = it - 3 * i;
             if (i >= np) continue;
@@ -967,6 +984,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         int lmax = -1;  // (warp 6) the deepest new level, and
         int mk = 0;     // the lane's member when at most 32 move
         if (warp == 6) nb = next_block(S.lev, S.ti, nact, n, tn);
+        #pragma unroll 1
         for (int a0 = 0; a0 < na; a0 += ACH) {
             const int nc = min(ACH, na - a0);
             // pair items on warps 0-6 (LA lanes per member), the star's pull
@@ -981,6 +999,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             const bool paired = nc <= NP;
             const int NR = paired ? nc : NU;
             CorrItem item;  // (warps 0-3)
+            #pragma unroll 1
             for (int s0 = 0; s0 < nc; s0 += NR) {
                 const int cnt = min(NR, nc - s0);
                 double *prb = S.pr;
@@ -990,6 +1009,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                         const int slot = s0 + (tid >> las), la = tid & (LA - 1);
                         if (slot < s0 + cnt) {
                             const int k = act[a0 + slot];
+                            #pragma unroll 1
                             for (int it = la; it < npart; it += LA)
                                 herm_item(S, k, it, mlo, npart, false, gm0, tc, h.eps2, f32, rcf, aj);
                         }
@@ -1009,6 +1029,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     double *xch = reinterpret_cast<double *>(S.need);
                     double acc[3] = {0.0, 0.0, 0.0};
                     int par = 0;
+                    #pragma unroll 1
                     for (int it0 = 0; it0 < npart; it0 += LA) {
                         const int l = mlo + it0 + la;
                         double *xs = xch + par * (3 * 96);
@@ -1099,6 +1120,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     if (tid == HTHREADS - 1) rbar_expect(buf, CLT * 6 * cnt * (int)sizeof(double));
                     double *rbb = S.rb + buf * (CLT * 6 * RSL);
                     const int g = wl & 7;
+                    #pragma unroll 1
                     for (int pi0 = warp * 4; pi0 < 6 * cnt; pi0 += HTHREADS / 8) {
                         const int pi = pi0 + (wl >> 3);
                         const bool live = pi < 6 * cnt;
@@ -1106,6 +1128,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                         const double *col = prb + c * HTHREADS + (sl << las);
                         double v = live && g < LA ? col[g] : 0.0;
                         if (live)
+                            #pragma unroll 1
                             for (int m = g + 8; m < LA; m += 8) v += col[m];
                         v += __shfl_xor_sync(0xffffffffu, v, 1);
                         v += __shfl_xor_sync(0xffffffffu, v, 2);
@@ -1116,6 +1139,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     if (warp < 4 && wl < 3 * nc) item.fetch(S, warp, act + a0, wl);
                     if (!rbar_wait(buf, par)) lost = true;
                     // pairwise tree over CLT lanes: rank r with rank r + w, halving w
+                    #pragma unroll 1
                     for (int t0 = warp * 32; t0 < 6 * cnt * CLT; t0 += HTHREADS) {
                         const int t = t0 + wl, pi = t / CLT, r = t % CLT;
                         const int sl = pi / 6, c = pi - 6 * sl;
@@ -1131,11 +1155,14 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     __syncthreads();
                     // sums over the LA lanes of each (member, component), one
                     // warp each, in a fixed order
+                    #pragma unroll 1
                     for (int pi = warp; pi < 6 * cnt; pi += HTHREADS / 32) {
                         const int sl = pi / 6, c = pi - 6 * sl;
                         const double *col = prb + c * HTHREADS + (sl << las);
                         double v = wl < LA ? col[wl] : 0.0;
+                        #pragma unroll 1
                         for (int m = wl + 32; m < LA; m += 32) v += col[m];
+                        #pragma unroll 1
                         for (int off = (LA < 32 ? LA : 32) >> 1; off > 0; off >>= 1)
                             v += __shfl_xor_sync(0xffffffffu, v, off);
                         if (wl == 0) S.a1s[c * ACH + s0 + sl] = v + prb[c * HTHREADS + 224 + sl];
@@ -1152,6 +1179,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // the criterion and twelve to the state.)
             if (warp < 4) {
                 const int f = warp;
+                #pragma unroll 1
                 for (int it = wl; it < 3 * nc; it += 32) {
                     if (it >= 32) item.fetch(S, f, act + a0, it);
                     const double r = item.value(S);
@@ -1199,6 +1227,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 int lv = S.lev[k];
                 bool up = (tn & ((1ll << (KMAX + 1 - lv)) - 1)) == 0;
                 asm volatile("bar.sync 5, 224;" ::: "memory");
+                #pragma unroll 1
                 for (int sl = wl; sl < nc; sl += 32) {
                     if (sl >= 32) {
                         k = act[a0 + sl];
@@ -1230,6 +1259,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 nn += __popc(m);
             } else if (tm == t) {
                 __syncwarp();
+                #pragma unroll 1
                 for (int b0 = 0; b0 < na; b0 += 32) {
                     const int k = b0 + wl < na ? act[b0 + wl] : -1;
                     const bool f = k >= 0 && S.lev[k] == deep;
@@ -1249,10 +1279,12 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     if (COOP) cl.sync(); else __syncthreads();
     if ((capped && tid == 0 && rank == 0) || lost) atomicOr(d.status, QYM_ST_HERMITE_CAP);
     // item 7: pre-remove the (1-K) part of the coming kick at q1 (own members)
+    #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) {
         S.ex[k] = S.x[k]; S.ey[k] = S.y[k]; S.ez[k] = S.z[k];
     }
     __syncthreads();
+    #pragma unroll 1
     for (int k0 = mlo; k0 < mhi; k0 += NG) {
         int k = k0 + grp;
         double c[3] = {0.0, 0.0, 0.0};
