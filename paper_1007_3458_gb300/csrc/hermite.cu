@@ -28,6 +28,7 @@
 
 #include <cooperative_groups.h>
 
+#include "pair64.cuh"
 #include "qym_internal.cuh"
 
 namespace qym {
@@ -108,7 +109,7 @@ struct TransC {
     double c;    // (pi / 2) a: K' = c cos, K'' = -c^2 sin
     double nc2;  // -c^2
     __device__ __forceinline__ explicit TransC(double rc)
-        : rc2(rc * rc), a(1.1 / rc), c(0.5 * kPi * (1.1 / rc)), nc2(-c * c) {}
+        : rc2(rc * rc), a(1.1 / rc), c(0.5 * kPi * a), nc2(-c * c) {}
 };
 
 // the transition's argument y = 1.1 s / r_crit - 0.1
@@ -243,16 +244,27 @@ static_assert(2 * 3 * 96 * sizeof(double) <= (4 * HCAP - 64) * sizeof(int32_t),
 // for the variables below)
 static_assert(2 * (kHermSmem + 128 + 1024) <= 228 * 1024, "Hermite shared memory above two CTAs per SM");
 
-// smallest k with T 2^-k <= dt_c, in [0, KMAX]: with T = fT 2^eT and
-// dt_c = fd 2^ed (fT, fd in [1/2, 1)), T 2^-k <= dt_c exactly when
-// k >= eT - ed + (fT > fd)
-__device__ __forceinline__ int level_of(double dt_c, double T) {
-    if (!(dt_c > 0.0)) return KMAX;
-    if (dt_c >= T) return 0;
+// The start-up level, the smallest k in [0, KMAX] with T 2^-k <= eta_s |a| / |adot|,
+// from the squares (no square root and one reciprocal): T^2 4^-k <= d2 with
+// T^2 = fT 2^eT and d2 = fd 2^ed (fT, fd in [1/2, 1)) holds exactly when
+// 2 k >= eT - ed + (fT > fd). T when the jerk is zero.
+__device__ __forceinline__ int first_level(const double *aj, double eta_s, double T2, double T) {
+    const double a2 = fma(aj[0], aj[0], fma(aj[1], aj[1], aj[2] * aj[2]));
+    const double j2 = fma(aj[3], aj[3], fma(aj[4], aj[4], aj[5] * aj[5]));
+    if (!(j2 > 0.0)) return 0;
+    const double d2 = (eta_s * eta_s) * (a2 * p64::rcp(j2));
+    if (!p64::mid_range(d2) || !p64::mid_range(T2)) {
+        // (out of the squares' range)
+        const double dt = eta_s * sqrt(a2) / sqrt(j2);
+        if (!(dt > 0.0)) return KMAX;
+        int eT, ed;
+        const double fT = frexp(T, &eT), fd = frexp(dt, &ed);
+        return dt >= T ? 0 : min(max(eT - ed + (fT > fd ? 1 : 0), 0), KMAX);
+    }
     int eT, ed;
-    const double fT = frexp(T, &eT), fd = frexp(dt_c, &ed);
-    const int k = eT - ed + (fT > fd ? 1 : 0);
-    return k < 0 ? 0 : (k > KMAX ? KMAX : k);
+    const double fT = frexp(T2, &eT), fd = frexp(d2, &ed);
+    const int k2 = eT - ed + (fT > fd ? 1 : 0);
+    return min(max((k2 + 1) >> 1, 0), KMAX);
 }
 
 // Work split inside a CTA: each member of a group of n is handled by P
@@ -274,7 +286,7 @@ __device__ __forceinline__ void group_sum(double *v, int cnt, int P) {
 // partial (1-K)-weighted pair acceleration of member k at the evaluation
 // point, unsmoothed (the kick used the bare separation):
 // sum_l -G m_l q_kl / q^3 [1 - K + q K'] over the partners of this lane
-__device__ void kcorr_part(const HermSmem &S, int lo, int hi, int k, int l0, int P,
+__device__ __forceinline__ void kcorr_part(const HermSmem &S, int lo, int hi, int k, int l0, int P,
                            const TransC &tc, double *c) {
     c[0] = c[1] = c[2] = 0.0;
     #pragma unroll 1
@@ -294,25 +306,30 @@ __device__ void kcorr_part(const HermSmem &S, int lo, int hi, int k, int l0, int
     }
 }
 
-// partial Hermite acceleration and jerk of member k at the evaluation point
-// (Sec. 2.2): with `star`, the star term on lane 0 of the group; the pair
-// terms with the transition bracket over this lane's partners (one
-// reciprocal square root per pair: q = q2 / sqrt(q2), 1/q^3, 1/q^2)
-__device__ void herm_part(const HermSmem &S, int lo, int hi, int k, int l0, int P, bool star,
-                          double gm0, const TransC &tc, double eps2, double *aj) {
+// the star's pull on member k at the evaluation point, fixed at the origin: a, adot
+__device__ __forceinline__ void star_pull(const HermSmem &S, int k, double gm0, double eps2,
+                                          double *aj) {
+    const double xk = S.ex[k], yk = S.ey[k], zk = S.ez[k];
+    const double uk = S.eu[k], vk = S.ev[k], wk = S.ew[k];
+    const double s2 = xk * xk + yk * yk + zk * zk + eps2;
+    const double si = rsqrt(s2);
+    const double si2 = si * si;
+    const double rv = xk * uk + yk * vk + zk * wk;
+    const double c = gm0 * (si2 * si);
+    const double t = 3.0 * rv * si2;
+    aj[0] += c * xk; aj[1] += c * yk; aj[2] += c * zk;
+    aj[3] += c * (uk - t * xk); aj[4] += c * (vk - t * yk); aj[5] += c * (wk - t * zk);
+}
+
+// partial Hermite acceleration and jerk of member k at the evaluation
+// point (Sec. 2.2): the pair terms with the transition bracket over this
+// lane's partners (one reciprocal square root per pair: q = q2 / sqrt(q2),
+// 1/q^3, 1/q^2)
+__device__ __forceinline__ void herm_part(const HermSmem &S, int lo, int hi, int k, int l0, int P,
+                                          const TransC &tc, double eps2, double *aj) {
     const double xk = S.ex[k], yk = S.ey[k], zk = S.ez[k];
     const double uk = S.eu[k], vk = S.ev[k], wk = S.ew[k];
     for (int c = 0; c < 6; ++c) aj[c] = 0.0;
-    if (star && l0 == 0) {  // star, fixed at the origin
-        double s2 = xk * xk + yk * yk + zk * zk + eps2;
-        double si = rsqrt(s2);
-        double si2 = si * si;
-        double rv = xk * uk + yk * vk + zk * wk;
-        double c = gm0 * (si2 * si);
-        double t = 3.0 * rv * si2;
-        aj[0] = c * xk; aj[1] = c * yk; aj[2] = c * zk;
-        aj[3] = c * (uk - t * xk); aj[4] = c * (vk - t * yk); aj[5] = c * (wk - t * zk);
-    }
     #pragma unroll 1
     for (int l = lo + l0; l < hi; l += P) {
         if (l == k) continue;
@@ -539,20 +556,12 @@ __device__ __forceinline__ void herm_item(const HermSmem &S, int k, int item, in
                                           bool star, double gm0, const TransC &tc, double eps2,
                                           bool f32, float rcf, double *aj) {
     if (item < npart && (mlo + item == k || (f32 && !maybe_near(S, k, mlo + item, rcf)))) return;
-    const double xk = S.ex[k], yk = S.ey[k], zk = S.ez[k];
-    const double uk = S.eu[k], vk = S.ev[k], wk = S.ew[k];
     if (item == npart) {
-        if (!star) return;
-        double s2 = xk * xk + yk * yk + zk * zk + eps2;
-        double si = rsqrt(s2);
-        double si2 = si * si;
-        double rv = xk * uk + yk * vk + zk * wk;
-        double c = gm0 * (si2 * si);
-        double t = 3.0 * rv * si2;
-        aj[0] += c * xk; aj[1] += c * yk; aj[2] += c * zk;
-        aj[3] += c * (uk - t * xk); aj[4] += c * (vk - t * yk); aj[5] += c * (wk - t * zk);
+        if (star) star_pull(S, k, gm0, eps2, aj);
         return;
     }
+    const double xk = S.ex[k], yk = S.ey[k], zk = S.ez[k];
+    const double uk = S.eu[k], vk = S.ev[k], wk = S.ew[k];
     const int l = mlo + item;
     const double qx = xk - S.ex[l], qy = yk - S.ey[l], qz = zk - S.ez[l];
     const double q2 = pair_q2(qx, qy, qz, eps2);
@@ -727,6 +736,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const int P = lanes_per_member(mhi - mlo, n);
     const int NG = HTHREADS / P;
     const int grp = tid / P, lane = tid % P;
+    const int64_t star_row = d.offsets[d.sys_of[d.set_mem[st]]];
+    const double gm0 = -h.G * d.m[star_row], rcrit = d.rcrit[set];
+    const TransC tc(rcrit);
     // members in ascending row order (rank sort)
     __syncthreads();
     #pragma unroll 1
@@ -738,7 +750,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         myid[c] = k < n ? S.ids[k] : 0;
         int rk = 0;
         if (k < n)
-            #pragma unroll 1
+            #pragma unroll 4
             for (int l = 0; l < n; ++l) rk += S.ids[l] < myid[c];
         myrank[c] = rk;
     }
@@ -748,9 +760,6 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         if (k < n) S.ids[myrank[c]] = myid[c];
     }
     __syncthreads();
-    const int64_t star_row = d.offsets[d.sys_of[S.ids[0]]];
-    const double gm0 = -h.G * d.m[star_row];
-    const TransC tc(d.rcrit[set]);
     const double tau = h.tau;
     // state entering the Kepler drift (after the first kick)
     #pragma unroll 1
@@ -798,21 +807,59 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const double T = fabs(tau);
     const long long TT = 1ll << KMAX;
     const double tick = T / (double)TT;
-    const double inv_T = 1.0 / T;
-    #pragma unroll 1
-    for (int k0 = mlo; k0 < mhi; k0 += NG) {
-        int k = k0 + grp;
+    const double T2d = T * T;
+    // The star's pull has lanes of its own (half the CTA at a time, its sums in the
+    // slots of the block steps' partials), and warp 7 sets up the corrector's constants
+    // per level meanwhile (products with powers of two): on one lane group the star's
+    // pull, the pairs' and the levels' square roots and division are one chain of FP64
+    // instructions, and scalars that every warp computes take the sub-partitions' FP64
+    // units eight times.
+    const int warp = tid >> 5, wl = tid & 31;
+    if (warp == 7) {
+        const double inv_T = 1.0 / T, iT2 = inv_T * inv_T, T3 = T2d * T;
+#pragma unroll 1
+        for (int lv = wl; lv <= KMAX; lv += 32) {
+            constexpr int LS = KMAX + 1;
+            double *L = S.lvt + lv;
+            const double ih = sgn * inv_T * pow2d(lv), ih2 = iT2 * pow2d(2 * lv);
+            const double hl = sgn * T * pow2d(-lv), h2 = T2d * pow2d(-2 * lv);
+            const double h3 = sgn * T3 * pow2d(-3 * lv);
+            L[(3 * LF_X) * LS] = h2 * (-3.0 / 20.0);
+            L[(3 * LF_X + 1) * LS] = h3 * (-7.0 / 60.0);
+            L[(3 * LF_X + 2) * LS] = h3 * (-1.0 / 30.0);
+            L[(3 * LF_V) * LS] = hl * -0.5;
+            L[(3 * LF_V + 1) * LS] = h2 * (-5.0 / 12.0);
+            L[(3 * LF_V + 2) * LS] = h2 * (-1.0 / 12.0);
+            L[(3 * LF_A2) * LS] = 6.0 * ih2;
+            L[(3 * LF_A2 + 1) * LS] = 2.0 * ih;
+            L[(3 * LF_A2 + 2) * LS] = 4.0 * ih;
+            L[(3 * LF_A3) * LS] = 12.0 * (sgn * (iT2 * inv_T) * pow2d(3 * lv));
+            L[(3 * LF_A3 + 1) * LS] = 6.0 * ih2;
+        }
+    }
+    const int NGS = min(NG, HTHREADS / 2);  // members per round
+#pragma unroll 1
+    for (int k0 = mlo; k0 < mhi; k0 += NGS) {
+        const int k = k0 + grp;
         double aj[6] = {0, 0, 0, 0, 0, 0};
-        if (k < mhi) herm_part(S, 0, n, k, lane, P, true, gm0, tc, h.eps2, aj);
+        const int ks = k0 + tid - HTHREADS / 2;
+        if (ks >= k0 && ks < min(k0 + NGS, mhi)) {
+            star_pull(S, ks, gm0, h.eps2, aj);
+            for (int c = 0; c < 6; ++c) S.pr[c * HTHREADS + ks - k0] = aj[c];
+        }
+        const bool mine = grp < NGS && k < mhi;
+        for (int c = 0; c < 6; ++c) aj[c] = 0.0;
+        if (mine) herm_part(S, 0, n, k, lane, P, tc, h.eps2, aj);
         group_sum(aj, 6, P);
-        if (k < mhi && lane == 0) {
+        __syncthreads();
+        if (mine && lane == 0) {
+            for (int c = 0; c < 6; ++c) aj[c] += S.pr[c * HTHREADS + grp];
             S.ax[k] = aj[0]; S.ay[k] = aj[1]; S.az[k] = aj[2];
             S.jx[k] = aj[3]; S.jy[k] = aj[4]; S.jz[k] = aj[5];
-            double jn = sqrt(aj[3] * aj[3] + aj[4] * aj[4] + aj[5] * aj[5]);
-            double dt_c = jn > 0.0 ? h.eta_s * sqrt(aj[0] * aj[0] + aj[1] * aj[1] + aj[2] * aj[2]) / jn : T;
-            S.lev[k] = level_of(dt_c, T);
+            S.lev[k] = first_level(aj, h.eta_s, T2d, T);
             S.ti[k] = 0;
         }
+        __syncthreads();
     }
     if (COOP) {
         cl.sync();
@@ -837,15 +884,12 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     // the sub-partitions serve in parallel): one warp per coordinate for the
     // predictor and the corrector, several warps per member for the forces,
     // one warp per (member, component) for the sums.
-    const int warp = tid >> 5, wl = tid & 31;
     const double stick = sgn * tick;
-    const double T2d = T * T, T3 = T2d * T;
-    const double iT2 = inv_T * inv_T, iT3 = iT2 * inv_T;
     const T2Split T2s((float)T2d);
     const float etaf = (float)h.eta;
     const float stickf = (float)stick;
-    const TickF tick1(stick), tick3(stick / 3.0);
-    const float rcf = __double2float_ru(d.rcrit[set] * (1.0 + 0x1p-20));
+    const TickF tick1(stick), tick3(stick * (1.0 / 3.0));
+    const float rcf = __double2float_ru(rcrit * (1.0 + 0x1p-20));
     const int npart = mhi - mlo;
     // the largest range of the cluster: every CTA derives its lane layout and
     // its round count from it, so all CTAs pass the same cluster barriers and
@@ -859,30 +903,11 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const int LA = 1 << las;
     const int NU = min(COOP ? RSL : 32, (HTHREADS - 32) >> las);
     const int NP = min(COOP ? RSL : 32, 96 >> las);
-    // FP32 copies of the start-up state; the corrector's constants per level
-    // (products with powers of two, so the table holds the same values)
+    const int N3 = min(COOP ? RSL : 32, 32 >> las);
+    // FP32 copies of the start-up state
     __syncthreads();
     #pragma unroll 1
     for (int k = tid; k < n; k += blockDim.x) store_f32(S, k);
-    #pragma unroll 1
-    for (int lv = tid; lv <= KMAX; lv += blockDim.x) {
-        double *L = S.lvt + lv;
-        constexpr int LS = KMAX + 1;
-        const double ih = sgn * inv_T * pow2d(lv), ih2 = iT2 * pow2d(2 * lv);
-        const double h = sgn * T * pow2d(-lv), h2 = T2d * pow2d(-2 * lv);
-        const double h3 = sgn * T3 * pow2d(-3 * lv);
-        L[(3 * LF_X) * LS] = h2 * (-3.0 / 20.0);
-        L[(3 * LF_X + 1) * LS] = h3 * (-7.0 / 60.0);
-        L[(3 * LF_X + 2) * LS] = h3 * (-1.0 / 30.0);
-        L[(3 * LF_V) * LS] = h * -0.5;
-        L[(3 * LF_V + 1) * LS] = h2 * (-5.0 / 12.0);
-        L[(3 * LF_V + 2) * LS] = h2 * (-1.0 / 12.0);
-        L[(3 * LF_A2) * LS] = 6.0 * ih2;
-        L[(3 * LF_A2 + 1) * LS] = 2.0 * ih;
-        L[(3 * LF_A2 + 2) * LS] = 4.0 * ih;
-        L[(3 * LF_A3) * LS] = 12.0 * (sgn * iT3 * pow2d(3 * lv));
-        L[(3 * LF_A3 + 1) * LS] = 6.0 * ih2;
-    }
     const bool with_star = rank == 0;
     int64_t steps = 0;
     bool capped = false, lost = false;
@@ -995,7 +1020,11 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // of different sub-partitions (pair_bar): the even warp takes sin,
             // q . p and the acceleration, the odd warp cos and the jerk, which
             // shortens each warp's FP64 instruction stream by about a third.
-            // Either way every partial is the same sum in the same order.
+            // When they fit one warp's worth (most block steps: one or two members
+            // move), a pair item runs on three warps: sin, cos, and everything that
+            // needs neither, then one coordinate each; its longest instruction stream
+            // is 34 FP64 instructions against the pair's 47, with the star's pull on
+            // the fourth sub-partition.
             const bool paired = nc <= NP;
             const int NR = paired ? nc : NU;
             CorrItem item;  // (warps 0-3)
@@ -1019,6 +1048,76 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     }
 #pragma unroll
                     for (int c = 0; c < 6; ++c) prb[c * HTHREADS + tid] = aj[c];
+                } else if (nc <= N3) {
+                    if (warp < 3) {
+                        // (LA >= npart: one partner per lane)
+                        const int role = warp, slot = wl >> las, la = wl & (LA - 1);
+                        const int k = slot < cnt ? act[a0 + slot] : 0, l = mlo + la;
+                        // exchange slots [8][32] in place of the idle FP32 lists
+                        double *xs = reinterpret_cast<double *>(S.need) + wl;
+                        bool valid = slot < cnt && la < npart && l != k &&
+                                     (!f32 || maybe_near(S, k, l, rcf));
+                        double qr = 0.0, sq = 0.0;
+                        bool fold = false;
+                        if (valid) {
+                            const double qx = S.ex[k] - S.ex[l];
+                            const double qy = S.ey[k] - S.ey[l];
+                            const double qz = S.ez[k] - S.ez[l];
+                            const double q2 = pair_q2(qx, qy, qz, h.eps2);
+                            valid = !at_least(q2, tc.rc2);  // beyond r_crit: no force, no jerk
+                            if (valid) {
+                                qr = role == 0 ? qx : (role == 1 ? qy : qz);
+                                const double qi = rsqrt(q2);
+                                sq = q2 * qi;
+                                const double y = trans_y(sq, tc);
+                                const bool zero = y_at_most_0(y), one = y_at_least_1(y);
+                                fold = !zero && !one && y_above_half(y);
+                                if (role < 2) {
+                                    // K = 0 (sin 0, cos taken as 0) and 1 outside (0, 1)
+                                    double p = one && role == 0 ? 1.0 : 0.0;
+                                    if (!zero && !one) {
+                                        const HalfPi arg = half_pi_arg(y);
+                                        p = role == 0 ? sin_w(arg) : cos_w(arg);
+                                    }
+                                    xs[32 * role] = p;
+                                } else {
+                                    const double qi2 = qi * qi;
+                                    const double px = S.eu[k] - S.eu[l];
+                                    const double py = S.ev[k] - S.ev[l];
+                                    const double pz = S.ew[k] - S.ew[l];
+                                    const double cl = pair_cl(S.gm[l], qi, qi2);
+                                    xs[32 * 2] = cl;
+                                    xs[32 * 3] = cl * pair_rv(qx, qy, qz, px, py, pz);
+                                    xs[32 * 4] = -3.0 * qi2;
+                                    xs[32 * 5] = px;
+                                    xs[32 * 6] = py;
+                                    xs[32 * 7] = pz;
+                                }
+                            }
+                        }
+                        __syncwarp();
+                        asm volatile("bar.sync 4, 96;" ::: "memory");
+                        double ar = 0.0, jr = 0.0;
+                        if (valid) {
+                            const double sw = xs[0], pc = xs[32];
+                            const double sn = fold ? pc : sw, cs = fold ? sw : pc;
+                            const double br = pair_br(sq, sn, tc.c * cs);
+                            const double cl = xs[32 * 2];
+                            const double cq = xs[32 * 3] * fma(xs[32 * 4], br, tc.nc2 * sn);
+                            const double cb = cl * br;
+                            ar = cb * qr;
+                            jr = fma(cb, xs[32 * (5 + role)], cq * qr);
+                        }
+                        prb[role * HTHREADS + wl] = ar;
+                        prb[(3 + role) * HTHREADS + wl] = jr;
+                    } else if (warp == 7) {
+                        double aj[6] = {0, 0, 0, 0, 0, 0};
+                        if (with_star && wl < cnt)
+                            herm_item(S, act[a0 + s0 + wl], npart, mlo, npart, true, gm0, tc,
+                                      h.eps2, f32, rcf, aj);
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) prb[c * HTHREADS + tid] = aj[c];
+                    }
                 } else if (warp < 6) {
                     const int role = warp & 1, vl = (warp >> 1) * 32 + wl;
                     const int slot = vl >> las, la = vl & (LA - 1);
