@@ -1582,12 +1582,12 @@ cudaError_t hermite_prepare() {
 
 // Cluster size for a batch (qym_params.hermite_cluster; 0 = automatic). One
 // system holds a few sets, and its longest set gains most from spreading its
-// partners over eight SMs (two CTAs per SM). A batch of many systems keeps
-// thousands of sets in flight that share the SMs' FP64 units; there the
-// longest set does best on a cluster of two CTAs, each alone on its SM
-// (measured on the 512-system ensemble: 20.2 ms per step, against 22.7 ms with
-// eight-CTA clusters at two CTAs per SM; the 16384-body disk: 1.38 ms against
-// 1.48 ms the other way round).
+// partners over eight SMs (16384-body disk: 1.38 ms per step against 1.48 ms on
+// two). A batch of many systems keeps thousands of sets in flight, and a set on
+// eight CTAs keeps seven from the queue: two (512-system ensemble: 16.5 ms per
+// step against 16.9-17.2 ms with eight). Either way two CTAs per SM: a CTA's chain
+// keeps its SM's FP64 units busy a third of the time (the ensemble with one per
+// SM: 17.4 ms).
 int hermite_cluster_size(const Dev &d, const qym_params &p) {
     if (p.hermite_cluster == 2 || p.hermite_cluster == 4 || p.hermite_cluster == 8)
         return p.hermite_cluster;
@@ -1603,8 +1603,8 @@ cudaError_t launch_hermite(const Dev &d, const qym_params &p, double tau, cudaSt
     h.tau = tau;
     h.max_steps = p.max_hermite_steps;
     const int cls = hermite_cluster_size(d, p);
-    const int grid = (cls == 2 ? 1 : 2) * 152;  // CTAs per SM x SMs
-    static_assert(2 * 152 / 4 <= kHermMaxClusters && 152 / 2 <= kHermMaxClusters,
+    const int grid = 2 * 152;  // CTAs per SM x SMs
+    static_assert(2 * 152 / 2 <= kHermMaxClusters,
                   "more clusters than plan entries");
     launch_chain(k_hermite_plan, 1, 1024, 0, st, d, grid / cls);
     cudaError_t e = cudaGetLastError();
