@@ -439,18 +439,18 @@ __device__ __forceinline__ double half_of(double v) {
 }
 // Coordinate c of member k predicted from its own time to tn: the position
 // x + h (u + h/2 (a + h/3 j)) or the velocity u + h (a + h/2 j). stick3 = stick / 3
-__device__ __forceinline__ void predict_x(const HermSmem &S, int k, int c, long long tn,
-                                          const TickF &stick, const TickF &stick3) {
+__device__ __forceinline__ double predict_x(const HermSmem &S, int k, int c, long long tn,
+                                            const TickF &stick, const TickF &stick3) {
     const long long dt = tn - S.ti[k];
     const int o = c * HCAP + k;
     const double h3 = ticks_times(dt, stick3), hs = ticks_times(dt, stick);
-    S.ex[o] = fma(hs, fma(half_of(hs), fma(h3, S.jx[o], S.ax[o]), S.u[o]), S.x[o]);
+    return fma(hs, fma(half_of(hs), fma(h3, S.jx[o], S.ax[o]), S.u[o]), S.x[o]);
 }
-__device__ __forceinline__ void predict_v(const HermSmem &S, int k, int c, long long tn,
-                                          const TickF &stick) {
+__device__ __forceinline__ double predict_v(const HermSmem &S, int k, int c, long long tn,
+                                            const TickF &stick) {
     const int o = c * HCAP + k;
     const double hs = ticks_times(tn - S.ti[k], stick);
-    S.eu[o] = fma(hs, fma(half_of(hs), S.jx[o], S.ax[o]), S.u[o]);
+    return fma(hs, fma(half_of(hs), S.jx[o], S.ax[o]), S.u[o]);
 }
 
 // FP32 copies of member k's state (truncated: within 2^-23 of the FP64
@@ -940,9 +940,59 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         // instead of eleven on each of three warps. Up to F32MIN members FP64 passes
         // over them all; above that the FP32 prediction first rules out the partners
         // that are surely beyond r_crit of every active member.
-        const bool f32 = npmax + na > F32MIN;
+        //
+        // One CTA's set whose moving members' partners would not fit one warp
+        // (na > N3) first lists the pairs that maybe_near leaves, by member and
+        // partner: few of a set's pairs lie within r_crit, and an FP64 instruction
+        // costs the same for one lane as for 32. Up to 96 pairs the block step then
+        // predicts and evaluates the list alone, packed into lanes (sparse).
+        int32_t *plist = S.need + 640, *poff = S.need + 736, *pcnt = S.need + 800;
+        bool sparse = false;
+        int npair = 0;
+        if (!COOP && na > N3 && na <= 32) {
+#pragma unroll 1
+            for (int k = tid; k < n; k += HTHREADS) predict_f32(S, k, tn, stickf);
+            __syncthreads();
+#pragma unroll 1
+            for (int ia = warp; ia < na; ia += HTHREADS / 32) {
+                const int k = act[ia];
+                int m = 0;
+#pragma unroll 1
+                for (int l = wl; l - wl < n; l += 32)
+                    m += __popc(__ballot_sync(0xffffffffu,
+                                              l < n && l != k && maybe_near(S, k, l, rcf)));
+                if (wl == 0) pcnt[ia] = m;
+            }
+            __syncthreads();
+            int to = wl < na ? pcnt[wl] : 0;  // end of member wl's pairs
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, to, o);
+                if (wl >= o) to += v;
+            }
+            npair = __shfl_sync(0xffffffffu, to, 31);
+            sparse = npair <= 96;
+            if (sparse) {
+                if (warp == 0) poff[wl] = to;
+#pragma unroll 1
+                for (int ia = warp; ia < na; ia += HTHREADS / 32) {
+                    const int k = act[ia];
+                    int m = __shfl_sync(0xffffffffu, to, (ia + 31) & 31);
+                    if (ia == 0) m = 0;
+#pragma unroll 1
+                    for (int l = wl; l - wl < n; l += 32) {
+                        const bool f = l < n && l != k && maybe_near(S, k, l, rcf);
+                        const unsigned b = __ballot_sync(0xffffffffu, f);
+                        if (f) plist[m + __popc(b & ((1u << wl) - 1u))] = (ia << 16) | l;
+                        m += __popc(b);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        const bool f32 = npmax + na > F32MIN && !sparse;
         const int32_t *list = nullptr;
-        int np = npart + na;
+        int np = sparse ? na + npair : npart + na;
         if (f32) {
             #pragma unroll 1
             for (int k = tid; k < n; k += HTHREADS) S.need[k] = 0;
@@ -989,19 +1039,30 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             const int it = (pq >> 1) * 32 + wl, i = it / 3, c = it - 3 * i;
             if (i >= np) continue;
             int k;
+            double *to = S.ex + c * HCAP;
             if (f32) {
                 k = list[i];
+                to += k;
+            } else if (sparse && i >= na) {
+                // a listed partner, into the list's own copy ([6][96], in place of
+                // the cluster's receive buffers)
+                k = plist[i - na] & 0xffff;
+                to = S.rb + c * 96 + (i - na);
+            } else if (sparse) {
+                k = act[i];
+                to += k;
             } else {
                 k = mlo + i;
                 if (i >= npart) {
                     k = act[i - npart];
                     if (k >= mlo && k < mhi) continue;
                 }
+                to += k;
             }
             if (pq & 1)
-                predict_v(S, k, c, tn, tick1);
+                to[sparse && i >= na ? 3 * 96 : 3 * HCAP] = predict_v(S, k, c, tn, tick1);
             else
-                predict_x(S, k, c, tn, tick1, tick3);
+                to[0] = predict_x(S, k, c, tn, tick1, tick3);
         }
         __syncthreads();
         uint16_t *nact = S.act + (~steps & 1) * HCAP;
@@ -1025,7 +1086,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // needs neither, then one coordinate each; its longest instruction stream
             // is 34 FP64 instructions against the pair's 47, with the star's pull on
             // the fourth sub-partition.
-            const bool paired = nc <= NP;
+            const bool paired = sparse || nc <= NP;
             const int NR = paired ? nc : NU;
             CorrItem item;  // (warps 0-3)
             #pragma unroll 1
@@ -1048,21 +1109,32 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     }
 #pragma unroll
                     for (int c = 0; c < 6; ++c) prb[c * HTHREADS + tid] = aj[c];
-                } else if (nc <= N3) {
+                } else if (sparse ? npair <= 32 : nc <= N3) {
                     if (warp < 3) {
                         // (LA >= npart: one partner per lane)
-                        const int role = warp, slot = wl >> las, la = wl & (LA - 1);
-                        const int k = slot < cnt ? act[a0 + slot] : 0, l = mlo + la;
+                        const int role = warp;
+                        int slot = wl >> las, l = mlo + (wl & (LA - 1));
+                        bool valid = slot < cnt && l < mhi;
+                        const double *pe = S.ex + l;  // the partner's x, y, z, u, v, w
+                        int pst = HCAP;
+                        if (sparse) {
+                            valid = wl < npair;
+                            const int e = valid ? plist[wl] : 0;
+                            slot = e >> 16;
+                            l = e & 0xffff;
+                            pe = S.rb + wl;
+                            pst = 96;
+                        }
+                        const int k = valid ? act[a0 + slot] : 0;
+                        valid = valid && l != k && (!f32 || maybe_near(S, k, l, rcf));
                         // exchange slots [8][32] in place of the idle FP32 lists
                         double *xs = reinterpret_cast<double *>(S.need) + wl;
-                        bool valid = slot < cnt && la < npart && l != k &&
-                                     (!f32 || maybe_near(S, k, l, rcf));
                         double qr = 0.0, sq = 0.0;
                         bool fold = false;
                         if (valid) {
-                            const double qx = S.ex[k] - S.ex[l];
-                            const double qy = S.ey[k] - S.ey[l];
-                            const double qz = S.ez[k] - S.ez[l];
+                            const double qx = S.ex[k] - pe[0];
+                            const double qy = S.ey[k] - pe[pst];
+                            const double qz = S.ez[k] - pe[2 * pst];
                             const double q2 = pair_q2(qx, qy, qz, h.eps2);
                             valid = !at_least(q2, tc.rc2);  // beyond r_crit: no force, no jerk
                             if (valid) {
@@ -1082,9 +1154,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                                     xs[32 * role] = p;
                                 } else {
                                     const double qi2 = qi * qi;
-                                    const double px = S.eu[k] - S.eu[l];
-                                    const double py = S.ev[k] - S.ev[l];
-                                    const double pz = S.ew[k] - S.ew[l];
+                                    const double px = S.eu[k] - pe[3 * pst];
+                                    const double py = S.ev[k] - pe[4 * pst];
+                                    const double pz = S.ew[k] - pe[5 * pst];
                                     const double cl = pair_cl(S.gm[l], qi, qi2);
                                     xs[32 * 2] = cl;
                                     xs[32 * 3] = cl * pair_rv(qx, qy, qz, px, py, pz);
@@ -1120,8 +1192,11 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     }
                 } else if (warp < 6) {
                     const int role = warp & 1, vl = (warp >> 1) * 32 + wl;
-                    const int slot = vl >> las, la = vl & (LA - 1);
-                    const bool sv = slot < cnt;
+                    int slot = vl >> las;
+                    const int la = vl & (LA - 1);
+                    const int e = sparse && vl < npair ? plist[vl] : 0;
+                    if (sparse) slot = e >> 16;
+                    const bool sv = sparse ? vl < npair : slot < cnt;
                     const int k = sv ? act[a0 + slot] : 0;
                     // exchange slots [2][3][96] (sin, q . p, cos): the FP32
                     // pass's lists, which are idle until the next block time
@@ -1129,18 +1204,20 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                     double acc[3] = {0.0, 0.0, 0.0};
                     int par = 0;
                     #pragma unroll 1
-                    for (int it0 = 0; it0 < npart; it0 += LA) {
-                        const int l = mlo + it0 + la;
+                    for (int it0 = 0; it0 < (sparse ? 1 : npart); it0 += LA) {
+                        const int l = sparse ? e & 0xffff : mlo + it0 + la;
+                        const double *pe = sparse ? S.rb + vl : S.ex + l;
+                        const int pst = sparse ? 96 : HCAP;
                         double *xs = xch + par * (3 * 96);
-                        bool valid = sv && it0 + la < npart && l != k &&
+                        bool valid = sv && (sparse || it0 + la < npart) && l != k &&
                                      (!f32 || maybe_near(S, k, l, rcf));
                         double qx = 0.0, qy = 0.0, qz = 0.0, qi2 = 0.0, sq = 0.0;
                         double y = 0.0, mine = 0.0, cl = 0.0, m3 = 0.0, px = 0.0, py = 0.0, pz = 0.0;
                         bool fold = false;
                         if (valid) {
-                            qx = S.ex[k] - S.ex[l];
-                            qy = S.ey[k] - S.ey[l];
-                            qz = S.ez[k] - S.ez[l];
+                            qx = S.ex[k] - pe[0];
+                            qy = S.ey[k] - pe[pst];
+                            qz = S.ez[k] - pe[2 * pst];
                             const double q2 = pair_q2(qx, qy, qz, h.eps2);
                             valid = !at_least(q2, tc.rc2);  // beyond r_crit: no force, no jerk
                             if (valid) {
@@ -1157,9 +1234,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                                 // what does not wait for the partner warp's
                                 // polynomial is done before the barrier
                                 cl = pair_cl(S.gm[l], qi, qi2);
-                                px = S.eu[k] - S.eu[l];
-                                py = S.ev[k] - S.ev[l];
-                                pz = S.ew[k] - S.ew[l];
+                                px = S.eu[k] - pe[3 * pst];
+                                py = S.ev[k] - pe[4 * pst];
+                                pz = S.ew[k] - pe[5 * pst];
                                 if (role == 0)
                                     xs[96 + vl] = pair_rv(qx, qy, qz, px, py, pz);
                                 else
@@ -1252,10 +1329,20 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 } else {
                     if (warp < 4 && wl < 3 * nc) item.fetch(S, warp, act + a0, wl);
                     __syncthreads();
+                    // sparse: each (member, component) on one thread, the star's pull
+                    // and its pairs in order
+                    if (sparse && tid < 6 * cnt) {
+                        const int sl = tid / 6, c = tid - 6 * sl;
+                        double v = prb[c * HTHREADS + 224 + sl];
+#pragma unroll 1
+                        for (int m = sl ? poff[sl - 1] : 0; m < poff[sl]; ++m)
+                            v += prb[c * HTHREADS + m];
+                        S.a1s[c * ACH + sl] = v;
+                    }
                     // sums over the LA lanes of each (member, component), one
                     // warp each, in a fixed order
                     #pragma unroll 1
-                    for (int pi = warp; pi < 6 * cnt; pi += HTHREADS / 32) {
+                    for (int pi = sparse ? 6 * cnt : warp; pi < 6 * cnt; pi += HTHREADS / 32) {
                         const int sl = pi / 6, c = pi - 6 * sl;
                         const double *col = prb + c * HTHREADS + (sl << las);
                         double v = wl < LA ? col[wl] : 0.0;
