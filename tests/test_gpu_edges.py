@@ -295,3 +295,37 @@ def test_pairs_once(torch, n, equal):
     assert big > 0 and max(x.max() for x in a) <= 2.0 ** -18 * big
     rms = [np.sqrt((x ** 2).mean()) for x in a]
     assert rms[0] <= 1.5 * rms[1] + 1e-16 * big, (rms, big)
+
+
+# (members, cluster, swarm mass, systems): either side of each lane layout of a block
+# step: partners of up to 8, 16 and 32 lanes a member, the list of near pairs up to a
+# warp's, up to three warps' (light swarm: only the planet pulls) and beyond (heavy
+# swarm: most pairs are near), one CTA, clusters, a batch with more large sets than
+# clusters
+HERM_CASES = [(2, 0, 1e-12, 1), (8, 0, 1e-12, 1), (9, 0, 1e-6, 1), (17, 0, 1e-12, 1), (23, 0, 1e-12, 1),
+              (23, 0, 1e-6, 1), (24, 8, 1e-12, 1), (33, 2, 1e-6, 1), (65, 4, 1e-12, 1), (130, 8, 1e-12, 1),
+              (33, 0, 1e-12, 156), (26, 0, 1e-6, 156)]
+
+
+@pytest.mark.parametrize("members,cluster,mass,systems", HERM_CASES)
+def test_hermite_layouts(torch, oracle, members, cluster, mass, systems):
+    """A planet's swarm as one encounter set through the Hermite: the oracle's
+    records, and positions within the larger of 1e-11 and 100 times what one ulp in
+    the initial positions moves a body (the sums run in another order)."""
+    from test_gpu_step import _chaos_spread, _check_positions, _compare_records, _planet_swarm, _run_gpu, _run_oracle
+    sw = [_planet_swarm(members - 1, seed=1000 + members + s) for s in range(systems)]
+    for x in sw:
+        x.m[2:] = mass
+    cat = [np.concatenate([getattr(x, k) for x in sw]) for k in "mqv"]
+    offs = np.cumsum([0] + [len(x.m) for x in sw])
+    w = W.Workload("swarms", *cat, offs, sw[0].tau, 2)
+    qg, vg, enc, st, E = _run_gpu(w, 2, kick_prec=q.QYM_KICK_FP64, hermite_cluster=cluster)
+    assert st["status_bits"] == 0 and st["max_set"] == members
+    for s in {0, systems // 2, systems - 1}:
+        a, b = int(offs[s]), int(offs[s + 1])
+        r, _ = _run_oracle(oracle, sw[s], 2)
+        mine = enc[(enc[:, 1] >= a) & (enc[:, 1] < b)].copy()
+        mine[:, 1:] -= a
+        skip = _compare_records(mine, r)
+        keep = np.array([i not in skip for i in range(b - a)])
+        _check_positions(qg[a:b][keep], r.q[keep], _chaos_spread(oracle, sw[s], 2)[keep], rel=1e-11)
