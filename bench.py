@@ -597,7 +597,8 @@ def run_ours(args):
     probe = probe_peaks(q, dev)
     peak = probe["fp32"] if prec else probe["dfma"]
     digest = source_digest("kick.cu")
-    roof = {"bound": "alu", "kernel": "k_kick_mixed" if prec else "k_kick_fp64",
+    once = prec and len(w.offsets) == 2 and st["kick_tile_i"] == 512
+    roof = {"bound": "alu", "kernel": "k_kick_sym" if once else "k_kick_mixed" if prec else "k_kick_fp64",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "peak_source": "measured (qym_probe_fma, %s)" % ("FP32 FMA pipe" if prec else "FP64"),
             "peak_probe": probe,

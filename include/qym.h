@@ -331,12 +331,15 @@ qym_status qym_time_drift(qym_ctx *ctx, double tau, int32_t reps, double *ms_mom
 /* Set the kick launch shape: threads per CTA (128 or 256), i rows per thread
  * (1, 2, or 4 for the mixed kick) and j splits per system (1 .. the largest
  * the context's buffers hold, at least 4); QYM_EINVAL otherwise. For
- * reproducing a shape the tuner chose (qym_stats kick_tile_i, _splits). */
+ * reproducing a shape the tuner chose (qym_stats kick_tile_i, _splits).
+ * One system of at least 8192 bodies forms each pair of the mixed kick once
+ * by default (kick_tile_i = 512 rows, kick_tile_splits its ranges); a shape
+ * set here replaces that form by the one-sided kick. */
 qym_status qym_set_kick_shape(qym_ctx *ctx, int32_t threads, int32_t ipt, int32_t splits);
 
 /* Pick the kick launch shape (threads per CTA, rows per thread, j splits)
- * by timing candidate shapes with qym_time_kick on the current state, and
- * keep the fastest. The state is unchanged; results can differ from the
+ * by timing candidate shapes with qym_time_kick on the current state, the
+ * pairs-once form among them where it applies, and keep the fastest. The state is unchanged; results can differ from the
  * default shape in the last bits (summation grouping). */
 qym_status qym_autotune(qym_ctx *ctx);
 

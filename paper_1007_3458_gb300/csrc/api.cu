@@ -183,7 +183,9 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // bodies from which a single system's kick holds them in Morton order
 constexpr int64_t kSortMinBodies = 2048;
-// bodies from which the mixed kick of one system forms each pair once (kick.cu)
+// bodies from which the mixed kick of one system forms each pair once (kick.cu):
+// 0.0384 against 0.0391 ms at 8192 bodies, 0.064 against 0.077 at 12288, 0.099
+// against 0.124 at 16384
 constexpr int64_t kSymMinBodies = 8192;
 // bodies from which QYM_SEARCH_AUTO takes the binned search for one system
 constexpr int64_t kBinnedMinBodies = 65536;

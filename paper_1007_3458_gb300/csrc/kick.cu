@@ -1057,12 +1057,13 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t, in
 // short CTAs even out the near and far tiles and the last wave: 16384 bodies
 // take 0.134 ms in 64 ranges, 0.150 in 16, 0.188 in 10 (four CTAs per SM);
 // 262144 bodies 26.9 ms in 12, 29.6 in one; 4096 bodies 20.5 us in 32, 1024
-// bodies 6.2 us in 32 (14.4 in 4).
+// bodies 6.2 us in 32 (14.4 in 4); each a twelfth less since windows of one G m
+// leave its multiplication to the fold.
 // FP64: as many CTAs as fit the GPU at once (eight of 128 threads per SM),
 // since a pair takes some 400 issue slots: 10240 bodies on 80 i-blocks fill
 // the chip with 15 splits; small systems take splits of at least 8 rows (a
 // 260-body kick is one warp's walk over its j-range: 185 us in one range in
-// plain FP64, 14 us in ranges of 16).
+// plain FP64, 14 us in ranges of 16, 8.1 us in ranges of 8).
 KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t max_splits) {
     KickTune t;
     const bool mixed = prec == QYM_KICK_MIXED;
