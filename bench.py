@@ -157,8 +157,8 @@ class ClockSampler:
 # particles (ncu sm__inst_executed_pipe_fp64.sum), per (solver, guess, source
 # digest of kepler.cu + mlp.cuh)
 KEPLER_FP64_WARP_INST = {
-    ("newton32", "standard", "52815e32767a71e8"): 12070789,
-    ("newton", "standard", "52815e32767a71e8"): 23102409,
+    ("newton32", "standard", "aad84024ce025248"): 7296855,
+    ("newton", "standard", "aad84024ce025248"): 12321900,
 }
 
 # DRAM bytes (read + written) per launch of the mixed kick, from one ncu
@@ -169,10 +169,8 @@ KEPLER_FP64_WARP_INST = {
 # with the splits. A shape or a kick source not captured reports null (the
 # capture commands sit with the ncu summaries under profiles/).
 KICK_DRAM_BYTES = {
-    ("disk_16384", 256, 64, "3d6b39905dba5b88"): 9.17e5,
-    ("disk_16384", 256, 128, "3d6b39905dba5b88"): 1.24e6,
-    ("disk_262144", 256, 64, "3d6b39905dba5b88"): 2.35e7,
-    ("disk_262144", 512, 64, "3d6b39905dba5b88"): 1.85e7,
+    ("disk_16384", 512, 160, "e3a78e7fc4b8f9ee"): 8.59e5,
+    ("disk_262144", 512, 128, "e3a78e7fc4b8f9ee"): 6.90e8,
 }
 
 
@@ -995,7 +993,7 @@ def run_kepler(args):
     pk = probe_peaks(q, dev)
     dfma_rate = pk["dfma"] / 2.0 * 1e3          # 1e9 FP64 thread-instructions/s
     achieved = fp64_inst * 32 / (head["ms_per_step"] / 1e3) / 1e9 if fp64_inst else None
-    roof = {"bound": "alu", "kernel": "k_kepler<%s>" % ("true" if args.guess == "learned" else "false"),
+    roof = {"bound": "alu", "kernel": "k_kepler<%d>" % (args.guess == "learned"),
             "achieved": achieved, "peak": dfma_rate, "unit": "G FP64 instr/s",
             "frac": achieved / dfma_rate if achieved else None,
             "peak_source": "measured (qym_probe_fma DFMA: %.3f TFLOP/s)" % pk["dfma"],

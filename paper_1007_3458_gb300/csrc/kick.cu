@@ -1070,7 +1070,7 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t, in
 // bodies 6.2 us in 32 (14.4 in 4); each a twelfth less since windows of one G m
 // leave its multiplication to the fold.
 // FP64: as many CTAs as fit the GPU at once (eight of 128 threads per SM),
-// since a pair takes some 400 issue slots: 10240 bodies on 80 i-blocks fill
+// since a pair takes some 300 issue slots: 10240 bodies on 80 i-blocks fill
 // the chip with 15 splits; small systems take splits of at least 8 rows (a
 // 260-body kick is one warp's walk over its j-range: 185 us in one range in
 // plain FP64, 14 us in ranges of 16, 8.1 us in ranges of 8).
