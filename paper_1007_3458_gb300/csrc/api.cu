@@ -915,7 +915,7 @@ static cudaError_t enqueue_step(qym_ctx *c, double tau, bool last, bool fresh = 
         // items 4-8: [binned search,] rigorous test, sets and r_crit, K corrections + Hermite
         if ((e = enqueue_binned_search(c, tau))) return e;
         if ((e = launch_refine(d, tau, p.a_E, st))) return e;
-        if ((e = launch_sets_impl(d, p.a_H, c->ss, st))) return e;
+        if ((e = launch_sets_impl(d, p, c->ss, st))) return e;
         // (the sets of a system integrated whole are left out of the Hermite)
         if (p.whole_hermite && (e = enqueue_whole(c, tau))) return e;
         if ((e = launch_hermite(d, p, tau, st))) return e;
@@ -936,7 +936,7 @@ static cudaError_t enqueue_step(qym_ctx *c, double tau, bool last, bool fresh = 
         return e;
     // kick [+ chunk re-test], finish, Kepler, [refine, sets, Hermite plan, Hermite], pack, kick,
     // finish, momentum [1 or 2], drift
-    c->launches += 7 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 3 + sets_launches(d.rows) : 0) + search_retest(p, fz);
+    c->launches += 7 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d.rows) : 0) + search_retest(p, fz);
     return cudaGetLastError();
 }
 
@@ -982,7 +982,7 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
     if (enc) {
         if ((e = enqueue_binned_search(c, tau))) return e;
         if ((e = launch_refine(d, tau, p.a_E, st))) return e;
-        if ((e = launch_sets_impl(d, p.a_H, c->ss, st))) return e;
+        if ((e = launch_sets_impl(d, p, c->ss, st))) return e;
         if ((e = launch_hermite(d, p, tau, st))) return e;
     }
     // (q1, v1) -> (q, v)
@@ -1004,7 +1004,7 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
             return e;
         // Kepler, [refine, sets, Hermite plan, Hermite], copy, momentum [1 or 2], drift, kick
         // [+ chunk re-test], finish
-        c->launches += 5 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 3 + sets_launches(d.rows) : 0) + search_retest(p, fz);
+        c->launches += 5 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d.rows) : 0) + search_retest(p, fz);
     } else {
         if ((e = launch_kick_tiles(d, p.kick_prec, 0, p.G, c->tune.threads, c->tune.ipt, st))) return e;
         if ((e = launch_kick_finish_v(d, d.v, d.q, 0.5 * tau, p.G, 0, p.hill_fixed, st))) return e;
@@ -1013,7 +1013,7 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
                                         p.hill_fixed, st, 0.5 * tau, 1.01, 1, 1)))
             return e;
         // Kepler, [refine, sets, Hermite plan, Hermite], copy, kick, finish, momentum [1 or 2], drift
-        c->launches += 5 + momentum_launches(d, true) + (enc ? 3 + sets_launches(d.rows) : 0);
+        c->launches += 5 + momentum_launches(d, true) + (enc ? 2 + sets_launches(d.rows) : 0);
     }
     return cudaGetLastError();
 }
@@ -1447,7 +1447,7 @@ extern "C" qym_status qym_split_phase(qym_ctx *c, int32_t phase, double tau, int
     }
     case QYM_PHASE_HERMITE: {
         if (enc) {
-            CK(c, launch_sets_impl(d, p.a_H, c->ss, st));
+            CK(c, launch_sets_impl(d, p, c->ss, st));
             CK(c, launch_hermite(d, p, tau, st));
             k_owned_members<<<1, 1, 0, st>>>(d, c->owned_info);
             CK(c, cudaGetLastError());

@@ -5,6 +5,7 @@
 // The rigorous test is evaluated in FP64 with explicitly rounded operations
 // (no contraction into FMA) in a fixed order, so that equal inputs give equal
 // bits on any IEEE-754 machine evaluating the same sequence.
+#include "hermite_plan.cuh"
 #include "qym_internal.cuh"
 
 namespace qym {
@@ -359,9 +360,11 @@ __global__ void __launch_bounds__(256) k_uf_place(Dev d, const int32_t *sid, int
 // the pairs of a step are few. A thread takes the rows tid, tid + 1024, ...: whether they are
 // members and roots stays in two bit masks; the roots' counts per (round, warp) are
 // numbered by one scan of 1024 entries.
+// The Hermite's plan follows in the same CTA (a launch of 3.7 us less: 16 steps of
+// 260 bodies 1636 -> 1618 us).
 constexpr int kSetsRounds = 8;
 constexpr int64_t kSetsOneRows = kSetsRounds * 1024;
-__global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a_H) {
+__global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a_H, int ncl) {
     chain_wait();
     __shared__ int s_cnt[32][32], s_warp[32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -422,12 +425,17 @@ __global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a
     }
     for (unsigned m = member; m; m &= m - 1)
         uf_place(d, (int64_t)(__ffs(m) - 1) * 1024 + tid, s.sid, s.fill);
+    __syncthreads();
+    hermite_plan(d, ncl);
 }
 
-int sets_launches(int64_t rows) { return rows <= kSetsOneRows ? 1 : 7; }
+bool sets_one(int64_t rows) { return rows <= kSetsOneRows; }
+int sets_launches(int64_t rows) { return sets_one(rows) ? 1 : 8; }
 
-cudaError_t launch_sets_impl(const Dev &d, double a_H, const SetScratch &s, cudaStream_t st) {
-    if (d.rows <= kSetsOneRows) return launch_chain(k_sets_one, 1, 1024, 0, st, d, s, a_H);
+cudaError_t launch_sets_impl(const Dev &d, const qym_params &p, const SetScratch &s, cudaStream_t st) {
+    const double a_H = p.a_H;
+    if (sets_one(d.rows))
+        return launch_chain(k_sets_one, 1, 1024, 0, st, d, s, a_H, hermite_clusters(d, p));
     int nblk = (int)((d.rows + 1023) / 1024);
     launch_chain(k_uf_hook, 152, 256, 0, st, d);
     launch_chain(k_uf_count, nblk, 1024, 0, st, d, s.blk);
