@@ -169,8 +169,8 @@ KEPLER_FP64_WARP_INST = {
 # with the splits. A shape or a kick source not captured reports null (the
 # capture commands sit with the ncu summaries under profiles/).
 KICK_DRAM_BYTES = {
-    ("disk_16384", 512, 160, "e3a78e7fc4b8f9ee"): 8.59e5,
-    ("disk_262144", 512, 128, "e3a78e7fc4b8f9ee"): 6.90e8,
+    ("disk_16384", 512, 160, "ef3860c9a9503734"): 8.59e5,
+    ("disk_262144", 512, 128, "ef3860c9a9503734"): 6.90e8,
 }
 
 

@@ -1071,9 +1071,10 @@ void kick_items_host(const int64_t *offsets, int32_t nsys, const KickTune &t, in
 // leave its multiplication to the fold.
 // FP64: as many CTAs as fit the GPU at once (eight of 128 threads per SM),
 // since a pair takes some 300 issue slots: 10240 bodies on 80 i-blocks fill
-// the chip with 15 splits; small systems take splits of at least 8 rows (a
-// 260-body kick is one warp's walk over its j-range: 185 us in one range in
-// plain FP64, 14 us in ranges of 16, 8.1 us in ranges of 8).
+// the chip with 15 splits; small systems take splits of at least 8 rows, of 4
+// while that makes at most 256 CTAs (a 260-body kick is one warp's walk over its
+// j-range: 185 us in one range in plain FP64, 14 us in ranges of 16, 6.8 in ranges
+// of 8, 5.2 in ranges of 4; 600 bodies 9.5 us in 75 ranges, 12.6 in 128).
 KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t max_splits) {
     KickTune t;
     const bool mixed = prec == QYM_KICK_MIXED;
@@ -1085,7 +1086,7 @@ KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t 
         const int64_t range = nbmax > 6144 ? 256 : (nbmax > 2048 ? 128 : 32);
         sp = std::min<int64_t>({(nbmax + range - 1) / range, 12288 / ib, 64});
     } else {
-        sp = std::min<int64_t>({8 * 152 / ib, nbmax / 8, 128});
+        sp = std::min<int64_t>({8 * 152 / ib, std::max(nbmax / 8, std::min(nbmax / 4, 256 / ib)), 128});
     }
     t.splits = (int32_t)std::max<int64_t>(1, std::min(sp, max_splits));
     return t;

@@ -340,7 +340,39 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
                        d.m, R, a.G, ax, ay, az);
         }
     }
-    if (L > 1) {
+    if (L == 32) {
+        // few rows: eight a CTA, 32 threads each (four of every warp), so that the
+        // slots' additions spread over the GPU and the tree is 16 FP64 additions deep,
+        // the last seven on a lane per (component, row) (L = 8 adds its warps' parts on
+        // one warp, 21; 260 rows: 5.7 us with 32 slots, 5.8 with the 65 that
+        // the shorter kick leaves)
+        __shared__ double sh[8][3][8];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+        for (int o = 8; o < 32; o *= 2) {
+            ax += __shfl_xor_sync(0xffffffffu, ax, o);
+            ay += __shfl_xor_sync(0xffffffffu, ay, o);
+            az += __shfl_xor_sync(0xffffffffu, az, o);
+        }
+        if (lane < 8) {
+            sh[warp][0][lane] = ax;
+            sh[warp][1][lane] = ay;
+            sh[warp][2][lane] = az;
+        }
+        __syncthreads();
+        if (warp > 0) return;
+        double p[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) p[k] = lane < 24 ? sh[k][lane >> 3][lane & 7] : 0.0;
+#pragma unroll
+        for (int w = 1; w < 8; w *= 2)
+#pragma unroll
+            for (int k = 0; k < 8; k += 2 * w) p[k] += p[k + w];
+        ax = __shfl_sync(0xffffffffu, p[0], lane & 7);
+        ay = __shfl_sync(0xffffffffu, p[0], 8 + (lane & 7));
+        az = __shfl_sync(0xffffffffu, p[0], 16 + (lane & 7));
+        if (lane >= 8) return;
+    } else if (L > 1) {
         __shared__ double sh[L > 1 ? L - 1 : 1][3][RB];
         if (q > 0) {
             sh[q - 1][0][t] = ax;
@@ -388,6 +420,10 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
     d.amag[r] = an;
 }
 
+// rows up to which the finisher takes 32 threads a row: a CTA of eight rows per SM
+// (steps of 600 rows 94.9 -> 89.2 us, 1200 rows 151 -> 139; 2400 rows 294 -> 296)
+constexpr int64_t kFewRows = 152 * 8;
+
 cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, double dt, double G,
                                  int check, int hill_fixed, cudaStream_t st, double a_allow,
                                  int skip_whole) {
@@ -403,7 +439,9 @@ cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, doubl
     // groups of 4 or 8 threads a row where there are that many slots to add (8
     // also halves the chain of a small system), one where there are few
     const int nslots = d.sym.G > 0 ? d.sym.splits : (d.kick_cnt ? 1 : d.splits);
-    if (nslots >= 16)
+    if (nslots >= 16 && d.rows <= kFewRows)
+        launch_chain(k_finish<32>, (unsigned)((d.rows + 7) / 8), 256, 0, st, d, a);
+    else if (nslots >= 16)
         launch_chain(k_finish<8>, (unsigned)((d.rows + 31) / 32), 256, 0, st, d, a);
     else if (nslots >= 4)
         launch_chain(k_finish<4>, (unsigned)((d.rows + 63) / 64), 256, 0, st, d, a);

@@ -329,3 +329,16 @@ def test_hermite_layouts(torch, oracle, members, cluster, mass, systems):
         skip = _compare_records(mine, r)
         keep = np.array([i not in skip for i in range(b - a)])
         _check_positions(qg[a:b][keep], r.q[keep], _chaos_spread(oracle, sw[s], 2)[keep], rel=1e-11)
+
+
+@pytest.mark.parametrize("n", [70, 1216, 1217])
+def test_finisher_rows(torch, oracle, n):
+    """The finisher with 32 threads a row (up to 1216 rows) and with eight, a ragged
+    last CTA: a step with the FP64 kick and no encounters against the oracle's,
+    within 1e-12 (as the plain step's parity)."""
+    from test_gpu_step import _relq, _run_gpu, _run_oracle
+    w = W.outer_disk(n - 5, 1e-9, seed=n)
+    assert len(w.m) == n
+    qg, vg, *_ = _run_gpu(w, 1, kick_prec=q.QYM_KICK_FP64, encounters=0)
+    r, vh = _run_oracle(oracle, w, 1, encounters=0)
+    assert _relq(qg, r.q).max() <= 1e-12 and _relq(vg, vh).max() <= 1e-12
