@@ -18,11 +18,11 @@
 // first rules out the pairs that are surely that far, and only the others
 // are predicted and evaluated in FP64 (the result is the same as evaluating
 // every pair). FP64 instructions issue at one per 64 cycles per warp here, so
-// each block step is split by instruction stream across warps: a warp per
-// coordinate for predictor and corrector, each pair item on two warps, the
-// star's pull on its own warp, fixed-order sums (a cluster's CTAs push their
-// parts to each other and add them in rank order, so every copy of the set
-// stays bit-identical). Every loop has a cap and reports through the status
+// each block step is split by instruction stream across warps: items
+// (member, coordinate) for predictor and corrector, each pair item on three or
+// two warps, the star's pull on its own warp, fixed-order sums (a cluster's CTAs
+// send their parts to each other and add them in rank order, so every copy of
+// the set stays bit-identical). Every loop has a cap and reports through the status
 // word.
 #include <climits>
 
@@ -695,10 +695,9 @@ __device__ __forceinline__ void pull_range(cg::cluster_group &cl, const HermSmem
 // COOP the cs CTAs of a cluster share the set: every CTA keeps a full copy of
 // the members' state; CTA `rank` evaluates the start-up forces and the K
 // corrections of its member range, exchanged once; in each block step it sums
-// the forces on the active members from its partner range, all partial sums
-// are read from the peers' shared memory in rank order, and every CTA applies
-// the same corrector, so the copies stay identical with one cluster barrier
-// per exchange round (partials double-buffered).
+// the forces on the active members from its partner range, sends its sums
+// to every CTA's receive buffer, adds all CTAs' sums in rank order and applies
+// the same corrector, so the copies stay identical.
 template <bool COOP, int CLT>
 __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set, int rank,
                                          int cs) {
@@ -878,9 +877,9 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     // Block steps. FP64 instructions are issued at about one warp-instruction
     // per 64 cycles per SM sub-partition here, whatever the number of active
     // lanes, so the work is split by instruction stream across warps (which
-    // the sub-partitions serve in parallel): one warp per coordinate for the
-    // predictor and the corrector, several warps per member for the forces,
-    // one warp per (member, component) for the sums.
+    // the sub-partitions serve in parallel): items (member, coordinate) of
+    // the predictor and of each of the corrector's forms on warps of their own,
+    // several warps per pair for the forces, lane groups for the sums.
     const double stick = sgn * tick;
     const T2Split T2s((float)T2d);
     const float etaf = (float)h.eta;
