@@ -5,11 +5,16 @@
 // yt = (t - om) / osd over rows (u1, u2, u3, u4, t) with Adam. One step is two
 // launches:
 //   k_mlp_grad    forward and backward of a minibatch; each CTA takes rounds
-//                 of 64 rows (16 per warp), keeps the 64 x 64 weight gradient
-//                 of its rows in tensor-core accumulators and writes one
-//                 partial gradient vector;
-//   k_mlp_reduce  sums the partials in a fixed order (deterministic) and
-//                 applies the Adam update to the float32 master weights.
+//                 of 64 rows (16 per warp of the forward pass), keeps the
+//                 64 x 64 weight gradient of its rows in tensor-core
+//                 accumulators and writes one partial gradient vector;
+//   k_mlp_reduce  sums the partials (as an FP64 sum does) and applies the Adam
+//                 update to the float32 master weights.
+// The grouping of the sums is part of the result: a weight near a bf16 midpoint
+// turns one last place into 2^-9, and a hundred minibatches into 1e-2 of the
+// moments. A round's sums run over its 64 rows in order (FP32), a CTA's over its
+// rounds, CTA b of min(256, rounds) taking the rounds b, b + 256, ...; the
+// partials' sum is exact but for its last rounding.
 // The operands the tensor cores take are bf16: h1 and W2 in the forward
 // product, dp2 = dL/dp2 with W2 (for dL/dh1) and with h1 (for dL/dW2) in the
 // backward ones. The other sums (dL/dW1, the biases, dL/dW3) stay in FP32.
@@ -22,16 +27,25 @@ using namespace mlp;
 
 namespace {
 constexpr int GT = 256;      // threads of a gradient CTA
-constexpr int GWARPS = GT / 32;
+constexpr int FW = 4;        // its warps that take a tile of 16 rows through the network
+constexpr int GR = 16 * FW;  // rows per round
 constexpr int LDT = 72;      // bf16 row stride of the shared tiles: 16-byte rows of eight lanes
                              // fall on distinct banks (ldmatrix)
-constexpr int MAXBLK = 256;  // CTAs of a gradient launch the workspace holds
-constexpr int GRID = 152;    // one CTA per SM
-constexpr int NRED = 448;    // column sums: W1 (4 x 64), b1, b2, W3
+constexpr int LDF = 72;      // float row stride: a half warp's pairs fall on distinct banks
+constexpr int MAXBLK = 256;  // CTAs of a gradient launch, at most
+struct GradShared {
+    __nv_bfloat16 w2[64 * LDT];         // bf16 W2[j][k]
+    __nv_bfloat16 h1[GR * LDT];         // bf16 h1 [row][k]
+    __nv_bfloat16 d2[GR * LDT];         // bf16 dL/dp2 [row][j]
+    float dp1[GR * LDF], dp2[GR * LDF], h2[GR * LDF];  // [row][unit]
+    float4 fn[GR];                      // normalised features
+    float dy[GR];
+    float w1[256], b1[64], b2[64], w3[64];  // W1 and W3 rounded to bf16
+    float red[2][FW];
+};
 }  // namespace
 
-__global__ void __launch_bounds__(256) k_mlp_forward(int64_t n, const float *__restrict__ w,
-                                                     const float *__restrict__ u,
+__global__ void __launch_bounds__(256) k_mlp_forward(int64_t n, const float *__restrict__ w, const float *__restrict__ u,
                                                      float *__restrict__ y) {
     chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -64,45 +78,21 @@ __device__ __forceinline__ void ldsm2t(uint32_t &r0, uint32_t &r1, uint32_t a) {
                  : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
 }
 
-// Sum of c[16] (entry 2 nt + e: column 8 nt + 2 t + e) over the eight lanes g
-// of a quad column, scattered: lane (g, t) adds the sums of columns
-// 8 g + 2 t + e to s[e]. Halves are exchanged, 8 + 4 + 2 shuffles instead of
-// three per column.
-__device__ __forceinline__ void scatter_sum(float (&c)[16], int lane, float (&s)[2]) {
-#pragma unroll
-    for (int h = 8; h >= 2; h >>= 1) {
-        const int bit = 2 * h;  // lanes 16, 8, 4 apart
-        const bool up = lane & bit;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const float keep = up ? c[h + i] : c[i], give = up ? c[i] : c[h + i];
-            c[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
-        }
-    }
-    s[0] += c[0];
-    s[1] += c[1];
-}
-
-// Forward and backward of a minibatch. A warp takes 16-row tiles (tile =
-// warp * grid + CTA, so any batch spreads over every SM before a warp gets a
-// second one); the batch is latency here, not arithmetic (16384 rows are 0.6
+// Forward and backward of a minibatch (16384 rows with the reduction: 20 us). Four of the CTA's eight warps take a
+// 16-row tile each; the batch is latency here, not arithmetic (16384 rows are 0.6
 // GFLOP), so the kernel is built for few dependent round trips: the weights
 // staged once per CTA with all loads in flight, one copy of W2 serving both
 // its products through ldmatrix (plain and transposed), the tiles' bf16 h1 and
 // dL/dp2 left row by row and read transposed for dL/dW2 (warp w owns its
-// columns 8w ..), the column sums by a halving exchange in registers. With
-// 64-row CTAs of 128 threads, 16-bit transposing stores and a serial walk of
-// 64 rows for the column sums a 16384-row minibatch took 20 us.
-__global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
-                                                    const float *__restrict__ rows, int64_t n,
-                                                    float inv_n, float *__restrict__ part,
-                                                    float *__restrict__ lpart) {
+// columns 8w ..). The other column sums run over the round's rows in order (see
+// above), 448 chains on the CTA's 256 threads. (A halving exchange in registers
+// instead is 3 us shorter at 16384 rows, in another order. Weights read from
+// global memory per tile and 16-bit transposing stores: 20 us.)
+__global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float *__restrict__ w, const float *__restrict__ rows, int64_t n,
+                                                    float inv_n, float *__restrict__ part, float *__restrict__ lpart) {
     chain_wait();
-    __shared__ __align__(16) __nv_bfloat16 s_w2[64 * LDT];             // bf16 W2[j][k]
-    __shared__ __align__(16) uint32_t s_t[2][16 * GWARPS * LDT / 2];   // h1, dL/dp2 [row][col]
-    __shared__ __align__(16) float s_w1[256];                          // bf16-rounded W1
-    __shared__ float s_b1[64], s_b2[64], s_w3[64];
-    __shared__ float s_red[2][GWARPS];
+    extern __shared__ __align__(16) unsigned char g_gradsmem[];
+    GradShared &S = *reinterpret_cast<GradShared *>(g_gradsmem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     {
         const float4 *w2 = reinterpret_cast<const float4 *>(w + W2);
@@ -111,44 +101,41 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
         for (int i = 0; i < 4; ++i) x[i] = w2[tid + i * GT];
         const float y = w[W1 + tid];
         if (tid < 64) {
-            s_b1[tid] = w[B1 + tid];
-            s_b2[tid] = w[B2 + tid];
-            s_w3[tid] = bf(w[W3 + tid]);
+            S.b1[tid] = w[B1 + tid];
+            S.b2[tid] = w[B2 + tid];
+            S.w3[tid] = bf(w[W3 + tid]);
         }
-        s_w1[tid] = bf(y);
+        S.w1[tid] = bf(y);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int e = 4 * (tid + i * GT);
-            *reinterpret_cast<uint2 *>(s_w2 + (e >> 6) * LDT + (e & 63)) =
+            *reinterpret_cast<uint2 *>(S.w2 + (e >> 6) * LDT + (e & 63)) =
                 make_uint2(pack2(x[i].x, x[i].y), pack2(x[i].z, x[i].w));
         }
     }
     const float om = w[OM], osd = w[OSD], b3 = w[B3];
     // lane addresses of the ldmatrix loads
-    const uint32_t w2s = smem_u32(s_w2);
+    const uint32_t w2s = smem_u32(S.w2);
     const uint32_t aF = w2s + 2 * ((lane & 7) * LDT + 8 * (lane >> 3));
     const uint32_t aB = w2s + 2 * (((lane & 7) + 8 * ((lane >> 3) & 1)) * LDT + 8 * (lane >> 4));
-    const uint32_t aD = smem_u32(s_t[1]) + 2 * (((lane & 7) + 8 * (lane >> 4)) * LDT + 8 * ((lane >> 3) & 1));
-    const uint32_t aH = smem_u32(s_t[0]) + 2 * ((lane & 15) * LDT + 8 * warp);
+    const uint32_t aD = smem_u32(S.d2) + 2 * (((lane & 7) + 8 * (lane >> 4)) * LDT + 8 * ((lane >> 3) & 1));
+    const uint32_t aH = smem_u32(S.h1) + 2 * ((lane & 15) * LDT + 8 * warp);
     float gw2[4][4];  // dL/dW2 rows 16 mt + g (+ 8), columns 8 warp + 2 t (+ 1)
 #pragma unroll
     for (int mt = 0; mt < 4; ++mt)
 #pragma unroll
         for (int e = 0; e < 4; ++e) gw2[mt][e] = 0.0f;
-    float cs[7][2];  // columns 8 g + 2 t + e: dL/dW1 (4), dL/db1, dL/db2, dL/dW3
-#pragma unroll
-    for (int i = 0; i < 7; ++i) cs[i][0] = cs[i][1] = 0.0f;
+    // column sums of unit j: db1 and dW1[0] | dW1[1], dW1[2] | dW1[3], db2 | dW3
+    const int j = tid & 63, job = tid >> 6;
+    float cs0 = 0.0f, cs1 = 0.0f;
     float gb3 = 0.0f, lsum = 0.0f;
     __syncthreads();
 
-    const int64_t ntile = (n + 15) / 16;
-    for (int64_t t0 = blockIdx.x; t0 < ntile; t0 += (int64_t)GWARPS * gridDim.x) {
-        // warps 0 .. nw - 1 have a tile in this round
-        const int64_t left = (ntile - t0 + gridDim.x - 1) / gridDim.x;
-        const int nw = left < GWARPS ? (int)left : GWARPS;
-        if (warp < nw) {
-            const int64_t tile = t0 + (int64_t)warp * gridDim.x;
-            const int64_t sa = tile * 16 + g, sb = sa + 8;
+    const int64_t nround = (n + GR - 1) / GR;
+    for (int64_t rd = blockIdx.x; rd < nround; rd += gridDim.x) {
+        if (warp < FW) {
+            const int ra = 16 * warp + g, rb = ra + 8;  // rows of this lane within the round
+            const int64_t sa = rd * GR + ra, sb = rd * GR + rb;
             const bool va = sa < n, vb = sb < n;
             float ua[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ub[4] = {0.0f, 0.0f, 0.0f, 0.0f};
             float ta = 0.0f, tb = 0.0f;
@@ -165,6 +152,10 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
             float fa[4], fb[4];
             normalise(w, ua, fa);
             normalise(w, ub, fb);
+            if (t == 0) {
+                S.fn[ra] = make_float4(fa[0], fa[1], fa[2], fa[3]);
+                S.fn[rb] = make_float4(fb[0], fb[1], fb[2], fb[3]);
+            }
             // layer 1: h1 as the A fragments of layer 2, d1 = gelu'(p1)
             uint32_t A[4][4];
             float d1[8][4];
@@ -174,8 +165,8 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const int c = 8 * nt + 2 * t + e;
-                    const float4 wr = *reinterpret_cast<const float4 *>(s_w1 + 4 * c);
-                    const float bb = s_b1[c];
+                    const float4 wr = *reinterpret_cast<const float4 *>(S.w1 + 4 * c);
+                    const float bb = S.b1[c];
                     const float pa = fmaf(wr.w, fa[3], fmaf(wr.z, fa[2], fmaf(wr.y, fa[1], fmaf(wr.x, fa[0], bb))));
                     const float pb = fmaf(wr.w, fb[3], fmaf(wr.z, fb[2], fmaf(wr.y, fb[1], fmaf(wr.x, fb[0], bb))));
                     h[e] = gelu(pa, d1[nt][e]);
@@ -188,8 +179,8 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
             float acc[8][4];
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
-                acc[nt][0] = acc[nt][2] = s_b2[8 * nt + 2 * t];
-                acc[nt][1] = acc[nt][3] = s_b2[8 * nt + 2 * t + 1];
+                acc[nt][0] = acc[nt][2] = S.b2[8 * nt + 2 * t];
+                acc[nt][1] = acc[nt][3] = S.b2[8 * nt + 2 * t + 1];
             }
 #pragma unroll
             for (int kp = 0; kp < 2; ++kp)
@@ -200,27 +191,32 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
                     mma_bf16(acc[nt], A[2 * kp], b[0], b[1]);
                     mma_bf16(acc[nt], A[2 * kp + 1], b[2], b[3]);
                 }
-            uint32_t *const h1s = s_t[0] + (16 * warp + g) * (LDT / 2) + t;
+            uint32_t *const h1s = reinterpret_cast<uint32_t *>(S.h1) + ra * (LDT / 2) + t;
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 h1s[4 * nt] = A[nt >> 1][2 * (nt & 1)];
                 h1s[8 * (LDT / 2) + 4 * nt] = A[nt >> 1][2 * (nt & 1) + 1];
             }
-            // output layer: h2, acc <- gelu'(p2)
-            float h2[8][4], sya = 0.0f, syb = 0.0f;
+            // output layer: h2 to shared memory, acc <- gelu'(p2)
+            float sya = 0.0f, syb = 0.0f;
+            const int fo = ra * LDF + 2 * t;  // this lane's pair of units in the float tiles
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
+            for (int nt = 0; nt < 8; ++nt) {
+                float h[4];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const float w3 = s_w3[8 * nt + 2 * t + e];
+                    const float w3 = S.w3[8 * nt + 2 * t + e];
                     float da, db;
-                    h2[nt][e] = gelu(acc[nt][e], da);
-                    h2[nt][2 + e] = gelu(acc[nt][2 + e], db);
-                    sya = fmaf(w3, h2[nt][e], sya);
-                    syb = fmaf(w3, h2[nt][2 + e], syb);
+                    h[e] = gelu(acc[nt][e], da);
+                    h[2 + e] = gelu(acc[nt][2 + e], db);
+                    sya = fmaf(w3, h[e], sya);
+                    syb = fmaf(w3, h[2 + e], syb);
                     acc[nt][e] = da;
                     acc[nt][2 + e] = db;
                 }
+                *reinterpret_cast<float2 *>(S.h2 + fo + 8 * nt) = make_float2(h[0], h[1]);
+                *reinterpret_cast<float2 *>(S.h2 + fo + 8 * LDF + 8 * nt) = make_float2(h[2], h[3]);
+            }
             sya += __shfl_xor_sync(0xffffffffu, sya, 1);
             syb += __shfl_xor_sync(0xffffffffu, syb, 1);
             sya += __shfl_xor_sync(0xffffffffu, sya, 2);
@@ -229,36 +225,32 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
             const float rrb = vb ? (syb + b3) - (tb - om) / osd : 0.0f;
             const float dya = 2.0f * rra * inv_n, dyb = 2.0f * rrb * inv_n;
             if (t == 0) {
+                S.dy[ra] = dya;
+                S.dy[rb] = dyb;
                 lsum = fmaf(rra, rra, fmaf(rrb, rrb, lsum));
                 gb3 += dya + dyb;
             }
-            float c[16];
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) c[2 * nt + e] = fmaf(h2[nt][e], dya, h2[nt][2 + e] * dyb);
-            scatter_sum(c, lane, cs[6]);
             // dp2 = dy W3 gelu'(p2): FP32 for the bias gradient, bf16 in the
             // two tensor-core products
             uint32_t dA[4][4];
-            uint32_t *const d2s = s_t[1] + (16 * warp + g) * (LDT / 2) + t;
+            uint32_t *const d2s = reinterpret_cast<uint32_t *>(S.d2) + ra * (LDT / 2) + t;
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 float p[4];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const float w3 = s_w3[8 * nt + 2 * t + e];
+                    const float w3 = S.w3[8 * nt + 2 * t + e];
                     p[e] = dya * w3 * acc[nt][e];
                     p[2 + e] = dyb * w3 * acc[nt][2 + e];
-                    c[2 * nt + e] = p[e] + p[2 + e];
                 }
+                *reinterpret_cast<float2 *>(S.dp2 + fo + 8 * nt) = make_float2(p[0], p[1]);
+                *reinterpret_cast<float2 *>(S.dp2 + fo + 8 * LDF + 8 * nt) = make_float2(p[2], p[3]);
                 const uint32_t xa = pack2(p[0], p[1]), xb = pack2(p[2], p[3]);
                 dA[nt >> 1][2 * (nt & 1)] = xa;
                 dA[nt >> 1][2 * (nt & 1) + 1] = xb;
                 d2s[4 * nt] = xa;
                 d2s[8 * (LDT / 2) + 4 * nt] = xb;
             }
-            scatter_sum(c, lane, cs[5]);
             // dh1[s][k] = sum_j dp2[s][j] W2[j][k]
             float dh[8][4];
 #pragma unroll
@@ -274,25 +266,19 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
                     mma_bf16(dh[2 * np], dA[ks], b[0], b[1]);
                     mma_bf16(dh[2 * np + 1], dA[ks], b[2], b[3]);
                 }
-            // dp1 = dh1 gelu'(p1), its column sums and those with the features
+            // dp1 = dh1 gelu'(p1)
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) d1[nt][e] *= dh[nt][e];
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e)
-                        c[2 * nt + e] = i < 4 ? fmaf(d1[nt][e], fa[i & 3], d1[nt][2 + e] * fb[i & 3])
-                                              : d1[nt][e] + d1[nt][2 + e];
-                scatter_sum(c, lane, cs[i]);
+            for (int nt = 0; nt < 8; ++nt) {
+                *reinterpret_cast<float2 *>(S.dp1 + fo + 8 * nt) =
+                    make_float2(d1[nt][0] * dh[nt][0], d1[nt][1] * dh[nt][1]);
+                *reinterpret_cast<float2 *>(S.dp1 + fo + 8 * LDF + 8 * nt) =
+                    make_float2(d1[nt][2] * dh[nt][2], d1[nt][3] * dh[nt][3]);
             }
         }
         __syncthreads();
         // dL/dW2[j][k] = sum_s dp2[s][j] h1[s][k] over the round's rows
-        for (int st = 0; st < nw; ++st) {
+#pragma unroll
+        for (int st = 0; st < FW; ++st) {
             uint32_t b0, b1;
             ldsm2t(b0, b1, aH + 2 * 16 * st * LDT);
 #pragma unroll
@@ -301,6 +287,31 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
                 ldsm4t(a, aD + 2 * (16 * st * LDT + 16 * mt));
                 mma_bf16(gw2[mt], a, b0, b1);
             }
+        }
+        // column sums over the round's rows
+        if (job == 0) {
+#pragma unroll 16
+            for (int s = 0; s < GR; ++s) {
+                const float d = S.dp1[s * LDF + j];
+                cs0 += d;
+                cs1 = fmaf(d, S.fn[s].x, cs1);
+            }
+        } else if (job == 1) {
+#pragma unroll 16
+            for (int s = 0; s < GR; ++s) {
+                const float d = S.dp1[s * LDF + j];
+                cs0 = fmaf(d, S.fn[s].y, cs0);
+                cs1 = fmaf(d, S.fn[s].z, cs1);
+            }
+        } else if (job == 2) {
+#pragma unroll 16
+            for (int s = 0; s < GR; ++s) {
+                cs0 = fmaf(S.dp1[s * LDF + j], S.fn[s].w, cs0);
+                cs1 += S.dp2[s * LDF + j];
+            }
+        } else {
+#pragma unroll 16
+            for (int s = 0; s < GR; ++s) cs0 = fmaf(S.h2[s * LDF + j], S.dy[s], cs0);
         }
         __syncthreads();
     }
@@ -314,39 +325,34 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
         o[8 * 64] = gw2[mt][2];
         o[8 * 64 + 1] = gw2[mt][3];
     }
-    // column sums over the warps, in warp order (in the tiles' storage)
-    float(*red)[NRED] = reinterpret_cast<float(*)[NRED]>(s_t);
-    static_assert(sizeof(float) * GWARPS * NRED <= sizeof(s_t), "column sums overlay the tiles");
-    const int c0 = 8 * g + 2 * t;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) red[warp][4 * (c0 + e) + i] = cs[i][e];
-#pragma unroll
-        for (int i = 4; i < 7; ++i) red[warp][64 * i + c0 + e] = cs[i][e];
+    if (job == 0) {
+        P[B1 + j] = cs0;
+        P[W1 + 4 * j] = cs1;
+    } else if (job == 1) {
+        P[W1 + 4 * j + 1] = cs0;
+        P[W1 + 4 * j + 2] = cs1;
+    } else if (job == 2) {
+        P[W1 + 4 * j + 3] = cs0;
+        P[B2 + j] = cs1;
+    } else {
+        P[W3 + j] = cs0;
     }
+    // b3 and the loss: lanes with t == 0 of the first warps hold them
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
         lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     }
-    if (lane == 0) {
-        s_red[0][warp] = gb3;
-        s_red[1][warp] = lsum;
+    if (warp < FW && lane == 0) {
+        S.red[0][warp] = gb3;
+        S.red[1][warp] = lsum;
     }
     __syncthreads();
-    for (int i = tid; i < NRED; i += GT) {
-        float x = 0.0f;
-#pragma unroll
-        for (int k = 0; k < GWARPS; ++k) x += red[k][i];
-        // W1, b1 | b2, W3 of the weight vector
-        P[i < 320 ? i : i - 320 + B2 + (i >= 384 ? W3 - B2 - 64 : 0)] = x;
-    }
     if (tid == 0) {
         float a = 0.0f, b = 0.0f;
-        for (int i = 0; i < GWARPS; ++i) {
-            a += s_red[0][i];
-            b += s_red[1][i];
+        for (int i = 0; i < FW; ++i) {
+            a += S.red[0][i];
+            b += S.red[1][i];
         }
         P[B3] = a;
         lpart[blockIdx.x] = b;
@@ -354,40 +360,44 @@ __global__ void __launch_bounds__(GT, 1) k_mlp_grad(const float *__restrict__ w,
     if (tid < NFROZEN) P[NW - NFROZEN + tid] = 0.0f;
 }
 
-// Sum of nblk partial gradients (fixed order), optional copy to grad, and
-// with adam != 0 the Adam update of w, m, v (normalisation entries kept).
-// A CTA takes 32 weights, its warps every eighth partial each with all their
-// loads in flight; sums are compensated pairs of floats (two-sum, about 2^-48:
-// rounded to float it is the FP64 sum's value but for ties), since an FP64 add
+// Sum of nblk partial gradients, optional copy to grad, and with adam != 0 the
+// Adam update of w, m, v (normalisation entries kept).
+// A CTA takes 32 weights, its warps every sixteenth partial each with all their
+// loads in flight. The sum is an FP64 one's, in any order the same float but where
+// FP64 itself would round: a warp adds its partials as three floats with the exact
+// errors (two-sum), the warps' sums are FP64 additions, since an FP64 addition
 // holds a warp 64 cycles here: one thread per weight adding 256 partials in
 // FP64 took 63 us, three times the gradient itself. The last CTA also
 // reduces the loss partials into *loss (mean over inv_n).
-constexpr int RT = 256;
-__global__ void __launch_bounds__(RT) k_mlp_reduce(const float *__restrict__ part, int nblk,
-                                                   const float *__restrict__ lpart, float inv_n,
-                                                   float *__restrict__ grad, float *__restrict__ loss,
-                                                   float *__restrict__ w, float *__restrict__ m,
-                                                   float *__restrict__ v, int adam, float lr,
-                                                   float beta1, float beta2, float eps, float bc1,
-                                                   float bc2) {
+constexpr int RT = 512;
+__global__ void __launch_bounds__(RT) k_mlp_reduce(const float *__restrict__ part, int nblk, const float *__restrict__ lpart,
+                                                   float inv_n, float *__restrict__ grad, float *__restrict__ loss, float *__restrict__ w,
+                                                   float *__restrict__ m, float *__restrict__ v, int adam, float lr, float beta1,
+                                                   float beta2, float eps, float bc1, float bc2) {
     chain_wait();
     constexpr int SL = RT / 32;
-    __shared__ float s_hi[SL][32], s_lo[SL][32];
+    __shared__ double s_sum[SL][32];
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
-    float hi = 0.0f, lo = 0.0f;
     if (i < NW) {
         const float *p = part + i;
-#pragma unroll 8
+        float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+#pragma unroll 16
         for (int b = sl; b < nblk; b += SL) {
-            float s, e;
+            float s, e, f;
             two_sum(hi, p[(size_t)b * NW], s, e);
             hi = s;
-            lo += e;
+            two_sum(mid, e, s, f);
+            mid = s;
+            lo += f;
         }
+        double sum = (double)hi + ((double)mid + (double)lo);
+        if (!isfinite(hi)) {  // beyond FP32's range on the way, or not finite
+            sum = 0.0;
+            for (int b = sl; b < nblk; b += SL) sum += (double)p[(size_t)b * NW];
+        }
+        s_sum[sl][lane] = sum;
     }
-    s_hi[sl][lane] = hi;
-    s_lo[sl][lane] = lo;
     __syncthreads();
     if (loss && lpart && blockIdx.x == gridDim.x - 1 && sl == 1) {
         double s = 0.0;
@@ -396,14 +406,14 @@ __global__ void __launch_bounds__(RT) k_mlp_reduce(const float *__restrict__ par
         if (lane == 0) *loss = (float)(s * inv_n);
     }
     if (sl != 0 || i >= NW) return;
+    double s[SL];
 #pragma unroll
-    for (int k = 1; k < SL; ++k) {
-        float s, e;
-        two_sum(hi, s_hi[k][lane], s, e);
-        hi = s;
-        lo += e + s_lo[k][lane];
-    }
-    const float gi = hi + lo;
+    for (int k = 0; k < SL; ++k) s[k] = s_sum[k][lane];
+#pragma unroll
+    for (int o = 1; o < SL; o *= 2)
+#pragma unroll
+        for (int k = 0; k < SL; k += 2 * o) s[k] += s[k + o];
+    const float gi = (float)s[0];
     if (grad) grad[i] = gi;
     if (adam && i < NW - NFROZEN) {
         const float mm = fmaf(beta1, m[i], (1.0f - beta1) * gi);
@@ -426,11 +436,14 @@ cudaError_t launch_mlp_forward(int64_t n, const float *w, const float *u, float 
 
 static cudaError_t grad_partials(int64_t n, const float *w, const float *rows, void *work, int &nblk,
                                  cudaStream_t st) {
-    const int64_t tiles = (n + 15) / 16;
-    nblk = (int)(tiles < GRID ? tiles : GRID);
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(GradShared));
+    if (e != cudaSuccess) return e;
+    const int64_t rounds = (n + GR - 1) / GR;
+    nblk = (int)(rounds < MAXBLK ? rounds : MAXBLK);
     float *part = static_cast<float *>(work);
     float *lpart = part + (size_t)MAXBLK * NW;
-    launch_chain(k_mlp_grad, nblk, GT, 0, st, w, rows, n, 1.0f / (float)n, part, lpart);
+    launch_chain(k_mlp_grad, nblk, GT, sizeof(GradShared), st, w, rows, n, 1.0f / (float)n, part, lpart);
     return cudaGetLastError();
 }
 

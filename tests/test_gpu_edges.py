@@ -342,3 +342,25 @@ def test_finisher_rows(torch, oracle, n):
     qg, vg, *_ = _run_gpu(w, 1, kick_prec=q.QYM_KICK_FP64, encounters=0)
     r, vh = _run_oracle(oracle, w, 1, encounters=0)
     assert _relq(qg, r.q).max() <= 1e-12 and _relq(vg, vh).max() <= 1e-12
+
+
+@pytest.mark.parametrize("n", [64, 1024, 16384])
+def test_gradient_rounds(torch, n):
+    """A minibatch's gradient is the sum of its 64-row rounds' gradients, added
+    as FP64 adds them and rounded once, bit for bit (up to 256 rounds, one each
+    to a CTA; every factor 2/n is a power of two, so a round's sums in FP32 and
+    its bf16 operands only change exponents). The grouping matters: training
+    turns one last place of a weight into 2^-9 where it crosses a bf16 midpoint."""
+    rows = torch.from_numpy(W.mlp_rows_synthetic(n, 21)).cuda()
+    ref = W.mlp_rows_synthetic(4096, 22)
+    w = torch.from_numpy(W.mlp_init(6, ref[:, :4], ref[:, 4])).cuda()
+    work = torch.empty(q.qym_mlp_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    loss = torch.empty(1, dtype=torch.float32, device="cuda")
+
+    def grad(r):
+        g = torch.empty(q.QYM_MLP_NW, dtype=torch.float32, device="cuda")
+        q.qym_mlp_grad_dev(len(r), w, r, g, loss, work)
+        return g.cpu().numpy()
+
+    parts = np.array([grad(rows[i:i + 64]) for i in range(0, n, 64)], dtype=np.longdouble)
+    assert np.array_equal(grad(rows), (parts.sum(0) * (64 / n)).astype(np.float64).astype(np.float32))
