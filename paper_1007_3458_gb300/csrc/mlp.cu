@@ -15,6 +15,9 @@
 // moments. A round's sums run over its 64 rows in order (FP32), a CTA's over its
 // rounds, CTA b of min(256, rounds) taking the rounds b, b + 256, ...; the
 // partials' sum is exact but for its last rounding.
+// The buffers are plain pointers, not const __restrict__: launches are chained, so
+// a kernel may be resident while the one before it still writes them, and every
+// load has to come after the wait and through the coherent path.
 // The operands the tensor cores take are bf16: h1 and W2 in the forward
 // product, dp2 = dL/dp2 with W2 (for dL/dh1) and with h1 (for dL/dW2) in the
 // backward ones. The other sums (dL/dW1, the biases, dL/dW3) stay in FP32.
@@ -45,8 +48,8 @@ struct GradShared {
 };
 }  // namespace
 
-__global__ void __launch_bounds__(256) k_mlp_forward(int64_t n, const float *__restrict__ w, const float *__restrict__ u,
-                                                     float *__restrict__ y) {
+__global__ void __launch_bounds__(256) k_mlp_forward(int64_t n, const float *w, const float *u,
+                                                     float *y) {
     chain_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float uu[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -88,8 +91,8 @@ __device__ __forceinline__ void ldsm2t(uint32_t &r0, uint32_t &r1, uint32_t a) {
 // above), 448 chains on the CTA's 256 threads. (A halving exchange in registers
 // instead is 3 us shorter at 16384 rows, in another order. Weights read from
 // global memory per tile and 16-bit transposing stores: 20 us.)
-__global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float *__restrict__ w, const float *__restrict__ rows, int64_t n,
-                                                    float inv_n, float *__restrict__ part, float *__restrict__ lpart) {
+__global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float *w, const float *rows, int64_t n,
+                                                    float inv_n, float *part, float *lpart) {
     chain_wait();
     extern __shared__ __align__(16) unsigned char g_gradsmem[];
     GradShared &S = *reinterpret_cast<GradShared *>(g_gradsmem);
@@ -370,9 +373,9 @@ __global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float *__restrict__ w,
 // FP64 took 63 us, three times the gradient itself. The last CTA also
 // reduces the loss partials into *loss (mean over inv_n).
 constexpr int RT = 512;
-__global__ void __launch_bounds__(RT) k_mlp_reduce(const float *__restrict__ part, int nblk, const float *__restrict__ lpart,
-                                                   float inv_n, float *__restrict__ grad, float *__restrict__ loss, float *__restrict__ w,
-                                                   float *__restrict__ m, float *__restrict__ v, int adam, float lr, float beta1,
+__global__ void __launch_bounds__(RT) k_mlp_reduce(const float *part, int nblk, const float *lpart,
+                                                   float inv_n, float *grad, float *loss, float *w,
+                                                   float *m, float *v, int adam, float lr, float beta1,
                                                    float beta2, float eps, float bc1, float bc2) {
     chain_wait();
     constexpr int SL = RT / 32;

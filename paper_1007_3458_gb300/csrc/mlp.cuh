@@ -69,7 +69,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 // normalised features fn = (u - mean) / std
-__device__ __forceinline__ void normalise(const float *__restrict__ w, const float (&u)[4],
+__device__ __forceinline__ void normalise(const float *w, const float (&u)[4],
                                           float (&fn)[4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) fn[i] = (u[i] - w[MEAN + i]) / w[STD + i];
@@ -92,7 +92,7 @@ struct W2FromGlobal {
 // rows g and g+8. Out: A = bf16(h1) as the A fragments of the four k-steps of
 // layer 2, acc = p2 = W2 h1 + b2 in C layout (n-tile nt: cols 8 nt + 2t, +1).
 template <class BLoad>
-__device__ __forceinline__ void layers12(const float *__restrict__ w, const BLoad &bload,
+__device__ __forceinline__ void layers12(const float *w, const BLoad &bload,
                                          const float (&fa)[4], const float (&fb)[4], int g, int t,
                                          uint32_t (&A)[4][4], float (&acc)[8][4]) {
 #pragma unroll
@@ -135,7 +135,7 @@ __device__ __forceinline__ void layers12(const float *__restrict__ w, const BLoa
 
 // Output layer of a tile: y for rows g and g+8 (summed over the quad, so
 // every lane of quad g holds both).
-__device__ __forceinline__ void output(const float *__restrict__ w, const float (&acc)[8][4], int t,
+__device__ __forceinline__ void output(const float *w, const float (&acc)[8][4], int t,
                                        float &ya, float &yb) {
     float sa = 0.0f, sb = 0.0f;
 #pragma unroll
@@ -157,7 +157,7 @@ __device__ __forceinline__ void output(const float *__restrict__ w, const float 
 
 // Network output y for the 32 samples of a warp, one per lane (fn: the
 // lane's normalised features). Every lane of the warp must call it.
-__device__ __forceinline__ float warp_forward(const float *__restrict__ w, const float (&fn)[4]) {
+__device__ __forceinline__ float warp_forward(const float *w, const float (&fn)[4]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     float mine = 0.0f;
 #pragma unroll 1

@@ -364,3 +364,31 @@ def test_gradient_rounds(torch, n):
 
     parts = np.array([grad(rows[i:i + 64]) for i in range(0, n, 64)], dtype=np.longdouble)
     assert np.array_equal(grad(rows), (parts.sum(0) * (64 / n)).astype(np.float64).astype(np.float32))
+
+
+def test_training_is_its_steps(torch):
+    """Training over many minibatches gives the bits of the gradient and Adam
+    calls with the stream synchronised after each: no kernel of the chain reads
+    a weight or a partial sum from before the kernel that writes it."""
+    n, batch, epochs, lr, lr1 = 40000, 1000, 3, 2e-3, 2e-5
+    rows = torch.from_numpy(W.mlp_rows_synthetic(n, 23)).cuda()
+    ref = W.mlp_rows_synthetic(4096, 24)
+    w0 = torch.from_numpy(W.mlp_init(7, ref[:, :4], ref[:, 4])).cuda()
+    work = torch.empty(q.qym_mlp_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    a = [w0.clone(), torch.zeros_like(w0), torch.zeros_like(w0)]
+    b = [x.clone() for x in a]
+    steps = n // batch * epochs
+    losses = torch.empty(steps, dtype=torch.float32, device="cuda")
+    q.qym_mlp_train_dev(*a, 0, rows, n, batch, epochs, lr, lr1, losses, work)
+    g = torch.empty(q.QYM_MLP_NW, dtype=torch.float32, device="cuda")
+    loss = torch.empty(1, dtype=torch.float32, device="cuda")
+    lr, lr1 = float(np.float32(lr)), float(np.float32(lr1))
+    for s in range(steps):
+        lo = s % (n // batch) * batch
+        q.qym_mlp_grad_dev(batch, b[0], rows[lo:lo + batch], g, loss, work)
+        torch.cuda.synchronize()
+        assert loss.item() == losses[s].item()
+        rate = lr1 + 0.5 * (lr - lr1) * (1.0 + np.cos(np.pi * s / steps))
+        q.qym_mlp_adam_dev(*b, g, s + 1, rate)
+        torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
