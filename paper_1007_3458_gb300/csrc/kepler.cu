@@ -10,8 +10,8 @@
 // SM, whatever the number of active lanes. So (1) only arithmetic on the state
 // goes there: comparisons, scalings by powers of two and conversions work on the
 // bits, the residual's scale and (until it matters) the root's bracket are FP32
-// with the margins stated at each, square roots and reciprocals take one step from FP32
-// (pair64.cuh); (2) F' and F'' are formed only where a step follows; (3) a warp
+// with the margins stated at each, square roots, reciprocals and quotients are rounded
+// from FP32 approximations (pair64.cuh); (2) F' and F'' are formed only where a step follows; (3) a warp
 // iterates while at least kPackBelow of its lanes do, then the CTA's unfinished
 // bodies are packed into full warps (some 5% of bodies need another evaluation,
 // that is four of five warps). 1,048,576 test particles with NEWTON32: 369 FP64
@@ -65,7 +65,11 @@ __device__ __forceinline__ void stumpff(double y, double &C, double &S) {
     }
 }
 
-// F, F', F'' of the universal Kepler equation (Appendix), sig = r0.v0/sqrt(mu)
+// F, F', F'' of the universal Kepler equation (Appendix), sig = r0.v0/sqrt(mu).
+// Sums and products that a compiler may fuse in one place and not in another are
+// written out with their roundings, here and at the state's dot products: the root
+// and the drifted state are the same bits whatever is compiled around them (a last
+// place here grows to 1e-8 of a velocity in an ensemble's encounters).
 struct KepEq {
     double sqmu_dt, r0, sig, alpha, b;  // b = 1 - r0 alpha
     // F at x with C, S; sc: the sum of F's terms' magnitudes in FP32 (within
@@ -76,7 +80,7 @@ struct KepEq {
         const double t1 = sig * x2, t2 = b * x2 * x;
         sc = fabsf(p64::lead(sqmu_dt, 0)) + fabsf(p64::lead(t1, 0) * p64::lead(C, 0)) +
              fabsf(p64::lead(t2, 0) * p64::lead(S, 0)) + p64::lead(r0, 0) * fabsf(p64::lead(x, 0));
-        return t1 * C + t2 * S + r0 * x - sqmu_dt;
+        return fma(r0, x, __dadd_rn(__dmul_rn(t1, C), __dmul_rn(t2, S))) - sqmu_dt;
     }
     __device__ __forceinline__ double scale(double x, double C, double S) const {
         const double x2 = x * x;
@@ -84,8 +88,8 @@ struct KepEq {
     }
     __device__ __forceinline__ void slopes(double x, double C, double S, double &Fp, double &Fpp) const {
         const double x2 = x * x, y = alpha * x2, oyS = 1.0 - y * S;
-        Fp = sig * x * oyS + b * x2 * C + r0;
-        Fpp = sig * (1.0 - y * C) + b * x * oyS;
+        Fp = __dadd_rn(fma(b * x2, C, __dmul_rn(sig * x, oyS)), r0);
+        Fpp = fma(sig, fma(-y, C, 1.0), __dmul_rn(b * x, oyS));
     }
 };
 
@@ -275,11 +279,12 @@ __device__ __forceinline__ bool kep_iterate(const KeplerArgs &a, int64_t r, doub
     const bool F_ok = p64::finite_bits(F);
     double scale = 0.0;
     if (F_ok) {
-        // |F| <= 1e-14 sum |terms|, in FP32 where its range holds (the factor
-        // covers the FP32 sum, so no residual above 1e-14 passes)
-        bool small;
-        if (sc > 1e-18f && sc < 1e30f) {
-            small = fabsf(p64::lead(F, 0)) <= 1e-14f * (1.0f - 4e-6f) * sc;
+        // |F| <= 1e-14 sum |terms|, in FP32 where its range holds and the two sides
+        // differ by more than the FP32 sum's error: the decision is the FP64 one
+        bool small = false;
+        const float Fa = fabsf(p64::lead(F, 0)), lim = 1e-14f * sc;
+        if (sc > 1e-18f && sc < 1e30f && !(fabsf(Fa - lim) <= 4e-6f * lim)) {
+            small = Fa < lim;
         } else {
             scale = eq.scale(x, s.C, s.S);
             small = fabs(F) <= 1e-14 * scale;
@@ -323,12 +328,12 @@ __device__ __forceinline__ bool kep_iterate(const KeplerArgs &a, int64_t r, doub
         if (p64::hi_abs(z) < 0x3eb0c6f7) {  // 1e-6
             dx = rf * fma(z, fma(13.0 / 32.0, z, 0.5), 1.0);
         } else {
-            const double w = fabs(16.0 - 20.0 * z);
-            const double rt = p64::mid_range(w) ? w * p64::rsqrt_mid(w) : sqrt(w);
-            dx = 5.0 * rf * p64::rcp(1.0 + rt);
+            double irt;
+            const double den = 1.0 + p64::sqrt_rcp(fabs(16.0 - 20.0 * z), irt);
+            dx = p64::div(5.0 * rf, den, p64::rcp(den));
         }
     } else {
-        dx = F * iFp;
+        dx = p64::div(F, Fp, iFp);
     }
     double xn = x - dx;
     // bisect when the step is not finite, leaves the bracket, or fails
@@ -396,12 +401,12 @@ __global__ void __launch_bounds__(T, 512 / T) k_kepler(const __grid_constant__ K
         }
     }
     const double dt = a.dt;
-    const double r0sq = qx * qx + qy * qy + qz * qz;
+    const double r0sq = fma(qz, qz, fma(qy, qy, qx * qx));
     double ir0 = 0.0;
     const double r0 = p64::sqrt_rcp(r0sq, ir0);
     const bool body = act && !(r0 == 0.0);
-    const double vv = vx * vx + vy * vy + vz * vz;
-    const double rv = qx * vx + qy * vy + qz * vz;
+    const double vv = fma(vz, vz, fma(vy, vy, vx * vx));
+    const double rv = fma(qz, vz, fma(qy, vy, qx * vx));
     float u[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     double sigma = 0.0;
     bool bound = false;  // in the learned guess's domain
@@ -491,7 +496,8 @@ __global__ void __launch_bounds__(T, 512 / T) k_kepler(const __grid_constant__ K
         const double f = 1.0 - x2C * ir0;
         const double g = dt - x2 * x * S * isqmu;
         const double nx = f * qx + g * vx, ny = f * qy + g * vy, nz = f * qz + g * vz;
-        const double irr = p64::rsqrt64(nx * nx + ny * ny + nz * nz);
+        double irr;
+        p64::sqrt_rcp(nx * nx + ny * ny + nz * nz, irr);
         const double fd = sqmu * x * (y * S - 1.0) * irr * ir0;
         const double gd = 1.0 - x2C * irr;
         const double ux = fd * qx + gd * vx, uy = fd * qy + gd * vy, uz = fd * qz + gd * vz;

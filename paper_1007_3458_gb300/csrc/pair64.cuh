@@ -314,25 +314,39 @@ __device__ __forceinline__ double to_double(float x) {
     return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
 }
 
-// Reciprocal, reciprocal square root and square root of a positive normal x by
-// one third-order step from the FP32 approximation (Householder's method: the
-// binomial series in the residual e = 1 - x y or 1 - x y^2, |e| < 2^-20, to e^2;
-// the next term is below 2^-61), within an ulp: three to eight FP64 instructions
-// where the library's correctly rounded forms take ten and more. Outside the
-// exponents [-1000, 1000] the library forms.
+// Reciprocal, quotient, reciprocal square root and square root of positive normal
+// numbers: one third-order step from the FP32 approximation (Householder's method:
+// the binomial series in the residual e = 1 - x y or 1 - x y^2, |e| < 2^-20, to e^2;
+// the next term is below 2^-61) gives y within an ulp, and one step with the exact
+// residual of a multiply-add the rounded value (Markstein 1990): 1/x, a/b, sqrt(x)
+// and 1/sqrt(x)'s rounded root are what the library's correctly rounded forms return,
+// for five to nine FP64 instructions where those take ten and more. Outside the
+// exponents [-1000, 1000] (quotient: [-500, 500]) the library forms.
 __device__ __forceinline__ bool mid_range(double x) {
     const int hi = __double2hiint(x);
     return hi > (23 << 20) && hi < (2023 << 20);
+}
+__device__ __forceinline__ bool near_one(double x) {
+    const int hi = hi_abs(x);
+    return hi > (523 << 20) && hi < (1523 << 20);
 }
 __device__ __forceinline__ double rcp(double x) {
     if (!mid_range(x)) return 1.0 / x;
     const int k = (__double2hiint(x) >> 20) - 1023;
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(lead(x, k)));
-    const double y = mul_pow2(to_double(r), -k);
+    double y = mul_pow2(to_double(r), -k);
     const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    y = fma(y, fma(e, e, e), y);
+    return fma(y, fma(-x, y, 1.0), y);
 }
+// a / b from ib = rcp(b)
+__device__ __forceinline__ double div(double a, double b, double ib) {
+    if (!near_one(a) || !near_one(b)) return a / b;
+    const double q = a * ib;
+    return fma(ib, fma(-b, q, a), q);
+}
+// within an ulp of 1 / sqrt(x)
 __device__ __forceinline__ double rsqrt_mid(double x) {
     const int k = ((__double2hiint(x) >> 20) - 1023) & ~1;  // even
     float r;
@@ -342,8 +356,7 @@ __device__ __forceinline__ double rsqrt_mid(double x) {
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 __device__ __forceinline__ double rsqrt64(double x) { return mid_range(x) ? rsqrt_mid(x) : rsqrt(x); }
-// square root (the correction s + y (x - s^2) / 2 rounds it correctly but for
-// rare ties, Markstein) with its reciprocal
+// square root and the reciprocal of that rounded root
 __device__ __forceinline__ double sqrt_rcp(double x, double &ir) {
     if (!mid_range(x)) {
         const double r = sqrt(x);

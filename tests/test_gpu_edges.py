@@ -392,3 +392,24 @@ def test_training_is_its_steps(torch):
         q.qym_mlp_adam_dev(*b, g, s + 1, rate)
         torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+def _batch_bits():
+    import os
+    return np.load(os.path.join(os.path.dirname(__file__), "golden", "batch_bits.npz"))
+
+
+def _same_bits(got, ref):
+    assert np.array_equal(got, ref), (np.mean(got != ref), np.abs(got - ref).max())
+
+
+@pytest.mark.parametrize("name,dt", [("fwd", 2 * np.pi / 40), ("back", -0.7)])
+def test_kepler_bits(torch, name, dt):
+    """E_Kep by Laguerre's method, bound and unbound orbits: the bits of the form
+    with IEEE square roots and divisions throughout (recorded)."""
+    g = _batch_bits()
+    q0, v0 = torch.from_numpy(g["kepler_q"]).cuda(), torch.from_numpy(g["kepler_v"]).cuda()
+    q1, v1 = torch.empty_like(q0), torch.empty_like(v0)
+    q.qym_kepler_drift_dev(q0.shape[1], q0, v0, q1, v1, 1.0, dt, q.QYM_SOLVER_LAGUERRE, q.QYM_GUESS_STANDARD)
+    _same_bits(q1.cpu().numpy(), g[f"kepler_{name}_q"])
+    _same_bits(v1.cpu().numpy(), g[f"kepler_{name}_v"])
