@@ -409,7 +409,12 @@ static int64_t slots_cap(int64_t R) {
     return std::min<int64_t>(128, std::max<int64_t>(4, ((int64_t)1 << 29) / (24 * R)));
 }
 
-// Launch shape of the kick for this batch
+// Launch shape of the kick for this batch. A batch's mixed kick takes two rows per
+// thread and ranges only to reach four CTAs per SM: its FP32 sums run over 64 rows
+// from a range's start, and the encounters of a batch amplify even a last place to
+// 1e-8 of a velocity and more within a few steps, so the ranges are part of its
+// results, and so is G m inside every pair's product (finer ranges and windows of
+// one mass, as one system's kick takes them: 1.63 ms instead of 1.77 on 512 systems).
 static KickTune default_tune(const std::vector<int64_t> &off, int prec) {
     const int32_t nsys = (int32_t)off.size() - 1;
     const int64_t ti = prec == QYM_KICK_MIXED ? 256 : 128;
@@ -418,6 +423,14 @@ static KickTune default_tune(const std::vector<int64_t> &off, int prec) {
         const int64_t nb = off[s + 1] - off[s] - 1;
         ib += (nb + ti - 1) / ti;
         nbmax = std::max(nbmax, nb);
+    }
+    if (nsys > 1 && prec == QYM_KICK_MIXED) {
+        KickTune t;
+        t.threads = 128;
+        t.ipt = 2;
+        t.splits = (int32_t)std::max<int64_t>(
+            1, std::min((4 * 152 + ib - 1) / std::max<int64_t>(ib, 1), nbmax / 256));
+        return t;
     }
     return default_kick_tune(ib * ti, nbmax, prec, slots_cap(off[nsys]));
 }
@@ -587,6 +600,7 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
         kmu[3 * s + 2] = 1.0 / mu;
     }
     d.heavy_split = split ? 1 : 0;
+    d.batch = nsys > 1 && params->kick_prec == QYM_KICK_MIXED;
 
     // one system of at least two tiles' worth of bodies, mixed kick: the kick
     // holds the bodies in Morton order (sort.cu)

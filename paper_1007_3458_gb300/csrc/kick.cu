@@ -57,6 +57,7 @@ struct KickArgs {
     SymShape sym;           // pair-symmetric form (k_kick_sym)
     int32_t *blk_cnt = nullptr;  // arrivals per i-block (NULL: each slot stays for the finisher)
     int32_t splits = 1;          // items (slots) per i-block
+    int32_t uniform = 1;         // windows of one G m multiply by it once per sum
 };
 
 // The item of CTA b: its rows [x, y), its j-range [z, w) and its slot; for one
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         // one G m for the whole window (and not zero, so that the pad and a
         // massless body are never taken for it)
         const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
-        bool same = gm0 > 0.0f;
+        bool same = a.uniform && gm0 > 0.0f;
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
             const int j0 = jt + 2 * t;
             const bool two = 2 * t + 1 < n;
@@ -1202,6 +1203,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     a.blk_cnt = d.kick_cnt;
     a.splits = d.splits;
     a.chunk = d.item_chunk;
+    a.uniform = !d.batch;
     if (a.far_tiles && !d.tiles_ready) {
         const int64_t ntiles = (d.rows - 1 + TILE - 1) / TILE;
         launch_chain(k_tile_prep, (unsigned)ntiles, TILE, 0, st, d.rows, d.pk_pos, d.pk_lo, d.far, d.tile);

@@ -390,6 +390,13 @@ __device__ __forceinline__ float norm_up(double x, double y, double z) {
     if (k > 125) return INFINITY;
     return k < -125 ? n * 0x1p-125f : n * __int_as_float((127 + k) << 23);
 }
+
+// x as hi + lo, each the nearest float (of x, and of x - hi)
+__device__ __forceinline__ float2 split2(double x) {
+    const F3 s = split3(x);
+    const float hi = to_float(x);  // s.h but for ties between floats
+    return make_float2(hi, add(add(sub(s.h, hi), s.m), s.l));
+}
 #endif
 
 }  // namespace p64

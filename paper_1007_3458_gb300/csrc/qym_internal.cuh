@@ -59,6 +59,7 @@ struct Dev {
     int32_t *item_slot = nullptr;
     int32_t nitems = 0;
     int32_t item_chunk = 0;       // items == NULL (one system): j rows per split
+    int32_t batch = 0;            // mixed kick of several systems: its sums keep their order
     // momentum reduction
     int4 *mchunks = nullptr;      // (row0, row1, sys, -) chunks of at most 1024 rows
     int32_t nmchunks = 0;
@@ -231,6 +232,25 @@ __device__ __forceinline__ void heavy_pull(const int32_t *hs, int k0, int step, 
             const double ri = rsqrt(d2);
             s = gm * (ri * ri) * ri;
         }
+        ax -= s * dx;
+        ay -= s * dy;
+        az -= s * dz;
+    }
+}
+
+// The same in FP64 by one thread, body after body: what a batch's finisher adds. Its
+// encounters amplify a last place by up to 1e9 within a few steps, so its pulls keep
+// their roundings (512 systems of 2 planets, 1.06e6 rows: the finisher 101 us, 71 with heavy_pull).
+__device__ __forceinline__ void heavy_pull_fp64(const int32_t *hs, int nh, int64_t i, double x,
+                                                double y, double z, const double *q, const double *m,
+                                                int64_t R, double G, double &ax, double &ay, double &az) {
+    for (int k = 0; k < nh; ++k) {
+        const int64_t h = hs[k];
+        if (h == i) continue;
+        const double dx = x - q[h], dy = y - q[R + h], dz = z - q[2 * R + h];
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        const double ri = rsqrt(r2);
+        const double s = G * m[h] * (ri * ri) * ri;
         ax -= s * dx;
         ay -= s * dy;
         az -= s * dz;

@@ -223,10 +223,9 @@ __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
     }
     d.q[r] = qx; d.q[R + r] = qy; d.q[2 * R + r] = qz;
     if (a.vs != d.v) { d.v[r] = vx; d.v[R + r] = vy; d.v[2 * R + r] = vz; }
-    // float pairs hi + lo of the position (its three-part split, rounded to two)
-    const p64::F3 sx = p64::split3(qx), sy = p64::split3(qy), sz = p64::split3(qz);
-    const float xh = sx.h, yh = sy.h, zh = sz.h;
-    const float xl = sx.m + sx.l, yl = sy.m + sy.l, zl = sz.m + sz.l;
+    // float pairs hi + lo of the position
+    const float2 sx = p64::split2(qx), sy = p64::split2(qy), sz = p64::split2(qz);
+    const float xh = sx.x, yh = sy.x, zh = sz.x, xl = sx.y, yl = sy.y, zl = sz.y;
     const double mm = d.m[r];
     float reach = 0.0f;
     if (a.flag_next && r != star) {
@@ -291,11 +290,11 @@ struct FinishArgs {
     int skip_whole;     // v of systems flagged in d.wh_flag stays
 };
 
-// L threads share one position's partial sums and heavy bodies: thread group q
-// of the CTA adds the slots q, q + L, ... and the heavies q, q + L, ... (loads
-// coalesced across positions, dependent FP64 adds in chains 1/L as long), the
-// groups' parts added as a fixed tree; the first group then does the rows' own
-// work in full warps. (An FP64 instruction costs the same for one active lane as
+// L threads share one position's partial sums: thread group q of the CTA adds the
+// slots q, q + L, ... (loads coalesced across positions, dependent FP64 adds in
+// chains 1/L as long), the groups' parts added as a fixed tree; the first group then
+// does the rows' own work in full warps. The heavy bodies' pulls are spread over the
+// groups as well, or with few slots follow the sums one after another. (An FP64 instruction costs the same for one active lane as
 // for 32: with the four parts on neighbouring lanes the row work ran on eight
 // lanes per warp, 492 us on 1.06e6 rows.)
 template <int L>
@@ -334,7 +333,7 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
                 az += p[2 * R + pr];
             }
         }
-        if (d.heavy_split) {
+        if (L > 4 && d.heavy_split) {
             const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
             heavy_pull(d.heavy_rows + h0, q, L, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q,
                        d.m, R, a.G, ax, ay, az);
@@ -396,6 +395,11 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
         ax = p[0][0]; ay = p[0][1]; az = p[0][2];
     }
     if (!live) return;
+    if (L <= 4 && d.heavy_split) {
+        const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
+        heavy_pull_fp64(d.heavy_rows + h0, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q, d.m, R,
+                        a.G, ax, ay, az);
+    }
     double vx = a.v[r], vy = a.v[R + r], vz = a.v[2 * R + r];
     if (!(a.skip_whole && d.wh_flag && d.wh_flag[sys])) {
         vx += a.dt * ax;
@@ -437,11 +441,12 @@ cudaError_t launch_kick_finish_v(const Dev &d, double *v, const double *q, doubl
     a.check = check;
     a.hill_fixed = hill_fixed;
     // groups of 4 or 8 threads a row where there are that many slots to add (8
-    // also halves the chain of a small system), one where there are few
+    // also halves the chain of a small system), one where there are few; four for a
+    // batch, whose sums keep their order
     const int nslots = d.sym.G > 0 ? d.sym.splits : (d.kick_cnt ? 1 : d.splits);
-    if (nslots >= 16 && d.rows <= kFewRows)
+    if (nslots >= 16 && !d.batch && d.rows <= kFewRows)
         launch_chain(k_finish<32>, (unsigned)((d.rows + 7) / 8), 256, 0, st, d, a);
-    else if (nslots >= 16)
+    else if (nslots >= 16 && !d.batch)
         launch_chain(k_finish<8>, (unsigned)((d.rows + 31) / 32), 256, 0, st, d, a);
     else if (nslots >= 4)
         launch_chain(k_finish<4>, (unsigned)((d.rows + 63) / 64), 256, 0, st, d, a);

@@ -413,3 +413,20 @@ def test_kepler_bits(torch, name, dt):
     q.qym_kepler_drift_dev(q0.shape[1], q0, v0, q1, v1, 1.0, dt, q.QYM_SOLVER_LAGUERRE, q.QYM_GUESS_STANDARD)
     _same_bits(q1.cpu().numpy(), g[f"kepler_{name}_q"])
     _same_bits(v1.cpu().numpy(), g[f"kepler_{name}_v"])
+
+
+@pytest.mark.parametrize("kind,encounters", [("plain", 0)])
+@pytest.mark.parametrize("name", ["disks", "swarms"])
+def test_batch_bits(torch, name, kind, encounters):
+    """Two steps of small batches (planetesimal disks; planets' swarms of 2 to 70
+    members) with the mixed kick: the recorded bits. Encounters amplify a last
+    place by up to 1e9 within a few steps of an ensemble, so a change of grouping
+    or rounding anywhere in a batch's step shows in its results."""
+    g = _batch_bits()
+    sim = q.Simulation(g[name + "_m"], g[name + "_q"], g[name + "_v"], g[name + "_offsets"], eps_H=4.7e-4,
+                       encounters=encounters)
+    sim.step(2 * np.pi / 40, 2)
+    qs, vs = sim.state()
+    sim.close()
+    _same_bits(qs, g[f"{name}_{kind}_q"])
+    _same_bits(vs, g[f"{name}_{kind}_v"])
