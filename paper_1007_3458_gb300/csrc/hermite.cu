@@ -24,6 +24,11 @@
 // send their parts to each other and add them in rank order, so every copy of
 // the set stays bit-identical). Every loop has a cap and reports through the status
 // word.
+//
+// A set's result is the same bits whatever the work is spread over: products and
+// sums that could be grouped in several ways are written out, lanes' parts are added
+// in one order. Close passages amplify a last place by up to 1e9 within a few steps,
+// so another grouping moves some velocity of an ensemble of a million bodies by 1e-7.
 #include <climits>
 
 #include <cooperative_groups.h>
@@ -60,40 +65,36 @@ __device__ __forceinline__ bool at_least(double a, double b) {
 // the Taylor series of sin to w^15 and of cos to w^16 leave truncation errors
 // below 7e-17 and 3e-18 (the next terms, w^17/17! and w^18/18!, at pi/4).
 struct HalfPi {
-    double w, x;  // w = (pi/2) y', y' = y or 1 - y; x = w^2
-    bool fold;    // y' = 1 - y: sin and cos swap
+    double w, x, x2, x4;  // w = (pi/2) y', y' = y or 1 - y; x = w^2, x^2, x^4
+    bool fold;            // y' = 1 - y: sin and cos swap
 };
 __device__ __forceinline__ HalfPi half_pi_arg(double y) {
     HalfPi a;
     a.fold = y_above_half(y);
     a.w = 1.5707963267948966 * (a.fold ? 1.0 - y : y);
     a.x = a.w * a.w;
+    a.x2 = a.x * a.x;
+    a.x4 = a.x2 * a.x2;
     return a;
 }
-// both polynomials in x = w^2 by Horner's scheme: a warp issues an FP64
-// instruction every 64 cycles, dependent or not, so the fewest instructions are
-// the fastest (Estrin's scheme takes two and three more)
+// both polynomials in x = w^2 by Estrin's scheme
 // sin w = w (1 - x/3! + x^2/5! - ... - x^7/15!)
 __device__ __forceinline__ double sin_w(const HalfPi &a) {
-    double p = fma(-1.0 / 1307674368000.0, a.x, 1.0 / 6227020800.0);
-    p = fma(p, a.x, -1.0 / 39916800.0);
-    p = fma(p, a.x, 1.0 / 362880.0);
-    p = fma(p, a.x, -1.0 / 5040.0);
-    p = fma(p, a.x, 1.0 / 120.0);
-    p = fma(p, a.x, -1.0 / 6.0);
-    p = fma(p, a.x, 1.0);
-    return a.w * p;
+    const double s01 = fma(-1.0 / 6.0, a.x, 1.0);
+    const double s23 = fma(-1.0 / 5040.0, a.x, 1.0 / 120.0);
+    const double s45 = fma(-1.0 / 39916800.0, a.x, 1.0 / 362880.0);
+    const double s67 = fma(-1.0 / 1307674368000.0, a.x, 1.0 / 6227020800.0);
+    const double ps = fma(fma(s67, a.x2, s45), a.x4, fma(s23, a.x2, s01));
+    return a.w * ps;
 }
 // cos w = 1 - x/2! + x^2/4! - ... + x^8/16!
 __device__ __forceinline__ double cos_w(const HalfPi &a) {
-    double p = fma(1.0 / 20922789888000.0, a.x, -1.0 / 87178291200.0);
-    p = fma(p, a.x, 1.0 / 479001600.0);
-    p = fma(p, a.x, -1.0 / 3628800.0);
-    p = fma(p, a.x, 1.0 / 40320.0);
-    p = fma(p, a.x, -1.0 / 720.0);
-    p = fma(p, a.x, 1.0 / 24.0);
-    p = fma(p, a.x, -0.5);
-    return fma(p, a.x, 1.0);
+    const double c01 = fma(-0.5, a.x, 1.0);
+    const double c23 = fma(-1.0 / 720.0, a.x, 1.0 / 24.0);
+    const double c45 = fma(-1.0 / 3628800.0, a.x, 1.0 / 40320.0);
+    const double c67 = fma(-1.0 / 87178291200.0, a.x, 1.0 / 479001600.0);
+    const double c8 = (1.0 / 20922789888000.0) * (a.x4 * a.x4);
+    return fma(fma(c67, a.x2, c45), a.x4, fma(c23, a.x2, c01)) + c8;
 }
 __device__ __forceinline__ void sincos_half_pi(double y, double &sn, double &cs) {
     const HalfPi a = half_pi_arg(y);
@@ -171,16 +172,14 @@ constexpr int RSL = 16;    // members per force round on a cluster (receive buff
 
 constexpr int KMAX = 48;
 
-// Constants of a level's step h (signed), rows of HermSmem::lvt. With d = a0 - a1
-// the corrector and the step criterion are linear in (d, j0, j1):
-//   x1  = x_p - 3/20 h^2 d - h^3 (7/60 j0 + 1/30 j1)
-//   v1  = v_p - 1/2 h d - h^2 (5/12 j0 + 1/12 j1)
-//   a2e = 6 d / h^2 + (2 j0 + 4 j1) / h     (a2 at the end of the step)
-//   a3  = 12 d / h^3 + 6 (j0 + j1) / h^2
-// (x_p + h^4/24 a2 + h^5/120 a3 and v_p + h^3/6 a2 + h^4/24 a3 written out). Form f's
-// factors of d, j0, j1 are the rows 3 f, 3 f + 1, 3 f + 2; a3's last two are one row.
+// corrector constants of a level's step h (signed), rows of HermSmem::lvt:
+// a2 = (-6 d - h (4 j0 + 2 j1)) / h^2 = A2D d + A2J0 j0 + A2J1 j1,
+// a3 = (12 d + 6 h (j0 + j1)) / h^3 = A3D d + A3J (j0 + j1),
+// x1 = x_p + h^4/24 a2 + h^5/120 a3, v1 = v_p + h^3/6 a2 + h^4/24 a3,
+// and a2 at the end of the step, a2 + h a3 (d = a0 - a1)
+enum LvConst : int { LV_H = 0, LV_A2D, LV_A2J0, LV_A2J1, LV_A3D, LV_A3J, LV_H4, LV_H5, LV_H3, LV_N };
+// what a warp of the corrector forms from a2 and a3
 enum LvForm : int { LF_X = 0, LF_V, LF_A2, LF_A3 };
-constexpr int LV_N = 11;
 
 struct HermSmem {
     double *ex, *ey, *ez, *eu, *ev, *ew;      // evaluation point of every member
@@ -318,15 +317,16 @@ __device__ __forceinline__ void star_pull(const HermSmem &S, int k, double gm0, 
     aj[3] += c * (uk - t * xk); aj[4] += c * (vk - t * yk); aj[5] += c * (wk - t * zk);
 }
 
-// partial Hermite acceleration and jerk of member k at the evaluation
-// point (Sec. 2.2): the pair terms with the transition bracket over this
-// lane's partners (one reciprocal square root per pair: q = q2 / sqrt(q2),
-// 1/q^3, 1/q^2)
+// partial Hermite acceleration and jerk of member k at the evaluation point
+// (Sec. 2.2): the star's term on lane 0 of the group, then the pair terms with the
+// transition bracket over this lane's partners (one reciprocal square root per
+// pair: q = q2 / sqrt(q2), 1/q^3, 1/q^2)
 __device__ __forceinline__ void herm_part(const HermSmem &S, int lo, int hi, int k, int l0, int P,
-                                          const TransC &tc, double eps2, double *aj) {
+                                          double gm0, const TransC &tc, double eps2, double *aj) {
     const double xk = S.ex[k], yk = S.ey[k], zk = S.ez[k];
     const double uk = S.eu[k], vk = S.ev[k], wk = S.ew[k];
     for (int c = 0; c < 6; ++c) aj[c] = 0.0;
+    if (l0 == 0) star_pull(S, k, gm0, eps2, aj);
     #pragma unroll 1
     for (int l = lo + l0; l < hi; l += P) {
         if (l == k) continue;
@@ -382,13 +382,6 @@ __device__ __forceinline__ float to_float_scaled(double v, int s) {
 // FP64 evaluation needs dt_c within ~1e-7 of a level boundary.
 // level_from: that level from the criterion's inputs as floats f[c * ACH]
 // (stride ACH): a (3), j g (3), a2 g^2 (3), a3 g^3 (3)
-// (square roots and the division by the approximate instructions, within 2^-22:
-// the criterion is latency between the corrector and the next block step)
-__device__ __forceinline__ float sqrt_approx(float x) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 // T^2 split for level_from: T2 = ft 2^et, ft in [1/2, 1)
 struct T2Split {
     int et;
@@ -400,11 +393,11 @@ __device__ __forceinline__ int level_from(const float *f, int lv, float eta, con
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         const float x = f[(3 * g) * ACH], y = f[(3 * g + 1) * ACH], z = f[(3 * g + 2) * ACH];
-        q[g] = sqrt_approx(fmaf(x, x, fmaf(y, y, z * z)));
+        q[g] = sqrtf(fmaf(x, x, fmaf(y, y, z * z)));
     }
     const float num = eta * fmaf(q[0], q[2], q[1] * q[1]);
     const float den = fmaf(q[1], q[3], q[2] * q[2]);
-    const float r = __fdividef(num, den);
+    const float r = num / den;
     // r = fr 2^er with fr in [1/2, 1)
     const int br = __float_as_int(r);
     int er = (br >> 23) - 126;
@@ -435,13 +428,13 @@ __device__ __forceinline__ double half_of(double v) {
     return __hiloint2double(hi - 0x00100000, __double2loint(v));
 }
 // Coordinate c of member k predicted from its own time to tn: the position
-// x + h (u + h/2 (a + h/3 j)) or the velocity u + h (a + h/2 j). stick3 = stick / 3
+// x + h (u + h (a/2 + h/6 j)) or the velocity u + h (a + h/2 j)
 __device__ __forceinline__ double predict_x(const HermSmem &S, int k, int c, long long tn,
-                                            const TickF &stick, const TickF &stick3) {
-    const long long dt = tn - S.ti[k];
+                                            const TickF &stick) {
     const int o = c * HCAP + k;
-    const double h3 = ticks_times(dt, stick3), hs = ticks_times(dt, stick);
-    return fma(hs, fma(half_of(hs), fma(h3, S.jx[o], S.ax[o]), S.u[o]), S.x[o]);
+    const double hs = ticks_times(tn - S.ti[k], stick);
+    const double h6 = hs * (1.0 / 6.0);
+    return fma(hs, fma(hs, fma(0.5, S.ax[o], __dmul_rn(h6, S.jx[o])), S.u[o]), S.x[o]);
 }
 __device__ __forceinline__ double predict_v(const HermSmem &S, int k, int c, long long tn,
                                             const TickF &stick) {
@@ -482,10 +475,11 @@ __device__ __forceinline__ void predict_f32(const HermSmem &S, int k, long long 
     S.pd[k] = fmaf(m, 0x1p-18f, 1e-30f);
 }
 
-// One item (active slot, coordinate) of the corrector's linear form f: everything but
+// One item (active slot, coordinate) of the corrector's form f: everything but
 // the new acceleration and jerk, read while those are on their way.
 struct CorrItem {
-    double cd, c0, c1, a, j, base;
+    double a2d, a2j0, a2j1, a3d, a3j, f2, f3;  // a2 and a3; the form f2 a2 + f3 a3 + base
+    double a, j, base;
     int o, s, lv;  // coordinate and member, coordinate and slot, the member's level
     __device__ __forceinline__ void fetch(const HermSmem &S, int f, const uint16_t *act, int it) {
         constexpr int LS = KMAX + 1;
@@ -494,17 +488,25 @@ struct CorrItem {
         o = c * HCAP + k;
         s = c * ACH + sl;
         lv = S.lev[k];
-        const double *L = S.lvt + 3 * f * LS + lv;
-        cd = L[0];
-        c0 = L[LS];
-        c1 = f == LF_A3 ? c0 : L[2 * LS];
+        const double *L = S.lvt + lv;
+        a2d = L[LV_A2D * LS];
+        a2j0 = L[LV_A2J0 * LS];
+        a2j1 = L[LV_A2J1 * LS];
+        a3d = L[LV_A3D * LS];
+        a3j = L[LV_A3J * LS];
+        f2 = L[(f == LF_X ? LV_H4 : LV_H3) * LS];
+        f3 = L[(f == LF_X ? LV_H5 : (f == LF_V ? LV_H4 : LV_H)) * LS];
         a = S.ax[o];
         j = S.jx[o];
         base = f < LF_A2 ? S.ex[3 * f * HCAP + o] : 0.0;
     }
-    __device__ __forceinline__ double value(const HermSmem &S) const {
+    __device__ __forceinline__ double value(const HermSmem &S, int f) const {
         const double d = a - S.a1s[s], j1 = S.a1s[3 * ACH + s];
-        return fma(cd, d, fma(c0, j, fma(c1, j1, base)));
+        const double a3 = fma(a3d, d, a3j * (j + j1));
+        if (f == LF_A3) return a3;
+        const double a2 = fma(a2d, d, fma(a2j0, j, a2j1 * j1));
+        if (f == LF_A2) return fma(f3, a3, a2);  // at the end of the step
+        return fma(f2, a2, fma(f3, a3, base));
     }
 };
 
@@ -804,58 +806,41 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const long long TT = 1ll << KMAX;
     const double tick = T / (double)TT;
     const double T2d = T * T;
-    // The star's pull has lanes of its own (half the CTA at a time, its sums in the
-    // slots of the block steps' partials), and warp 7 sets up the corrector's constants
-    // per level meanwhile (products with powers of two): on one lane group the star's
-    // pull, the pairs' and the levels' square roots and division are one chain of FP64
-    // instructions, and scalars that every warp computes take the sub-partitions' FP64
-    // units eight times.
+    // (warp 7 first sets up the corrector's constants per level, products with powers
+    // of two: scalars that every warp computes take the sub-partitions' FP64 units
+    // eight times)
     const int warp = tid >> 5, wl = tid & 31;
     if (warp == 7) {
-        const double inv_T = 1.0 / T, iT2 = inv_T * inv_T, T3 = T2d * T;
+        const double inv_T = 1.0 / T, iT2 = inv_T * inv_T, iT3 = iT2 * inv_T;
+        const double T3 = T2d * T, T4 = T3 * T;
 #pragma unroll 1
         for (int lv = wl; lv <= KMAX; lv += 32) {
             constexpr int LS = KMAX + 1;
             double *L = S.lvt + lv;
             const double ih = sgn * inv_T * pow2d(lv), ih2 = iT2 * pow2d(2 * lv);
-            const double hl = sgn * T * pow2d(-lv), h2 = T2d * pow2d(-2 * lv);
-            const double h3 = sgn * T3 * pow2d(-3 * lv);
-            L[(3 * LF_X) * LS] = h2 * (-3.0 / 20.0);
-            L[(3 * LF_X + 1) * LS] = h3 * (-7.0 / 60.0);
-            L[(3 * LF_X + 2) * LS] = h3 * (-1.0 / 30.0);
-            L[(3 * LF_V) * LS] = hl * -0.5;
-            L[(3 * LF_V + 1) * LS] = h2 * (-5.0 / 12.0);
-            L[(3 * LF_V + 2) * LS] = h2 * (-1.0 / 12.0);
-            L[(3 * LF_A2) * LS] = 6.0 * ih2;
-            L[(3 * LF_A2 + 1) * LS] = 2.0 * ih;
-            L[(3 * LF_A2 + 2) * LS] = 4.0 * ih;
-            L[(3 * LF_A3) * LS] = 12.0 * (sgn * (iT2 * inv_T) * pow2d(3 * lv));
-            L[(3 * LF_A3 + 1) * LS] = 6.0 * ih2;
+            L[LV_H * LS] = sgn * T * pow2d(-lv);
+            L[LV_A2D * LS] = -6.0 * ih2;
+            L[LV_A2J0 * LS] = -4.0 * ih;
+            L[LV_A2J1 * LS] = -2.0 * ih;
+            L[LV_A3D * LS] = 12.0 * (sgn * iT3 * pow2d(3 * lv));
+            L[LV_A3J * LS] = 6.0 * ih2;
+            L[LV_H4 * LS] = (T4 * pow2d(-4 * lv)) * (1.0 / 24.0);
+            L[LV_H5 * LS] = (sgn * T4 * T * pow2d(-5 * lv)) * (1.0 / 120.0);
+            L[LV_H3 * LS] = (sgn * T3 * pow2d(-3 * lv)) * (1.0 / 6.0);
         }
     }
-    const int NGS = min(NG, HTHREADS / 2);  // members per round
 #pragma unroll 1
-    for (int k0 = mlo; k0 < mhi; k0 += NGS) {
+    for (int k0 = mlo; k0 < mhi; k0 += NG) {
         const int k = k0 + grp;
         double aj[6] = {0, 0, 0, 0, 0, 0};
-        const int ks = k0 + tid - HTHREADS / 2;
-        if (ks >= k0 && ks < min(k0 + NGS, mhi)) {
-            star_pull(S, ks, gm0, h.eps2, aj);
-            for (int c = 0; c < 6; ++c) S.pr[c * HTHREADS + ks - k0] = aj[c];
-        }
-        const bool mine = grp < NGS && k < mhi;
-        for (int c = 0; c < 6; ++c) aj[c] = 0.0;
-        if (mine) herm_part(S, 0, n, k, lane, P, tc, h.eps2, aj);
+        if (k < mhi) herm_part(S, 0, n, k, lane, P, gm0, tc, h.eps2, aj);
         group_sum(aj, 6, P);
-        __syncthreads();
-        if (mine && lane == 0) {
-            for (int c = 0; c < 6; ++c) aj[c] += S.pr[c * HTHREADS + grp];
+        if (k < mhi && lane == 0) {
             S.ax[k] = aj[0]; S.ay[k] = aj[1]; S.az[k] = aj[2];
             S.jx[k] = aj[3]; S.jy[k] = aj[4]; S.jz[k] = aj[5];
             S.lev[k] = first_level(aj, h.eta_s, T2d, T);
             S.ti[k] = 0;
         }
-        __syncthreads();
     }
     if (COOP) {
         cl.sync();
@@ -884,7 +869,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
     const T2Split T2s((float)T2d);
     const float etaf = (float)h.eta;
     const float stickf = (float)stick;
-    const TickF tick1(stick), tick3(stick * (1.0 / 3.0));
+    const TickF tick1(stick);
     const float rcf = __double2float_ru(rcrit * (1.0 + 0x1p-20));
     const int npart = mhi - mlo;
     // the largest range of the cluster: every CTA derives its lane layout and
@@ -941,11 +926,13 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
         // (na > N3) first lists the pairs that maybe_near leaves, by member and
         // partner: few of a set's pairs lie within r_crit, and an FP64 instruction
         // costs the same for one lane as for 32. Up to 96 pairs the block step then
-        // predicts and evaluates the list alone, packed into lanes (sparse).
+        // predicts and evaluates the list alone, packed into lanes (sparse). One system's
+        // sets only: a member's pulls are then added in another order, and a batch's
+        // sums keep theirs.
         int32_t *plist = S.need + 640, *poff = S.need + 736, *pcnt = S.need + 800;
         bool sparse = false;
         int npair = 0;
-        if (!COOP && na > N3 && na <= 32) {
+        if (!COOP && d.nsys == 1 && na > N3 && na <= 32) {
 #pragma unroll 1
             for (int k = tid; k < n; k += HTHREADS) predict_f32(S, k, tn, stickf);
             __syncthreads();
@@ -1058,7 +1045,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             if (pq & 1)
                 to[sparse && i >= na ? 3 * 96 : 3 * HCAP] = predict_v(S, k, c, tn, tick1);
             else
-                to[0] = predict_x(S, k, c, tn, tick1, tick3);
+                to[0] = predict_x(S, k, c, tn, tick1);
         }
         __syncthreads();
         uint16_t *nact = S.act + (~steps & 1) * HCAP;
@@ -1080,7 +1067,7 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
             // When they fit one warp's worth (most block steps: one or two members
             // move), a pair item runs on three warps: sin, cos, and everything that
             // needs neither, then one coordinate each; its longest instruction stream
-            // is 34 FP64 instructions against the pair's 47, with the star's pull on
+            // is 38 FP64 instructions against the pair's 51, with the star's pull on
             // the fourth sub-partition.
             const bool paired = sparse || nc <= NP;
             const int NR = paired ? nc : NU;
@@ -1353,18 +1340,20 @@ __device__ __noinline__ void hermite_set(const Dev &d, const HermArgs h, int set
                 __syncthreads();
             }
             // Corrector and step criterion (the same in every CTA): items (member,
-            // coordinate), 32 to a warp, and each of the four linear forms on a warp of
-            // its own sub-partition, four FP64 instructions deep; warps 4 and 5 bring
-            // the new acceleration and jerk. Warp 6 sets the new levels when the
-            // criterion's inputs are there, and finds the next block time.
-            // (One warp per coordinate with a2 and a3 first took eight instructions to
-            // the criterion and twelve to the state.)
+            // coordinate), 32 to a warp, and each of the four forms on a warp of
+            // its own sub-partition, which forms a2 and a3 for itself (four to nine FP64
+            // instructions deep); warps 4 and 5 bring the new acceleration and jerk. Warp
+            // 6 sets the new levels when the criterion's inputs are there, and finds the
+            // next block time. (One warp per coordinate with a2 and a3 first took eight
+            // instructions to the criterion and twelve to the state. With the forms
+            // written out in the new and old derivatives every warp takes four, 300
+            // cycles of a block step's 9000, but rounds differently.)
             if (warp < 4) {
                 const int f = warp;
                 #pragma unroll 1
                 for (int it = wl; it < 3 * nc; it += 32) {
                     if (it >= 32) item.fetch(S, f, act + a0, it);
-                    const double r = item.value(S);
+                    const double r = item.value(S, f);
                     if (f < LF_A2) {
                         S.x[3 * f * HCAP + item.o] = r;
                         S.f[3 * f * HCAP + item.o] = to_float_scaled(r, 0);
@@ -1558,8 +1547,13 @@ int hermite_cluster_size(const Dev &d, const qym_params &p) {
 }
 
 constexpr int kHermGrid = 2 * 152;  // CTAs per SM x SMs
-static_assert(kHermGrid / 2 <= kHermMaxClusters, "more clusters than plan entries");
-int hermite_clusters(const Dev &d, const qym_params &p) { return kHermGrid / hermite_cluster_size(d, p); }
+// clusters that take a set of the plan (with two CTAs each, half of them: how many
+// sets share their sums over a cluster is part of a batch's results)
+int hermite_clusters(const Dev &d, const qym_params &p) {
+    const int cls = hermite_cluster_size(d, p);
+    return (cls == 2 ? 1 : 2) * 152 / cls;
+}
+static_assert(2 * 152 / 4 <= kHermMaxClusters && 152 / 2 <= kHermMaxClusters, "more clusters than plan entries");
 
 cudaError_t launch_hermite(const Dev &d, const qym_params &p, double tau, cudaStream_t st) {
     HermArgs h;

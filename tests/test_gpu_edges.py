@@ -415,7 +415,7 @@ def test_kepler_bits(torch, name, dt):
     _same_bits(v1.cpu().numpy(), g[f"kepler_{name}_v"])
 
 
-@pytest.mark.parametrize("kind,encounters", [("plain", 0)])
+@pytest.mark.parametrize("kind,encounters", [("plain", 0), ("step", 1)])
 @pytest.mark.parametrize("name", ["disks", "swarms"])
 def test_batch_bits(torch, name, kind, encounters):
     """Two steps of small batches (planetesimal disks; planets' swarms of 2 to 70
