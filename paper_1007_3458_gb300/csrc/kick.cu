@@ -195,7 +195,26 @@ struct JPairs {
 // the minimum. Without FORCE only the search runs (the same separations and
 // r^2). With UNI every j has the same G m, which the caller multiplies the sums
 // by: one product a pair less on the FMA pipe that bounds the kick (planetesimals
-// of one mass fill nearly every window; heavy bodies are summed elsewhere).
+// of one mass fill nearly every window; heavy bodies are summed elsewhere). r^-3
+// alone has to stay in FP32's range then: the callers take UNI for coordinates
+// below kUniMax, where every r^-3 is a normal float, and repeat a chunk whose sums
+// are not finite (a pair closer than about 2^-43) with G m in the product.
+constexpr float kUniMax = 0x1p40f;  // r < 2^42, r^-3 > 2^-126
+__device__ __forceinline__ bool uni_range(const float4 &p) {
+    return fmaxf(fabsf(p.x), fmaxf(fabsf(p.y), fabsf(p.z))) < kUniMax;
+}
+// whether the sums of a thread's rows are finite
+template <int N>
+__device__ __forceinline__ bool finite_sums(const float2 (&x)[N], const float2 (&y)[N], const float2 (&z)[N]) {
+    float2 m = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < N; ++k) m = __ffma2_rn(x[k], make_float2(0.0f, 0.0f), m);
+#pragma unroll
+    for (int k = 0; k < N; ++k) m = __ffma2_rn(y[k], make_float2(0.0f, 0.0f), m);
+#pragma unroll
+    for (int k = 0; k < N; ++k) m = __ffma2_rn(z[k], make_float2(0.0f, 0.0f), m);
+    return m.x + m.y == 0.0f;  // (0 times infinity is NaN)
+}
 template <int IPT, bool FLAG, bool DIAG, bool FORCE, bool UNI>
 __device__ __forceinline__ void mixed_chunk(const JPairs &s, int p0, int p1, int jt,
                                             const int (&gi)[IPT],
@@ -334,6 +353,9 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         nyl[k] = make_float2(-l.y, -l.y); nzl[k] = make_float2(-l.z, -l.z);
         ahx[k] = ahy[k] = ahz[k] = alx[k] = aly[k] = alz[k] = 0.0f;
     }
+    bool i_in = a.uniform;  // this thread's rows let a window take the form without G m
+#pragma unroll
+    for (int k = 0; k < IPT; ++k) i_in = i_in && (gi[k] >= it.y || uni_range(make_float4(nxh[k].x, nyh[k].x, nzh[k].x, 0.0f)));
     const int i_lo = it.x, i_hi = it.x + (int)(IPT * blockDim.x);
     for (int jt = it.z, n = 0; jt < it.w; jt += n) {
         // windows of at most TILE positions; with far tiles never across the
@@ -359,11 +381,13 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         bool quiet = false;
         float2 dxi[IPT], dyi[IPT], dzi[IPT];
         float4 m0 = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool j_in = true;
         if (a.far_tiles && !diag) {
             const float4 *tm = a.tile + 3 * ((jt - 1) / TILE);
             m0 = tm[0];
             const float4 m1 = tm[1], m2 = tm[2];
             const float R = m0.w;
+            j_in = uni_range(m1) && uni_range(m2);
             bool mine = true, calm = true;
 #pragma unroll
             for (int k = 0; k < IPT; ++k) {
@@ -385,7 +409,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         // one G m for the whole window (and not zero, so that the pad and a
         // massless body are never taken for it)
         const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
-        bool same = a.uniform && gm0 > 0.0f;
+        bool same = i_in && j_in && gm0 > 0.0f;
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
             const int j0 = jt + 2 * t;
             const bool two = 2 * t + 1 < n;
@@ -398,7 +422,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     l1 = a.lo[j0 + 1];
                 }
                 s_a[t] = make_float4(p0.x, p1.x, p0.y, p1.y);
-                same = same && p0.w == gm0 && (!two || p1.w == gm0);
+                same = same && p0.w == gm0 && uni_range(p0) && (!two || (p1.w == gm0 && uni_range(p1)));
                 s_b[t] = make_float4(p0.z, p1.z, p0.w, p1.w);
                 s_c[t] = make_float4(l0.x, l1.x, l0.y, l1.y);
                 s_d[t] = make_float4(l0.z, l1.z, -l0.w, -l1.w);
@@ -418,7 +442,6 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
             }
         }
         const bool uni = FORCE ? __syncthreads_and(same) : (__syncthreads(), false);
-        const float gw = uni ? gm0 : 1.0f;
         if (far) {
             // d_i = c - Q_i = (c - x_hi) - x_lo rounded once, duplicated for
             // the packed form
@@ -436,11 +459,6 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
             const int ce = min(c + FOLD / 2, np);
             float2 fx[IPT], fy[IPT], fz[IPT];
             float mind[IPT];
-#pragma unroll
-            for (int k = 0; k < IPT; ++k) {
-                fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
-                mind[k] = 3.0e38f;
-            }
             const auto run = [&](auto u) {
                 constexpr bool U = decltype(u)::value;
                 if (far && quiet)
@@ -457,7 +475,21 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     mixed_chunk<IPT, FLAG, false, FORCE, U>(sp, c, ce, jt, gi, nxh, nyh, nzh, nxl, nyl,
                                                             nzl, fx, fy, fz, mind);
             };
-            if (FORCE && uni) run(std::integral_constant<bool, FORCE>{}); else run(std::false_type{});
+            float gw = uni ? gm0 : 1.0f;
+            for (;;) {
+#pragma unroll
+                for (int k = 0; k < IPT; ++k) {
+                    fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
+                    mind[k] = 3.0e38f;
+                }
+                if (!FORCE || gw == 1.0f) {
+                    run(std::false_type{});
+                    break;
+                }
+                run(std::integral_constant<bool, FORCE>{});
+                if (finite_sums(fx, fy, fz)) break;
+                gw = 1.0f;
+            }
 #pragma unroll
             for (int k = 0; k < IPT; ++k) {
                 if (FORCE) {
@@ -489,9 +521,9 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
 
 // ---------------------------------------------------------------- pairs once
 // The mixed kick of one system in Morton order with each pair formed once: the
-// separation, r^2 and r^-3 serve both bodies (Newton's third law), 14 FMA-pipe
-// instructions a far pair of equal masses instead of 2 x 11, which is what bounds
-// the kick.
+// separation, r^2, 1/r and r^-2 serve both bodies (Newton's third law), 14 FMA-pipe
+// instructions a far pair of equal masses instead of 2 x 11 (17 instead of 2 x 12 of
+// several masses), which is what bounds the kick.
 //
 // An i-block is 512 consecutive positions, four per thread, a warp's 128
 // consecutive ones (compact along the Morton curve, so that more windows are far
@@ -509,7 +541,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
 // Work unit: G consecutive i-blocks against a range of rh half tiles (the part
 // past each block). Rows get one slot of partial sums per range from their own
 // block, and one per group of earlier i-blocks from the j side, added up in the
-// group's order by the unit that owns the slot. sym_slots (qym_internal.cuh)
+// group's order by the unit that owns the slot. SymSlots (qym_internal.cuh)
 // gives a row's valid slots.
 constexpr int SYM_T = 128, SYM_R = 4, SYM_BLK = SYM_T * SYM_R, SYM_W = SYM_T / 32;
 static_assert(SYM_BLK == kSymBlock, "i-block of the pair-symmetric kick");
@@ -564,9 +596,9 @@ __device__ __forceinline__ void sym_chunk(const SymShared &S, int p0, const floa
             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             if (FORCE) {
                 const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-                const float2 r3 = __fmul2_rn(ri, __fmul2_rn(ri, ri));
-                const float2 si = UNI ? r3 : __fmul2_rn(gm, r3);
-                const float2 sj = UNI ? r3 : __fmul2_rn(make_float2(gi[k], gi[k]), r3);
+                const float2 w = __fmul2_rn(ri, ri);
+                const float2 si = __fmul2_rn(UNI ? ri : __fmul2_rn(gm, ri), w);
+                const float2 sj = UNI ? si : __fmul2_rn(__fmul2_rn(make_float2(gi[k], gi[k]), ri), w);
                 fx[k] = __ffma2_rn(si, dx, fx[k]);
                 fy[k] = __ffma2_rn(si, dy, fy[k]);
                 fz[k] = __ffma2_rn(si, dz, fz[k]);
@@ -624,7 +656,7 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
                 p = a.pos[i];
                 l = a.lo[i];
             }
-            i_same = i_same && p.w == gi0;
+            i_same = i_same && p.w == gi0 && uni_range(p);
             rho[k] = l.w;
             gmi[k] = p.w;
             S.ip[o] = p;
@@ -638,12 +670,13 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
             n = min(min(1 + ((jt - 1) / TILE + 1) * TILE, 1 + u.w * (TILE / 2)), npos) - jt;
             const int np = (n + 1) >> 1;
             const bool diag = jt < i_hi;
-            bool far = false, quiet = false;
+            bool far = false, quiet = false, j_in = true;
             float4 m0 = make_float4(0.f, 0.f, 0.f, 0.f);
             if (!diag) {
                 const float4 *tm = a.tile + 3 * ((jt - 1) / TILE);
                 m0 = tm[0];
                 const float4 m1 = tm[1], m2 = tm[2];
+                j_in = uni_range(m1) && uni_range(m2);
                 bool mine = true, calm = true;
 #pragma unroll
                 for (int k = 0; k < SYM_R; ++k) {
@@ -663,7 +696,7 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
             const bool any_far = __syncthreads_or(far);
             const bool any_near = __syncthreads_or(!far);
             const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
-            bool same = gm0 > 0.0f;
+            bool same = j_in && gm0 > 0.0f;
             // (padded to whole chunks of 32 pairs with massless bodies far from everything)
             for (int t = tid; t < ((np + 31) & ~31); t += SYM_T) {
                 const int j0 = jt + 2 * t;
@@ -689,7 +722,6 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
             }
             const bool j_uni = FORCE ? __syncthreads_and(same) : (__syncthreads(), false);
             const bool uni = j_uni && i_uni && !diag;
-            const float gw = uni ? gm0 : 1.0f, gv = uni ? -gi0 : -1.0f;
             float2 ix[SYM_R], iy[SYM_R], iz[SYM_R], lx[SYM_R], ly[SYM_R], lz[SYM_R];
 #pragma unroll
             for (int k = 0; k < SYM_R; ++k) {
@@ -708,37 +740,40 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
             for (int c = 0; c < np; c += 32) {
                 float2 fx[SYM_R], fy[SYM_R], fz[SYM_R], jx, jy, jz;
                 float mind[SYM_R];
+                const auto run = [&](auto U, auto F, auto Q) {
+                    sym_chunk<FLAG && decltype(Q)::value, FORCE, decltype(U)::value, decltype(F)::value>(
+                        S, c, ix, iy, iz, lx, ly, lz, gmi, fx, fy, fz, mind, jx, jy, jz);
+                };
+                using T1 = std::true_type;
+                using T0 = std::false_type;
+                bool u = uni && (quiet || !FLAG);
+                for (;;) {
 #pragma unroll
-                for (int k = 0; k < SYM_R; ++k) {
-                    fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
-                    mind[k] = 3.0e38f;
-                }
-                if (diag) {
-                    mixed_chunk<SYM_R, FLAG, true, FORCE, false>(sp, c, min(c + 32, np), jt, gi, ix, iy, iz,
-                                                                 lx, ly, lz, fx, fy, fz, mind);
-                } else {
-                    const auto run = [&](auto U, auto F, auto Q) {
-                        sym_chunk<FLAG && decltype(Q)::value, FORCE, decltype(U)::value, decltype(F)::value>(
-                            S, c, ix, iy, iz, lx, ly, lz, gmi, fx, fy, fz, mind, jx, jy, jz);
-                    };
-                    using T1 = std::true_type;
-                    using T0 = std::false_type;
-                    if (far && (quiet || !FLAG)) {
-                        if (uni) run(T1{}, T1{}, T0{}); else run(T0{}, T1{}, T0{});
+                    for (int k = 0; k < SYM_R; ++k) {
+                        fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
+                        mind[k] = 3.0e38f;
+                    }
+                    if (diag) {
+                        mixed_chunk<SYM_R, FLAG, true, FORCE, false>(sp, c, min(c + 32, np), jt, gi, ix, iy,
+                                                                     iz, lx, ly, lz, fx, fy, fz, mind);
+                    } else if (far && (quiet || !FLAG)) {
+                        if (u) run(T1{}, T1{}, T0{}); else run(T0{}, T1{}, T0{});
                     } else if (far) {
                         run(T0{}, T1{}, T1{});
                     } else if (quiet || !FLAG) {
-                        if (uni) run(T1{}, T0{}, T0{}); else run(T0{}, T0{}, T0{});
+                        if (u) run(T1{}, T0{}, T0{}); else run(T0{}, T0{}, T0{});
                     } else {
                         run(T0{}, T0{}, T1{});
                     }
-                    if (FORCE) {
-                        const float v = (FLAG && !quiet) ? -1.0f : gv;
-                        S.jxy[warp][c + lane] = make_float4(v * jx.x, v * jx.y, v * jy.x, v * jy.y);
-                        S.jz[warp][c + lane] = make_float2(v * jz.x, v * jz.y);
-                    }
+                    if (!FORCE || !u || __all_sync(0xffffffffu, finite_sums(fx, fy, fz))) break;
+                    u = false;
                 }
-                const float g = (FLAG && !quiet) ? 1.0f : gw;
+                if (FORCE && !diag) {
+                    const float v = u ? -gi0 : -1.0f;
+                    S.jxy[warp][c + lane] = make_float4(v * jx.x, v * jx.y, v * jy.x, v * jy.y);
+                    S.jz[warp][c + lane] = make_float2(v * jz.x, v * jz.y);
+                }
+                const float g = u ? gm0 : 1.0f;
 #pragma unroll
                 for (int k = 0; k < SYM_R; ++k) {
                     const int o = i_of + 32 * k;

@@ -430,3 +430,75 @@ def test_batch_bits(torch, name, kind, encounters):
     sim.close()
     _same_bits(qs, g[f"{name}_{kind}_q"])
     _same_bits(vs, g[f"{name}_{kind}_v"])
+
+
+# lengths and masses in cgs, SI and parsecs, and around AU and solar masses (G folded
+# into the masses): r^-3 of a disk's pairs lies below, at the end of, above and inside
+# FP32's range
+UNITS = [(1.5e13, 1.3e26), (1.5e11, 1.3e20), (4.85e-6, 4.3e-3), (1e-6, 1.0), (1e-12, 1e-9), (1.0, 1.0)]
+
+
+@pytest.mark.parametrize("n", [300, 2100, 9000])
+@pytest.mark.parametrize("lu,mu", UNITS)
+@pytest.mark.parametrize("equal", [True, False])
+def test_mixed_accel_units(torch, n, lu, mu, equal):
+    """The mixed kick in the caller's units, bodies of one mass (windows that
+    multiply by it once) and of several, with two close pairs and one body far
+    outside: the bound of test_mixed_accel_sizes."""
+    rng = np.random.default_rng(n)
+    w = W.outer_disk(n - 4, 1e-9, seed=3)
+    x, m = w.q.copy(), w.m.copy()
+    if not equal:
+        m[5:] = 10.0 ** rng.uniform(-11, -8, n - 4)
+    x[60] *= 1e3
+    x, m = x * lu, m * mu
+    sep = max(1e-13 * lu, 1e-14)  # (r^2 stays a normal float)
+    x[10] = x[9] + [sep, 0.0, 0.0]
+    x[40] = x[39] + [0.0, 3 * sep, -2 * sep]
+    # (the split positions resolve 2^-48 of a coordinate: the close pairs as the kernel sees them)
+    hi = x.astype(np.float32)
+    x = hi.astype(np.float64) + (x - hi).astype(np.float32)
+    md, xd = torch.from_numpy(m).cuda(), torch.from_numpy(np.ascontiguousarray(x.T)).cuda()
+    a = torch.empty((3, n + 1), dtype=torch.float64, device="cuda")
+    work = torch.empty(q.qym_accel_workspace_bytes(n + 1, q.QYM_KICK_MIXED), dtype=torch.uint8, device="cuda")
+    q.qym_accel_dev(n + 1, md, xd, a, 1.0, q.QYM_KICK_MIXED, work)
+    ref, mag = _accel_ref64(torch, m, x)
+    err = np.abs(a.cpu().numpy().T - ref)
+    assert np.all(err <= 2.0 ** -18 * mag), float((err / (mag + 1e-300)).max())
+
+
+@pytest.mark.parametrize("lu,mu", UNITS)
+@pytest.mark.parametrize("equal", [True, False])
+def test_pairs_once_units(torch, lu, mu, equal):
+    """The pairs-once kick in the caller's units: test_pairs_once's bound against
+    the FP64 kick, and a step's encounters those of the one-sided kick and of the
+    FP64 kick."""
+    n = 8705
+    w = W.outer_disk(n - 4, 1e-10, seed=n)
+    m = w.m.copy()
+    if not equal:
+        m[5:] *= 10.0 ** np.random.default_rng(n).uniform(-1, 1, n - 4)
+    # unit time: that of the disk's own units, lu^3 = G mu
+    t, G = np.sqrt(lu ** 3 / mu), 1.0
+    dv, rec = [], []
+    for prec, shape in ((q.QYM_KICK_FP64, None), (q.QYM_KICK_MIXED, None), (q.QYM_KICK_MIXED, (128, 2, 16))):
+        sim = q.Simulation(m * mu, w.q * lu, np.zeros_like(w.v), w.offsets, kick_prec=prec, encounters=0,
+                           heavy_mass=0.0, coords=1, G=1e-6 * G)
+        if shape:
+            q.qym_set_kick_shape(sim.ctx, *shape)
+        sim.step(1e-3 * t, 1)
+        dv.append(sim.state()[1] / (lu / t))
+        sim.close()
+        sim = q.Simulation(m * mu, w.q * lu, w.v * (lu / t), w.offsets, kick_prec=prec, eps_H=w.eps_H * lu, G=G)
+        if shape:
+            q.qym_set_kick_shape(sim.ctx, *shape)
+        sim.step(w.tau * t, 2)
+        rec.append(sim.encounters())
+        assert sim.stats()["status_bits"] == 0
+        sim.close()
+    a = [np.linalg.norm(x - dv[0], axis=1) for x in dv[1:]]
+    big = np.linalg.norm(dv[0], axis=1).max()
+    assert big > 0 and max(x.max() for x in a) <= 2.0 ** -18 * big
+    rms = [np.sqrt((x ** 2).mean()) for x in a]
+    assert rms[0] <= 1.5 * rms[1] + 1e-16 * big, (rms, big)
+    assert len(rec[0]) > 0 and np.array_equal(rec[0], rec[1]) and np.array_equal(rec[0], rec[2])
