@@ -333,8 +333,11 @@ qym_status qym_time_drift(qym_ctx *ctx, double tau, int32_t reps, double *ms_mom
  * the context's buffers hold, at least 4); QYM_EINVAL otherwise. For
  * reproducing a shape the tuner chose (qym_stats kick_tile_i, _splits).
  * One system of at least 8192 bodies forms each pair of the mixed kick once
- * by default (kick_tile_i = 512 rows, kick_tile_splits its ranges); a shape
- * set here replaces that form by the one-sided kick. */
+ * by default (kick_tile_i = 512 rows, kick_tile_splits its ranges), as long
+ * as its partial sums fit 2 GB (24 bytes a row and range, 0.8 GB for 262144
+ * bodies): up to about 0.7 million bodies, larger systems take the one-sided
+ * kick and hold 0.5 GB. A shape set here replaces the form by the one-sided
+ * kick. */
 qym_status qym_set_kick_shape(qym_ctx *ctx, int32_t threads, int32_t ipt, int32_t splits);
 
 /* Pick the kick launch shape (threads per CTA, rows per thread, j splits)

@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
 
 // Units of the pair-symmetric kick of nb bodies with at most max_slots slots a
 // row: about 2000 (four CTAs on each SM, several waves), ranges and groups of the
-// same length where the slots allow; G = 0 where they do not.
+// same length where the slots allow; no shape (G = 0, no slots) where they do not.
 SymShape sym_shape(int64_t nb, int64_t max_slots) {
     SymShape y;
     const int64_t nblk = (nb + SYM_BLK - 1) / SYM_BLK, nhalf = (nb + TILE / 2 - 1) / (TILE / 2);
@@ -847,8 +847,7 @@ SymShape sym_shape(int64_t nb, int64_t max_slots) {
     y.rh = (int32_t)std::max<int64_t>(1, (nhalf + want - 1) / want);
     y.nc = (int32_t)((nhalf + y.rh - 1) / y.rh);
     y.splits = (int32_t)(y.nc + ng);
-    if (y.splits > max_slots) y.G = 0;
-    return y;
+    return y.splits <= max_slots ? y : SymShape();
 }
 
 void sym_items_host(int64_t nb, const SymShape &y, std::vector<int4> &items) {

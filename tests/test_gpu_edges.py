@@ -502,3 +502,19 @@ def test_pairs_once_units(torch, lu, mu, equal):
     rms = [np.sqrt((x ** 2).mean()) for x in a]
     assert rms[0] <= 1.5 * rms[1] + 1e-16 * big, (rms, big)
     assert len(rec[0]) > 0 and np.array_equal(rec[0], rec[1]) and np.array_equal(rec[0], rec[2])
+
+
+def test_partial_sums_memory(torch):
+    """A system whose pairs-once partial sums would pass 2 GB (24 bytes a row and
+    range, 128 ranges: 699050 rows) takes the one-sided kick and holds no such
+    slots: less device memory than a somewhat smaller one, by most of 2 GB."""
+    held = []
+    for n in (690000, 705000):
+        w = W.outer_disk(n - 4, 1e-12, seed=1)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        sim = q.Simulation(w.m, w.q, w.v, w.offsets, encounters=0)
+        held.append((free - torch.cuda.mem_get_info()[0], sim.stats()["kick_tile_i"]))
+        sim.close()
+    assert held[0][1] == 512 and held[1][1] == 256
+    assert held[1][0] < held[0][0] - (1 << 30), held
