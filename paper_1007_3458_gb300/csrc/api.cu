@@ -45,7 +45,8 @@ struct qym_ctx {
     // energy
     EnergyPlan eplan;
     int4 *eblocks = nullptr;
-    int32_t *eblock0 = nullptr;
+    int2 *eitems = nullptr;
+    int32_t *eblock0 = nullptr, *eitem0 = nullptr;
     double *epart = nullptr, *E = nullptr;
     double *mt = nullptr;  // [nsys] total masses
     void *flush = nullptr; // L2 flush buffer (params.l2_flush_bytes)
@@ -307,8 +308,12 @@ static void carve_all(qym_ctx *c, Carver &k) {
     c->ss.size = k.take<int32_t>(R + 1);
     c->ss.fill = k.take<int32_t>(R + 1);
     c->ss.rc_bits = k.take<unsigned long long>(R + 1);
-    c->eblocks = k.take<int4>(c->eplan.nblocks);
-    c->eblock0 = k.take<int32_t>(d.nsys + 1);
+    if (d.nsys > 1) {
+        c->eblocks = k.take<int4>(c->eplan.nblocks);
+        c->eitems = k.take<int2>(c->eplan.nitems);
+        c->eblock0 = k.take<int32_t>(d.nsys + 1);
+        c->eitem0 = k.take<int32_t>(d.nsys + 1);
+    }
     c->epart = k.take<double>(energy_partials(c->eplan));
     c->E = k.take<double>(d.nsys);
     c->mt = k.take<double>(d.nsys);
@@ -562,7 +567,8 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     d.max_log = params->max_log ? params->max_log : (int64_t)1 << 22;
     d.max_sets = (int32_t)R;
     d.max_members = (int32_t)R;
-    c->eplan = energy_plan(offsets, nsys, nullptr, nullptr);
+    EnergyTables et;
+    c->eplan = energy_plan(offsets, nsys, nsys > 1 ? &et : nullptr);
     // heavy bodies per system (mixed kick): m >= heavy_mass m0, at most
     // QYM_HEAVY_CAP of them, else the system keeps all bodies in FP32
     std::vector<int32_t> hrows, hstart(nsys + 1);
@@ -667,11 +673,10 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
     int32_t ni = 0, spu = 0;
     kick_items_host(offsets, nsys, c->tune, items.data(), slots.data(), &ni, &spu, d.nitems, 0,
                     INT64_MAX, c->sort_rows ? kKickTile / 2 : 1);
-    std::vector<int4> eblk(c->eplan.nblocks);
-    std::vector<int32_t> eb0(nsys + 1);
-    energy_plan(offsets, nsys, eblk.data(), eb0.data());
     c->eplan.blocks = c->eblocks;
+    c->eplan.items = c->eitems;
     c->eplan.block0 = c->eblock0;
+    c->eplan.item0 = c->eitem0;
     CKI(cudaMemcpyAsync(d.offsets, offsets, sizeof(int64_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
     if (!c->h_wh_heavy.empty())
         CKI(cudaMemcpyAsync(c->wh_heavy, c->h_wh_heavy.data(), sizeof(int32_t) * c->h_wh_heavy.size(),
@@ -685,8 +690,12 @@ extern "C" qym_status qym_init(const qym_params *params, int32_t nsys, const int
                             cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.mchunks, mch.data(), sizeof(int4) * d.nmchunks, cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.sys_chunk0, sc0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
-    CKI(cudaMemcpyAsync(c->eblocks, eblk.data(), sizeof(int4) * eblk.size(), cudaMemcpyHostToDevice, c->stream));
-    CKI(cudaMemcpyAsync(c->eblock0, eb0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
+    if (nsys > 1) {
+        CKI(cudaMemcpyAsync(c->eblocks, et.blocks.data(), sizeof(int4) * et.blocks.size(), cudaMemcpyHostToDevice, c->stream));
+        CKI(cudaMemcpyAsync(c->eitems, et.items.data(), sizeof(int2) * et.items.size(), cudaMemcpyHostToDevice, c->stream));
+        CKI(cudaMemcpyAsync(c->eblock0, et.block0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
+        CKI(cudaMemcpyAsync(c->eitem0, et.item0.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
+    }
     if (!hrows.empty())
         CKI(cudaMemcpyAsync(d.heavy_rows, hrows.data(), sizeof(int32_t) * hrows.size(), cudaMemcpyHostToDevice, c->stream));
     CKI(cudaMemcpyAsync(d.heavy_start, hstart.data(), sizeof(int32_t) * (nsys + 1), cudaMemcpyHostToDevice, c->stream));
@@ -1696,7 +1705,7 @@ extern "C" qym_status qym_encounter_test_dev(int64_t rows, const double *q0, con
 extern "C" size_t qym_energy_workspace_bytes(int64_t rows) {
     if (rows < 2) return 0;
     const int64_t off[2] = {0, rows};
-    return al256(sizeof(double) * energy_partials(energy_plan(off, 1, nullptr, nullptr)));
+    return al256(sizeof(double) * energy_partials(energy_plan(off, 1, nullptr)));
 }
 
 extern "C" qym_status qym_energy_dev(int64_t rows, const double *m, const double *q, const double *v,
@@ -1706,7 +1715,7 @@ extern "C" qym_status qym_energy_dev(int64_t rows, const double *m, const double
     if (work_bytes < qym_energy_workspace_bytes(rows)) FAIL(nullptr, QYM_EINVAL, "qym_energy_dev: workspace too small");
     const int64_t off[2] = {0, rows};
     cudaStream_t st = (cudaStream_t)stream;
-    CK(nullptr, launch_energy(energy_plan(off, 1, nullptr, nullptr), 1, nullptr, rows, m, q, v, G,
+    CK(nullptr, launch_energy(energy_plan(off, 1, nullptr), 1, nullptr, rows, m, q, v, G,
                               (double *)work, E, st));
     CK(nullptr, cudaStreamSynchronize(st));
     return QYM_OK;

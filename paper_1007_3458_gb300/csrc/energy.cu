@@ -38,9 +38,10 @@ __global__ void __launch_bounds__(ET) k_energy_pairs(EnergyPlan pl, int64_t R, c
     __shared__ float s_c[ET];            // z.l
     __shared__ int s_hi[ET / 32];
     __shared__ double red[4][ET / 32];
-    const int64_t I = blockIdx.x / pl.nranges;
-    const int c = (int)(blockIdx.x - I * pl.nranges);
-    // (first row, last row + 1, end of the system, its star row)
+    const int2 it = pl.items ? pl.items[blockIdx.x]
+                             : make_int2((int)(blockIdx.x / pl.nranges), (int)(blockIdx.x % pl.nranges));
+    const int64_t I = it.x;
+    const int c = it.y;
     const int4 bk = pl.blocks ? pl.blocks[I]
                               : make_int4((int)(1 + I * ET), (int)min(1 + (I + 1) * (int64_t)ET, R), (int)R, 0);
     const int64_t jb = bk.x + (int64_t)c * pl.range;
@@ -127,8 +128,9 @@ __global__ void __launch_bounds__(256) k_energy_final(EnergyPlan pl, const int64
     chain_wait();
     const int s = blockIdx.x;
     const int64_t b0 = pl.block0 ? pl.block0[s] : 0, b1 = pl.block0 ? pl.block0[s + 1] : pl.nblocks;
+    const int64_t i0 = pl.item0 ? pl.item0[s] : 0, i1 = pl.item0 ? pl.item0[s + 1] : pl.nitems;
     double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t k = b0 * pl.nranges + threadIdx.x; k < b1 * pl.nranges; k += blockDim.x) t[0] += pe[k];
+    for (int64_t k = i0 + threadIdx.x; k < i1; k += blockDim.x) t[0] += pe[k];
     for (int64_t k = b0 + threadIdx.x; k < b1; k += blockDim.x)
         for (int c = 0; c < 3; ++c) t[1 + c] += ps[3 * k + c];
     __shared__ double sh[4][8];
@@ -146,40 +148,49 @@ __global__ void __launch_bounds__(256) k_energy_final(EnergyPlan pl, const int64
     }
 }
 
-// host: i-blocks of at most 128 rows of each system (blocks and block0 may be
-// NULL: counted only) and the ranges' length: about 16 CTAs per SM over the
-// batch's pairs, ranges of 8 (a small system's walk is latency) to 4096 rows
-EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, int4 *blocks, int32_t *block0) {
+// host: i-blocks of at most 128 rows of each system and the ranges' length: about 16
+// CTAs per SM over the batch's pairs, ranges of 8 (a small system's walk is latency)
+// to 4096 rows. A batch's items are its non-empty ranges: one count of ranges for all
+// i-blocks, the largest system's, made a million systems of two bodies beside one of
+// 3000 launch 1.9e8 CTAs and hold 1.5 GB of partial sums.
+EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, EnergyTables *t) {
     EnergyPlan pl;
     double pairs = 0.0;
-    int64_t nbmax = 0;
-    int32_t n = 0;
     for (int32_t s = 0; s < nsys; ++s) {
-        if (block0) block0[s] = n;
-        const int64_t b0 = offsets[s] + 1, b1 = offsets[s + 1];
-        pairs += 0.5 * (double)(b1 - b0) * (double)(b1 - b0);
-        nbmax = std::max(nbmax, b1 - b0);
-        for (int64_t i0 = b0; i0 < b1; i0 += ET) {
-            if (blocks)
-                blocks[n] = make_int4((int)i0, (int)std::min<int64_t>(i0 + ET, b1), (int)b1, (int)offsets[s]);
-            ++n;
-        }
+        const int64_t nb = offsets[s + 1] - offsets[s] - 1;
+        pairs += 0.5 * (double)nb * (double)nb;
+        pl.nblocks += (int32_t)((nb + ET - 1) / ET);
     }
-    if (block0) block0[nsys] = n;
     const double want = pairs / (16.0 * 152.0 * ET);
     pl.range = (int32_t)std::min(4096.0, std::max(8.0, 8.0 * (double)(int64_t)(want / 8.0 + 1.0)));
-    pl.nranges = (int32_t)((nbmax + pl.range - 1) / pl.range);
-    pl.nblocks = n;
+    if (!t) {
+        pl.nranges = (int32_t)((offsets[1] - offsets[0] - 1 + pl.range - 1) / pl.range);
+        pl.nitems = pl.nblocks * pl.nranges;
+        return pl;
+    }
+    for (int32_t s = 0; s < nsys; ++s) {
+        t->block0.push_back((int32_t)t->blocks.size());
+        t->item0.push_back((int32_t)t->items.size());
+        const int64_t b1 = offsets[s + 1];
+        for (int64_t i0 = offsets[s] + 1; i0 < b1; i0 += ET) {
+            for (int64_t j0 = i0; j0 < b1; j0 += pl.range)
+                t->items.push_back(make_int2((int)t->blocks.size(), (int)((j0 - i0) / pl.range)));
+            t->blocks.push_back(make_int4((int)i0, (int)std::min<int64_t>(i0 + ET, b1), (int)b1, (int)offsets[s]));
+        }
+    }
+    t->block0.push_back((int32_t)t->blocks.size());
+    t->item0.push_back((int32_t)t->items.size());
+    pl.nitems = (int32_t)t->items.size();
     return pl;
 }
 
-int64_t energy_partials(const EnergyPlan &pl) { return (int64_t)pl.nblocks * (pl.nranges + 3); }
+int64_t energy_partials(const EnergyPlan &pl) { return (int64_t)pl.nitems + 3 * (int64_t)pl.nblocks; }
 
 cudaError_t launch_energy(const EnergyPlan &pl, int32_t nsys, const int64_t *offsets, int64_t R,
                           const double *m, const double *q, const double *v, double G, double *part,
                           double *E, cudaStream_t st) {
-    double *ps = part + (int64_t)pl.nblocks * pl.nranges;
-    launch_chain(k_energy_pairs, (unsigned)((int64_t)pl.nblocks * pl.nranges), ET, 0, st, pl, R, m, q, v, G, part, ps);
+    double *ps = part + pl.nitems;
+    launch_chain(k_energy_pairs, (unsigned)pl.nitems, ET, 0, st, pl, R, m, q, v, G, part, ps);
     launch_chain(k_energy_final, nsys, 256, 0, st, pl, offsets, m, part, ps, E);
     return cudaGetLastError();
 }

@@ -531,13 +531,22 @@ cudaError_t launch_wh_blocks(const WholeArgs &w, int nblocks, cudaStream_t st);
 cudaError_t launch_wh_store(const WholeArgs &w, double *q1, double *v1, cudaStream_t st);
 
 // energy.cu
+// One system: nranges items (CTAs) per i-block, no tables. A batch: tables (device) of
+// the i-blocks (first row, last row + 1, end of the system, its star row), of the items
+// (i-block, range), and of each system's first i-block and item.
 struct EnergyPlan {
-    const int4 *blocks = nullptr;     // i-blocks (device; NULL: one system of R rows)
-    const int32_t *block0 = nullptr;  // [nsys+1] first i-block of each system (NULL: one system)
-    int32_t nblocks = 0;
-    int32_t range = 0, nranges = 0;   // j rows per CTA, ranges per i-block
+    const int4 *blocks = nullptr;
+    const int2 *items = nullptr;
+    const int32_t *block0 = nullptr, *item0 = nullptr;  // [nsys+1]
+    int32_t nblocks = 0, nitems = 0;
+    int32_t range = 0, nranges = 0;  // j rows per item; items per i-block (one system)
 };
-EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, int4 *blocks, int32_t *block0);
+struct EnergyTables {
+    std::vector<int4> blocks;
+    std::vector<int2> items;
+    std::vector<int32_t> block0, item0;
+};
+EnergyPlan energy_plan(const int64_t *offsets, int32_t nsys, EnergyTables *t);  // t: for a batch
 int64_t energy_partials(const EnergyPlan &pl);  // doubles of `part`
 cudaError_t launch_energy(const EnergyPlan &pl, int32_t nsys, const int64_t *offsets, int64_t R,
                           const double *m, const double *q, const double *v, double G, double *part,

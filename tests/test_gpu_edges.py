@@ -518,3 +518,47 @@ def test_partial_sums_memory(torch):
         sim.close()
     assert held[0][1] == 512 and held[1][1] == 256
     assert held[1][0] < held[0][0] - (1 << 30), held
+
+
+def _energy_ref(w, lo, hi):
+    """Energy of the system of rows [lo, hi) in extended precision (DH velocities),
+    and the sum of its terms' magnitudes."""
+    L = np.longdouble
+    m, x, v = (a[lo:hi].astype(L) for a in (w.m, w.q, w.v))
+    mb, xb, vb = m[1:], x[1:], v[1:]
+    S = (mb[:, None] * vb).sum(0)
+    kin, star, pair = (mb * (vb * vb).sum(1) / 2).sum(), (m[0] * mb / np.sqrt((xb * xb).sum(1))).sum(), L(0)
+    for i in range(len(mb)):
+        pair += (mb[i] * mb[i + 1:] / np.sqrt(((xb[i + 1:] - xb[i]) ** 2).sum(1))).sum()
+    return (S * S).sum() / (2 * m[0]) + kin - star - pair, kin + star + pair
+
+
+def test_energy_unbalanced_batch(torch):
+    """Energy of many two-body systems beside a large one, against extended
+    precision (bound of test_energy_blocks) for the large one and a sample, and
+    the device memory that the batch holds: with the large system's count of
+    ranges for every i-block the partial sums alone would take 20000 x 125 x 8
+    bytes more than they do."""
+    pairs, big = 20000, 3000
+    one = W.outer_disk(big - 4, 1e-9, seed=1)
+    rng = np.random.default_rng(2)
+    m2 = np.stack([np.ones(pairs), 10.0 ** rng.uniform(-9, -3, pairs), 10.0 ** rng.uniform(-9, -3, pairs)], 1)
+    x2, v2 = rng.normal(size=(2, pairs, 3, 3))
+    x2[:, 0] = v2[:, 0] = 0.0
+    cat = lambda a, b: np.concatenate([a.reshape(-1, *b.shape[1:]), b, a[:100].reshape(-1, *b.shape[1:])])
+    n = np.concatenate([np.full(pairs, 3), [big + 1], np.full(100, 3)])
+    w = W.Workload("mix", cat(m2, one.m), cat(x2, one.q), cat(v2, one.v), np.concatenate([[0], np.cumsum(n)]), one.tau, 1)
+    held = []
+    for k in (pairs + 101, pairs):  # with and without the large system (the last 101)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        rows = int(w.offsets[k])
+        sim = q.Simulation(w.m[:rows], w.q[:rows], w.v[:rows], w.offsets[:k + 1], coords=1, encounters=0)
+        held.append(free - torch.cuda.mem_get_info()[0])
+        if k > pairs:
+            E = sim.energy()
+        sim.close()
+    for s in [0, 1, 777, pairs - 1, pairs, pairs + 1, pairs + 100]:
+        ref, mag = _energy_ref(w, int(w.offsets[s]), int(w.offsets[s + 1]))
+        assert abs(E[s] - ref) <= (n[s] + 8) * np.longdouble(2.0) ** -53 * mag, s
+    assert held[0] - held[1] < (12 << 20), held
