@@ -959,7 +959,7 @@ static cudaError_t enqueue_step(qym_ctx *c, double tau, bool last, bool fresh = 
         return e;
     // kick [+ chunk re-test], finish, Kepler, [refine, sets, Hermite plan, Hermite], pack, kick,
     // finish, momentum [1 or 2], drift
-    c->launches += 7 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d.rows) : 0) + search_retest(p, fz);
+    c->launches += 7 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d) : 0) + search_retest(p, fz);
     return cudaGetLastError();
 }
 
@@ -1027,7 +1027,7 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
             return e;
         // Kepler, [refine, sets, Hermite plan, Hermite], copy, momentum [1 or 2], drift, kick
         // [+ chunk re-test], finish
-        c->launches += 5 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d.rows) : 0) + search_retest(p, fz);
+        c->launches += 5 + momentum_launches(d, true) + (c->binned ? 1 : 0) + (enc ? 2 + sets_launches(d) : 0) + search_retest(p, fz);
     } else {
         if ((e = launch_kick_tiles(d, p.kick_prec, 0, p.G, c->tune.threads, c->tune.ipt, st))) return e;
         if ((e = launch_kick_finish_v(d, d.v, d.q, 0.5 * tau, p.G, 0, p.hill_fixed, st))) return e;
@@ -1036,7 +1036,7 @@ static cudaError_t enqueue_unit(qym_ctx *c, double tau, bool last) {
                                         p.hill_fixed, st, 0.5 * tau, 1.01, 1, 1)))
             return e;
         // Kepler, [refine, sets, Hermite plan, Hermite], copy, kick, finish, momentum [1 or 2], drift
-        c->launches += 5 + momentum_launches(d, true) + (enc ? 2 + sets_launches(d.rows) : 0);
+        c->launches += 5 + momentum_launches(d, true) + (enc ? 2 + sets_launches(d) : 0);
     }
     return cudaGetLastError();
 }
@@ -1464,7 +1464,7 @@ extern "C" qym_status qym_split_phase(qym_ctx *c, int32_t phase, double tau, int
     case QYM_PHASE_REFINE: {
         if (enc) {
             CK(c, launch_refine(d, tau, p.a_E, st));
-            c->launches += 2;
+            c->launches += 1;
         }
         break;
     }
@@ -1474,7 +1474,8 @@ extern "C" qym_status qym_split_phase(qym_ctx *c, int32_t phase, double tau, int
             CK(c, launch_hermite(d, p, tau, st));
             k_owned_members<<<1, 1, 0, st>>>(d, c->owned_info);
             CK(c, cudaGetLastError());
-            c->launches += 12;
+            // sets [and plan], Hermite, the union-find's reset, the owned members
+            c->launches += sets_launches(d) + 3;
         }
         break;
     }

@@ -429,12 +429,12 @@ __global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a
     hermite_plan(d, ncl);
 }
 
-bool sets_one(int64_t rows) { return rows <= kSetsOneRows; }
-int sets_launches(int64_t rows) { return sets_one(rows) ? 1 : 8; }
+bool sets_one(const Dev &d) { return d.rows <= kSetsOneRows; }
+int sets_launches(const Dev &d) { return sets_one(d) ? 1 : 8; }
 
 cudaError_t launch_sets_impl(const Dev &d, const qym_params &p, const SetScratch &s, cudaStream_t st) {
     const double a_H = p.a_H;
-    if (sets_one(d.rows))
+    if (sets_one(d))
         return launch_chain(k_sets_one, 1, 1024, 0, st, d, s, a_H, hermite_clusters(d, p));
     int nblk = (int)((d.rows + 1023) / 1024);
     launch_chain(k_uf_hook, 152, 256, 0, st, d);

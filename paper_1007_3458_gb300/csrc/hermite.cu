@@ -1566,7 +1566,7 @@ cudaError_t launch_hermite(const Dev &d, const qym_params &p, double tau, cudaSt
     const int cls = hermite_cluster_size(d, p);
     const int grid = kHermGrid;
     cudaError_t e;
-    if (!sets_one(d.rows)) {  // (else at the end of the set builder)
+    if (!sets_one(d)) {  // (else at the end of the set builder)
         launch_chain(k_hermite_plan, 1, 1024, 0, st, d, hermite_clusters(d, p));
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -483,8 +483,8 @@ struct SetScratch {
 };
 cudaError_t launch_refine(const Dev &d, double tau, double a_E, cudaStream_t st);
 cudaError_t launch_sets_impl(const Dev &d, const qym_params &p, const SetScratch &s, cudaStream_t st);
-bool sets_one(int64_t rows);      // whether one CTA builds the sets and plans the Hermite
-int sets_launches(int64_t rows);  // kernels from the sets to the Hermite's plan
+bool sets_one(const Dev &d);      // whether one CTA builds the sets and plans the Hermite
+int sets_launches(const Dev &d);  // kernels from the sets to the Hermite's plan
 int hermite_clusters(const Dev &d, const qym_params &p);
 cudaError_t launch_pair_test(int64_t rows, const double *q0, const double *v0, const double *q1,
                              const double *v1, const double *rH, double tau, double a_E,

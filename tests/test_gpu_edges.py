@@ -562,3 +562,30 @@ def test_energy_unbalanced_batch(torch):
         ref, mag = _energy_ref(w, int(w.offsets[s]), int(w.offsets[s + 1]))
         assert abs(E[s] - ref) <= (n[s] + 8) * np.longdouble(2.0) ** -53 * mag, s
     assert held[0] - held[1] < (12 << 20), held
+
+
+@pytest.mark.parametrize("n", [1000, 9000])
+def test_split_launch_count(torch, n):
+    """qym_stats.launches of a split step: the library's kernels that the
+    profiler sees, with the set builder in one kernel and in seven (FP64 kick: no
+    tile preparation, which no count includes)."""
+    from torch.profiler import ProfilerActivity, profile
+    from paper_1007_3458_gb300 import split as SP
+    from test_gpu_split import LocalComm
+    w = W.outer_disk(n - 5, 1e-9, seed=n)
+    sim = q.Simulation(w.m, w.q, w.v, w.offsets, eps_H=w.eps_H, kick_prec=q.QYM_KICK_FP64)
+    run = SP.SplitRun(SP.GpuEngine(sim, 0, 1), LocalComm())
+    run.step(w.tau, 1)
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]):  # (the first session of a process may record nothing)
+        torch.zeros(8, device="cuda").add_(1)
+        torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        run.step(w.tau, 3)
+        torch.cuda.synchronize()
+    seen = [e.name for e in prof.events() if e.name.replace("void ", "").startswith(("qym::", "k_"))]
+    launches = sim.stats()["launches"]
+    sim.close()
+    if not seen:
+        pytest.skip("no kernel records from the profiler")
+    assert launches == len(seen), (launches, len(seen))
