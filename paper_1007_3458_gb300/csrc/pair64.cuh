@@ -387,7 +387,7 @@ __device__ __forceinline__ float norm_up(double x, double y, double z) {
     const int k = (hm >> 20) - 1023;
     const float a = lead(x, k), b = lead(y, k), c = lead(z, k);
     const float n = sqrtf(fmaf(a, a, fmaf(b, b, c * c))) * (1.0f + 0x1p-21f);
-    if (k > 125) return INFINITY;
+    if (k > 127) return INFINITY;
     return k < -125 ? n * 0x1p-125f : n * __int_as_float((127 + k) << 23);
 }
 

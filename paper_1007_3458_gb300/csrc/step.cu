@@ -109,7 +109,7 @@ struct DriftArgs {
 // 2 rho^2: kernels test r^2 < c_i + c_j with c = 2 rho^2 >= ... a superset of
 // r < rho_i + rho_j, as (rho_i + rho_j)^2 <= 2 rho_i^2 + 2 rho_j^2; the factor
 // covers the FP32 rounding of r^2 (a few 1e-7 relative, also in the kick's
-// far-tile form). Out of line: only the escape mode and positions outside
+// far-tile form). Out of line: only the escape mode and quantities outside
 // FP32's range come here.
 __device__ __noinline__ float crude_reach_fp64(const Dev &d, const DriftArgs &a, int64_t r, double m0,
                                                double qx, double qy, double qz, double vx, double vy,
@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(256) k_drift_pack(Dev d, DriftArgs a) {
         if (!d.escape_reach && r2 > 1e-24f && r2 < 1e24f)
             reach = crude_reach(d, a, r, sys, xh, yh, zh, r2, p64::lead(vx, 0), p64::lead(vy, 0),
                                 p64::lead(vz, 0));
-        else
+        // (FP64 also where some quantity of the FP32 form may have left its range)
+        if (!(reach > 1e-30f && reach < 1e30f))
             reach = crude_reach_fp64(d, a, r, d.m[star], qx, qy, qz, vx, vy, vz);
     }
     // heavy bodies enter the FP32 tiles with zero mass (their pull is added

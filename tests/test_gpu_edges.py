@@ -589,3 +589,26 @@ def test_split_launch_count(torch, n):
     if not seen:
         pytest.skip("no kernel records from the profiler")
     assert launches == len(seen), (launches, len(seen))
+
+
+@pytest.mark.parametrize("lu,mu", [(1e6, 1e40), (1e9, 1e40), (1e-9, 1e-40), (1e-8, 1e24), (1.5e13, 1.3e26)])
+@pytest.mark.parametrize("prec", [q.QYM_KICK_FP64, q.QYM_KICK_MIXED])
+def test_crude_reach_units(torch, lu, mu, prec):
+    """A step's encounters in units where the star's G m (1e40, 1e-40) or its
+    quotient by r^3 leaves FP32's range, or pulls come near its end, and in cgs:
+    those of the disk's own units."""
+    n = 2000
+    if prec == q.QYM_KICK_MIXED and mu in (1e24, 1e-40):
+        pytest.skip("pulls or weights of the bodies outside FP32's range")
+    w = W.outer_disk(n - 4, 1e-9, seed=5, a_lo=9.0, a_hi=14.0)
+    rec = []
+    for a, b in ((1.0, 1.0), (lu, mu)):
+        t = np.sqrt(a ** 3 / b)
+        sim = q.Simulation(w.m * b, w.q * a, w.v * (a / t), w.offsets, eps_H=w.eps_H * a, kick_prec=prec)
+        for k in range(2):  # (the first step's search follows its kick, later ones are part of it)
+            sim.set_state(w.q * a, w.v * (a / t)) if k else None
+            sim.step(w.tau * t, 1)
+            assert sim.stats()["status_bits"] == 0
+            rec.append(sim.encounters())
+        sim.close()
+    assert len(rec[0]) > 0 and all(np.array_equal(rec[0], r) for r in rec[1:])
