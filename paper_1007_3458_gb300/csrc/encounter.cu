@@ -429,7 +429,10 @@ __global__ void __launch_bounds__(1024) k_sets_one(Dev d, SetScratch s, double a
     hermite_plan(d, ncl);
 }
 
-bool sets_one(const Dev &d) { return d.rows <= kSetsOneRows; }
+// A batch can have a pair for nearly every row (swarms about its planets), and one CTA
+// takes them in more rounds then: 1980 rows 240 us a step either way, 4320 rows 409
+// against 394 in the seven kernels, 6600 rows 309 against 287.
+bool sets_one(const Dev &d) { return d.rows <= (d.nsys == 1 ? kSetsOneRows : 2048); }
 int sets_launches(const Dev &d) { return sets_one(d) ? 1 : 8; }
 
 cudaError_t launch_sets_impl(const Dev &d, const qym_params &p, const SetScratch &s, cudaStream_t st) {
