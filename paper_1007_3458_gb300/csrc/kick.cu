@@ -353,7 +353,10 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         nyl[k] = make_float2(-l.y, -l.y); nzl[k] = make_float2(-l.z, -l.z);
         ahx[k] = ahy[k] = ahz[k] = alx[k] = aly[k] = alz[k] = 0.0f;
     }
-    bool i_in = a.uniform;  // this thread's rows let a window take the form without G m
+    // whether this thread's rows let a window take the form without G m (one and two
+    // rows a thread; four have no registers for both forms)
+    constexpr bool HAS_UNI = FORCE && IPT <= 2;
+    bool i_in = HAS_UNI && a.uniform;
 #pragma unroll
     for (int k = 0; k < IPT; ++k) i_in = i_in && (gi[k] >= it.y || uni_range(make_float4(nxh[k].x, nyh[k].x, nzh[k].x, 0.0f)));
     const int i_lo = it.x, i_hi = it.x + (int)(IPT * blockDim.x);
@@ -408,7 +411,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
         const bool any_near = __syncthreads_or(!far);
         // one G m for the whole window (and not zero, so that the pad and a
         // massless body are never taken for it)
-        const float gm0 = FORCE ? a.pos[jt].w : 0.0f;
+        const float gm0 = HAS_UNI ? a.pos[jt].w : 0.0f;
         bool same = i_in && j_in && gm0 > 0.0f;
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
             const int j0 = jt + 2 * t;
@@ -441,7 +444,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                 if (FLAG && !any_near) s_d[t] = make_float4(0.f, 0.f, -a.lo[j0].w, -c1);
             }
         }
-        const bool uni = FORCE ? __syncthreads_and(same) : (__syncthreads(), false);
+        const bool uni = HAS_UNI ? __syncthreads_and(same) : (__syncthreads(), false);
         if (far) {
             // d_i = c - Q_i = (c - x_hi) - x_lo rounded once, duplicated for
             // the packed form
@@ -482,11 +485,11 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     fx[k] = fy[k] = fz[k] = make_float2(0.0f, 0.0f);
                     mind[k] = 3.0e38f;
                 }
-                if (!FORCE || gw == 1.0f) {
+                if (!HAS_UNI || gw == 1.0f) {
                     run(std::false_type{});
                     break;
                 }
-                run(std::integral_constant<bool, FORCE>{});
+                run(std::integral_constant<bool, HAS_UNI>{});
                 if (finite_sums(fx, fy, fz)) break;
                 gw = 1.0f;
             }
@@ -1127,27 +1130,36 @@ KickTune default_kick_tune(int64_t iblocks_nb, int64_t nbmax, int prec, int64_t 
     return t;
 }
 
-template <bool FLAG, bool FORCE>
-static cudaError_t launch_mixed(const KickArgs &a, int nitems, int threads, int ipt,
-                                cudaStream_t st) {
-    switch (ipt) {
-    case 1: launch_chain(k_kick_mixed<1, FLAG, FORCE>, nitems, threads, 0, st, a); break;
-    case 2: launch_chain(k_kick_mixed<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
-    case 4: launch_chain(k_kick_mixed<4, FLAG, FORCE>, nitems, threads, 0, st, a); break;
-    default: return cudaErrorInvalidValue;
-    }
+// One-sided kicks: chained where a CTA's walk is short (the launch counts), a plain
+// launch from 2^18 pairs a CTA (some 20 us): chained CTAs settle on the SMs beside the
+// kernel before, two and three to some of them, and with few long CTAs that stays the
+// kick's length. 16384 bodies: 128 threads x 4 rows in 4 ranges 0.254 ms, chained
+// 0.363; 256 x 2 in 4 0.199 and 0.326; 3000 bodies, 128 x 2 in 8: 18.9 and 16.5 us.
+constexpr int64_t kPlainPairs = 1 << 18;
+template <class... P>
+static cudaError_t launch_kick(void (*kernel)(P...), int nitems, int threads, int ipt, int64_t nj,
+                               cudaStream_t st, const KickArgs &a) {
+    if (nj * threads * ipt < kPlainPairs) return launch_chain(kernel, nitems, threads, 0, st, a);
+    kernel<<<nitems, threads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 template <bool FLAG, bool FORCE>
-static cudaError_t launch_f64(const KickArgs &a, int nitems, int threads, int ipt,
-                              cudaStream_t st) {
+static cudaError_t launch_mixed(const KickArgs &a, int nitems, int threads, int ipt, int64_t nj,
+                                cudaStream_t st) {
     switch (ipt) {
-    case 1: launch_chain(k_kick_fp64<1, FLAG, FORCE>, nitems, threads, 0, st, a); break;
-    case 2: launch_chain(k_kick_fp64<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
-    default: launch_chain(k_kick_fp64<2, FLAG, FORCE>, nitems, threads, 0, st, a); break;
+    case 1: return launch_kick(k_kick_mixed<1, FLAG, FORCE>, nitems, threads, ipt, nj, st, a);
+    case 2: return launch_kick(k_kick_mixed<2, FLAG, FORCE>, nitems, threads, ipt, nj, st, a);
+    case 4: return launch_kick(k_kick_mixed<4, FLAG, FORCE>, nitems, threads, ipt, nj, st, a);
+    default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+}
+
+template <bool FLAG, bool FORCE>
+static cudaError_t launch_f64(const KickArgs &a, int nitems, int threads, int ipt, int64_t nj,
+                              cudaStream_t st) {
+    return ipt == 1 ? launch_kick(k_kick_fp64<1, FLAG, FORCE>, nitems, threads, ipt, nj, st, a)
+                    : launch_kick(k_kick_fp64<2, FLAG, FORCE>, nitems, threads, ipt, nj, st, a);
 }
 
 // Per tile of TILE consecutive positions (from position 1; the bodies in
@@ -1246,6 +1258,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     }
     if (flag != KICK_FORCE && flag != KICK_SEARCH && flag != KICK_SEARCH_ONLY)
         return cudaErrorInvalidValue;
+    const int64_t nj = d.rows / std::max(1, d.nsys) / d.splits;  // j rows of a CTA, about
     if (prec == QYM_KICK_MIXED) {
         const bool sym = d.sym.G > 0;
         if (sym) {
@@ -1254,12 +1267,12 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
         }
         if (flag == KICK_FORCE)
             return sym ? launch_sym<false, true>(a, d.sym_nitems, st)
-                       : launch_mixed<false, true>(a, d.nitems, threads, ipt, st);
+                       : launch_mixed<false, true>(a, d.nitems, threads, ipt, nj, st);
         cudaError_t e = flag == KICK_SEARCH
                             ? (sym ? launch_sym<true, true>(a, d.sym_nitems, st)
-                                   : launch_mixed<true, true>(a, d.nitems, threads, ipt, st))
+                                   : launch_mixed<true, true>(a, d.nitems, threads, ipt, nj, st))
                             : (sym ? launch_sym<true, false>(a, d.sym_nitems, st)
-                                   : launch_mixed<true, false>(a, d.nitems, threads, ipt, st));
+                                   : launch_mixed<true, false>(a, d.nitems, threads, ipt, nj, st));
         if (e) return e;
         // about one entry per row (its own chunk) plus the close pairs
         int64_t blocks = (d.rows + 63) / 64;
@@ -1268,9 +1281,9 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
         launch_chain(k_flag_chunks, (int)blocks, 256, 0, st, a, d.ctr + C_FCDONE);
         return cudaGetLastError();
     }
-    if (flag == KICK_FORCE) return launch_f64<false, true>(a, d.nitems, threads, ipt, st);
-    return flag == KICK_SEARCH ? launch_f64<true, true>(a, d.nitems, threads, ipt, st)
-                               : launch_f64<true, false>(a, d.nitems, threads, ipt, st);
+    if (flag == KICK_FORCE) return launch_f64<false, true>(a, d.nitems, threads, ipt, nj, st);
+    return flag == KICK_SEARCH ? launch_f64<true, true>(a, d.nitems, threads, ipt, nj, st)
+                               : launch_f64<true, false>(a, d.nitems, threads, ipt, nj, st);
 }
 
 // ---------------------------------------------------------------- single system
@@ -1455,7 +1468,7 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
         KickArgs ka{};
         ka.q = q; ka.m = m; ka.G = G; ka.apart = d.apart; ka.rows = rows;
         ka.splits = d.splits; ka.chunk = d.item_chunk;
-        e = launch_f64<false, true>(ka, L.nitems, L.tune.threads, L.tune.ipt, st);
+        e = launch_f64<false, true>(ka, L.nitems, L.tune.threads, L.tune.ipt, L.chunk, st);
     }
     if (e != cudaSuccess) return e;
     launch_chain(k_sum_partials, (unsigned)((rows + 256 / SL - 1) / (256 / SL)), 256, 0, st, rows, d.splits, d.apart, hl, m,
