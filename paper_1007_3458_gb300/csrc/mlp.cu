@@ -432,8 +432,12 @@ size_t mlp_workspace_bytes() { return (size_t)MAXBLK * NW * sizeof(float) + MAXB
 
 cudaError_t launch_mlp_forward(int64_t n, const float *w, const float *u, float *y, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const int64_t blocks = (n + 255) / 256;
-    launch_chain(k_mlp_forward, (unsigned)blocks, 256, 0, st, n, w, u, y);
+    // chained up to a CTA per SM; a plain launch above, where the next call's CTAs
+    // would settle on the SMs while this one's still run, two and three to some of
+    // them (65536 rows: 28 us, chained 31; 4096 rows: 24 us, chained 22)
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (blocks <= 152) return launch_chain(k_mlp_forward, blocks, 256, 0, st, n, w, u, y);
+    k_mlp_forward<<<blocks, 256, 0, st>>>(n, w, u, y);
     return cudaGetLastError();
 }
 
