@@ -295,13 +295,15 @@ struct FinishArgs {
 // slots q, q + L, ... (loads coalesced across positions, dependent FP64 adds in
 // chains 1/L as long), the groups' parts added as a fixed tree; the first group then
 // does the rows' own work in full warps. The heavy bodies' pulls are spread over the
-// groups as well, or with few slots follow the sums one after another. (An FP64 instruction costs the same for one active lane as
+// groups as well, or in a batch follow the sums one after another. (An FP64
+// instruction costs the same for one active lane as
 // for 32: with the four parts on neighbouring lanes the row work ran on eight
 // lanes per warp, 492 us on 1.06e6 rows.)
 template <int L>
 __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
     chain_wait();
     constexpr int RB = 256 / L;
+    const bool late = L <= 4 && d.batch;  // the heavy bodies' pulls follow the sums
     const int t = threadIdx.x % RB, q = threadIdx.x / RB;
     const int64_t pr = (int64_t)blockIdx.x * RB + t;
     const int64_t R = d.rows;
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
                 az += p[2 * R + pr];
             }
         }
-        if (L > 4 && d.heavy_split) {
+        if (d.heavy_split && !late) {
             const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
             heavy_pull(d.heavy_rows + h0, q, L, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q,
                        d.m, R, a.G, ax, ay, az);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(256) k_finish(Dev d, FinishArgs a) {
         ax = p[0][0]; ay = p[0][1]; az = p[0][2];
     }
     if (!live) return;
-    if (L <= 4 && d.heavy_split) {
+    if (d.heavy_split && late) {
         const int h0 = d.heavy_start[sys], h1 = d.heavy_start[sys + 1];
         heavy_pull_fp64(d.heavy_rows + h0, h1 - h0, r, a.q[r], a.q[R + r], a.q[2 * R + r], a.q, d.m, R,
                         a.G, ax, ay, az);
