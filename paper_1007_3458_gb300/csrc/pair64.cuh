@@ -321,7 +321,8 @@ __device__ __forceinline__ double to_double(float x) {
 // residual of a multiply-add the rounded value (Markstein 1990): 1/x, a/b, sqrt(x)
 // and 1/sqrt(x)'s rounded root are what the library's correctly rounded forms return,
 // for five to nine FP64 instructions where those take ten and more. Outside the
-// exponents [-1000, 1000] (quotient: [-500, 500]) the library forms.
+// exponents [-1000, 1000] (quotient and root, whose residuals are the operands'
+// size: [-500, 500]) the library forms.
 __device__ __forceinline__ bool mid_range(double x) {
     const int hi = __double2hiint(x);
     return hi > (23 << 20) && hi < (2023 << 20);
@@ -358,7 +359,7 @@ __device__ __forceinline__ double rsqrt_mid(double x) {
 __device__ __forceinline__ double rsqrt64(double x) { return mid_range(x) ? rsqrt_mid(x) : rsqrt(x); }
 // square root and the reciprocal of that rounded root
 __device__ __forceinline__ double sqrt_rcp(double x, double &ir) {
-    if (!mid_range(x)) {
+    if (!mid_range(x) || !near_one(x)) {
         const double r = sqrt(x);
         ir = 1.0 / r;
         return r;
@@ -366,6 +367,8 @@ __device__ __forceinline__ double sqrt_rcp(double x, double &ir) {
     const double y = rsqrt_mid(x), s = x * y;
     const double r = fma(mul_pow2(y, -1), fma(-s, s, x), s);
     ir = fma(y, fma(-r, y, 1.0), y);
+    // (the one mantissa that the step can miss: all ones)
+    if (__double2loint(r) == -1 && (__double2hiint(r) & 0xfffff) == 0xfffff) ir = 1.0 / r;
     return r;
 }
 
