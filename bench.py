@@ -157,8 +157,8 @@ class ClockSampler:
 # particles (ncu sm__inst_executed_pipe_fp64.sum), per (solver, guess, source
 # digest of kepler.cu + mlp.cuh)
 KEPLER_FP64_WARP_INST = {
-    ("newton32", "standard", "aad84024ce025248"): 7296855,
-    ("newton", "standard", "aad84024ce025248"): 12321900,
+    ("newton32", "standard", "63c5031f74eabaed"): 7691697,
+    ("newton", "standard", "63c5031f74eabaed"): 13124208,
 }
 
 # DRAM bytes (read + written) per launch of the mixed kick, from one ncu
@@ -169,8 +169,8 @@ KEPLER_FP64_WARP_INST = {
 # with the splits. A shape or a kick source not captured reports null (the
 # capture commands sit with the ncu summaries under profiles/).
 KICK_DRAM_BYTES = {
-    ("disk_16384", 512, 160, "ef3860c9a9503734"): 8.59e5,
-    ("disk_262144", 512, 128, "ef3860c9a9503734"): 6.90e8,
+    ("disk_16384", 512, 160, "ea93f9fec5721a94"): 8.60e5,
+    ("disk_262144", 512, 128, "ea93f9fec5721a94"): 6.91e8,
 }
 
 

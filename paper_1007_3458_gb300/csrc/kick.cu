@@ -539,7 +539,8 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
 // the warp's 128 rows: added per step as sums of four, 32 in a row, as the i side
 // adds its own. The warps' sums are added as two floats (hi, lo) and converted once:
 // added in FP64 they took 54 FP64 instructions per 64 x 512 pairs, a quarter of the
-// FMA pipe's time for them (16384 bodies 0.0988 -> 0.0970 ms, 262144 20.15 -> 19.98).
+// FMA pipe's time for them (16384 bodies 0.0988 -> 0.0970 ms, 262144 20.15 -> 19.98;
+// with the checks of r^-3's range 0.098 and 20.1).
 //
 // Work unit: G consecutive i-blocks against a range of rh half tiles (the part
 // past each block). Rows get one slot of partial sums per range from their own
@@ -932,7 +933,7 @@ __device__ __noinline__ double weight_fp64(double dx, double dy, double dz, doub
 // accuracy on the FP32 pipes (pair64.cuh, about 400 issue slots); beside them the
 // FP64 pipe, one warp instruction per ~19 cycles and SM, forms the separation
 // again and sums the pair's acceleration, six instructions where the plain form
-// has 22: 10240 bodies take 1.26 ms, 112 cycles of an SM per warp of pairs, both
+// has 22: 10240 bodies take 1.20 ms, 107 cycles of an SM per warp of pairs, both
 // pipes full (4.08 ms before; assembling the separation's doubles from the floats
 // instead of three FP64 subtractions, 1.34 ms). Rows and partners are split into
 // three floats once per CTA and tile, scaled by powers of two; pairs outside the
