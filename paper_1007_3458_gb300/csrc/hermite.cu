@@ -1534,12 +1534,12 @@ cudaError_t hermite_prepare() {
 
 // Cluster size for a batch (qym_params.hermite_cluster; 0 = automatic). One
 // system holds a few sets, and its longest set gains most from spreading its
-// partners over eight SMs (16384-body disk: 1.38 ms per step against 1.48 ms on
+// partners over eight SMs (16384-body disk: 0.96 ms per step against 1.08 ms on
 // two). A batch of many systems keeps thousands of sets in flight, and a set on
-// eight CTAs keeps seven from the queue: two (512-system ensemble: 16.5 ms per
-// step against 16.9-17.2 ms with eight). Either way two CTAs per SM: a CTA's chain
+// eight CTAs keeps seven from the queue: two (512-system ensemble: 17.4 ms per
+// step against 18.4 ms with eight). Either way two CTAs per SM: a CTA's chain
 // keeps its SM's FP64 units busy a third of the time (the ensemble with one per
-// SM: 17.4 ms).
+// SM: 18.4 ms).
 int hermite_cluster_size(const Dev &d, const qym_params &p) {
     if (p.hermite_cluster == 2 || p.hermite_cluster == 4 || p.hermite_cluster == 8)
         return p.hermite_cluster;
