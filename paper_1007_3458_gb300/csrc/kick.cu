@@ -203,16 +203,13 @@ constexpr float kUniMax = 0x1p40f;  // r < 2^42, r^-3 > 2^-126
 __device__ __forceinline__ bool uni_range(const float4 &p) {
     return fmaxf(fabsf(p.x), fmaxf(fabsf(p.y), fabsf(p.z))) < kUniMax;
 }
-// whether the sums of a thread's rows are finite
+// whether the sums of a thread's rows are finite: one component tells, as an infinite
+// r^-3 makes all three infinite or NaN (also times a zero difference)
 template <int N>
-__device__ __forceinline__ bool finite_sums(const float2 (&x)[N], const float2 (&y)[N], const float2 (&z)[N]) {
+__device__ __forceinline__ bool finite_sums(const float2 (&x)[N]) {
     float2 m = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int k = 0; k < N; ++k) m = __ffma2_rn(x[k], make_float2(0.0f, 0.0f), m);
-#pragma unroll
-    for (int k = 0; k < N; ++k) m = __ffma2_rn(y[k], make_float2(0.0f, 0.0f), m);
-#pragma unroll
-    for (int k = 0; k < N; ++k) m = __ffma2_rn(z[k], make_float2(0.0f, 0.0f), m);
     return m.x + m.y == 0.0f;  // (0 times infinity is NaN)
 }
 template <int IPT, bool FLAG, bool DIAG, bool FORCE, bool UNI>
@@ -490,7 +487,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
                     break;
                 }
                 run(std::integral_constant<bool, HAS_UNI>{});
-                if (finite_sums(fx, fy, fz)) break;
+                if (finite_sums(fx)) break;
                 gw = 1.0f;
             }
 #pragma unroll
@@ -540,7 +537,7 @@ __global__ void __launch_bounds__(256) k_kick_mixed(KickArgs a) {
 // adds its own. The warps' sums are added as two floats (hi, lo) and converted once:
 // added in FP64 they took 54 FP64 instructions per 64 x 512 pairs, a quarter of the
 // FMA pipe's time for them (16384 bodies 0.0988 -> 0.0970 ms, 262144 20.15 -> 19.98;
-// with the checks of r^-3's range 0.098 and 20.1).
+// with the checks of r^-3's range 0.0972 and 20.16).
 //
 // Work unit: G consecutive i-blocks against a range of rh half tiles (the part
 // past each block). Rows get one slot of partial sums per range from their own
@@ -769,7 +766,7 @@ __global__ void __launch_bounds__(SYM_T, 4) k_kick_sym(KickArgs a) {
                     } else {
                         run(T0{}, T0{}, T1{});
                     }
-                    if (!FORCE || !u || __all_sync(0xffffffffu, finite_sums(fx, fy, fz))) break;
+                    if (!FORCE || !u || __all_sync(0xffffffffu, finite_sums(fx))) break;
                     u = false;
                 }
                 if (FORCE && !diag) {
