@@ -169,8 +169,8 @@ KEPLER_FP64_WARP_INST = {
 # with the splits. A shape or a kick source not captured reports null (the
 # capture commands sit with the ncu summaries under profiles/).
 KICK_DRAM_BYTES = {
-    ("disk_16384", 512, 160, "1791546550912ebd"): 8.60e5,
-    ("disk_262144", 512, 128, "1791546550912ebd"): 6.86e8,
+    ("disk_16384", 512, 160, "9540600f9292031f"): 8.60e5,
+    ("disk_262144", 512, 128, "9540600f9292031f"): 6.86e8,
 }
 
 

@@ -36,6 +36,7 @@ struct KickArgs {
     const int4 *items;      // NULL: one system of `rows` rows, items by kick_item
     const int32_t *slots;
     int32_t chunk = 0;      // j rows per split (items == NULL)
+    int32_t parts = 1;      // splits per chunk, of FOLD rows each (items == NULL; 1: whole chunks)
     const float4 *pos;      // (x_hi, y_hi, z_hi, G m)
     const float4 *lo;       // (x_lo, y_lo, z_lo, c = 2 rho^2 of the crude reach rho)
     const double *q;        // [3][rows] (FP64 path)
@@ -61,7 +62,8 @@ struct KickArgs {
 };
 
 // The item of CTA b: its rows [x, y), its j-range [z, w) and its slot; for one
-// system (items == NULL) i-blocks of `ti` rows times `splits` ranges of `chunk`
+// system (items == NULL) i-blocks of `ti` rows times `splits` ranges of `chunk`, or
+// of the `parts` parts of FOLD rows of each
 __device__ __forceinline__ int4 kick_item(const KickArgs &a, int ti, int &slot) {
     if (a.items) {
         slot = a.slots[blockIdx.x];
@@ -69,9 +71,10 @@ __device__ __forceinline__ int4 kick_item(const KickArgs &a, int ti, int &slot) 
     }
     const int64_t ib = blockIdx.x / a.splits;
     slot = (int)(blockIdx.x - ib * a.splits);
-    const int64_t i0 = 1 + ib * ti, j0 = 1 + (int64_t)slot * a.chunk;
-    return make_int4((int)i0, (int)min(i0 + ti, a.rows), (int)min(j0, a.rows),
-                     (int)min(j0 + a.chunk, a.rows));
+    const int64_t i0 = 1 + ib * ti, c = slot / a.parts;
+    const int64_t j0 = 1 + c * a.chunk + (slot - c * a.parts) * FOLD;
+    const int64_t j1 = a.parts == 1 ? j0 + a.chunk : min(j0 + FOLD, 1 + (c + 1) * a.chunk);
+    return make_int4((int)i0, (int)min(i0 + ti, a.rows), (int)min(j0, a.rows), (int)min(j1, a.rows));
 }
 
 // The last CTA of an i-block to finish (arrivals counted per i-block, the
@@ -1247,6 +1250,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
     a.blk_cnt = d.kick_cnt;
     a.splits = d.splits;
     a.chunk = d.item_chunk;
+    a.parts = d.item_parts;
     a.uniform = !d.batch;
     if (a.far_tiles && !d.tiles_ready) {
         const int64_t ntiles = (d.rows - 1 + TILE - 1) / TILE;
@@ -1288,7 +1292,7 @@ cudaError_t launch_kick_tiles(const Dev &d, int prec, int flag, double G, int th
 // Workspace for qym_accel_dev: packs + items + partials for one system.
 struct SingleLayout {
     size_t off_pos, off_lo, off_apart, off_heavy, total;
-    int32_t nitems, chunk;
+    int32_t nitems, chunk, parts;
     KickTune tune;
     bool sorted;   // bodies held in Morton order (mixed kick, >= kSortMinBodies bodies)
     size_t off_perm, off_inv, off_box, off_k0, off_k1, off_v0, off_v1, off_hist, off_far, off_tile;
@@ -1297,6 +1301,14 @@ struct SingleLayout {
 // bodies from which a system's mixed kick holds them in Morton order (sort.cu)
 constexpr int64_t kSingleSortMin = 2048;
 
+// An acceleration is dominated by its closest pair, so how a pair's pull is rounded and
+// which 64 bodies share an FP32 sum are part of a mixed call's result (1e-8 of it where
+// a close pair stands out). Pulls carry G m in each product (as a batch's do; windows of
+// one mass would give 16384 bodies 176 us instead of 184, 260 bodies 12.6 instead of
+// 13.5), and the ranges end where sums of FOLD bodies end: on tiles or their halves in
+// Morton order (4500 bodies 50.6 us in halves, 52.5 in tiles), else the system in equal
+// chunks of at most a tile, each in parts of FOLD rows (2040 bodies 18.3 us). Two rows a
+// thread in Morton order: a tile is near or far to a warp by all of its 64 rows.
 static SingleLayout single_layout(int64_t rows, int prec) {
     SingleLayout L;
     int64_t nb = rows - 1;
@@ -1304,13 +1316,20 @@ static SingleLayout single_layout(int64_t rows, int prec) {
     // row of packs, order and tiles; beyond its sizes, 16
     L.tune = default_kick_tune(nb, nb, prec, rows <= QYM_STATIC_MAX_ROWS ? (((8 << 20) - (1 << 17)) / rows - 60) / 24 : 16);
     KickTune &t = L.tune;
-    int64_t ti = (int64_t)t.threads * t.ipt;
     L.sorted = prec == QYM_KICK_MIXED && nb >= kSingleSortMin;
-    const int64_t align = L.sorted ? TILE : 1;
+    L.parts = 1;
+    if (L.sorted) t.ipt = 2;
+    int64_t ti = (int64_t)t.threads * t.ipt;
+    const int64_t align = L.sorted ? (nb > 6144 ? TILE : TILE / 2) : 1;
+    if (prec == QYM_KICK_MIXED && !L.sorted) t.splits = (int32_t)((nb + TILE - 1) / TILE);
     int64_t chunk = (nb + t.splits - 1) / t.splits;
-    chunk = (chunk + align - 1) / align * align;  // j-ranges start on tiles
+    chunk = (chunk + align - 1) / align * align;
     t.splits = (int32_t)((nb + chunk - 1) / chunk);
     L.chunk = (int32_t)chunk;
+    if (prec == QYM_KICK_MIXED && !L.sorted) {
+        L.parts = (int32_t)((chunk + FOLD - 1) / FOLD);
+        t.splits *= L.parts;
+    }
     L.nitems = (int32_t)((nb + ti - 1) / ti * t.splits);
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     size_t o = 0;
@@ -1435,6 +1454,8 @@ cudaError_t launch_accel_single(int64_t rows, const double *m, const double *q, 
     d.nitems = L.nitems;
     d.splits = L.tune.splits;
     d.item_chunk = L.chunk;
+    d.item_parts = L.parts;
+    d.batch = 1;
     // heavy split (mixed kick only): threshold relative to the star mass m[0],
     // read on the device
     int32_t *hl = prec == QYM_KICK_MIXED && heavy_mass > 0.0 ? (int32_t *)(w + L.off_heavy) : nullptr;

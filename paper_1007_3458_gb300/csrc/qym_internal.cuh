@@ -59,6 +59,7 @@ struct Dev {
     int32_t *item_slot = nullptr;
     int32_t nitems = 0;
     int32_t item_chunk = 0;       // items == NULL (one system): j rows per split
+    int32_t item_parts = 1;       // splits per chunk, of FOLD rows each (mixed kick; 1: whole)
     int32_t batch = 0;            // mixed kick of several systems: its sums keep their order
     // momentum reduction
     int4 *mchunks = nullptr;      // (row0, row1, sys, -) chunks of at most 1024 rows

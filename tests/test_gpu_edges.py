@@ -432,6 +432,42 @@ def test_batch_bits(torch, name, kind, encounters):
     _same_bits(vs, g[f"{name}_{kind}_v"])
 
 
+def _sums_case(n):
+    """Bodies in a flat box by exact arithmetic (the same on every machine), each
+    eighth beside its neighbour, of one mass (odd n) or several, four heavy ones;
+    and the rows whose accelerations are recorded."""
+    rng = np.random.default_rng(n)
+    x = (rng.random((n + 1, 3)) - 0.5) * np.array([2.0, 2.0, 0.125])
+    near = np.arange(8, n, 8)
+    x[near] = x[near + 1] + (rng.random((len(near), 3)) - 0.5) * 2.0 ** -9
+    m = np.full(n + 1, 1.3 * 2.0 ** -30) * (1.0 if n % 2 else 1.0 + 7.0 * rng.random(n + 1))
+    m[0], m[3:7] = 1.0, 2.0 ** -10
+    x[0] = 0.0
+    return m, x, np.unique(np.concatenate([near[:: max(1, len(near) // 64)], np.arange(1, n + 1, max(1, n // 64))]))
+
+
+SUMS = [65, 110, 259, 1023, 1493, 2047, 2048, 2443, 6145, 9001, 20490]
+
+
+@pytest.mark.parametrize("n", SUMS)
+def test_mixed_accel_sums(torch, n):
+    """Mixed accelerations against recorded ones: the same roundings of each pair's
+    pull and the same FP32 sums of 64 bodies, whatever the ranges of a launch. What
+    the ranges leave free are sums of at most 320 two-float parts (2^-48 each) and of
+    64 doubles: below 2^-39 of the terms' magnitudes, while another rounding of a
+    dominating pair is some 2^-24."""
+    import os
+    ref = np.load(os.path.join(os.path.dirname(__file__), "golden", "accel_sums.npz"))["a%d" % n]
+    m, x, rows = _sums_case(n)
+    md, xd = torch.from_numpy(m).cuda(), torch.from_numpy(np.ascontiguousarray(x.T)).cuda()
+    a = torch.empty((3, n + 1), dtype=torch.float64, device="cuda")
+    work = torch.empty(q.qym_accel_workspace_bytes(n + 1, q.QYM_KICK_MIXED), dtype=torch.uint8, device="cuda")
+    q.qym_accel_dev(n + 1, md, xd, a, 1.0, q.QYM_KICK_MIXED, work)
+    mag = _accel_ref64(torch, m, x)[1][rows]
+    err = np.abs(a.cpu().numpy().T[rows] - ref)
+    assert np.all(err <= 2.0 ** -39 * mag), float((err / mag).max())
+
+
 # lengths and masses in cgs, SI and parsecs, and around AU and solar masses (G folded
 # into the masses): r^-3 of a disk's pairs lies below, at the end of, above and inside
 # FP32's range
